@@ -415,40 +415,46 @@ __device__ __forceinline__ S pull_pad(const S* const* arr, const PullOffsets& o)
 // Whether a node sits next to a wall (then some of its outgoing values also
 // go to bounce-back ghost cells).  The periodic images of the ghost band are
 // written after each step by halo_kernel, not by the step kernels.
+template <int LAT>
+__device__ __forceinline__ bool wall_adjacent(const Geom& G, int x, int y, int z) {
+    return (G.wall[0] && (x == 0 || x == G.NX - 1)) ||
+           (Lattice<LAT>::kHasY && G.wall[1] && (y == 0 || y == G.NY - 1)) ||
+           (G.wall[2] && (z == 0 || z == G.NZ - 1));
+}
+
+// The bounce-back cells of a node next to a wall, once per node: the ends it
+// touches and the offsets of the cells around it.  The cell x + c_J that the
+// value of direction J goes to is the cell the node's own pull of opp(J)
+// reads (x - c_opp(J)): a ghost cell across a wall, wrapped along periodic axes.
 struct NodeWrites {
-    bool wall_adj;
+    bool lo[3], hi[3];
+    PullOffsets at;
 };
 
-template <int LAT>
 __device__ __forceinline__ NodeWrites node_writes(const Geom& G, int x, int y, int z) {
     NodeWrites w;
-    w.wall_adj = (G.wall[0] && (x == 0 || x == G.NX - 1)) ||
-                 (Lattice<LAT>::kHasY && G.wall[1] && (y == 0 || y == G.NY - 1)) ||
-                 (G.wall[2] && (z == 0 || z == G.NZ - 1));
+    w.lo[0] = G.wall[0] && x == 0;
+    w.hi[0] = G.wall[0] && x == G.NX - 1;
+    w.lo[1] = G.wall[1] && y == 0;
+    w.hi[1] = G.wall[1] && y == G.NY - 1;
+    w.lo[2] = G.wall[2] && z == 0;
+    w.hi[2] = G.wall[2] && z == G.NZ - 1;
+    w.at = pull_offsets(G, x, y, z);
     return w;
 }
 
-// Write the post-collision value v of direction J at node (x, y, z): its own
-// cell `own` and, if the grid has walls (WALLS) and x + c_J crosses one, the
-// bounce-back ghost cell of array opp(J).
+// Write the post-collision value v of direction J at a node: its own cell
+// `own` and, next to a wall (WALLS) that x + c_J crosses, the bounce-back
+// ghost cell of array opp(J).
 template <int LAT, int J, bool WALLS, typename S>
-__device__ __forceinline__ void write_dir(S* const* arr, const Geom& G, int x, int y, int z, int own,
-                                          const NodeWrites& nw, S v) {
+__device__ __forceinline__ void write_dir(S* const* arr, const Geom& G, int own, const NodeWrites& nw, S v) {
     using L = Lattice<LAT>;
     constexpr int CX = L::cx[J], CY = L::cy[J], CZ = L::cz[J];
     arr[J][checked_write(own, G.NP)] = v;
-    if constexpr (WALLS) {
-        if (nw.wall_adj) {
-            const int tx = x + CX, ty = y + CY, tz = z + CZ;
-            const bool wall_cross = (CX != 0 && G.wall[0] && (tx < 0 || tx >= G.NX)) ||
-                                    (CY != 0 && G.wall[1] && (ty < 0 || ty >= G.NY)) ||
-                                    (CZ != 0 && G.wall[2] && (tz < 0 || tz >= G.NZ));
-            // the ghost cell lies across a wall; along the periodic axes the
-            // pull wraps, so the cell does too
-            if (wall_cross)
-                arr[L::opp(J)][checked_write(pidx(G, wrap1(tx, G.NX, G.wall[0]), wrap1(ty, G.NY, G.wall[1]),
-                                                  wrap1(tz, G.NZ, G.wall[2])), G.NP)] = v;
-        }
+    if constexpr (WALLS && (CX != 0 || CY != 0 || CZ != 0)) {
+        const bool cross = (CX < 0 && nw.lo[0]) || (CX > 0 && nw.hi[0]) || (CY < 0 && nw.lo[1]) ||
+                           (CY > 0 && nw.hi[1]) || (CZ < 0 && nw.lo[2]) || (CZ > 0 && nw.hi[2]);
+        if (cross) arr[L::opp(J)][checked_write(nw.at.z[1 - CZ] + nw.at.r[1 - CY] + nw.at.c[1 - CX], G.NP)] = v;
     }
 }
 
@@ -891,7 +897,8 @@ __device__ __forceinline__ void collide_node(const DirPtrs<typename Storage<ST>:
     s.gz = gz * (R)3;
     s.lap = lap * (R)6;
     node_state<R, L::kHasY>(s, p, m.m0, m.mx, m.my, m.mz, m.mxx, m.myy, m.mzz, m.mxy, m.mxz, m.myz);
-    const NodeWrites nw = node_writes<LAT>(G, x, y, z);
+    NodeWrites nw;
+    if constexpr (WALLS) nw = node_writes(G, x, y, z);
     const int own = G.base + (z + G.GZ) * G.PXY + rb;
     // moving directions first; the rest population closes sum_i h*_i = phi
     // (Eq. 1 conserves phi at every node; closing it keeps FP32 rounding of
@@ -912,12 +919,12 @@ __device__ __forceinline__ void collide_node(const DirPtrs<typename Storage<ST>:
                 float2 hs, gs;
                 collide_pair<LAT, i, SH>(s, q, make_float2(hv(i), hv(o)), &hs, &gs);
                 hsum2 = add2(hsum2, hs);
-                write_dir<LAT, i, WALLS>(D.hout, G, x, y, z, own, nw, St::pack(hs.x));
-                write_dir<LAT, o, WALLS>(D.hout, G, x, y, z, own, nw, St::pack(hs.y));
-                write_dir<LAT, i, WALLS>(D.gout, G, x, y, z, own, nw, St::pack(gs.x));
-                write_dir<LAT, o, WALLS>(D.gout, G, x, y, z, own, nw, St::pack(gs.y));
+                write_dir<LAT, i, WALLS>(D.hout, G, own, nw, St::pack(hs.x));
+                write_dir<LAT, o, WALLS>(D.hout, G, own, nw, St::pack(hs.y));
+                write_dir<LAT, i, WALLS>(D.gout, G, own, nw, St::pack(gs.x));
+                write_dir<LAT, o, WALLS>(D.gout, G, own, nw, St::pack(gs.y));
                 if constexpr (WALLS) {
-                    if (p.moving && nw.wall_adj) {
+                    if (p.moving) {
                         // the wall term of g in the units of the stored g
                         const R srho = SH ? s.rho * p.g_scale : s.rho;
                         moving_wall_write<LAT, i>(D.hout, G, x, y, z, hs.x, s.phi, p, pk);
@@ -936,10 +943,10 @@ __device__ __forceinline__ void collide_node(const DirPtrs<typename Storage<ST>:
             R hs, gs;
             collide_dir<LAT, i, R>(s, p, hv(i), &hs, &gs);
             hsum += hs;
-            write_dir<LAT, i, WALLS>(D.hout, G, x, y, z, own, nw, St::store(hs, (R)W * p.h_shift, (R)1));
-            write_dir<LAT, i, WALLS>(D.gout, G, x, y, z, own, nw, St::store(gs, (R)W * p.g_shift, p.g_scale));
+            write_dir<LAT, i, WALLS>(D.hout, G, own, nw, St::store(hs, (R)W * p.h_shift, (R)1));
+            write_dir<LAT, i, WALLS>(D.gout, G, own, nw, St::store(gs, (R)W * p.g_shift, p.g_scale));
             if constexpr (WALLS) {
-                if (p.moving && nw.wall_adj) {
+                if (p.moving) {
                     moving_wall_write<LAT, i>(D.hout, G, x, y, z, hs, s.phi, p,
                                               [&](R v) { return St::store(v, (R)W * p.h_shift, (R)1); });
                     moving_wall_write<LAT, i>(D.gout, G, x, y, z, gs, s.rho, p,
@@ -956,10 +963,10 @@ __device__ __forceinline__ void collide_node(const DirPtrs<typename Storage<ST>:
         // with 16-bit storage hsum sums the stored values h*_i - w_i h_shift,
         // so phi - h_shift - hsum is the stored h*_0 - w_0 h_shift (sum w = 1)
         if constexpr (St::kShifted)
-            write_dir<LAT, 0, WALLS>(D.hout, G, x, y, z, own, nw, St::pack((s.phi - p.h_shift) - hsum));
+            write_dir<LAT, 0, WALLS>(D.hout, G, own, nw, St::pack((s.phi - p.h_shift) - hsum));
         else
-            write_dir<LAT, 0, WALLS>(D.hout, G, x, y, z, own, nw, St::store(s.phi - hsum, (R)W0 * p.h_shift, (R)1));
-        write_dir<LAT, 0, WALLS>(D.gout, G, x, y, z, own, nw, St::store(gs, (R)W0 * p.g_shift, p.g_scale));
+            write_dir<LAT, 0, WALLS>(D.hout, G, own, nw, St::store(s.phi - hsum, (R)W0 * p.h_shift, (R)1));
+        write_dir<LAT, 0, WALLS>(D.gout, G, own, nw, St::store(gs, (R)W0 * p.g_shift, p.g_scale));
     }
 }
 
@@ -1148,7 +1155,7 @@ __device__ __forceinline__ void march(const DirPtrs<typename Storage<ST>::S, Lat
             auto hv = [&](int i) { return hown[(j + 1) & 1][i - 1][tid]; };   // i >= 1
             // only a node next to a wall writes bounce-back ghost cells: the
             // rest take the wall-free collision (fewer live registers)
-            if (WALLS && node_writes<LAT>(G, x, y, z).wall_adj)
+            if (WALLS && wall_adjacent<LAT>(G, x, y, z))
                 collide_node<LAT, ST, true>(D, G, p, phis, j & 3, (j + 1) & 3, (j + 2) & 3, tx + 1, ty + HY, m, hv, x,
                                             y, z, rb);
             else

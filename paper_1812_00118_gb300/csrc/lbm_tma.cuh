@@ -303,7 +303,8 @@ step_tma_kernel(const __grid_constant__ TmaMaps maps, const DirPtrs<typename Sto
                 s.gz = gz * (R)3;
                 s.lap = lap * (R)6;
                 node_state<R, L::kHasY>(s, p, m0, mx, my, mz, mxx, myy, mzz, mxy, mxz, myz);
-                const NodeWrites nw = node_writes<LAT>(G, x, y, z);
+                NodeWrites nw;
+                if constexpr (WALLS) nw = node_writes(G, x, y, z);
                 const int own = (z + G.GZ) * G.PXY + rb;
                 R hsum = 0;
                 Unroll<1, Q>::run([&](auto ic) {
@@ -314,10 +315,10 @@ step_tma_kernel(const __grid_constant__ TmaMaps maps, const DirPtrs<typename Sto
                     R hs, gs;
                     collide_dir<LAT, i, R>(s, p, hv, &hs, &gs);
                     hsum += hs;
-                    write_dir<LAT, i, WALLS>(D.hout, G, x, y, z, own, nw, St::store(hs, (R)W * p.h_shift, (R)1));
-                    write_dir<LAT, i, WALLS>(D.gout, G, x, y, z, own, nw, St::store(gs, (R)W * p.g_shift, p.g_scale));
+                    write_dir<LAT, i, WALLS>(D.hout, G, own, nw, St::store(hs, (R)W * p.h_shift, (R)1));
+                    write_dir<LAT, i, WALLS>(D.gout, G, own, nw, St::store(gs, (R)W * p.g_shift, p.g_scale));
                     if constexpr (WALLS) {
-                        if (p.moving && nw.wall_adj) {
+                        if (p.moving) {
                             moving_wall_write<LAT, i>(D.hout, G, x, y, z, hs, s.phi, p,
                                                       [&](R v) { return St::store(v, (R)W * p.h_shift, (R)1); });
                             moving_wall_write<LAT, i>(D.gout, G, x, y, z, gs, s.rho, p,
@@ -329,8 +330,8 @@ step_tma_kernel(const __grid_constant__ TmaMaps maps, const DirPtrs<typename Sto
                     constexpr double W0 = L::w[0];
                     R hs, gs;
                     collide_dir<LAT, 0, R>(s, p, (R)0, &hs, &gs);
-                    write_dir<LAT, 0, WALLS>(D.hout, G, x, y, z, own, nw, St::store(s.phi - hsum, (R)W0 * p.h_shift, (R)1));
-                    write_dir<LAT, 0, WALLS>(D.gout, G, x, y, z, own, nw, St::store(gs, (R)W0 * p.g_shift, p.g_scale));
+                    write_dir<LAT, 0, WALLS>(D.hout, G, own, nw, St::store(s.phi - hsum, (R)W0 * p.h_shift, (R)1));
+                    write_dir<LAT, 0, WALLS>(D.gout, G, own, nw, St::store(gs, (R)W0 * p.g_shift, p.g_scale));
                 }
             }
         }

@@ -167,8 +167,12 @@ int lbm_init_fields_ex(lbm_ctx* ctx, const double* phi, const double* u, const d
                        int flags);
 
 /* Advance n >= 0 time steps: each step is one launch of the fused
- * collide-and-pull-stream kernel (Eqs. 1-14) and a buffer swap; the
- * bulk-copy tile (see lbm_set_tile) adds one launch of a small kernel that
+ * collide-and-pull-stream kernel (Eqs. 1-14) and a buffer swap.  A grid small
+ * enough to be resident on the chip as a whole (and whose tile the caller has
+ * not chosen) takes all n steps in one cooperative launch instead, split only
+ * where lbm_set_phi_correction asks for a correction; the waits inside it are
+ * bounded, and one that gives up is reported by lbm_diagnostics as
+ * LBM_ETIMEOUT, like a bulk-copy step's.  The bulk-copy tile (see lbm_set_tile) adds one launch of a small kernel that
  * writes the periodic images into the ghost band of the buffer just written
  * (and one more before its first step on a state another tile wrote).
  * Asynchronous on the context stream; returns LBM_ECUDA if a launch fails,
@@ -266,15 +270,17 @@ int lbm_set_wall_velocity(lbm_ctx* ctx, int axis, int side, const double u[3]);
  * arithmetic.  lbm_create picks tile 1 with lz = 16 for D2Q9, and for D3Q19
  * tile 8 with lz = 16, or tile 3 with lz = 32 for FP32 storage on grids of
  * 2^24 nodes or more; lbm_get_tile reports the current choice and its CTA
- * shape.
+ * shape.  Until lbm_set_tile or lbm_autotune chooses, lz is an upper limit
+ * (a grid that would leave the chip idle is cut into shorter chunks) and
+ * small grids step in the resident form (see lbm_step).
  * Errors: LBM_EINVAL for an unknown tile or lz < 1, LBM_ENOTSUP for a
  * bulk-copy or asynchronous-copy tile this grid, layout or storage type
  * cannot use. */
 int lbm_set_tile(lbm_ctx* ctx, int tile, int lz);
 int lbm_get_tile(const lbm_ctx* ctx, int* tile, int* lz, int* tx, int* ty);
 
-/* Poll limit of the bounded waits of the bulk-copy step pipeline (tile 4;
- * the other step kernels do not wait).  A wait whose copies have not landed
+/* Poll limit of the bounded waits of the bulk-copy step pipeline (tile 4; of
+ * the other forms only the resident step waits, with a limit of its own).  A wait whose copies have not landed
  * after `polls` tries gives up: the kernel raises the context's error flag,
  * lets the copies it has in flight land (a separate bounded wait) and
  * returns, so the GPU context stays usable, lbm_diagnostics returns
@@ -286,7 +292,7 @@ int lbm_get_tile(const lbm_ctx* ctx, int* tile, int* lz, int* tx, int* ty);
 int lbm_set_wait_limit(lbm_ctx* ctx, long long polls);
 
 /* Autotuner: times every compiled tile (those the grid supports) with lz in
- * {4, 8, 16, 32} for `steps` steps each on the current state, keeps the
+ * {4, 8, 16, 32}, and the form a context takes before any choice, for `steps` steps each on the current state, keeps the
  * fastest configuration, and restores the state it started from (the state
  * is saved to, and copied back from, a temporary device copy).  Reports the
  * choice and its time per step (step kernel plus ghost update) in ms; any

@@ -289,6 +289,23 @@ int copy_field(lbm_ctx* c, double* dst, const double* src, size_t n, int on_devi
                                       on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
 }
 
+// The resident step (lbm_box.cuh) keeps its box counts in the half of the
+// reduction scratch that the reductions leave free (they use the first
+// 4 x 1024 doubles and the 4 after them).
+constexpr int kMaxBoxes = 8000;
+int* box_flags(lbm_ctx* c) { return (int*)(c->partial + 4 * 1024 + 8); }
+bool resident(const lbm_ctx* c) {
+    return c->box.variant >= 0 && c->box.boxes <= kMaxBoxes && c->partial && !c->owner;
+}
+
+// A new state: the error flag of the bounded waits, and the box counts a wait
+// that gave up left uneven.
+int clear_wait_state(lbm_ctx* c) {
+    if (check_cuda(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream))) return LBM_ECUDA;
+    if (!resident(c)) return LBM_OK;
+    return check_cuda(cudaMemsetAsync(box_flags(c), 0, sizeof(int) * c->box.boxes, c->stream));
+}
+
 // rho_bar for force_mode 1 from the current state's phi (scratch fields must be fresh)
 int update_rho_bar(lbm_ctx* c) {
     double d[4];
@@ -471,6 +488,7 @@ int lbm_create_ex(const lbm_grid* grid, int lattice, const lbm_params* params, v
         return LBM_ENOMEM;
     }
     cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
+    if (c->K->box_plan(c->G, &c->box) != cudaSuccess) { cudaGetLastError(); lbm_destroy(c); return LBM_ECUDA; }
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) { lbm_destroy(c); return LBM_ECUDA; }
     *out = c;
     return LBM_OK;
@@ -543,7 +561,7 @@ int lbm_init_fields_ex(lbm_ctx* c, const double* phi, const double* u, const dou
         return LBM_ECUDA;
     c->ghosts[b] = true;   // the initialisation writes the periodic images too
     c->diverged = false;
-    if (check_cuda(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream))) return LBM_ECUDA;
+    if (clear_wait_state(c)) return LBM_ECUDA;
     c->launches += 1;
     return check_cuda(cudaStreamSynchronize(c->stream));
 }
@@ -590,10 +608,39 @@ static int step_impl(lbm_ctx* c, int n, cudaEvent_t* ev) {
     a.p = c->P;
     a.tile = c->tile;
     a.lz = c->lz;
+    a.fit = !c->tile_chosen;
     a.stream = c->stream;
     a.error_flag = c->d_err;
     a.wait_polls = c->wait_polls;
-    for (int s = 0; s < n; ++s) {
+    int s = 0;
+    while (s < n && resident(c) && !c->tile_chosen) {
+        // one launch up to the end or the next re-imposition of phi's total
+        int m = ev ? 1 : n - s;
+        if (c->phi_fix_every > 0) {
+            const int left = c->phi_fix_every - c->phi_fix_count;
+            if (m > left) m = left > 1 ? left : 1;
+        }
+        const int i = c->cur, o = 1 - c->cur;
+        a.hin = c->h[i]; a.gin = c->g[i]; a.hout = c->h[o]; a.gout = c->g[o];
+        if (ev) cudaEventRecord(ev[2 * s], c->stream);
+        const cudaError_t e = c->K->box_steps(a, c->box, m, box_flags(c));
+        if (e == cudaErrorCooperativeLaunchTooLarge) {   // fewer SMs than the device reports: the march
+            cudaGetLastError();
+            c->box.variant = -1;
+            break;
+        }
+        if (check_cuda(e)) return LBM_ECUDA;
+        if (ev) cudaEventRecord(ev[2 * s + 1], c->stream);
+        c->launches += 1;
+        c->ghosts[0] = c->ghosts[1] = false;
+        c->cur = (c->cur + m) & 1;
+        s += m;
+        if (c->phi_fix_every > 0 && (c->phi_fix_count += m) >= c->phi_fix_every) {
+            if (phi_fix(c)) return LBM_ECUDA;
+            c->phi_fix_count = 0;
+        }
+    }
+    for (; s < n; ++s) {
         const int i = c->cur, o = 1 - c->cur;
         a.hin = c->h[i]; a.gin = c->g[i]; a.hout = c->h[o]; a.gout = c->g[o];
         a.maps = &c->maps[i];
@@ -704,7 +751,7 @@ int lbm_set_populations(lbm_ctx* c, const double* h, const double* g, int on_dev
     int rc = check_cuda(c->K->set(c->h[b], c->g[b], c->G, c->P, dh, dg, c->stream));
     c->ghosts[b] = true;
     c->diverged = false;
-    if (!rc) rc = check_cuda(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
+    if (!rc) rc = clear_wait_state(c);
     c->launches += 1;
     if (th) { cudaFreeAsync(th, c->stream); cudaFreeAsync(tg, c->stream); }
     if (!rc) {
@@ -780,6 +827,7 @@ int lbm_autotune(lbm_ctx* c, int steps, int* best_tile, int* best_lz, double* be
     const bool saved_ghosts = c->ghosts[c->cur];
     const bool saved_diverged = c->diverged;
     const int saved_tile = c->tile, saved_lz = c->lz, saved_fix_count = c->phi_fix_count;
+    const bool saved_chosen = c->tile_chosen;
     int rc = check_cuda(cudaMemcpyAsync(save_h, c->h[c->cur], bytes, cudaMemcpyDeviceToDevice, c->stream));
     if (!rc) rc = check_cuda(cudaMemcpyAsync(save_g, c->g[c->cur], bytes, cudaMemcpyDeviceToDevice, c->stream));
     const bool saved = rc == LBM_OK;
@@ -788,12 +836,17 @@ int lbm_autotune(lbm_ctx* c, int steps, int* best_tile, int* best_lz, double* be
     cudaEventCreate(&e1);
     const int lzs[4] = {4, 8, 16, 32};
     int bt = c->tile, bl = c->lz;
+    bool bc = saved_chosen;
     float bms = 1e30f;
-    for (int t = 0; t < c->K->n_tiles && !rc; ++t) {
-        if (!c->K->tile_ok(t, c->G)) continue;
-        for (int k = 0; k < 4 && !rc; ++k) {
-            c->tile = t;
-            c->lz = lzs[k];
+    // the last trial is the context's own configuration before any choice
+    // (the resident step, or the default tile fitted to one wave)
+    for (int t = 0; t <= c->K->n_tiles && !rc; ++t) {
+        const bool own = t == c->K->n_tiles;
+        if (own ? saved_chosen : !c->K->tile_ok(t, c->G)) continue;
+        for (int k = 0; k < (own ? 1 : 4) && !rc; ++k) {
+            c->tile = own ? saved_tile : t;
+            c->lz = own ? saved_lz : lzs[k];
+            c->tile_chosen = !own;
             rc = lbm_step(c, 2);
             if (rc) break;
             cudaEventRecord(e0, c->stream);
@@ -803,7 +856,7 @@ int lbm_autotune(lbm_ctx* c, int steps, int* best_tile, int* best_lz, double* be
             rc = check_cuda(cudaEventSynchronize(e1));
             float ms = 0;
             cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < bms) { bms = ms; bt = t; bl = lzs[k]; }
+            if (ms < bms) { bms = ms; bt = c->tile; bl = c->lz; bc = c->tile_chosen; }
         }
     }
     cudaEventDestroy(e0);
@@ -824,6 +877,7 @@ int lbm_autotune(lbm_ctx* c, int steps, int* best_tile, int* best_lz, double* be
     cudaFreeAsync(save_g, c->stream);
     c->tile = rc ? saved_tile : bt;
     c->lz = rc ? saved_lz : bl;
+    c->tile_chosen = rc ? saved_chosen : bc;
     if (!rc) rc = check_cuda(cudaStreamSynchronize(c->stream));
     if (best_tile) *best_tile = bt;
     if (best_lz) *best_lz = bl;
@@ -883,6 +937,7 @@ int lbm_set_tile(lbm_ctx* c, int tile, int lz) {
     if (!c->K->tile_ok(tile, c->G)) return LBM_ENOTSUP;
     c->tile = tile;
     c->lz = lz;
+    c->tile_chosen = true;
     return LBM_OK;
 }
 

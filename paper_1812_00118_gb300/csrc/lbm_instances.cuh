@@ -6,6 +6,7 @@
 
 #include <new>
 
+#include "lbm_box.cuh"
 #include "lbm_internal.h"
 #include "lbm_tma.cuh"
 
@@ -49,7 +50,8 @@ cudaError_t resident_slots(K kern, int threads, size_t smem, int* out) {
     return cudaSuccess;
 }
 
-// Grid = tile columns x chunks along z.  Chunks of lz planes, or with BAL
+// Grid = tile columns x chunks along z.  Chunks of lz planes (with StepArgs::fit
+// as few as keep the launch in one wave), or with BAL
 // (one-wave launch) as many equal chunks as the resident slots (occupancy x
 // SMs, looked up once per instantiation) allow for every column, with at
 // least lz planes each.
@@ -62,12 +64,25 @@ cudaError_t launch_step_tile(const StepArgs& a) {
                       : step_kernel<LAT, ST, TX, TY, MINB, HOIST, BAL, false>;
     dim3 block(TX, TY);
     dim3 grid((G.NX + TX - 1) / TX, (G.NY + TY - 1) / TY, (G.NZ + a.lz - 1) / a.lz);
-    if (BAL) {
+    int lz = a.lz, slots = 0;
+    if (BAL || a.fit) {
         static PerDevice slots_cache;
-        int slots = 0;
         cudaError_t e = per_device(slots_cache, walls ? 1 : 0,
                                    [&](int* v) { return resident_slots(kern, TX * TY, 0, v); }, &slots);
         if (e != cudaSuccess) return e;
+    }
+    if (a.fit) {
+        // chunks as short as one wave allows: a grid that does not fill the
+        // chip with chunks of a.lz planes is bound by the length of the march,
+        // not by the planes the chunks read twice (one wave / 16 planes, us
+        // per step in FP32: 64^3 22.6 / 45.2, 80^3 47.2 / 71.8, 117 x 75 x 90
+        // 63.8 / 85.9, 1000^2 35.6 / 52.2; 128^3 and 1500^2 fill it either way)
+        const long long per_column = slots / ((long long)grid.x * grid.y);
+        const int one_wave = (int)((G.NZ - 1) / (per_column > 0 ? per_column : 1)) + 1;
+        if (one_wave < lz) lz = one_wave;
+        grid.z = (G.NZ - 1) / lz + 1;
+    }
+    if (BAL) {
         long long nzc = slots / ((long long)grid.x * grid.y);
         const long long by_lz = (G.NZ + a.lz - 1) / a.lz;
         if (nzc > by_lz) nzc = by_lz;
@@ -76,7 +91,7 @@ cudaError_t launch_step_tile(const StepArgs& a) {
     }
     const auto d = dir_ptrs<S, Lattice<LAT>::Q>(a.hin, a.gin, a.hout, a.gout, G.NP);
     const auto ph = phys_as<typename Storage<ST>::R>(a.p);
-    kern<<<grid, block, 0, a.stream>>>(d, G, ph, a.lz);
+    kern<<<grid, block, 0, a.stream>>>(d, G, ph, lz);
     return cudaGetLastError();
 }
 
@@ -110,6 +125,56 @@ cudaError_t launch_async_tile(const StepArgs& a) {
                                                       G, phys_as<float>(a.p), a.lz);
         return cudaGetLastError();
     }
+}
+
+// ---------------------------------------------------------------- resident step
+template <int BX_, int BY_, int BZ_, int MINB_>
+struct Box {
+    static constexpr int BX = BX_, BY = BY_, BZ = BZ_, MINB = MINB_, NT = BX_ * BY_ * BZ_;
+    // boxes of a cut axis are at least two nodes wide: the step's reach
+    static_assert(BX >= 3 && (BY == 1 || BY >= 3) && BZ >= 3, "box_bound gives at least (B + 1) / 2 nodes");
+    static BoxPlan cut(const Geom& G, int variant) {
+        BoxPlan q;
+        q.variant = variant;
+        q.nx = (G.NX - 1) / BX + 1;
+        q.ny = (G.NY - 1) / BY + 1;
+        q.nz = (G.NZ - 1) / BZ + 1;
+        const long long n = (long long)q.nx * q.ny * q.nz;
+        q.boxes = n < (1LL << 31) ? (int)n : 0;
+        return q;
+    }
+    template <int LAT, int ST>
+    static auto kernel(const Geom& G) {
+        return G.wall[0] || G.wall[1] || G.wall[2] ? box_kernel<LAT, ST, BX, BY, BZ, MINB, true>
+                                                   : box_kernel<LAT, ST, BX, BY, BZ, MINB, false>;
+    }
+};
+
+template <int LAT, int ST, typename B>
+cudaError_t box_slots(const Geom& G, int* out) {
+    static PerDevice cache;
+    return per_device(cache, G.wall[0] || G.wall[1] || G.wall[2] ? 1 : 0,
+                      [&](int* v) { return resident_slots(B::template kernel<LAT, ST>(G), B::NT, 0, v); }, out);
+}
+
+template <int LAT, int ST, typename B>
+cudaError_t launch_box(const StepArgs& a, const BoxPlan& pl, int n, int* flags) {
+    using S = typename Storage<ST>::S;
+    const Geom& G = a.G;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n > 1 ? pl.ctas : pl.boxes);
+    cfg.blockDim = dim3(B::NT);
+    cfg.stream = a.stream;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeCooperative;   // boxes that wait for one another are all resident
+    at.val.cooperative = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = n > 1 ? 1 : 0;
+    BoxPtrs<S, Lattice<LAT>::Q> ptrs;
+    ptrs.d[0] = dir_ptrs<S, Lattice<LAT>::Q>(a.hin, a.gin, a.hout, a.gout, G.NP);
+    ptrs.d[1] = dir_ptrs<S, Lattice<LAT>::Q>(a.hout, a.gout, const_cast<void*>(a.hin), const_cast<void*>(a.gin), G.NP);
+    return cudaLaunchKernelEx(&cfg, B::template kernel<LAT, ST>(G), ptrs, G, phys_as<typename Storage<ST>::R>(a.p), pl,
+                              n, flags, a.error_flag);
 }
 
 // ---------------------------------------------------------------- batches

@@ -5,6 +5,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "lbm.h"
+#include "lbm_box.cuh"
 #include "lbm_kernels.cuh"
 #include "lbm_tma.cuh"
 
@@ -33,6 +34,7 @@ struct StepArgs {
     Geom G;
     Phys p;
     int tile, lz;
+    bool fit = false;      // lz is an upper limit: shorter chunks while one wave holds them
     cudaStream_t stream;
     const TmaMaps* maps;   // tensor maps of (hin, gin) for a bulk-copy tile
     int* error_flag;       // raised by a bounded wait that gave up
@@ -58,6 +60,10 @@ constexpr int kMaxBatchTiles = 4;
 
 struct KernelTable {
     cudaError_t (*step)(const StepArgs& a);
+    // resident step of small grids: its plan for a grid on the current device
+    // (variant -1: not for this grid), and n steps in one launch
+    cudaError_t (*box_plan)(const Geom& G, BoxPlan* plan);
+    cudaError_t (*box_steps)(const StepArgs& a, const BoxPlan& plan, int n, int* flags);
     // tensor maps of one input buffer pair for bulk-copy tile `tile`
     cudaError_t (*make_maps)(int tile, TmaMaps* out, const void* h, const void* g, const Geom& G);
     // true if tile `tile` can run this grid and storage type (shared memory,
@@ -124,6 +130,10 @@ struct lbm_ctx {
     int cur = 0;           // buffer holding the current state
     int tile = 0;          // step tile shape index
     int lz = 16;           // planes per CTA chunk
+    bool tile_chosen = false;   // by lbm_set_tile or lbm_autotune; until then
+                           // tile and lz are the march's limits and small
+                           // grids take the resident step
+    lbm::BoxPlan box;      // the resident step's cut of the grid
     lbm::TmaMaps maps[2];  // tensor maps of buffer pair 0 and 1 for a bulk-copy tile
     int maps_tile = -1;    // tile the maps were made for
     bool ghosts[2] = {false, false};   // ghost band of buffer b holds the periodic images

@@ -44,6 +44,26 @@ namespace {
     X(9, splitbal, 128, 1, 7)
 #endif
 
+// Boxes of the resident step (lbm_box.cuh): nodes along the internal axes and
+// the CTAs per SM the registers are bounded for; the larger box first.
+// Measured, us per step of a periodic grid (FP32, 100 steps per launch):
+//   D2Q9   32x8 / 32x4: 64^2 3.8 / 3.1, 128^2 4.0 / 3.3, 256^2 4.9 / 4.8, 512^2 11.5 / 15.4
+//   D3Q19  16x4x4 / 8x4x4: 16^3 6.6 / 5.9, 24^3 6.9 / 6.0, 32^3 6.4 / 7.0, 40^3 9.8 / 11.1
+// so the larger box pays once it gives at least half the SMs a box (D3Q19) or
+// every SM one (D2Q9).  At 64 registers (4 CTAs of 256) the D2Q9 box spills
+// nothing; D3Q19 needs 128.
+#if LBM_LAT == 1
+using BoxA = Box<16, 4, 4, 2>;
+using BoxB = Box<8, 4, 4, 4>;
+constexpr int kBoxAHalves = 1;    // box A from this many half boxes per SM on
+constexpr int kBoxRounds = 1;     // boxes of one CTA per step at most
+#else
+using BoxA = Box<32, 1, 8, 4>;
+using BoxB = Box<32, 1, 4, 4>;
+constexpr int kBoxAHalves = 2;
+constexpr int kBoxRounds = 2;
+#endif
+
 #define LBM_LAUNCH_hoist(TX, TY, MB) launch_step_tile<LBM_LAT, LBM_ST, TX, TY, MB, true, false>(a)
 #define LBM_LAUNCH_split(TX, TY, MB) launch_step_tile<LBM_LAT, LBM_ST, TX, TY, MB, false, false>(a)
 #define LBM_LAUNCH_hoistbal(TX, TY, MB) launch_step_tile<LBM_LAT, LBM_ST, TX, TY, MB, true, true>(a)
@@ -89,6 +109,36 @@ bool ok_dispatch(int tile, const Geom& G) {
     switch (tile) {
         LBM_TILES(LBM_OK_CASE)
         default: return false;
+    }
+}
+
+// How a grid is cut into boxes; plan->variant stays -1 where the march is the
+// faster form.  The march of as many CTAs as the chip holds (StepArgs::fit)
+// overtakes once the boxes need more than one round per step (D3Q19: 40^3 9.8
+// against 14.4 us, 48^3 16.4 against 14.5) or two (D2Q9: 512^2 11.5 against
+// 12.4, 707^2 23.2 against 18.8).
+cudaError_t box_plan(const Geom& G, BoxPlan* plan) {
+    *plan = BoxPlan();
+    int dev = 0, sms = 0, slots = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    BoxPlan q = BoxA::cut(G, 0);
+    if (2LL * q.boxes < (long long)kBoxAHalves * sms) q = BoxB::cut(G, 1);
+    if (q.boxes < 1) return cudaSuccess;   // more boxes than fit an int
+    e = q.variant == 0 ? box_slots<LBM_LAT, LBM_ST, BoxA>(G, &slots) : box_slots<LBM_LAT, LBM_ST, BoxB>(G, &slots);
+    if (e != cudaSuccess) return e;
+    if (q.boxes > (long long)slots * kBoxRounds) return cudaSuccess;
+    q.ctas = q.boxes < slots ? q.boxes : slots;
+    *plan = q;
+    return cudaSuccess;
+}
+
+cudaError_t box_dispatch(const StepArgs& a, const BoxPlan& pl, int n, int* flags) {
+    switch (pl.variant) {
+        case 0: return launch_box<LBM_LAT, LBM_ST, BoxA>(a, pl, n, flags);
+        case 1: return launch_box<LBM_LAT, LBM_ST, BoxB>(a, pl, n, flags);
+        default: return cudaErrorInvalidValue;
     }
 }
 
@@ -139,7 +189,7 @@ int checked_status() {
 #endif
 }
 
-const KernelTable kTable = {step_dispatch, maps_dispatch, ok_dispatch,
+const KernelTable kTable = {step_dispatch, box_plan, box_dispatch, maps_dispatch, ok_dispatch,
                             Launchers<LBM_LAT, LBM_ST>::phi, Launchers<LBM_LAT, LBM_ST>::macro,
                             Launchers<LBM_LAT, LBM_ST>::init, Launchers<LBM_LAT, LBM_ST>::get,
                             Launchers<LBM_LAT, LBM_ST>::set, Launchers<LBM_LAT, LBM_ST>::halo,

@@ -124,7 +124,7 @@ double* f_u(lbm_ctx* c, int a) { return c->fields + (2 + a) * c->G.N; }
 int compute_fields(lbm_ctx* c) {
     int rc = ensure_scratch(c);
     if (rc) return rc;
-    if (check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, f_phi(c), c->stream))) return LBM_ECUDA;
+    if (check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, f_phi(c), nullptr, c->stream))) return LBM_ECUDA;
     if (check_cuda(c->K->macro(c->g[c->cur], c->G, c->P, f_phi(c), f_P(c), f_u(c, 0), f_u(c, 1), f_u(c, 2),
                                c->stream)))
         return LBM_ECUDA;
@@ -245,13 +245,6 @@ __global__ void phi_delta_kernel(const double* __restrict__ part, int nb, double
     *delta = (target - s) / (double)n;
 }
 
-// rho u = rho(phi) u
-__global__ void rho_times_u_kernel(const double* __restrict__ phi, const double* __restrict__ u, long long N,
-                                   double rho_L, double rho_dif, double* out) {
-    const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (n < N) out[n] = (rho_L + phi[n] * rho_dif) * u[n];
-}
-
 int partial_blocks(const lbm_ctx* c) {
     long long b = (c->G.N + kRedThreads - 1) / kRedThreads;
     return (int)(b < c->n_partial_blocks ? b : c->n_partial_blocks);
@@ -273,7 +266,7 @@ int reduce_diag(lbm_ctx* c, double out[4]) {
 // Total of phi restored to phi_target (FP64 sums on the GPU, uniform shift of
 // the rest population); stream-ordered, no host synchronisation.
 int phi_fix(lbm_ctx* c) {
-    if (check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, f_phi(c), c->stream))) return LBM_ECUDA;
+    if (check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, f_phi(c), nullptr, c->stream))) return LBM_ECUDA;
     long long nb = (c->G.N + kRedThreads - 1) / kRedThreads;
     if (nb > kFixBlocks) nb = kFixBlocks;
     sum_partial_kernel<<<(unsigned)nb, kRedThreads, 0, c->stream>>>(f_phi(c), c->G.N, c->d_fix);
@@ -670,33 +663,47 @@ static int step_impl(lbm_ctx* c, int n, cudaEvent_t* ev) {
     return LBM_OK;
 }
 
+// Two launches, straight into the caller's device arrays; host outputs, and
+// device outputs that overlap one another, go through scratch fields.
 int lbm_macro(lbm_ctx* c, double* phi, double* P, double* rho_u, int on_device) {
     lbm::NvtxRange range("lbm_macro");
     if (!c) return LBM_EINVAL;
-    int rc = compute_fields(c);
+    int rc = ensure_scratch(c);
     if (rc) return rc;
     const long long N = c->G.N;
-    if (phi && copy_field(c, phi, f_phi(c), N, on_device)) return LBM_ECUDA;
-    if (P && copy_field(c, P, f_P(c), N, on_device)) return LBM_ECUDA;
-    if (rho_u) {
-        double* dst = rho_u;
-        if (!on_device && cudaMallocAsync((void**)&dst, sizeof(double) * c->dim * (size_t)N, c->stream) != cudaSuccess) {
-            cudaGetLastError();
-            return LBM_ENOMEM;
-        }
-        const unsigned nb = (unsigned)((N + 255) / 256);
-        for (int d = 0; d < c->dim; ++d)
-            rho_times_u_kernel<<<nb, 256, 0, c->stream>>>(f_phi(c), f_u(c, internal_axis(c, d)), N, c->P.rho_L,
-                                                          c->P.rho_dif, dst + d * N);
-        c->launches += c->dim;
-        rc = check_cuda(cudaGetLastError());
-        if (!on_device) {
-            if (!rc) rc = check_cuda(cudaMemcpyAsync(rho_u, dst, sizeof(double) * c->dim * (size_t)N,
-                                                     cudaMemcpyDeviceToHost, c->stream));
-            cudaFreeAsync(dst, c->stream);
-        }
-        if (rc) return rc;
+    auto apart = [](const double* a, long long na, const double* b, long long nb) {
+        return !a || !b || a + na <= b || b + nb <= a;
+    };
+    const bool direct = on_device && apart(phi, N, P, N) && apart(phi, N, rho_u, c->dim * N) &&
+                        apart(P, N, rho_u, c->dim * N);
+    double* d_phi = direct && phi ? phi : f_phi(c);
+    double* d_P = direct ? P : (P ? f_P(c) : nullptr);
+    double* d_ru = rho_u;
+    if (rho_u && !direct &&
+        cudaMallocAsync((void**)&d_ru, sizeof(double) * c->dim * (size_t)N, c->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return LBM_ENOMEM;
     }
+    // the stencils read phi in the kernels' arithmetic type: FP64 storage as
+    // it is, else a rounded copy in the scratch of the velocity (unused here)
+    void* rounded = c->store == LBM_F64 ? nullptr : (void*)f_u(c, 0);
+    const bool flow = d_P || d_ru;
+    rc = check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, d_phi, flow ? rounded : nullptr, c->stream));
+    c->launches += 1;
+    if (!rc && flow) {
+        double* ru[3] = {nullptr, nullptr, nullptr};   // internal axes
+        for (int d = 0; d < c->dim && d_ru; ++d) ru[internal_axis(c, d)] = d_ru + d * N;
+        rc = check_cuda(c->K->momentum(c->g[c->cur], c->G, c->P, d_phi, rounded ? rounded : d_phi, d_P, ru[0], ru[1],
+                                       ru[2], c->stream));
+        c->launches += 1;
+    }
+    if (!direct) {
+        if (!rc && phi) rc = copy_field(c, phi, d_phi, N, on_device);
+        if (!rc && P) rc = copy_field(c, P, d_P, N, on_device);
+        if (!rc && rho_u) rc = copy_field(c, rho_u, d_ru, c->dim * N, on_device);
+        if (d_ru) cudaFreeAsync(d_ru, c->stream);
+    }
+    if (rc) return rc;
     return check_cuda(cudaStreamSynchronize(c->stream));
 }
 

@@ -297,16 +297,25 @@ template <int LAT, int ST>
 struct Launchers {
     using S = typename Storage<ST>::S;
     static constexpr int Q = Lattice<LAT>::Q;
-    static cudaError_t phi(const void* hin, const Geom& G, const Phys& p, double* out, cudaStream_t s) {
+    static cudaError_t phi(const void* hin, const Geom& G, const Phys& p, double* out, void* rounded,
+                           cudaStream_t s) {
         phi_kernel<LAT, ST><<<blocks_for(G.N, 256), 256, 0, s>>>(
-            dir_ptrs<S, Q>(hin, hin, nullptr, nullptr, G.NP), G, p, out);
+            dir_ptrs<S, Q>(hin, hin, nullptr, nullptr, G.NP), G, p, out, (typename Storage<ST>::R*)rounded);
         return cudaGetLastError();
     }
     static cudaError_t macro(const void* gin, const Geom& G, const Phys& p, const double* phi, double* P,
                              double* ux, double* uy, double* uz, cudaStream_t s) {
-        macro_kernel<LAT, ST><<<blocks_for(G.N, 256), 256, 0, s>>>(
-            dir_ptrs<S, Q>(gin, gin, nullptr, nullptr, G.NP), G, phys_as<typename Storage<ST>::R>(p), phi, P, ux, uy,
-            uz);
+        macro_kernel<LAT, ST, double, false><<<blocks_for(G.N, 256), 256, 0, s>>>(
+            dir_ptrs<S, Q>(gin, gin, nullptr, nullptr, G.NP), G, phys_as<typename Storage<ST>::R>(p), phi, phi, p.rho_L,
+            p.rho_dif, P, ux, uy, uz);
+        return cudaGetLastError();
+    }
+    static cudaError_t momentum(const void* gin, const Geom& G, const Phys& p, const double* phi, const void* rounded,
+                                double* P, double* rux, double* ruy, double* ruz, cudaStream_t s) {
+        using R = typename Storage<ST>::R;
+        macro_kernel<LAT, ST, R, true><<<blocks_for(G.N, 256), 256, 0, s>>>(
+            dir_ptrs<S, Q>(gin, gin, nullptr, nullptr, G.NP), G, phys_as<R>(p), phi, (const R*)rounded, p.rho_L,
+            p.rho_dif, P, rux, ruy, ruz);
         return cudaGetLastError();
     }
     static cudaError_t init(void* hout, void* gout, const Geom& G, const Phys& p, const double* phi,

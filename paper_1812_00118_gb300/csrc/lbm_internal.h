@@ -69,9 +69,13 @@ struct KernelTable {
     // true if tile `tile` can run this grid and storage type (shared memory,
     // sizes; bulk-copy and asynchronous-load tiles have limits)
     bool (*tile_ok)(int tile, const Geom& G);
-    cudaError_t (*phi)(const void* hin, const Geom& G, const Phys& p, double* phi, cudaStream_t s);
+    // phi in double and (rounded not null) in the kernels' arithmetic type
+    cudaError_t (*phi)(const void* hin, const Geom& G, const Phys& p, double* phi, void* rounded, cudaStream_t s);
     cudaError_t (*macro)(const void* gin, const Geom& G, const Phys& p, const double* phi, double* P,
                          double* ux, double* uy, double* uz, cudaStream_t s);
+    // P and rho u (null outputs left out) from phi and its rounded copy
+    cudaError_t (*momentum)(const void* gin, const Geom& G, const Phys& p, const double* phi, const void* rounded,
+                            double* P, double* rux, double* ruy, double* ruz, cudaStream_t s);
     cudaError_t (*init)(void* hout, void* gout, const Geom& G, const Phys& p, const double* phi,
                         const double* ux, const double* uy, const double* uz, const double* P, int neq,
                         cudaStream_t s);

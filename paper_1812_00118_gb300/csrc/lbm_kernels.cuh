@@ -1389,9 +1389,43 @@ __global__ void shift_rest_kernel(typename Storage<ST>::S* __restrict__ h0, Geom
     h0[k] = St::store(St::load(h0[k], sh, (R)1) + (R)*delta, sh, (R)1);
 }
 
-// phi = sum_i of the pulled h at every node (double output, node order).
+// A sum of FP32 values as a non-overlapping triple of FP32 (two levels of
+// TwoSum), converted to FP64 once: at least as close to the exact sum as a
+// chain of FP64 additions.  FP64 operations, conversions from and to FP32
+// included, run at two lanes per clock and SM on this chip; 19 conversions and
+// additions per node took 2.0 ms for 2^25 nodes, this 0.5 ms.
+template <typename R>
+struct WideSum {
+    double s = 0;
+    __device__ __forceinline__ void add(R v) { s += (double)v; }
+    __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct WideSum<float> {
+    float a = 0.0f, b = 0.0f, c = 0.0f;
+    static __device__ __forceinline__ float two_sum(float x, float y, float* err) {
+        const float s = __fadd_rn(x, y);
+        const float t = __fsub_rn(s, x);
+        *err = __fadd_rn(__fsub_rn(x, __fsub_rn(s, t)), __fsub_rn(y, t));
+        return s;
+    }
+    __device__ __forceinline__ void add(float v) {
+        float e, f;
+        a = two_sum(a, v, &e);
+        b = two_sum(b, e, &f);
+        c = __fadd_rn(c, f);
+    }
+    // a sum that is not finite goes as it is: its error terms are NaN
+    __device__ __forceinline__ double value() const {
+        return isfinite(a) ? (double)a + ((double)b + (double)c) : (double)a;
+    }
+};
+
+// phi = sum_i of the pulled h at every node: in double (node order) and, where
+// asked for, rounded to the kernels' arithmetic type for the stencils.
 template <int LAT, int ST>
-__global__ void phi_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::Q> D, Geom G, Phys p, double* phi) {
+__global__ void phi_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::Q> D, Geom G, Phys p, double* phi,
+                           typename Storage<ST>::R* rounded) {
     using L = Lattice<LAT>;
     using St = Storage<ST>;
     using R = typename St::R;
@@ -1400,21 +1434,23 @@ __global__ void phi_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::
     int x, y, z;
     node_coords(G, n, &x, &y, &z);
     const PullOffsets po = pull_offsets(G, x, y, z);
-    double acc = 0;
+    WideSum<R> acc;
     Unroll<0, L::Q>::run([&](auto ic) {
         constexpr int i = decltype(ic)::value;
         constexpr double W = L::w[i];
-        acc += (double)St::load(pull_pad<LAT, i, false>(D.hin, po), (R)(W * p.h_shift), (R)1);
+        acc.add(St::load(pull_pad<LAT, i, false>(D.hin, po), (R)(W * p.h_shift), (R)1));
     });
-    phi[n] = acc;
+    const double f = acc.value();
+    phi[n] = f;
+    if (rounded) rounded[n] = (R)f;
 }
 
 // CD stencils of a double field (node order) at node (x, y, z), in the
 // arithmetic type R (the values are rounded to R first): FP64 for the
 // diagnostics and FP64 storage, FP32 for initialising FP32 and 16-bit
 // storage (whose kernels compute in FP32; GB300's FP64 rate is low).
-template <int LAT, typename R = double>
-__device__ __forceinline__ void stencils(const double* __restrict__ phi, const Geom& G, int x, int y, int z,
+template <int LAT, typename R = double, typename F = double>
+__device__ __forceinline__ void stencils(const F* __restrict__ phi, const Geom& G, int x, int y, int z,
                                          R* gx, R* gy, R* gz, R* lap) {
     using L = Lattice<LAT>;
     auto at = [&](int a, int b, int c) { return (R)phi[a + G.NX * (b + G.NY * c)]; };
@@ -1434,15 +1470,16 @@ __device__ __forceinline__ void stencils(const double* __restrict__ phi, const G
     *gx = (R)3 * ax; *gy = (R)3 * ay; *gz = (R)3 * az; *lap = (R)6 * l;
 }
 
-// Macroscopic fields (phi given): P and u (internal axes), written in
-// double.  Computed in the kernels' arithmetic type R: FP64 for FP64 storage,
-// FP32 for FP32 and 16-bit storage (their values carry FP32 rounding
-// already, and GB300's FP64 rate is low).  Only the flow fields of the step
-// (node_flow), not the collision's second moments.
-template <int LAT, int ST>
+// Macroscopic fields (phi given, in double and as the stencils' input f of
+// type F): P and, in double, u or (with MOMENTUM) rho(phi) u along the internal
+// axes; a null output is left out.  Computed in the kernels' arithmetic type
+// R: FP64 for FP64 storage, FP32 for FP32 and 16-bit storage (their values
+// carry FP32 rounding already, and GB300's FP64 rate is low).  Only the flow
+// fields of the step (node_flow), not the collision's second moments.
+template <int LAT, int ST, typename F, bool MOMENTUM>
 __global__ void macro_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::Q> D, Geom G,
-                             PhysT<typename Storage<ST>::R> p, const double* __restrict__ phi, double* P, double* ux,
-                             double* uy, double* uz) {
+                             PhysT<typename Storage<ST>::R> p, const double* __restrict__ phi, const F* __restrict__ f,
+                             double rho_L, double rho_dif, double* P, double* ux, double* uy, double* uz) {
     using L = Lattice<LAT>;
     using St = Storage<ST>;
     using R = typename St::R;
@@ -1452,8 +1489,8 @@ __global__ void macro_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>
     node_coords(G, n, &x, &y, &z);
     const PullOffsets po = pull_offsets(G, x, y, z);
     NodeState<R> s;
-    s.phi = (R)phi[n];
-    stencils<LAT, R>(phi, G, x, y, z, &s.gx, &s.gy, &s.gz, &s.lap);
+    s.phi = (R)f[n];
+    stencils<LAT, R>(f, G, x, y, z, &s.gx, &s.gy, &s.gz, &s.lap);
     R m0 = 0, mx = 0, my = 0, mz = 0;
     Unroll<0, L::Q>::run([&](auto ic) {
         constexpr int i = decltype(ic)::value;
@@ -1466,10 +1503,12 @@ __global__ void macro_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>
         if (CZ) mz += cmul<CZ>(v);
     });
     node_flow<R, L::kHasY>(s, p, m0, mx, my, mz);
-    P[n] = (double)s.P;
-    ux[n] = (double)s.ux;
-    uy[n] = (double)s.uy;
-    uz[n] = (double)s.uz;
+    if (P) P[n] = (double)s.P;
+    if (MOMENTUM && !ux) return;
+    const double k = MOMENTUM ? rho_L + phi[n] * rho_dif : 1.0;
+    ux[n] = MOMENTUM ? k * (double)s.ux : (double)s.ux;
+    if (uy) uy[n] = MOMENTUM ? k * (double)s.uy : (double)s.uy;
+    uz[n] = MOMENTUM ? k * (double)s.uz : (double)s.uz;
 }
 
 // Where the value pulled by node (x, y, z) for direction I lives: x - c_I

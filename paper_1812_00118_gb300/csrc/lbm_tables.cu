@@ -191,6 +191,7 @@ int checked_status() {
 
 const KernelTable kTable = {step_dispatch, box_plan, box_dispatch, maps_dispatch, ok_dispatch,
                             Launchers<LBM_LAT, LBM_ST>::phi, Launchers<LBM_LAT, LBM_ST>::macro,
+                            Launchers<LBM_LAT, LBM_ST>::momentum,
                             Launchers<LBM_LAT, LBM_ST>::init, Launchers<LBM_LAT, LBM_ST>::get,
                             Launchers<LBM_LAT, LBM_ST>::set, Launchers<LBM_LAT, LBM_ST>::halo,
                             Launchers<LBM_LAT, LBM_ST>::shift_rest, kMaxTiles,

@@ -46,6 +46,12 @@ extern "C" {
 int lbm_sg_conv3x3(const void* x, int csx, const void* w, const float* bias, float* y, int csy, int N, int H, int W,
                    int Ci, int Co, void* stream);
 
+/* lbm_sg_conv3x3 with the ReLU in its epilogue: y (bf16, stride csy) =
+ * max(convolution + bias, 0) rounded to bf16, the values lbm_sg_relu gives for
+ * lbm_sg_conv3x3's output.  Arguments and errors as lbm_sg_conv3x3. */
+int lbm_sg_conv3x3_relu(const void* x, int csx, const void* w, const float* bias, void* y, int csy, int N, int H,
+                        int W, int Ci, int Co, void* stream);
+
 /* Synchronises `stream` and reports whether a bounded wait of a surrogate
  * kernel gave up since the last call: LBM_ETIMEOUT (the flag is cleared),
  * else LBM_OK; LBM_ECUDA if the copy or the synchronisation failed. */
@@ -104,6 +110,30 @@ int lbm_sg_upsample(const void* x, int csx, void* y, int csy, int N, int H, int 
 int lbm_sg_upsample_bwd(const float* g, int csg, float* gx, int csx, int N, int H, int W, int C, int f,
                         void* stream);
 
+#define LBM_SG_GRAD_BLOCKS 512
+
+/* Gradient through a layer's ReLU and its bias gradient in one pass: ga (bf16,
+ * stride C) = v rounded, v = gradient where act (bf16, stride csa, the layer's
+ * output after the ReLU) is positive, else 0; gb[c] = sum of the FP32 v over
+ * the pixels (fixed order).  The gradient of the H x W layer's output is g
+ * (float, stride csg; up = 1), the sums of g over 2 x 2 blocks of a 2H x 2W
+ * image (up = 2: the layer's output was upsampled), or g + gp / 4 spread over
+ * 2 x 2 blocks (gp not NULL, float, H/2 x W/2, stride csp, up = 1: it was
+ * pooled as well).  C and the strides are multiples of 4, C at most 1024; g, gp
+ * and scratch start on 16-byte boundaries, act and ga on 8-byte ones, else
+ * LBM_EINVAL.  scratch: LBM_SG_GRAD_BLOCKS * C floats are always enough. */
+int lbm_sg_relu_grad(const float* g, int csg, int up, const float* gp, int csp, const void* act, int csa, void* ga,
+                     float* gb, float* scratch, long long scratch_floats, int N, int H, int W, int C, void* stream);
+
+/* lbm_sg_mse for the four-channel output layer, with what its backward pass
+ * reads: *loss as there; g16 (bf16, 16 channels, the last 12 zero) = the
+ * gradient rounded; gb (16 floats, the last 12 zero) = its sums over the pixels
+ * from the FP32 values.  x and target have 4 channels, delta 16; x, delta,
+ * target, g16 and scratch start on 16-byte boundaries.  scratch: 3 *
+ * LBM_SG_GRAD_BLOCKS doubles. */
+int lbm_sg_mse_grad(const float* x, const float* delta, const float* target, void* g16, float* gb, double* scratch,
+                    double* loss, long long npix, void* stream);
+
 /* Mean squared error of out = x + delta against target over the first C
  * channels: *loss (device double) = mean (out - target)^2 (FP64 sums), and
  * g (float, stride csd) = d loss / d delta (zero in channels C..csd-1).
@@ -116,6 +146,23 @@ int lbm_sg_mse(const float* x, int csx, const float* delta, int csd, const float
  * weights the convolutions read. */
 int lbm_sg_adam(float* w, float* m, float* v, const float* g, long long n, float lr, float b1, float b2, float eps,
                 int step, void* w16, void* stream);
+
+/* A layer as lbm_sg_adam_layers takes it. */
+typedef struct {
+    float *w, *mw, *vw;
+    const float* gw;
+    float *b, *mb, *vb;
+    const float* gb;
+    void *w16, *wt;
+    int ci, co;
+} lbm_sg_layer;
+
+/* One Adam update (as lbm_sg_adam) of the weights [co][9][ci] and biases [co]
+ * of up to 16 layers in one launch; w16 receives the rounded weights and wt
+ * their flipped form (lbm_sg_weight_flip of w16).  No pointer may be NULL; ci
+ * and co are at most 4096. */
+int lbm_sg_adam_layers(const lbm_sg_layer* layers, int n, float lr, float b1, float b2, float eps, int step,
+                       void* stream);
 
 /* Network input from one grid's fields (device FP64, x fastest, as
  * lbm_macro writes them: phi, the two components of rho u, P): x32 (float,

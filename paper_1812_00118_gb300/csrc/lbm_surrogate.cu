@@ -143,9 +143,49 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 16 channels of one pixel of a convolution's output, as FP32 or (ACT) as the
+// bf16 values after the ReLU, which is all the next layer and the backward
+// pass read of them; `vec`: the row starts on a 16-byte boundary.
+template <bool ACT>
+__device__ __forceinline__ void conv_store16(void* y, long long at, float (&v)[16], const float* __restrict__ bias,
+                                             bool vec) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] += bias ? bias[i] : 0.0f;
+    if constexpr (ACT) {
+        bf16* out = (bf16*)y + at;
+        __nv_bfloat162 h[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            h[i] = __floats2bfloat162_rn(fmaxf(v[2 * i], 0.0f), fmaxf(v[2 * i + 1], 0.0f));
+        if (vec) {
+            const uint4* q = reinterpret_cast<const uint4*>(h);
+            reinterpret_cast<uint4*>(out)[0] = q[0];
+            reinterpret_cast<uint4*>(out)[1] = q[1];
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) { out[2 * i] = h[i].x; out[2 * i + 1] = h[i].y; }
+        }
+    } else {
+        float* out = (float*)y + at;
+        if (vec) {
+#pragma unroll
+            for (int i = 0; i < 16; i += 4)
+                *reinterpret_cast<float4*>(out + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) out[i] = v[i];
+        }
+    }
+}
+template <bool ACT>
+__device__ __forceinline__ bool conv_vec(const void* y, int csy) {
+    return (csy & (ACT ? 7 : 3)) == 0 && ((uintptr_t)y & 15) == 0;
+}
+
+template <bool ACT>
 __global__ void __launch_bounds__(128, 1)
 conv_tc_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, const float* __restrict__ bias,
-               float* __restrict__ y, int csy, long long M, int H, int W, int Ci, int Co, int* err) {
+               void* __restrict__ y, int csy, long long M, int H, int W, int Ci, int Co, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[kTcBuf];
     __shared__ uint32_t tmem_slot;
@@ -244,23 +284,11 @@ conv_tc_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, 
     if (ok) {
         const long long pr = p0 + 32 * warp + lane;
         const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);
-        const bool vec = (csy & 3) == 0 && ((uintptr_t)y & 15) == 0;
+        const bool vec = conv_vec<ACT>(y, csy);
         for (int c0 = 0; c0 < Co; c0 += 16) {
             float v[16];
             tc_ld16(trow + (uint32_t)c0, v);
-            if (pr < M) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] += bias ? bias[c0 + i] : 0.0f;
-                float* out = y + pr * csy + c0;
-                if (vec) {
-#pragma unroll
-                    for (int i = 0; i < 16; i += 4)
-                        *reinterpret_cast<float4*>(out + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) out[i] = v[i];
-                }
-            }
+            if (pr < M) conv_store16<ACT>(y, pr * csy + c0, v, bias ? bias + c0 : nullptr, vec);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -310,9 +338,10 @@ __host__ __device__ inline uint32_t row_tmem_cols(int Co) {
     return need <= 32 ? 32u : (need <= 64 ? 64u : (need <= 128 ? 128u : 256u));
 }
 
+template <bool ACT>
 __global__ void __launch_bounds__(128, 1)
 conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, const float* __restrict__ bias,
-                float* __restrict__ y, int csy, int N, int H, int W, int Ci, int Co, int rows_per_cta, int* err) {
+                void* __restrict__ y, int csy, int N, int H, int W, int Ci, int Co, int rows_per_cta, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[2];
     __shared__ uint32_t tmem_slot;
@@ -375,21 +404,11 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
         const int r = y0 + j;
         const uint32_t acc = tmem + (uint32_t)((j & 1) * Co) + ((uint32_t)(32 * warp) << 16);
         const long long pix = img + (long long)r * W + x0 + 32 * warp + lane;
-        float* out = y + pix * csy;
-        const bool vec = (csy & 3) == 0 && ((uintptr_t)y & 15) == 0;
+        const bool vec = conv_vec<ACT>(y, csy);
         for (int c0 = 0; c0 < Co; c0 += 16) {
             float v[16];
             tc_ld16(acc + (uint32_t)c0, v);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] += bias ? bias[c0 + i] : 0.0f;
-            if (vec) {
-#pragma unroll
-                for (int i = 0; i < 16; i += 4)
-                    *reinterpret_cast<float4*>(out + c0 + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) out[c0 + i] = v[i];
-            }
+            conv_store16<ACT>(y, pix * csy + c0, v, bias ? bias + c0 : nullptr, vec);
         }
     };
     const int nrows = y1 - y0;
@@ -787,6 +806,64 @@ __global__ void pool_kernel(const bf16* __restrict__ x, int csx, bf16* __restric
     y[q * csy + c] = __float2bfloat16_rn(s / (float)(f * f));
 }
 
+// 2 x 2 pooling and upsampling on 8 channels (16 bytes) per thread: the
+// per-element kernels spend their time on 64-bit index divisions (8 x 256^2 x
+// 32 channels: pooling 53 us, upsampling 121 us).  The sums are formed in the
+// order of pool_kernel.
+__device__ __forceinline__ void unpack8(uint4 q, float (&v)[8]) {
+    const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        v[2 * i] = __uint_as_float(u[i] << 16);
+        v[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u);
+    }
+}
+
+__global__ void pool2_kernel(const bf16* __restrict__ x, int csx, bf16* __restrict__ y, int csy, int nrows, int Wc,
+                             int C8) {
+    // blockIdx.y: coarse row over all images; its two fine rows are 2 r, 2 r + 1
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= Wc * C8) return;
+    const int xc = k / C8, c = (k - xc * C8) * 8;
+    for (int r = blockIdx.y; r < nrows; r += gridDim.y) {
+        const bf16* p = x + ((long long)(2 * r) * (2 * Wc) + 2 * xc) * csx + c;
+        const bf16* q = p + (long long)(2 * Wc) * csx;
+        float a[8], b[8], d[8], e[8];
+        unpack8(*reinterpret_cast<const uint4*>(p), a);
+        unpack8(*reinterpret_cast<const uint4*>(p + csx), b);
+        unpack8(*reinterpret_cast<const uint4*>(q), d);
+        unpack8(*reinterpret_cast<const uint4*>(q + csx), e);
+        __nv_bfloat162 o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float s[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int m = 2 * i + j;
+                s[j] = (((a[m] + b[m]) + d[m]) + e[m]) * 0.25f;
+            }
+            o[i] = __floats2bfloat162_rn(s[0], s[1]);
+        }
+        *reinterpret_cast<uint4*>(y + ((long long)r * Wc + xc) * csy + c) = *reinterpret_cast<uint4*>(o);
+    }
+}
+
+__global__ void upsample2_kernel(const bf16* __restrict__ x, int csx, bf16* __restrict__ y, int csy, int nrows, int Wc,
+                                 int C8) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= Wc * C8) return;
+    const int xc = k / C8, c = (k - xc * C8) * 8;
+    for (int r = blockIdx.y; r < nrows; r += gridDim.y) {
+        const uint4 v = *reinterpret_cast<const uint4*>(x + ((long long)r * Wc + xc) * csx + c);
+        bf16* p = y + ((long long)(2 * r) * (2 * Wc) + 2 * xc) * csy + c;
+        bf16* q = p + (long long)(2 * Wc) * csy;
+        *reinterpret_cast<uint4*>(p) = v;
+        *reinterpret_cast<uint4*>(p + csy) = v;
+        *reinterpret_cast<uint4*>(q) = v;
+        *reinterpret_cast<uint4*>(q + csy) = v;
+    }
+}
+
 // gx[fine] = g[coarse] / f^2
 __global__ void pool_bwd_kernel(const float* __restrict__ g, int csg, float* __restrict__ gx, int csx, int N, int H,
                                 int W, int C, int f) {
@@ -859,6 +936,141 @@ __global__ void colsum_finish_kernel(const float* __restrict__ part, int nb, int
     out[c] = s;
 }
 
+// Gradient through a layer's ReLU, fused with what feeds it and with what reads
+// it: v = act > 0 ? gradient : 0 as bf16 (the operand of the two gradient
+// convolutions), and the bias gradient's block partials from the FP32 v.  The
+// gradient of the activation is g (MODE 0), the sum of g over the 2 x 2 fine
+// pixels of an upsampling (MODE 1), or g plus a quarter of the pooled path's
+// gradient gp (MODE 2).  One pass over memory where the separate kernels
+// (pooling or upsampling backward, addition, ReLU, column sums) took up to
+// seven and an FP32 copy of v in between (the 8 x 256^2 x 32 level: 342 us).
+// Four channels per thread; H x W the layer's own size.
+template <int MODE>
+__global__ void __launch_bounds__(kThreads)
+relu_grad_kernel(const float* __restrict__ g, int csg, const float* __restrict__ gp, int csp,
+                 const bf16* __restrict__ act, int csa, bf16* __restrict__ out, int H, int W, int npix, int C,
+                 float* __restrict__ part) {
+    __shared__ float4 sh[kThreads];
+    const int C4 = C / 4, lanes = kThreads / C4;       // pixels a block takes at a time
+    const int c = (threadIdx.x % C4) * 4, lane = threadIdx.x / C4;
+    float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int p = blockIdx.x * lanes + lane; lane < lanes && p < npix; p += gridDim.x * lanes) {
+        float4 v;
+        if constexpr (MODE == 0) {
+            v = *reinterpret_cast<const float4*>(g + (long long)p * csg + c);
+        } else {
+            const int row = p / W, x = p - row * W;     // row over all images
+            if constexpr (MODE == 1) {
+                const float* q = g + ((long long)(2 * row) * (2 * W) + 2 * x) * csg + c;
+                const float4 a = *reinterpret_cast<const float4*>(q);
+                const float4 b = *reinterpret_cast<const float4*>(q + csg);
+                q += (long long)(2 * W) * csg;
+                const float4 d = *reinterpret_cast<const float4*>(q);
+                const float4 e = *reinterpret_cast<const float4*>(q + csg);
+                v = make_float4(((a.x + b.x) + d.x) + e.x, ((a.y + b.y) + d.y) + e.y, ((a.z + b.z) + d.z) + e.z,
+                                ((a.w + b.w) + d.w) + e.w);
+            } else {
+                const float4 a = *reinterpret_cast<const float4*>(g + (long long)p * csg + c);
+                const float4 b = *reinterpret_cast<const float4*>(
+                    gp + ((long long)(row >> 1) * (W >> 1) + (x >> 1)) * csp + c);
+                v = make_float4(a.x + b.x * 0.25f, a.y + b.y * 0.25f, a.z + b.z * 0.25f, a.w + b.w * 0.25f);
+            }
+        }
+        const uint2 m = *reinterpret_cast<const uint2*>(act + (long long)p * csa + c);
+        v.x = __uint_as_float(m.x << 16) > 0.0f ? v.x : 0.0f;
+        v.y = __uint_as_float(m.x & 0xffff0000u) > 0.0f ? v.y : 0.0f;
+        v.z = __uint_as_float(m.y << 16) > 0.0f ? v.z : 0.0f;
+        v.w = __uint_as_float(m.y & 0xffff0000u) > 0.0f ? v.w : 0.0f;
+        __nv_bfloat162 o[2] = {__floats2bfloat162_rn(v.x, v.y), __floats2bfloat162_rn(v.z, v.w)};
+        *reinterpret_cast<uint2*>(out + (long long)p * C + c) = *reinterpret_cast<uint2*>(o);
+        sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+    }
+    sh[threadIdx.x] = sum;
+    __syncthreads();
+    if ((int)threadIdx.x < C4) {
+        for (int l = 1; l < lanes; ++l) {
+            const float4 t = sh[threadIdx.x + l * C4];
+            sum.x += t.x; sum.y += t.y; sum.z += t.z; sum.w += t.w;
+        }
+        *reinterpret_cast<float4*>(part + (long long)blockIdx.x * C + c) = sum;
+    }
+}
+
+// out[c] = sum of part[b][c] over the blocks: one warp per channel, fixed order
+__global__ void channel_finish_kernel(const float* __restrict__ part, int nb, int C, float* __restrict__ out) {
+    const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (c >= C) return;
+    float s = 0.0f;
+    for (int b = lane; b < nb; b += 32) s += part[(long long)b * C + c];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) out[c] = s;
+}
+
+// Loss of out = x + delta against t over four channels, its gradient as the
+// bf16 operand of the output layer's gradient convolutions (16 channels, the
+// padded ones zero) and the output layer's bias gradient: one thread per pixel.
+// part: the block's FP64 loss sum; gpart: its sums of the FP32 gradient.
+__global__ void __launch_bounds__(kThreads)
+mse_grad_kernel(const float4* __restrict__ x, const float* __restrict__ delta, const float4* __restrict__ t,
+                bf16* __restrict__ g16, int npix, double inv, double* __restrict__ part, float* __restrict__ gpart) {
+    __shared__ double sh[kThreads];
+    __shared__ float4 gs[kThreads];
+    double s = 0.0;
+    float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int p = blockIdx.x * kThreads + threadIdx.x; p < npix; p += gridDim.x * kThreads) {
+        const float4 a = x[p], d = *reinterpret_cast<const float4*>(delta + (long long)p * 16), b = t[p];
+        const double e[4] = {(double)a.x + (double)d.x - (double)b.x, (double)a.y + (double)d.y - (double)b.y,
+                             (double)a.z + (double)d.z - (double)b.z, (double)a.w + (double)d.w - (double)b.w};
+        float g[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            s += e[k] * e[k];
+            g[k] = (float)(2.0 * e[k] * inv);
+        }
+        sum.x += g[0]; sum.y += g[1]; sum.z += g[2]; sum.w += g[3];
+        __nv_bfloat162 o[4] = {__floats2bfloat162_rn(g[0], g[1]), __floats2bfloat162_rn(g[2], g[3]),
+                               __floats2bfloat162_rn(0.0f, 0.0f), __floats2bfloat162_rn(0.0f, 0.0f)};
+        uint4* q = reinterpret_cast<uint4*>(g16 + (long long)p * 16);
+        q[0] = *reinterpret_cast<uint4*>(o);
+        q[1] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    sh[threadIdx.x] = s;
+    gs[threadIdx.x] = sum;
+    __syncthreads();
+    for (int o = kThreads / 2; o > 0; o >>= 1) {
+        if (threadIdx.x < o) {
+            sh[threadIdx.x] += sh[threadIdx.x + o];
+            float4& u = gs[threadIdx.x];
+            const float4 v = gs[threadIdx.x + o];
+            u.x += v.x; u.y += v.y; u.z += v.z; u.w += v.w;
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = sh[0];
+        *reinterpret_cast<float4*>(gpart + 4 * blockIdx.x) = gs[0];
+    }
+}
+
+// loss and the 16 entries of the output layer's bias gradient (4 real) from the
+// block partials: one warp each
+__global__ void mse_grad_finish_kernel(const double* __restrict__ part, const float* __restrict__ gpart, int nb,
+                                       double inv_count, double* __restrict__ loss, float* __restrict__ gb) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w == 0) {
+        double s = 0.0;
+        for (int b = lane; b < nb; b += 32) s += part[b];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) loss[0] = s * inv_count;
+        if (lane >= 4 && lane < 16) gb[lane] = 0.0f;
+    } else if (w <= 4) {
+        float s = 0.0f;
+        for (int b = lane; b < nb; b += 32) s += gpart[4 * b + w - 1];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) gb[w - 1] = s;
+    }
+}
+
 // out = x + delta on the first C channels; g = 2 (out - t) / (npix C) (zero beyond C up to csd);
 // block partials of sum (out - t)^2 in FP64
 __global__ void mse_kernel(const float* __restrict__ x, int csx, const float* __restrict__ delta, int csd,
@@ -909,6 +1121,40 @@ __global__ void adam_kernel(float* __restrict__ w, float* __restrict__ m, float*
     const float wk = w[k] - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
     w[k] = wk;
     if (w16) w16[k] = __float2bfloat16_rn(wk);
+}
+
+// Adam on every layer of a network at once: the weights (with their bf16 copy
+// and its flipped form, the operand of the input-gradient convolution) and the
+// biases.  blockIdx.y is the layer.
+constexpr int kMaxLayers = 16;
+struct AdamLayers {
+    lbm_sg_layer l[kMaxLayers];
+};
+__device__ __forceinline__ float adam_one(float* w, float* m, float* v, const float* g, long long k, float lr, float b1,
+                                          float b2, float eps, float c1, float c2) {
+    const float gk = g[k];
+    const float mk = b1 * m[k] + (1.0f - b1) * gk;
+    const float vk = b2 * v[k] + (1.0f - b2) * gk * gk;
+    m[k] = mk;
+    v[k] = vk;
+    const float wk = w[k] - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
+    w[k] = wk;
+    return wk;
+}
+__global__ void adam_layers_kernel(const __grid_constant__ AdamLayers a, float lr, float b1, float b2, float eps,
+                                   float c1, float c2) {
+    const lbm_sg_layer& l = a.l[blockIdx.y];
+    const int n = l.co * 9 * l.ci;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n + l.co; k += gridDim.x * blockDim.x) {
+        if (k < n) {
+            const bf16 h = __float2bfloat16_rn(adam_one(l.w, l.mw, l.vw, l.gw, k, lr, b1, b2, eps, c1, c2));
+            ((bf16*)l.w16)[k] = h;
+            const int row = k / l.ci, ci = k - row * l.ci, co = row / 9, tap = row - co * 9;
+            ((bf16*)l.wt)[((long long)ci * 9 + (8 - tap)) * l.co + co] = h;
+        } else {
+            adam_one(l.b, l.mb, l.vb, l.gb, k - n, lr, b1, b2, eps, c1, c2);
+        }
+    }
 }
 
 // LB fields (FP64, x fastest: phi, rho u_x, rho u_y, P) -> normalised channels-last input: channel c = field c / scale c
@@ -1112,22 +1358,23 @@ size_t conv_row_launch_smem(size_t need, int Co) {
 
 // Resident row-march CTAs on the current device (SMs x CTAs per SM), with the
 // attribute for large dynamic shared memory set once per device.
+template <bool ACT>
 cudaError_t conv_row_slots(size_t need, int Co, int* out) {
     static bool attr_set[64] = {};
     int dev = 0, sms = 0, occ = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        e = cudaFuncSetAttribute(conv_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
+        e = cudaFuncSetAttribute(conv_row_kernel<ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(conv_row_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+            e = cudaFuncSetAttribute(conv_row_kernel<ACT>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, conv_row_kernel, kRowM, conv_row_launch_smem(need, Co));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, conv_row_kernel<ACT>, kRowM, conv_row_launch_smem(need, Co));
     if (e != cudaSuccess) return e;
     *out = sms * (occ > 0 ? occ : 1);
     return cudaSuccess;
@@ -1194,7 +1441,10 @@ bool conv_dims_ok(long long M, int Ci, int Co) { return M > 0 && M % 16 == 0 && 
 
 extern "C" {
 
-int lbm_sg_conv3x3(const void* x, int csx, const void* w, const float* bias, float* y, int csy, int N, int H, int W,
+}  // extern "C"
+
+template <bool ACT>
+static int conv3x3(const void* x, int csx, const void* w, const float* bias, void* y, int csy, int N, int H, int W,
                    int Ci, int Co, void* stream) {
     const long long M = (long long)N * H * W;
     if (!x || !w || !y || N < 1 || H < 1 || W < 1 || !conv_dims_ok(M, Ci, Co) || csx < Ci || csx % 2 || csy < Co)
@@ -1208,7 +1458,7 @@ int lbm_sg_conv3x3(const void* x, int csx, const void* w, const float* bias, flo
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return LBM_ECUDA;
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        if (cudaFuncSetAttribute(conv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(conv_tc_kernel<ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)conv_tc_smem_bytes(kTcK, 128)) != cudaSuccess)
             return LBM_ECUDA;
         attr_set[dev] = true;
@@ -1220,7 +1470,7 @@ int lbm_sg_conv3x3(const void* x, int csx, const void* w, const float* bias, flo
     const size_t row_smem = conv_row_smem_bytes(Ci, Co);
     if (W % kRowM == 0 && H >= 2 && row_smem <= kRowSmemMax) {
         int slots = 0;
-        if (conv_row_slots(row_smem, Co, &slots) != cudaSuccess) {
+        if (conv_row_slots<ACT>(row_smem, Co, &slots) != cudaSuccess) {
             cudaGetLastError();
             return LBM_ECUDA;
         }
@@ -1237,13 +1487,25 @@ int lbm_sg_conv3x3(const void* x, int csx, const void* w, const float* bias, flo
         if (chunks > H) chunks = H;
         const int rows = (int)((H + chunks - 1) / chunks);
         const long long nb = cols * ((H + rows - 1) / rows);
-        conv_row_kernel<<<(unsigned)nb, kRowM, conv_row_launch_smem(row_smem, Co), s>>>(
+        conv_row_kernel<ACT><<<(unsigned)nb, kRowM, conv_row_launch_smem(row_smem, Co), s>>>(
             (const bf16*)x, csx, (const bf16*)w, bias, y, csy, N, H, W, Ci, Co, rows, err);
         return check(cudaGetLastError());
     }
     const unsigned nb = (unsigned)((M + kTcM - 1) / kTcM);
-    conv_tc_kernel<<<nb, kTcM, smem, s>>>((const bf16*)x, csx, (const bf16*)w, bias, y, csy, M, H, W, Ci, Co, err);
+    conv_tc_kernel<ACT><<<nb, kTcM, smem, s>>>((const bf16*)x, csx, (const bf16*)w, bias, y, csy, M, H, W, Ci, Co, err);
     return check(cudaGetLastError());
+}
+
+extern "C" {
+
+int lbm_sg_conv3x3(const void* x, int csx, const void* w, const float* bias, float* y, int csy, int N, int H, int W,
+                   int Ci, int Co, void* stream) {
+    return conv3x3<false>(x, csx, w, bias, y, csy, N, H, W, Ci, Co, stream);
+}
+
+int lbm_sg_conv3x3_relu(const void* x, int csx, const void* w, const float* bias, void* y, int csy, int N, int H,
+                        int W, int Ci, int Co, void* stream) {
+    return conv3x3<true>(x, csx, w, bias, y, csy, N, H, W, Ci, Co, stream);
 }
 
 int lbm_sg_status(void* stream) {
@@ -1361,9 +1623,86 @@ static bool pool_dims_ok(int N, int H, int W, int C, int f) {
     return N >= 1 && f >= 1 && f <= 64 && H >= f && W >= f && H % f == 0 && W % f == 0 && C >= 1;
 }
 
+// 2 x 2 blocks of 16-byte channel groups (pool2_kernel, upsample2_kernel), with
+// 32-bit row and column counts
+static bool wide_ok(const void* x, int csx, const void* y, int csy, int N, int H, int W, int C, int f) {
+    return f == 2 && C % 8 == 0 && csx % 8 == 0 && csy % 8 == 0 && ((uintptr_t)x & 15) == 0 && ((uintptr_t)y & 15) == 0 &&
+           (long long)N * H < (1LL << 31) && (long long)W * C < (1LL << 31);
+}
+static dim3 wide_grid(int N, int H, int W, int C) {
+    const int rows = N * (H / 2);
+    return dim3(blocks((long long)(W / 2) * (C / 8)), rows < 16384 ? rows : 16384);
+}
+
+int lbm_sg_relu_grad(const float* g, int csg, int up, const float* gp, int csp, const void* act, int csa, void* ga,
+                     float* gb, float* scratch, long long scratch_floats, int N, int H, int W, int C, void* stream) {
+    const long long npix = (long long)N * H * W;
+    if (!g || !act || !ga || !gb || !scratch || N < 1 || H < 1 || W < 1 || npix >= (1LL << 30)) return LBM_EINVAL;
+    if ((up != 1 && up != 2) || (gp && (up != 1 || H % 2 || W % 2 || csp < C || csp % 4))) return LBM_EINVAL;
+    if (C < 4 || C % 4 || C > 4 * kThreads || csg < C || csg % 4 || csa < C || csa % 4) return LBM_EINVAL;
+    if (((uintptr_t)g & 15) || ((uintptr_t)gp & 15) || ((uintptr_t)act & 7) || ((uintptr_t)ga & 7) ||
+        ((uintptr_t)scratch & 15))
+        return LBM_EINVAL;
+    // about 16 pixels per thread, at most the blocks the scratch holds partials of
+    const int lanes = kThreads / (C / 4);
+    long long nb = (npix + 16LL * lanes - 1) / (16LL * lanes);
+    if (nb > LBM_SG_GRAD_BLOCKS) nb = LBM_SG_GRAD_BLOCKS;
+    if (scratch_floats < nb * C) return LBM_EINVAL;
+    cudaStream_t s = (cudaStream_t)stream;
+    const bf16* a = (const bf16*)act;
+    bf16* o = (bf16*)ga;
+    const int np = (int)npix;
+    if (gp) relu_grad_kernel<2><<<(unsigned)nb, kThreads, 0, s>>>(g, csg, gp, csp, a, csa, o, H, W, np, C, scratch);
+    else if (up == 2) relu_grad_kernel<1><<<(unsigned)nb, kThreads, 0, s>>>(g, csg, gp, csp, a, csa, o, H, W, np, C, scratch);
+    else relu_grad_kernel<0><<<(unsigned)nb, kThreads, 0, s>>>(g, csg, gp, csp, a, csa, o, H, W, np, C, scratch);
+    channel_finish_kernel<<<(C + 7) / 8, kThreads, 0, s>>>(scratch, (int)nb, C, gb);
+    return check(cudaGetLastError());
+}
+
+int lbm_sg_mse_grad(const float* x, const float* delta, const float* target, void* g16, float* gb, double* scratch,
+                    double* loss, long long npix, void* stream) {
+    if (!x || !delta || !target || !g16 || !gb || !scratch || !loss || npix < 1 || npix >= (1LL << 30)) return LBM_EINVAL;
+    if (((uintptr_t)x & 15) || ((uintptr_t)delta & 15) || ((uintptr_t)target & 15) || ((uintptr_t)g16 & 15) ||
+        ((uintptr_t)scratch & 15))
+        return LBM_EINVAL;
+    long long nb = (npix + kThreads - 1) / kThreads;
+    if (nb > LBM_SG_GRAD_BLOCKS) nb = LBM_SG_GRAD_BLOCKS;
+    cudaStream_t s = (cudaStream_t)stream;
+    float* gpart = (float*)(scratch + LBM_SG_GRAD_BLOCKS);
+    const double inv = 1.0 / ((double)npix * 4);
+    mse_grad_kernel<<<(unsigned)nb, kThreads, 0, s>>>((const float4*)x, delta, (const float4*)target, (bf16*)g16, (int)npix,
+                                                      inv, scratch, gpart);
+    mse_grad_finish_kernel<<<1, 160, 0, s>>>(scratch, gpart, (int)nb, inv, loss, gb);
+    return check(cudaGetLastError());
+}
+
+int lbm_sg_adam_layers(const lbm_sg_layer* layers, int n, float lr, float b1, float b2, float eps, int step,
+                       void* stream) {
+    if (!layers || n < 1 || n > kMaxLayers || step < 1 || !(lr > 0) || !(b1 >= 0 && b1 < 1) || !(b2 >= 0 && b2 < 1))
+        return LBM_EINVAL;
+    AdamLayers a = {};
+    int most = 0;
+    for (int k = 0; k < n; ++k) {
+        const lbm_sg_layer& l = layers[k];
+        if (!l.w || !l.mw || !l.vw || !l.gw || !l.b || !l.mb || !l.vb || !l.gb || !l.w16 || !l.wt || l.ci < 1 || l.co < 1 ||
+            l.ci > 4096 || l.co > 4096)
+            return LBM_EINVAL;
+        a.l[k] = l;
+        if (l.co * 9 * l.ci + l.co > most) most = l.co * 9 * l.ci + l.co;
+    }
+    const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
+    adam_layers_kernel<<<dim3(blocks(most), n), kThreads, 0, (cudaStream_t)stream>>>(a, lr, b1, b2, eps, c1, c2);
+    return check(cudaGetLastError());
+}
+
 int lbm_sg_pool(const void* x, int csx, void* y, int csy, int N, int H, int W, int C, int f, void* stream) {
     if (!x || !y || !pool_dims_ok(N, H, W, C, f) || csx < C || csy < C) return LBM_EINVAL;
     const long long n = (long long)N * (H / f) * (W / f) * C;
+    if (wide_ok(x, csx, y, csy, N, H, W, C, f)) {
+        pool2_kernel<<<wide_grid(N, H, W, C), kThreads, 0, (cudaStream_t)stream>>>((const bf16*)x, csx, (bf16*)y, csy,
+                                                                                  N * (H / 2), W / 2, C / 8);
+        return check(cudaGetLastError());
+    }
     pool_kernel<<<blocks(n), kThreads, 0, (cudaStream_t)stream>>>((const bf16*)x, csx, (bf16*)y, csy, N, H, W, C, f);
     return check(cudaGetLastError());
 }
@@ -1377,6 +1716,11 @@ int lbm_sg_pool_bwd(const float* g, int csg, float* gx, int csx, int N, int H, i
 
 int lbm_sg_upsample(const void* x, int csx, void* y, int csy, int N, int H, int W, int C, int f, void* stream) {
     if (!x || !y || !pool_dims_ok(N, H, W, C, f) || csx < C || csy < C) return LBM_EINVAL;
+    if (wide_ok(x, csx, y, csy, N, H, W, C, f)) {
+        upsample2_kernel<<<wide_grid(N, H, W, C), kThreads, 0, (cudaStream_t)stream>>>(
+            (const bf16*)x, csx, (bf16*)y, csy, N * (H / 2), W / 2, C / 8);
+        return check(cudaGetLastError());
+    }
     upsample_kernel<<<blocks((long long)N * H * W * C), kThreads, 0, (cudaStream_t)stream>>>((const bf16*)x, csx,
                                                                                             (bf16*)y, csy, N, H, W, C,
                                                                                             f);

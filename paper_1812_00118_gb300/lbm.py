@@ -53,6 +53,11 @@ class lbm_params(ctypes.Structure):
                 ("C_dtheta", ctypes.c_double)]
 
 
+class lbm_sg_layer(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_void_p) for k in ("w", "mw", "vw", "gw", "b", "mb", "vb", "gb", "w16", "wt")] + \
+               [("ci", ctypes.c_int), ("co", ctypes.c_int)]
+
+
 _lib = None
 
 # (name, restype, argtypes) of every symbol include/lbm.h declares
@@ -98,6 +103,7 @@ SIGNATURES = [
                                       ctypes.c_int]),
     ("lbm_batch_destroy", None, [_VP]),
     ("lbm_sg_conv3x3", ctypes.c_int, [_VP, ctypes.c_int, _VP, _VP, _VP, ctypes.c_int] + [ctypes.c_int] * 5 + [_VP]),
+    ("lbm_sg_conv3x3_relu", ctypes.c_int, [_VP, ctypes.c_int, _VP, _VP, _VP, ctypes.c_int] + [ctypes.c_int] * 5 + [_VP]),
     ("lbm_sg_wgrad_scratch_floats", ctypes.c_longlong, [ctypes.c_int] * 5),
     ("lbm_sg_conv3x3_wgrad", ctypes.c_int, [_VP, ctypes.c_int, _VP, ctypes.c_int, _VP, _VP, ctypes.c_longlong]
      + [ctypes.c_int] * 5 + [_VP]),
@@ -118,6 +124,11 @@ SIGNATURES = [
     ("lbm_sg_upsample_bwd", ctypes.c_int, [_VP, ctypes.c_int, _VP, ctypes.c_int] + [ctypes.c_int] * 5 + [_VP]),
     ("lbm_sg_mse", ctypes.c_int, [_VP, ctypes.c_int, _VP, ctypes.c_int, _VP, ctypes.c_int, _VP, _VP, _VP,
                                   ctypes.c_longlong, ctypes.c_int, _VP]),
+    ("lbm_sg_relu_grad", ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int, _VP, ctypes.c_int, _VP, ctypes.c_int, _VP, _VP,
+                                        _VP, ctypes.c_longlong] + [ctypes.c_int] * 4 + [_VP]),
+    ("lbm_sg_mse_grad", ctypes.c_int, [_VP] * 7 + [ctypes.c_longlong, _VP]),
+    ("lbm_sg_adam_layers", ctypes.c_int, [ctypes.POINTER(lbm_sg_layer), ctypes.c_int, ctypes.c_float, ctypes.c_float,
+                                          ctypes.c_float, ctypes.c_float, ctypes.c_int, _VP]),
     ("lbm_sg_adam", ctypes.c_int, [_VP, _VP, _VP, _VP, ctypes.c_longlong, ctypes.c_float, ctypes.c_float,
                                    ctypes.c_float, ctypes.c_float, ctypes.c_int, _VP, _VP]),
     ("lbm_sg_pack", ctypes.c_int, [_VP, _VP, _VP, _VP, _DP, _VP, ctypes.c_int, _VP, ctypes.c_int, ctypes.c_longlong,

@@ -30,6 +30,7 @@ LAYERS = [("e1", 4, 32), ("e2", 32, 64), ("e3", 64, 128), ("b", 128, 128),
 POOL = 2      # pooling / upsampling factor between levels
 LEVELS = 4
 NC = 4        # real channels of the input and output: phi, rho u_x, rho u_y, P
+GRAD_BLOCKS = 512   # LBM_SG_GRAD_BLOCKS of include/lbm_surrogate.h
 CO_MAX = 128  # output channels one lbm_sg_conv3x3 call produces at most
 
 
@@ -90,23 +91,19 @@ class Surrogate:
                                      gW=z(cop, 9, cip), gb=z(cop))
         self.set_params(params if params is not None else init_params(seed))
         M1, M2, M3, M4 = self.M
-        # forward activations: pre-activations (FP32) for the ReLU backward,
-        # post-activations (bf16) as the next layer's input
+        # forward activations after the ReLU (bf16): the next layer's input, and
+        # the mask of the ReLU's backward
         self.x16, self.x32 = z(M1, 16, dt=b16), z(M1, NC)
-        self.a = {"e1": z(M1, 32), "e2": z(M2, 64), "e3": z(M3, 128), "b": z(M4, 128),
-                  "d3": z(M3, 64), "d2": z(M2, 32), "d1": z(M1, 32)}
         self.cat1, self.cat2, self.cat3 = z(M1, 64, dt=b16), z(M2, 128, dt=b16), z(M3, 256, dt=b16)
         self.p1, self.p2, self.p3 = z(M2, 32, dt=b16), z(M3, 64, dt=b16), z(M4, 128, dt=b16)
         self.hb, self.h3, self.h2, self.h1 = z(M4, 128, dt=b16), z(M3, 64, dt=b16), z(M2, 32, dt=b16), z(M1, 32, dt=b16)
         self.delta = z(M1, 16)
-        # backward buffers (FP32 gradients and their bf16 copies per level)
-        self.g_delta, self.g16_1 = z(M1, 16), z(M1, 64, dt=b16)
-        self.gc1, self.gs1, self.ga1 = z(M1, 64), z(M1, 32), z(M1, 32)
-        self.gc2, self.gs2, self.ga2, self.g16_2 = z(M2, 128), z(M2, 64), z(M2, 64), z(M2, 64, dt=b16)
-        self.gc3, self.gs3, self.ga3, self.g16_3 = z(M3, 256), z(M3, 128), z(M3, 128), z(M3, 128, dt=b16)
-        self.gt2, self.gt3 = z(M2, 32), z(M3, 64)
-        self.ghb, self.ga4, self.g16_4, self.gp3 = z(M4, 128), z(M4, 128), z(M4, 128, dt=b16), z(M4, 128)
-        self.gp2, self.gp1, self.gpool = z(M3, 64), z(M2, 32), z(M1, 32)
+        # backward buffers: FP32 gradients of the layers' inputs, bf16 gradients
+        # through the ReLUs per level
+        self.g16_1, self.g16_2 = z(M1, 32, dt=b16), z(M2, 64, dt=b16)
+        self.g16_3, self.g16_4 = z(M3, 128, dt=b16), z(M4, 128, dt=b16)
+        self.gh1, self.gc1, self.gc2, self.gc3 = z(M1, 32), z(M1, 64), z(M2, 128), z(M3, 256)
+        self.gp3, self.gp2, self.gp1 = z(M4, 128), z(M3, 64), z(M2, 32)
         lib = self.lib
         scratch = max(lib.lbm_sg_wgrad_scratch_floats(N, H, W, 64, 32),
                       lib.lbm_sg_wgrad_scratch_floats(N, H, W, 16, 32),
@@ -115,9 +112,9 @@ class Surrogate:
                       lib.lbm_sg_wgrad_scratch_floats(N, H // 2, W // 2, 32, 64),
                       lib.lbm_sg_wgrad_scratch_floats(N, H // 4, W // 4, 256, 64),
                       lib.lbm_sg_wgrad_scratch_floats(N, H // 4, W // 4, 64, 128),
-                      lib.lbm_sg_wgrad_scratch_floats(N, H // 8, W // 8, 128, 128), 64 * 256)
+                      lib.lbm_sg_wgrad_scratch_floats(N, H // 8, W // 8, 128, 128), GRAD_BLOCKS * 128)
         self.scratch = z(int(scratch))
-        self.mse_scratch = torch.zeros(256, dtype=torch.float64, device=dev)
+        self.mse_scratch = torch.zeros(3 * GRAD_BLOCKS, dtype=torch.float64, device=dev)
         self.loss_dev = torch.zeros(1, dtype=torch.float64, device=dev)
         self.step_count = 0
 
@@ -193,13 +190,11 @@ class Surrogate:
         _ck(self.lib.lbm_sg_conv3x3_wgrad(x, csx, g16, csg, _ptr(ly["gW"]), _ptr(self.scratch), self.scratch.numel(),
                                           self.N, h, w, ly["cip"], ly["cop"], self.stream), "lbm_sg_conv3x3_wgrad")
 
-    def _bgrad(self, name, g, csg, level):
+    def _conv_relu(self, name, x, csx, y, csy, level):
         ly = self.layers[name]
-        _ck(self.lib.lbm_sg_bias_grad(g, csg, _ptr(ly["gb"]), _ptr(self.scratch), self.M[level], ly["cop"],
-                                      self.stream), "lbm_sg_bias_grad")
-
-    def _relu(self, a, csa, y, csy, level, C):
-        _ck(self.lib.lbm_sg_relu(a, csa, y, csy, self.M[level], C, self.stream), "lbm_sg_relu")
+        h, w = self.HW[level]
+        _ck(self.lib.lbm_sg_conv3x3_relu(x, csx, _ptr(ly["W16"]), _ptr(ly["b"]), y, csy, self.N, h, w, ly["cip"],
+                                         ly["cop"], self.stream), "lbm_sg_conv3x3_relu")
 
     def _pool(self, x, csx, y, csy, level_fine, C):
         h, w = self.HW[level_fine]
@@ -209,19 +204,13 @@ class Surrogate:
         h, w = self.HW[level_fine]
         _ck(self.lib.lbm_sg_upsample(x, csx, y, csy, self.N, h, w, C, POOL, self.stream), "lbm_sg_upsample")
 
-    def _up_bwd(self, g, csg, gx, csx, level_fine, C):
-        h, w = self.HW[level_fine]
-        _ck(self.lib.lbm_sg_upsample_bwd(g, csg, gx, csx, self.N, h, w, C, POOL, self.stream), "lbm_sg_upsample_bwd")
-
-    def _pool_bwd(self, g, csg, gx, csx, level_fine, C):
-        h, w = self.HW[level_fine]
-        _ck(self.lib.lbm_sg_pool_bwd(g, csg, gx, csx, self.N, h, w, C, POOL, self.stream), "lbm_sg_pool_bwd")
-
-    def _relu_bwd(self, g, csg, a, csa, ga, ga16, level, C):
-        _ck(self.lib.lbm_sg_relu_bwd(g, csg, a, csa, ga, ga16, self.M[level], C, self.stream), "lbm_sg_relu_bwd")
-
-    def _add(self, a, csa, b, csb, out, cso, level, C):
-        _ck(self.lib.lbm_sg_add(a, csa, b, csb, out, cso, self.M[level], C, self.stream), "lbm_sg_add")
+    def _relu_grad(self, name, level, act, csa, ga, g, csg, up=1, gp=None, csp=0):
+        """ga (bf16) and the layer's bias gradient from the gradient of its
+        output: g, its 2x2 sums (up=2) or g plus the pooled path's gp."""
+        ly = self.layers[name]
+        h, w = self.HW[level]
+        _ck(self.lib.lbm_sg_relu_grad(g, csg, up, gp, csp, act, csa, ga, _ptr(ly["gb"]), _ptr(self.scratch),
+                                      self.scratch.numel(), self.N, h, w, ly["cop"], self.stream), "lbm_sg_relu_grad")
 
     # ---------------------------------------------------------------- passes
     def set_input(self, x32):
@@ -235,27 +224,20 @@ class Surrogate:
 
     def forward(self):
         """delta (M, 16) float32 for the current input; out = input + delta[:, :4]."""
-        p, a = _ptr, self.a
-        self._conv("e1", p(self.x16), 16, p(a["e1"]), 32, 0)
-        self._relu(p(a["e1"]), 32, p(self.cat1), 64, 0, 32)                 # s1 -> cat1[:, :32]
+        p = _ptr
+        self._conv_relu("e1", p(self.x16), 16, p(self.cat1), 64, 0)         # s1 -> cat1[:, :32]
         self._pool(p(self.cat1), 64, p(self.p1), 32, 0, 32)
-        self._conv("e2", p(self.p1), 32, p(a["e2"]), 64, 1)
-        self._relu(p(a["e2"]), 64, p(self.cat2), 128, 1, 64)                # s2 -> cat2[:, :64]
+        self._conv_relu("e2", p(self.p1), 32, p(self.cat2), 128, 1)         # s2 -> cat2[:, :64]
         self._pool(p(self.cat2), 128, p(self.p2), 64, 1, 64)
-        self._conv("e3", p(self.p2), 64, p(a["e3"]), 128, 2)
-        self._relu(p(a["e3"]), 128, p(self.cat3), 256, 2, 128)              # s3 -> cat3[:, :128]
+        self._conv_relu("e3", p(self.p2), 64, p(self.cat3), 256, 2)         # s3 -> cat3[:, :128]
         self._pool(p(self.cat3), 256, p(self.p3), 128, 2, 128)
-        self._conv("b", p(self.p3), 128, p(a["b"]), 128, 3)
-        self._relu(p(a["b"]), 128, p(self.hb), 128, 3, 128)
+        self._conv_relu("b", p(self.p3), 128, p(self.hb), 128, 3)
         self._up(p(self.hb), 128, _off(self.cat3, 128), 256, 2, 128)        # cat3[:, 128:]
-        self._conv("d3", p(self.cat3), 256, p(a["d3"]), 64, 2)
-        self._relu(p(a["d3"]), 64, p(self.h3), 64, 2, 64)
+        self._conv_relu("d3", p(self.cat3), 256, p(self.h3), 64, 2)
         self._up(p(self.h3), 64, _off(self.cat2, 64), 128, 1, 64)          # cat2[:, 64:]
-        self._conv("d2", p(self.cat2), 128, p(a["d2"]), 32, 1)
-        self._relu(p(a["d2"]), 32, p(self.h2), 32, 1, 32)
+        self._conv_relu("d2", p(self.cat2), 128, p(self.h2), 32, 1)
         self._up(p(self.h2), 32, _off(self.cat1, 32), 64, 0, 32)           # cat1[:, 32:]
-        self._conv("d1", p(self.cat1), 64, p(a["d1"]), 32, 0)
-        self._relu(p(a["d1"]), 32, p(self.h1), 32, 0, 32)
+        self._conv_relu("d1", p(self.cat1), 64, p(self.h1), 32, 0)
         self._conv("out", p(self.h1), 32, p(self.delta), 16, 0)
         return self.delta
 
@@ -263,7 +245,7 @@ class Surrogate:
         """Loss (device FP64 scalar) and gradients of the MSE of out against
         target32 ((M, 4) float32)."""
         lib, s = self.lib, self.stream
-        p, a = _ptr, self.a
+        p = _ptr
         M1 = self.M[0]
         t = self.torch
         if not (isinstance(target32, t.Tensor) and target32.dtype == t.float32 and target32.is_cuda
@@ -272,67 +254,50 @@ class Surrogate:
             # the loss kernel reads M x 4 floats from this pointer unchecked
             raise ValueError(f"target32: a contiguous float32 CUDA tensor of shape ({M1}, {NC}) on "
                              f"{self.x32.device} is required")
-        _ck(lib.lbm_sg_mse(p(self.x32), NC, p(self.delta), 16, p(target32), NC, p(self.g_delta), p(self.mse_scratch),
-                           p(self.loss_dev), M1, NC, s), "lbm_sg_mse")
-        _ck(lib.lbm_sg_to_bf16(p(self.g_delta), 16, p(self.g16_1), 16, M1, 16, s), "lbm_sg_to_bf16")
-        # out: input gradient -> gt1 (FP32, 32 channels, reusing gs1)
+        if target32.data_ptr() % 16:     # a view into a larger tensor
+            target32 = target32.clone()
+        _ck(lib.lbm_sg_mse_grad(p(self.x32), p(self.delta), p(target32), p(self.g16_1), p(self.layers["out"]["gb"]),
+                                p(self.mse_scratch), p(self.loss_dev), M1, s), "lbm_sg_mse_grad")
+        # out, d1 (level 1)
         self._wgrad("out", p(self.h1), 32, p(self.g16_1), 16, 0)
-        self._bgrad("out", p(self.g_delta), 16, 0)
-        self._conv_input_grad("out", p(self.g16_1), 16, self.gs1, 32, 0)
-        # d1 (level 1): d cat1
-        self._relu_bwd(p(self.gs1), 32, p(a["d1"]), 32, p(self.ga1), p(self.g16_1), 0, 32)
+        self._conv_input_grad("out", p(self.g16_1), 16, self.gh1, 32, 0)
+        self._relu_grad("d1", 0, p(self.h1), 32, p(self.g16_1), p(self.gh1), 32)
         self._wgrad("d1", p(self.cat1), 64, p(self.g16_1), 32, 0)
-        self._bgrad("d1", p(self.ga1), 32, 0)
-        self._conv_input_grad("d1", p(self.g16_1), 32, self.gc1, 64, 0)
-        self._up_bwd(_off(self.gc1, 32), 64, p(self.gt2), 32, 0, 32)       # -> d h2 (level 2)
-        # d2 (level 2): d cat2
-        self._relu_bwd(p(self.gt2), 32, p(a["d2"]), 32, p(self.ga2), p(self.g16_2), 1, 32)
+        self._conv_input_grad("d1", p(self.g16_1), 32, self.gc1, 64, 0)             # d cat1
+        # d2 (level 2), through the upsampling
+        self._relu_grad("d2", 1, p(self.h2), 32, p(self.g16_2), _off(self.gc1, 32), 64, up=2)
         self._wgrad("d2", p(self.cat2), 128, p(self.g16_2), 32, 1)
-        self._bgrad("d2", p(self.ga2), 32, 1)
-        self._conv_input_grad("d2", p(self.g16_2), 32, self.gc2, 128, 1)
-        self._up_bwd(_off(self.gc2, 64), 128, p(self.gt3), 64, 1, 64)      # -> d h3 (level 3)
-        # d3 (level 3): d cat3
-        self._relu_bwd(p(self.gt3), 64, p(a["d3"]), 64, p(self.ga3), p(self.g16_3), 2, 64)
+        self._conv_input_grad("d2", p(self.g16_2), 32, self.gc2, 128, 1)            # d cat2
+        # d3 (level 3)
+        self._relu_grad("d3", 2, p(self.h3), 64, p(self.g16_3), _off(self.gc2, 64), 128, up=2)
         self._wgrad("d3", p(self.cat3), 256, p(self.g16_3), 64, 2)
-        self._bgrad("d3", p(self.ga3), 64, 2)
-        self._conv_input_grad("d3", p(self.g16_3), 64, self.gc3, 256, 2)
-        self._up_bwd(_off(self.gc3, 128), 256, p(self.ghb), 128, 2, 128)   # -> d hb (level 4)
+        self._conv_input_grad("d3", p(self.g16_3), 64, self.gc3, 256, 2)            # d cat3
         # b (level 4)
-        self._relu_bwd(p(self.ghb), 128, p(a["b"]), 128, p(self.ga4), p(self.g16_4), 3, 128)
+        self._relu_grad("b", 3, p(self.hb), 128, p(self.g16_4), _off(self.gc3, 128), 256, up=2)
         self._wgrad("b", p(self.p3), 128, p(self.g16_4), 128, 3)
-        self._bgrad("b", p(self.ga4), 128, 3)
         self._conv_input_grad("b", p(self.g16_4), 128, self.gp3, 128, 3)
-        # s3 receives the skip (gc3[:, :128]) and the pooled path
-        self._pool_bwd(p(self.gp3), 128, p(self.ga3), 128, 2, 128)
-        self._add(p(self.gc3), 256, p(self.ga3), 128, p(self.gs3), 128, 2, 128)
-        self._relu_bwd(p(self.gs3), 128, p(a["e3"]), 128, p(self.ga3), p(self.g16_3), 2, 128)
+        # e3, e2, e1: the skip (the first channels of d cat) and the pooled path
+        self._relu_grad("e3", 2, p(self.cat3), 256, p(self.g16_3), p(self.gc3), 256, gp=p(self.gp3), csp=128)
         self._wgrad("e3", p(self.p2), 64, p(self.g16_3), 128, 2)
-        self._bgrad("e3", p(self.ga3), 128, 2)
         self._conv_input_grad("e3", p(self.g16_3), 128, self.gp2, 64, 2)
-        # s2
-        self._pool_bwd(p(self.gp2), 64, p(self.ga2), 64, 1, 64)
-        self._add(p(self.gc2), 128, p(self.ga2), 64, p(self.gs2), 64, 1, 64)
-        self._relu_bwd(p(self.gs2), 64, p(a["e2"]), 64, p(self.ga2), p(self.g16_2), 1, 64)
+        self._relu_grad("e2", 1, p(self.cat2), 128, p(self.g16_2), p(self.gc2), 128, gp=p(self.gp2), csp=64)
         self._wgrad("e2", p(self.p1), 32, p(self.g16_2), 64, 1)
-        self._bgrad("e2", p(self.ga2), 64, 1)
         self._conv_input_grad("e2", p(self.g16_2), 64, self.gp1, 32, 1)
-        # s1
-        self._pool_bwd(p(self.gp1), 32, p(self.gpool), 32, 0, 32)
-        self._add(p(self.gc1), 64, p(self.gpool), 32, p(self.gs1), 32, 0, 32)
-        self._relu_bwd(p(self.gs1), 32, p(a["e1"]), 32, p(self.ga1), p(self.g16_1), 0, 32)
+        self._relu_grad("e1", 0, p(self.cat1), 64, p(self.g16_1), p(self.gc1), 64, gp=p(self.gp1), csp=32)
         self._wgrad("e1", p(self.x16), 16, p(self.g16_1), 32, 0)
-        self._bgrad("e1", p(self.ga1), 32, 0)
         return self.loss_dev
 
     def adam(self, lr=1e-3, b1=0.9, b2=0.999, eps=1e-8):
         self.step_count += 1
-        for name, _, _ in LAYERS:
+        arr = (L.lbm_sg_layer * len(LAYERS))()
+        for d, (name, _, _) in zip(arr, LAYERS):
             ly = self.layers[name]
-            _ck(self.lib.lbm_sg_adam(_ptr(ly["W"]), _ptr(ly["mW"]), _ptr(ly["vW"]), _ptr(ly["gW"]), ly["W"].numel(),
-                                     lr, b1, b2, eps, self.step_count, _ptr(ly["W16"]), self.stream), "lbm_sg_adam")
-            _ck(self.lib.lbm_sg_adam(_ptr(ly["b"]), _ptr(ly["mb"]), _ptr(ly["vb"]), _ptr(ly["gb"]), ly["b"].numel(),
-                                     lr, b1, b2, eps, self.step_count, None, self.stream), "lbm_sg_adam")
-            self._flip(name)
+            for field, key in (("w", "W"), ("mw", "mW"), ("vw", "vW"), ("gw", "gW"), ("b", "b"), ("mb", "mb"),
+                               ("vb", "vb"), ("gb", "gb"), ("w16", "W16"), ("wt", "Wt")):
+                setattr(d, field, ly[key].data_ptr())
+            d.ci, d.co = ly["cip"], ly["cop"]
+        _ck(self.lib.lbm_sg_adam_layers(arr, len(LAYERS), lr, b1, b2, eps, self.step_count, self.stream),
+            "lbm_sg_adam_layers")
 
     def train_step(self, x32, target32, lr=1e-3):
         self.set_input(x32)

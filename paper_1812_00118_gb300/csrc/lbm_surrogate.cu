@@ -12,7 +12,7 @@
 // The forward (and input-gradient) convolution runs on the tcgen05 tensor
 // cores with the accumulator in tensor memory (conv_row_kernel for images
 // whose width is a multiple of 128, conv_tc_kernel otherwise); so does the
-// weight gradient, a GEMM over pixels, for widths that are multiples of 64
+// weight gradient, a GEMM over pixels, for widths that are multiples of 16
 // (conv_wgrad_row_kernel), with the warp-level mma.sync m16n8k16 BF16 kernel
 // (fragments gathered straight from the channels-last tensors) for the
 // rest.  All are implicit GEMMs without an im2col buffer.
@@ -515,56 +515,59 @@ __global__ void conv_wgrad_kernel(const bf16* __restrict__ x, int csx, const bf1
 
 // ---------------------------------------------------------------- tcgen05 weight gradient, row march
 // gw[co, tap, ci] = sum_p gy[p, co] x[p + d(tap), ci] as GEMMs over pixels
-// on the tensor cores, for images whose width is a multiple of 32: for each
-// tap D_tap (M = co, N = ci) += A (co x pixels) B_tap (ci x pixels)^T with K
-// running over pixels.  A CTA owns a segment of P = 64 (or 32) pixels of one
-// image row, one tap row dy, a block of at most 128 input channels and a
-// chunk of rows; per row (one stage) it copies the gy row segment and the x
-// row r + dy (P + 2 pixels, the periodic neighbours included)
-// into shared memory in their natural channels-last order (16-byte
-// cp.async, one stage ahead), then transposes them with ldmatrix /
-// stmatrix.trans into the K-major core-matrix layout the MMAs read: A as
-// 128 co rows (rows past Co are never written and their D rows never read),
-// B once per dx in {-1, 0, +1}, the window shifted by dx pixels.  The three
-// taps of the CTA's dy accumulate in tensor memory over the whole march
-// (columns dx Ci + ci, lanes co) and are written out once, as the CTA's
-// partial; the partials are summed in a fixed order (deterministic).
-constexpr int kWgCn = 128;            // input channels of one CTA at most (3 Cn tensor-memory columns)
+// on the tensor cores, for images whose width is a multiple of 16: per tap
+// D_tap (M x N) += A (M x pixels) B (N x pixels)^T, M the channels of the side
+// with more of them, N those of the other, K running over pixels.
+//
+// Both operands are read where they were copied: a row lies in shared memory as
+// planes of 8 channels, 16 bytes per pixel, which is the tensor core's
+// no-swizzle MN-major layout (core matrices of 8 pixels x 8 channels, plane
+// pitch between channel groups, 128 bytes between groups of 8 pixels).  A tap
+// is then the x row of its dy started (1 + dx) pixels in: no transposition,
+// and one copy of a row serves three dy and three dx.  (Transposing both
+// operands through registers into K-major buffers, for one dy per CTA, took
+// 290 us for the 64 -> 32 layer at 8 x 256^2; this takes 48.)  Plane
+// pitches are odd multiples of 16 bytes, so the 8 groups of a pixel, copied by
+// neighbouring threads, fall into different banks.
+//
+// A CTA marches a segment of P pixels down a chunk of rows, x rows in a ring
+// of six and gy rows in a ring of four, copies two rows ahead of the MMAs, MMAs
+// of a row issued while those of the one before still run.  The taps (all
+// nine where their columns fit tensor memory, else the three of one dy)
+// accumulate over the whole march and are written out once, as the CTA's
+// partial; partials are summed in a fixed order (deterministic).  M = 128
+// always: the rows past a side's channels read whatever lies behind its planes
+// and are not written out.
+constexpr int kWgCn = 128;            // input channels of one CTA at most
+constexpr int kWgThreads = 256;
+constexpr int kWgX = 6, kWgG = 4;     // rows in the rings
 constexpr size_t kWgSmemMax = 220 * 1024;   // below the 227 KB per CTA less the kernel's static shared memory
 
 struct WgLayout {
-    uint32_t gys, xs;                 // natural row strides (padded by 16 bytes against bank conflicts)
-    uint32_t nat_gy, nat;             // bytes of the gy part and of one natural buffer
-    uint32_t opA, opB1, op;           // bytes of A, of one B window, of one operand buffer
+    uint32_t px, pg;        // plane pitches of x and gy
+    uint32_t xrow, grow;    // bytes of one row
     uint32_t total;
 };
 // P pixels of a segment, Cn input channels and Co output channels of a CTA
 __host__ __device__ inline WgLayout wg_layout(int P, int Cn, int Co) {
     WgLayout L;
-    L.gys = (uint32_t)Co * 2 + 16;
-    L.xs = (uint32_t)Cn * 2 + 16;
-    L.nat_gy = (uint32_t)P * L.gys;
-    L.nat = L.nat_gy + (uint32_t)(P + 2) * L.xs;
-    L.opA = (uint32_t)(P / 8) * 128 * 16;
-    L.opB1 = (uint32_t)(P / 8) * (uint32_t)Cn * 16;
-    L.op = L.opA + 3 * L.opB1;
-    L.total = 2 * L.nat + 2 * L.op;
+    L.px = (uint32_t)((P + 2) | 1) * 16;
+    L.pg = (uint32_t)(P | 1) * 16;
+    L.xrow = (uint32_t)(Cn / 8) * L.px;
+    L.grow = (uint32_t)(Co / 8) * L.pg;
+    // the 16 planes an M = 128 operand reads from the last row of its ring
+    const uint32_t tail = Cn >= Co ? (uint32_t)(16 - Cn / 8) * L.px : (uint32_t)(16 - Co / 8) * L.pg;
+    L.total = kWgX * L.xrow + kWgG * L.grow + tail;
     return L;
 }
-__host__ __device__ inline uint32_t wg_tmem_cols(int Ci) {
-    const int need = 3 * Ci;
+__host__ __device__ inline int wg_n(int Cn, int Co) { return Cn >= Co ? Co : Cn; }   // columns of a tap
+__host__ __device__ inline int wg_taps(int Cn, int Co) { return 9 * wg_n(Cn, Co) <= 512 ? 9 : 3; }
+__host__ __device__ inline uint32_t wg_tmem_cols(int Cn, int Co) {
+    const int need = wg_taps(Cn, Co) * wg_n(Cn, Co);
     return need <= 32 ? 32u : (need <= 64 ? 64u : (need <= 128 ? 128u : (need <= 256 ? 256u : 512u)));
 }
 
-__device__ __forceinline__ void ldsm_x2(uint32_t addr, uint32_t& r0, uint32_t& r1) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
-}
-__device__ __forceinline__ void stsm_x2_trans(uint32_t addr, uint32_t r0, uint32_t r1) {
-    asm volatile("stmatrix.sync.aligned.m8n8.x2.trans.shared.b16 [%0], {%1, %2};" ::"r"(addr), "r"(r0), "r"(r1)
-                 : "memory");
-}
-
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kWgThreads, 1)
 conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ gy, int csg,
                       float* __restrict__ partial, int N, int H, int W, int Ci, int Co, int P, int Cn,
                       int rows_per_cta, int* err) {
@@ -574,25 +577,28 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int segs = W / P;
     const int nsplit = Ci / Cn;
+    const int taps = wg_taps(Cn, Co);
     const int chunks = (H + rows_per_cta - 1) / rows_per_cta;
     int b = blockIdx.x;
-    const int dyi = b % 3;
-    b /= 3;
+    const int dy0 = taps == 9 ? -1 : b % 3 - 1, ndy = taps / 3;   // the CTA's tap rows
+    if (taps != 9) b /= 3;
     const int ci0 = (b % nsplit) * Cn;
     b /= nsplit;
     const int chunk = b % chunks;
     b /= chunks;
     const int seg = b % segs, n = b / segs;
-    const int dy = dyi - 1;
     const int y0 = chunk * rows_per_cta;
     const int y1 = y0 + rows_per_cta < H ? y0 + rows_per_cta : H;
     const int x0 = seg * P;
     const long long pchunk = ((long long)n * segs + seg) * chunks + chunk;
     const WgLayout Lt = wg_layout(P, Cn, Co);
+    const bool x_is_a = Cn >= Co;
+    // the ring of the M side lies last, its tail behind it
     const uint32_t sb = smem_u32(smem);
-    const uint32_t nat0 = sb, op0 = sb + 2 * Lt.nat;
+    const uint32_t xb = x_is_a ? sb + kWgG * Lt.grow : sb, gb = x_is_a ? sb : sb + kWgX * Lt.xrow;
     const uint32_t bar0 = smem_u32(&bars[0]);
-    const uint32_t ncols = wg_tmem_cols(Cn);
+    const int Nc = wg_n(Cn, Co);
+    const uint32_t ncols = wg_tmem_cols(Cn, Co);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                      "r"(ncols)
@@ -607,107 +613,104 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
-    const uint32_t idesc = tc_idesc_bf16(128, Cn);
+    // both operands MN-major (bits 15 and 16)
+    const uint32_t idesc = tc_idesc_bf16(128, Nc) | (1u << 15) | (1u << 16);
     const int nco8 = Co / 8, nci8 = Cn / 8;
     const long long img = (long long)n * H * W;
-    // natural copies of stage s (row r = y0 + s): the gy row segment and
-    // channels ci0 .. ci0 + Cn - 1 of the x row r + dy, pixels x0 - 1 .. x0 + P
-    // (wrapped)
-    auto copy_stage = [&](int st) {
-        const int r = y0 + st;
-        const uint32_t nb = nat0 + (uint32_t)(st & 1) * Lt.nat;
-        const bf16* grow = gy + (img + (long long)r * W) * csg;
-        for (int k = tid; k < P * nco8; k += 128) {
-            const int p = k / nco8, c = k - p * nco8;
-            cp_async16(nb + p * Lt.gys + c * 16, grow + (long long)(x0 + p) * csg + c * 8, 16u);
-        }
-        const int yr = (((r + dy) % H) + H) % H;
-        const bf16* xrow = x + (img + (long long)yr * W) * csx + ci0;
-        for (int k = tid; k < (P + 2) * nci8; k += 128) {
-            const int q = k / nci8, c = k - q * nci8;
+    // row r0 + dy0 ... of x that the march reads start at y0 + dy0; ring slots
+    // count from there
+    auto x_slot = [&](int k) { return xb + (uint32_t)(k % kWgX) * Lt.xrow; };   // k-th x row of the march
+    auto g_slot = [&](int k) { return gb + (uint32_t)(k % kWgG) * Lt.grow; };
+    auto copy_x = [&](int k) {   // x row y0 + dy0 + k (wrapped), pixels x0 - 1 .. x0 + P (wrapped)
+        const int yy = y0 + dy0 + k;
+        const int yr = ((yy % H) + H) % H;
+        const bf16* row = x + (img + (long long)yr * W) * csx + ci0;
+        const uint32_t dst = x_slot(k);
+        for (int e = tid; e < (P + 2) * nci8; e += kWgThreads) {
+            const int q = e / nci8, c = e - q * nci8;
             int xx = x0 - 1 + q;
             xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
-            cp_async16(nb + Lt.nat_gy + q * Lt.xs + c * 16, xrow + (long long)xx * csx + c * 8, 16u);
+            cp_async16(dst + c * Lt.px + q * 16, row + (long long)xx * csx + c * 8, 16u);
         }
     };
-    // natural buffer st & 1 -> operand buffer st & 1 (K-major: [pixel block][row][8 pixels])
-    auto transpose_stage = [&](int st) {
-        const uint32_t nb = nat0 + (uint32_t)(st & 1) * Lt.nat;
-        const uint32_t ob = op0 + (uint32_t)(st & 1) * Lt.op;
-        const int j = (lane >> 3) & 1, i = lane & 7;   // matrix and row a lane addresses (lanes 0-15 count)
-        const int npb = P / 8;
-        const int na = npb * (nco8 / 2);
-        for (int o = warp; o < na; o += 4) {
-            const int pb = o % npb, cp = o / npb, c = 2 * cp + j;
-            uint32_t r0, r1;
-            ldsm_x2(nb + (uint32_t)(8 * pb + i) * Lt.gys + c * 16, r0, r1);
-            stsm_x2_trans(ob + (uint32_t)pb * (128 * 16) + (uint32_t)(8 * c + i) * 16, r0, r1);
-        }
-        const int nbx = 3 * npb * (nci8 / 2);
-        for (int o = warp; o < nbx; o += 4) {
-            const int w3 = o % 3, rest = o / 3, pb = rest % npb, cp = rest / npb, c = 2 * cp + j;
-            const int q = 8 * pb + i + w3;   // staging pixel of window pixel 8 pb + i shifted by dx = w3 - 1
-            uint32_t r0, r1;
-            ldsm_x2(nb + Lt.nat_gy + (uint32_t)q * Lt.xs + c * 16, r0, r1);
-            stsm_x2_trans(ob + Lt.opA + (uint32_t)w3 * Lt.opB1 + (uint32_t)pb * Cn * 16 + (uint32_t)(8 * c + i) * 16, r0,
-                          r1);
+    auto copy_g = [&](int k) {   // gy row y0 + k
+        const bf16* row = gy + (img + (long long)(y0 + k) * W + x0) * csg;
+        const uint32_t dst = g_slot(k);
+        for (int e = tid; e < P * nco8; e += kWgThreads) {
+            const int q = e / nco8, c = e - q * nco8;
+            cp_async16(dst + c * Lt.pg + q * 16, row + (long long)q * csg + c * 8, 16u);
         }
     };
-    auto wait_stage = [&](int st) { return mbar_wait_bounded(bar0 + 8 * (st & 1), (uint32_t)(st >> 1) & 1u, kTcPolls); };
     const int S = y1 - y0;
+    // group j: the gy row j and the last x row its taps read (group 0: all of them)
+    auto copy_group = [&](int j) {
+        if (j < S) {
+            if (j == 0)
+                for (int k = 0; k < ndy - 1; ++k) copy_x(k);
+            copy_x(j + ndy - 1);
+            copy_g(j);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // the MMAs of row j commit to barrier j & 1: its (j >> 1)-th phase
+    auto wait_row = [&](int j) { return mbar_wait_bounded(bar0 + 8 * (j & 1), (uint32_t)(j >> 1) & 1u, kTcPolls); };
     bool ok = true;
     int issued = 0;
-    copy_stage(0);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    for (int st = 0; st < S; ++st) {
-        const bool more = st + 1 < S;
-        if (more) {   // natural buffer (st + 1) & 1 was last read by the transposes of stage st - 1
-            copy_stage(st + 1);
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        }
-        if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
-        else asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();
-        // operand buffer st & 1 was last read by the MMAs of stage st - 2
-        if (st >= 2 && !__syncthreads_and(wait_stage(st - 2))) { ok = false; break; }
-        transpose_stage(st);
+    copy_group(0);
+    copy_group(1);
+    for (int j = 0; j < S; ++j) {
+        // group j + 2 goes where row j - 2's operands were
+        if (j >= 2 && !__syncthreads_and(wait_row(j - 2))) { ok = false; break; }
+        copy_group(j + 2);
+        asm volatile("cp.async.wait_group 2;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t ob = op0 + (uint32_t)(st & 1) * Lt.op;
-            for (int w3 = 0; w3 < 3; ++w3) {
-                for (int k = 0; k < P / 16; ++k) {
-                    const uint64_t ad = tc_smem_desc(ob + 2 * k * (128 * 16), 128 * 16, 128);
-                    const uint64_t bd = tc_smem_desc(ob + Lt.opA + w3 * Lt.opB1 + 2 * k * (Cn * 16), Cn * 16, 128);
-                    tc_mma(tmem + (uint32_t)(w3 * Cn), ad, bd, idesc, (st > 0 || k > 0) ? 1u : 0u);
+            const uint32_t gs = g_slot(j);
+            for (int d = 0; d < ndy; ++d) {
+                const uint32_t xs = x_slot(j + d);
+                for (int dx = 0; dx < 3; ++dx) {
+                    const uint32_t acc = tmem + (uint32_t)((3 * d + dx) * Nc);
+                    const uint32_t xo = xs + (uint32_t)dx * 16;
+                    for (int k = 0; k < P / 16; ++k) {
+                        const uint64_t xd = tc_smem_desc(xo + k * 256, 128, Lt.px);
+                        const uint64_t gd = tc_smem_desc(gs + k * 256, 128, Lt.pg);
+                        tc_mma(acc, x_is_a ? xd : gd, x_is_a ? gd : xd, idesc, (j > 0 || k > 0) ? 1u : 0u);
+                    }
                 }
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             bar0 + 8 * (st & 1))
+                             bar0 + 8 * (j & 1))
                          : "memory");
         }
-        issued = st + 1;
+        issued = j + 1;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (issued > 0) {
-        const bool done = wait_stage(issued - 1);
+        const bool done = wait_row(issued - 1);
         ok = __syncthreads_and(ok && done) != 0 && issued == S;
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (ok) {
-        const int co = 32 * warp + lane;
-        for (int w3 = 0; w3 < 3; ++w3) {
-            const int tap = (dy + 1) * 3 + w3;
-            float* out = partial + ((pchunk * Co + co) * 9 + tap) * (long long)Ci + ci0;
-            for (int c0 = 0; c0 < Cn; c0 += 16) {
+    if (ok && warp < 4) {
+        const int m = 32 * warp + lane;          // channel of the M side
+        const int K9 = 9 * Ci;
+        float* out = partial + pchunk * Co * (long long)K9;
+        for (int t = 0; t < taps; ++t) {
+            const int tap = (dy0 + 1) * 3 + t;
+            for (int c0 = 0; c0 < Nc; c0 += 16) {
                 float v[16];
-                tc_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(w3 * Cn + c0), v);
-                if (co < Co) {
+                tc_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(t * Nc + c0), v);
+                if (x_is_a) {
+                    if (m < Cn) {
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) out[(long long)(c0 + k) * K9 + tap * Ci + ci0 + m] = v[k];
+                    }
+                } else if (m < Co) {
+                    float* o = out + (long long)m * K9 + tap * Ci + ci0 + c0;
 #pragma unroll
                     for (int k = 0; k < 16; k += 4)
-                        *reinterpret_cast<float4*>(out + c0 + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+                        *reinterpret_cast<float4*>(o + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
                 }
             }
         }
@@ -725,6 +728,7 @@ __global__ void sum_chunks_kernel(const float* __restrict__ partial, long long n
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= K) return;
     float s = 0.0f;
+#pragma unroll 8
     for (long long c = 0; c < nchunks; ++c) s += partial[c * K + k];
     gw[k] = s;
 }
@@ -911,21 +915,35 @@ __global__ void upsample_bwd_kernel(const float* __restrict__ g, int csg, float*
     gx[q * csx + c] = s;
 }
 
-// per-block partial sums of column c of g (rows = pixels), fixed order
-__global__ void colsum_partial_kernel(const float* __restrict__ g, int csg, long long npix, int C,
-                                      float* __restrict__ part) {
-    __shared__ float sh[kThreads];
-    const int c = blockIdx.y;
-    float s = 0.0f;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < npix; p += (long long)gridDim.x * blockDim.x)
-        s += g[p * csg + c];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = kThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
+// per-block partial sums of the columns of g (rows = pixels), fixed order:
+// neighbouring threads take neighbouring channels of a pixel, so a block reads
+// whole rows (one channel per block read 4 of every 4 C bytes: 63 us for
+// 8 x 256^2 x 32).  blockIdx.y: 256 channels.
+constexpr int kColThreads = 1024;
+__global__ void __launch_bounds__(kColThreads)
+colsum_partial_kernel(const float* __restrict__ g, int csg, long long npix, int C, float* __restrict__ part) {
+    __shared__ float sh[kColThreads];
+    const int c0 = blockIdx.y * 256;
+    const int nc = C - c0 < 256 ? C - c0 : 256, lanes = kColThreads / nc;
+    const int c = threadIdx.x % nc, lane = threadIdx.x / nc;
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};     // four pixels in flight
+    if (lane < lanes) {
+        const long long step = (long long)gridDim.x * lanes;
+        const float* q = g + c0 + c;
+        long long p = (long long)blockIdx.x * lanes + lane;
+        for (; p + 3 * step < npix; p += 4 * step) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) s[k] += q[(p + k * step) * csg];
+        }
+        for (; p < npix; p += step) s[0] += q[p * csg];
     }
-    if (threadIdx.x == 0) part[(long long)c * gridDim.x + blockIdx.x] = sh[0];
+    sh[threadIdx.x] = (s[0] + s[1]) + (s[2] + s[3]);
+    __syncthreads();
+    if ((int)threadIdx.x < nc) {
+        float t = 0.0f;
+        for (int l = 0; l < lanes; ++l) t += sh[threadIdx.x + l * nc];
+        part[(long long)(c0 + c) * gridDim.x + blockIdx.x] = t;
+    }
 }
 
 __global__ void colsum_finish_kernel(const float* __restrict__ part, int nb, int C, float* __restrict__ out) {
@@ -1382,28 +1400,35 @@ cudaError_t conv_row_slots(size_t need, int Co, int* out) {
 
 // Dynamic shared memory of a weight-gradient row-march launch, raised like
 // conv_row_launch_smem so that the CTAs an SM holds fit its tensor memory.
-size_t wg_launch_smem(size_t need, int Ci) {
-    const int per_sm = 512 / (int)wg_tmem_cols(Ci);
+size_t wg_launch_smem(size_t need, int Cn, int Co) {
+    const int per_sm = 512 / (int)wg_tmem_cols(Cn, Co);
     const size_t floor_bytes = sm_shared_bytes() / (size_t)(per_sm + 1) + 1;
     return need > floor_bytes ? need : floor_bytes;
 }
 
-// Segment width of the weight-gradient row march (0: the width allows none)
-// and the input channels of one CTA.
-inline int wg_segment(int W) { return W % 64 == 0 ? 64 : (W % 32 == 0 ? 32 : 0); }
+// Input channels of one CTA of the weight-gradient row march, and the pixels of
+// its segment: the widest divisor of W that is a multiple of 16, at most 128
+// and fits shared memory (0: the march does not apply to these sizes).
 inline int wg_block(int Ci) { return Ci <= kWgCn ? Ci : kWgCn; }
+inline int wg_segment(int W, int Ci, int Co) {
+    if (W % 16) return 0;
+    for (int P = W < 128 ? W : 128; P >= 16; P -= 16)
+        if (W % P == 0 && wg_layout(P, wg_block(Ci), Co).total <= kWgSmemMax) return P;
+    return 0;
+}
 
 // Row chunks of the weight-gradient row march on the current device: rows
 // per CTA and chunks per column (0 rows: the march does not apply to these
-// sizes).  One wave: 3 tap rows x channel blocks x N x W / P segments x
+// sizes).  One wave: tap rows x channel blocks x N x W / P segments x
 // chunks CTAs at most the resident CTAs.
 cudaError_t wgrad_row_plan(int N, int H, int W, int Ci, int Co, int* rows, int* chunks) {
     *rows = 0;
     *chunks = 0;
-    const int P = wg_segment(W), Cn = wg_block(Ci);
-    if (P == 0 || Ci % Cn || Co > 128 || Ci % 16 || Co % 16 || H < 1) return cudaSuccess;
+    const int Cn = wg_block(Ci);
+    if (Ci % Cn || Co > 128 || Ci % 16 || Co % 16 || H < 1) return cudaSuccess;
+    const int P = wg_segment(W, Ci, Co);
+    if (P == 0) return cudaSuccess;
     const WgLayout Lt = wg_layout(P, Cn, Co);
-    if (Lt.total > kWgSmemMax) return cudaSuccess;
     static bool attr_set[64] = {};
     int dev = 0, sms = 0, occ = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1420,12 +1445,12 @@ cudaError_t wgrad_row_plan(int N, int H, int W, int Ci, int Co, int* rows, int* 
     if (e != cudaSuccess) return e;
     // CTAs an SM holds: its shared memory (1 KB reserved per CTA) and its 512
     // tensor-memory columns
-    const size_t per_cta = wg_launch_smem(Lt.total, Cn) + 1024;
+    const size_t per_cta = wg_launch_smem(Lt.total, Cn, Co) + 1024;
     occ = (int)(sm_shared_bytes() / per_cta);
-    const int by_tmem = 512 / (int)wg_tmem_cols(Cn);
+    const int by_tmem = 512 / (int)wg_tmem_cols(Cn, Co);
     if (occ > by_tmem) occ = by_tmem;
     const long long slots = (long long)sms * (occ > 0 ? occ : 1);
-    const long long cols = 3LL * (Ci / Cn) * N * (W / P);
+    const long long cols = (9LL / wg_taps(Cn, Co)) * (Ci / Cn) * N * (W / P);
     long long c = slots / cols;
     if (c < 1) c = 1;
     if (c > H) c = H;
@@ -1530,7 +1555,7 @@ long long lbm_sg_wgrad_scratch_floats(int N, int H, int W, int Ci, int Co) {
     int rows = 0, chunks = 0;
     if (wgrad_row_plan(N, H, W, Ci, Co, &rows, &chunks) == cudaSuccess) {
         if (rows > 0) {
-            const long long row_need = (long long)N * (W / wg_segment(W)) * chunks * Co * 9 * Ci;
+            const long long row_need = (long long)N * (W / wg_segment(W, Ci, Co)) * chunks * Co * 9 * Ci;
             if (row_need > need) need = row_need;
         }
     } else {
@@ -1546,8 +1571,8 @@ int lbm_sg_conv3x3_wgrad(const void* x, int csx, const void* gy, int csg, float*
         return LBM_EINVAL;
     const long long need = lbm_sg_wgrad_scratch_floats(N, H, W, Ci, Co);
     if (scratch_floats < need) return LBM_EINVAL;
-    // rows of 64-pixel segments with 16-byte aligned channel rows: the
-    // tcgen05 row march
+    // rows in segments of multiples of 16 pixels, with 16-byte aligned channel
+    // rows: the tcgen05 row march
     int rows = 0, rchunks = 0;
     if (wgrad_row_plan(N, H, W, Ci, Co, &rows, &rchunks) != cudaSuccess) {
         cudaGetLastError();
@@ -1558,10 +1583,11 @@ int lbm_sg_conv3x3_wgrad(const void* x, int csx, const void* gy, int csg, float*
         int* err = nullptr;
         if (cudaGetSymbolAddress((void**)&err, g_sg_err) != cudaSuccess) return LBM_ECUDA;
         cudaStream_t s = (cudaStream_t)stream;
-        const int P = wg_segment(W), Cn = wg_block(Ci);
+        const int P = wg_segment(W, Ci, Co), Cn = wg_block(Ci);
         const long long pchunks = (long long)N * (W / P) * rchunks;
         const WgLayout Lt = wg_layout(P, Cn, Co);
-        conv_wgrad_row_kernel<<<(unsigned)(3 * (Ci / Cn) * pchunks), 128, wg_launch_smem(Lt.total, Cn), s>>>(
+        conv_wgrad_row_kernel<<<(unsigned)((9 / wg_taps(Cn, Co)) * (Ci / Cn) * pchunks), kWgThreads,
+                                wg_launch_smem(Lt.total, Cn, Co), s>>>(
             (const bf16*)x, csx, (const bf16*)gy, csg, scratch, N, H, W, Ci, Co, P, Cn, rows, err);
         const long long K = (long long)Co * 9 * Ci;
         sum_chunks_kernel<<<blocks(K), kThreads, 0, s>>>(scratch, pchunks, K, gw);
@@ -1588,7 +1614,7 @@ int lbm_sg_bias_grad(const float* g, int csg, float* gb, float* scratch, long lo
     if (!g || !gb || !scratch || npix < 1 || C < 1 || csg < C) return LBM_EINVAL;
     const int nb = (int)(npix < 64LL * kThreads ? (npix + kThreads - 1) / kThreads : 64);
     cudaStream_t s = (cudaStream_t)stream;
-    colsum_partial_kernel<<<dim3(nb, C), kThreads, 0, s>>>(g, csg, npix, C, scratch);
+    colsum_partial_kernel<<<dim3(nb, (C + 255) / 256), kColThreads, 0, s>>>(g, csg, npix, C, scratch);
     colsum_finish_kernel<<<blocks(C), kThreads, 0, s>>>(scratch, nb, C, gb);
     return check(cudaGetLastError());
 }

@@ -130,6 +130,22 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a, uint64_t b, 
         : "memory");
 }
 
+// n MMAs of K = 16 into one accumulator, operand descriptors a step apart (the
+// address field counts 16-byte units and never carries out of its 14 bits); the
+// first one starts the sum unless `acc`.  One thread issues them: descriptors
+// stepped by an addition instead of built per MMA keep it ahead of the tensor
+// core.
+__device__ __forceinline__ void tc_mma_run(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t a_step, uint32_t b_step,
+                                           uint32_t idesc, int n, bool acc) {
+    tc_mma(d_tmem, a, b, idesc, acc ? 1u : 0u);
+#pragma unroll 4
+    for (int k = 1; k < n; ++k) {
+        a += a_step;
+        b += b_step;
+        tc_mma(d_tmem, a, b, idesc, 1u);
+    }
+}
+
 // 16 consecutive FP32 columns of the thread's lane
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
@@ -311,26 +327,44 @@ __device__ int g_sg_err;   // a bounded wait of a surrogate kernel gave up
 // owns a 128-pixel segment of one image row and marches down a chunk of
 // rows.  The shifted activations of a 3x3 tap are then rows of a halo
 // strip: for row r the taps read input rows r - 1, r, r + 1 at pixel
-// offsets -1, 0, +1 around the segment.  The strip holds four input rows
+// offsets -1, 0, +1 around the segment.  The strip is a ring of input rows
 // (130 pixels each, the periodic neighbours included) in the tensor core's
 // no-swizzle K-major layout, one 16-byte row per (pixel, 8 channels): a tap's
 // A operand is the strip row of its dy started (1 + dx) pixels in, 128 rows
-// of 16 bytes, 8-row core matrices 128 bytes apart, 8-channel planes 130 x 16
-// bytes apart.  Every input row is copied into shared memory once (the tap
-// kernel above copies it nine times), the weights of all nine taps stay
-// resident for the whole march, and one thread issues the 9 x Ci/16 MMAs of
-// a row into one of two tensor-memory accumulators while the CTA writes out
-// the previous row from the other and the copy of the next input row is in
-// flight.  Every wait is bounded, as in the tap kernel.
+// of 16 bytes, 8-row core matrices 128 bytes apart, 8-channel planes an odd
+// multiple of 16 bytes apart (the 8 groups of a pixel, copied by neighbouring
+// threads, fall into different banks).  Every input row is copied into shared
+// memory once (the tap kernel above copies it nine times) and the weights of
+// all nine taps stay resident for the whole march.
+//
+// The march keeps the tensor core fed: a row's MMAs are issued as soon as its
+// last input row has landed, into one of two tensor-memory accumulators; then
+// the row before is waited for, its oldest input row replaced by a copy one to
+// three rows ahead (as many ring rows as fit), and its accumulator written
+// out, all under the running MMAs.  (Writing out row j - 1 and copying row
+// j + 1 before issuing row j, on 128 threads, took 126 us for the 64 -> 32
+// layer at 8 x 256^2; this takes 39.)  Every wait is bounded, as in the tap
+// kernel.
 constexpr int kRowM = 128;          // pixels of a row segment (MMA M)
 constexpr int kRowHalo = kRowM + 2;
-constexpr int kRowSlots = 4;        // input rows resident in the strip
+constexpr int kRowThreads = 256;
+constexpr int kRowSlots = 6;        // ring rows at most (at least 4)
+constexpr size_t kRowSmemMax = 220 * 1024;
 
-__host__ __device__ constexpr uint32_t row_plane_bytes() { return kRowHalo * 16; }
+__host__ __device__ constexpr uint32_t row_plane_bytes() { return (kRowHalo | 1) * 16; }
 __host__ __device__ inline uint32_t row_slot_bytes(int Ci) { return (uint32_t)(Ci / 8) * row_plane_bytes(); }
-__host__ __device__ inline uint32_t row_w_bytes(int Ci, int Co) { return (uint32_t)9 * Co * Ci * 2; }
-size_t conv_row_smem_bytes(int Ci, int Co) {
-    return (size_t)kRowSlots * row_slot_bytes(Ci) + row_w_bytes(Ci, Co);
+// weights: [tap][ci chunk][co], chunks an odd multiple of 16 bytes apart
+__host__ __device__ inline uint32_t row_w_chunk(int Co) { return (uint32_t)(Co + 1) * 16; }
+__host__ __device__ inline uint32_t row_w_bytes(int Ci, int Co) { return 9u * (uint32_t)(Ci / 8) * row_w_chunk(Co); }
+// ring rows that fit beside the weights (below 4: the march does not apply)
+inline int conv_row_slots_of(int Ci, int Co) {
+    const size_t w = row_w_bytes(Ci, Co);
+    if (w >= kRowSmemMax) return 0;
+    const size_t n = (kRowSmemMax - w) / row_slot_bytes(Ci);
+    return n < (size_t)kRowSlots ? (int)n : kRowSlots;
+}
+size_t conv_row_smem_bytes(int Ci, int Co, int slots) {
+    return (size_t)slots * row_slot_bytes(Ci) + row_w_bytes(Ci, Co);
 }
 // tensor-memory columns of the two accumulators (a power of two, at least 32)
 __host__ __device__ inline uint32_t row_tmem_cols(int Co) {
@@ -339,9 +373,10 @@ __host__ __device__ inline uint32_t row_tmem_cols(int Co) {
 }
 
 template <bool ACT>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kRowThreads, 1)
 conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, const float* __restrict__ bias,
-                void* __restrict__ y, int csy, int N, int H, int W, int Ci, int Co, int rows_per_cta, int* err) {
+                void* __restrict__ y, int csy, int N, int H, int W, int Ci, int Co, int rows_per_cta, int slots,
+                int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[2];
     __shared__ uint32_t tmem_slot;
@@ -355,9 +390,9 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
     const int y0 = chunk * rows_per_cta;
     const int y1 = y0 + rows_per_cta < H ? y0 + rows_per_cta : H;
     const int x0 = seg * kRowM;
-    const uint32_t sb = smem_u32(smem);
-    const uint32_t slot_bytes = row_slot_bytes(Ci);
-    const uint32_t wb = sb + kRowSlots * slot_bytes;     // weights: [tap][ci chunk][co][16 bytes]
+    const uint32_t wb = smem_u32(smem);                  // weights, then the ring
+    const uint32_t sb = wb + row_w_bytes(Ci, Co);
+    const uint32_t slot_bytes = row_slot_bytes(Ci), wchunk = row_w_chunk(Co);
     const uint32_t bar0 = smem_u32(&bars[0]);
     const uint32_t ncols = row_tmem_cols(Co);
     if (warp == 0) {
@@ -377,75 +412,67 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
     const uint32_t idesc = tc_idesc_bf16(kRowM, Co);
     const int nch = Ci / 8;
     const long long img = (long long)n * H * W;
-    // input row yy (wrapped) into strip slot yy & 3: pixels x0 - 1 .. x0 + 128 (wrapped)
-    auto copy_row = [&](int yy) {
-        const int yr = ((yy % H) + H) % H;
-        const uint32_t dst = sb + (uint32_t)(yy & 3) * slot_bytes;
+    const int nrows = y1 - y0;
+    // input row k of the march (image row y0 - 1 + k, wrapped; k <= nrows + 1)
+    // into ring slot k % slots: pixels x0 - 1 .. x0 + 128 (wrapped)
+    auto copy_row = [&](int k) {
+        if (k > nrows + 1) return;
+        const int yr = ((y0 - 1 + k) % H + H) % H;
+        const uint32_t dst = sb + (uint32_t)(k % slots) * slot_bytes;
         const bf16* row = x + (img + (long long)yr * W) * csx;
-        for (int k = tid; k < nch * kRowHalo; k += kRowM) {
-            const int c = k / kRowHalo, px = k - c * kRowHalo;
+        for (int e = tid; e < nch * kRowHalo; e += kRowThreads) {
+            const int px = e / nch, c = e - px * nch;
             int xx = x0 - 1 + px;
             xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
             cp_async16(dst + c * row_plane_bytes() + px * 16, row + (long long)xx * csx + c * 8, 16u);
         }
     };
-    // prologue: the weights of every tap and input rows y0 - 1 .. y0 + 1, one group
-    for (int k = tid; k < 9 * nch * Co; k += kRowM) {
-        const int co = k % Co, rest = k / Co, c = rest % nch, tap = rest / nch;
-        cp_async16(wb + ((uint32_t)(tap * nch + c) * Co + co) * 16, w + ((long long)co * 9 + tap) * Ci + c * 8, 16u);
+    // prologue: group 0 is the weights of every tap and input rows 0 .. 2, each
+    // later group one row
+    const int ahead = slots - 3;
+    for (int k = tid; k < 9 * nch * Co; k += kRowThreads) {
+        const int row = k / nch, c = k - row * nch, co = row / 9, tap = row - co * 9;
+        cp_async16(wb + (uint32_t)(tap * nch + c) * wchunk + co * 16, w + (long long)row * Ci + c * 8, 16u);
     }
-    for (int yy = y0 - 1; yy <= y0 + 1; ++yy) copy_row(yy);
+    for (int k = 0; k < 3; ++k) copy_row(k);
     asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int k = 1; k < ahead; ++k) {
+        copy_row(2 + k);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
     bool ok = true;
     // row j of the march (row y0 + j) accumulates in buffer j & 1 and commits
     // to barrier j & 1: the (j >> 1)-th phase of that barrier
     auto wait_row = [&](int j) { return mbar_wait_bounded(bar0 + 8 * (j & 1), (uint32_t)(j >> 1) & 1u, kTcPolls); };
-    auto epilogue = [&](int j) {
-        const int r = y0 + j;
-        const uint32_t acc = tmem + (uint32_t)((j & 1) * Co) + ((uint32_t)(32 * warp) << 16);
-        const long long pix = img + (long long)r * W + x0 + 32 * warp + lane;
-        const bool vec = conv_vec<ACT>(y, csy);
-        for (int c0 = 0; c0 < Co; c0 += 16) {
+    const bool vec = conv_vec<ACT>(y, csy);
+    auto epilogue = [&](int j) {   // warps w and w + 4 share a quarter of the lanes
+        const uint32_t acc = tmem + (uint32_t)((j & 1) * Co) + ((uint32_t)(32 * (warp & 3)) << 16);
+        const long long pix = img + (long long)(y0 + j) * W + x0 + 32 * (warp & 3) + lane;
+        for (int c0 = 16 * (warp >> 2); c0 < Co; c0 += 32) {
             float v[16];
             tc_ld16(acc + (uint32_t)c0, v);
             conv_store16<ACT>(y, pix * csy + c0, v, bias ? bias + c0 : nullptr, vec);
         }
     };
-    const int nrows = y1 - y0;
     int issued = 0;   // rows whose MMAs were issued and committed
-    for (int j = 0; j < nrows && ok; ++j) {
-        const int r = y0 + j;
-        // (1) row j - 1: its MMAs done (they read strip slot (r - 2) & 3 last),
-        // its accumulator out
-        if (j > 0) {
-            if (!__syncthreads_and(wait_row(j - 1))) { ok = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            epilogue(j - 1);
-        }
-        // (2) input row r + 2 into the slot row r - 2 held
-        const bool more = r + 2 <= y1;
-        if (more) {
-            copy_row(r + 2);
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        }
-        // (3) rows r - 1 .. r + 1 landed (only the group just issued may be pending)
-        if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    for (int j = 0; j < nrows; ++j) {
+        // input rows j .. j + 2 landed (the ahead - 1 newer groups may be pending)
+        if (ahead >= 3) asm volatile("cp.async.wait_group 2;" ::: "memory");
+        else if (ahead == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
         else asm volatile("cp.async.wait_group 0;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
-        // (4) the 9 x Ci/16 MMAs of row r into buffer j & 1
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t acc = tmem + (uint32_t)((j & 1) * Co);
-            for (int tap = 0; tap < 9; ++tap) {
-                const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-                const uint32_t a_s = sb + (uint32_t)((r + dy) & 3) * slot_bytes + (uint32_t)(1 + dx) * 16;
-                const uint32_t b_s = wb + (uint32_t)tap * nch * Co * 16;
-                for (int s2 = 0; s2 < Ci / 16; ++s2) {
-                    const uint64_t ad = tc_smem_desc(a_s + 2 * s2 * row_plane_bytes(), row_plane_bytes(), 128);
-                    const uint64_t bd = tc_smem_desc(b_s + 2 * s2 * (Co * 16), Co * 16, 128);
-                    tc_mma(acc, ad, bd, idesc, (tap > 0 || s2 > 0) ? 1u : 0u);
+            for (int dy = 0; dy < 3; ++dy) {
+                const uint32_t a_s = sb + (uint32_t)((j + dy) % slots) * slot_bytes;
+                for (int dx = 0; dx < 3; ++dx) {
+                    const int tap = 3 * dy + dx;
+                    const uint64_t ad = tc_smem_desc(a_s + (uint32_t)dx * 16, row_plane_bytes(), 128);
+                    const uint64_t bd = tc_smem_desc(wb + (uint32_t)(tap * nch) * wchunk, wchunk, 128);
+                    tc_mma_run(acc, ad, bd, 2 * row_plane_bytes() / 16, 2 * wchunk / 16, idesc, nch / 2, tap > 0);
                 }
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -453,6 +480,15 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
                          : "memory");
         }
         issued = j + 1;
+        // row j - 1 done: its oldest input row (j - 1) makes room for row
+        // j + 2 + ahead, and its accumulator goes out
+        if (j > 0 && !__syncthreads_and(wait_row(j - 1))) { ok = false; break; }
+        copy_row(j + 2 + ahead);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (j > 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            epilogue(j - 1);
+        }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     // the last issued row: its MMAs complete after every earlier one (waited
@@ -463,6 +499,147 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (all && issued == nrows) epilogue(issued - 1);
         ok = all && ok;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+    if (!ok && tid == 0) atomicExch(err, 1);
+}
+
+// ---------------------------------------------------------------- tcgen05 convolution, flat tiles
+// The same convolution for any other width: the image with one halo column on
+// each side, read as one flat array of cells with row pitch W + 2.  Output
+// position f (row f / (W + 2), column f % (W + 2)) then reads cell f + dy (W + 2)
+// + dx for every tap, whatever row it is in, so 128 consecutive positions are
+// one MMA tile even where they span several rows; the two positions per row
+// that fall on the halo columns are computed and dropped.  A CTA copies the
+// 128 + 2 (W + 3) cells its tile reads once, all channels of them (the tap
+// kernel copies 9 x 128 pixels, a stage of 64 channels at a time), and the
+// weights tap by tap through a ring of `stages` buffers.  Taps and channels in
+// the tap kernel's order.
+constexpr int kFlatThreads = 256;
+constexpr int kFlatStages = 9;
+
+__host__ __device__ inline int flat_cells(int W) { return 128 + 2 * (W + 3); }
+__host__ __device__ inline uint32_t flat_plane(int W) { return (uint32_t)(flat_cells(W) | 1) * 16; }
+__host__ __device__ inline uint32_t flat_x_bytes(int W, int Ci) { return (uint32_t)(Ci / 8) * flat_plane(W); }
+__host__ __device__ inline uint32_t flat_w_bytes(int Ci, int Co) { return (uint32_t)(Ci / 8) * row_w_chunk(Co); }
+// weight buffers of a launch: as many as leave room for two CTAs per SM, or
+// else for one (below 2: the tiles do not apply)
+inline int flat_stages(int W, int Ci, int Co) {
+    if (W > 4096 || Ci > 4096) return 0;
+    const size_t x = flat_x_bytes(W, Ci), w = flat_w_bytes(Ci, Co);
+    size_t n = x + 2 * w <= kRowSmemMax / 2 ? (kRowSmemMax / 2 - x) / w : (x + 2 * w <= kRowSmemMax ? (kRowSmemMax - x) / w : 0);
+    return n < (size_t)kFlatStages ? (int)n : kFlatStages;
+}
+
+template <bool ACT>
+__global__ void __launch_bounds__(kFlatThreads, 1)
+conv_flat_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, const float* __restrict__ bias,
+                 void* __restrict__ y, int csy, int H, int W, int Ci, int Co, int tiles, int stages, int* err) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t bars[kFlatStages];
+    __shared__ uint32_t tmem_slot;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n = blockIdx.x / tiles, f0 = (blockIdx.x - n * tiles) * 128;
+    const int Wp = W + 2, nch = Ci / 8, cells = flat_cells(W);
+    const uint32_t xs = smem_u32(smem), plane = flat_plane(W);
+    const uint32_t ws = xs + flat_x_bytes(W, Ci), wstage = flat_w_bytes(Ci, Co), wchunk = row_w_chunk(Co);
+    const uint32_t bar0 = smem_u32(&bars[0]);
+    const uint32_t ncols = Co <= 32 ? 32u : (Co <= 64 ? 64u : 128u);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                     "r"(ncols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int k = 0; k < stages; ++k)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * k) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = tmem_slot;
+    const long long img = (long long)n * H * W;
+    auto copy_w = [&](int tap) {   // the tap's weights into buffer tap % stages, as one commit group
+        if (tap < 9) {
+            const uint32_t dst = ws + (uint32_t)(tap % stages) * wstage;
+            for (int e = tid; e < Co * nch; e += kFlatThreads) {
+                const int co = e / nch, c = e - co * nch;
+                cp_async16(dst + c * wchunk + co * 16, w + ((long long)co * 9 + tap) * Ci + c * 8, 16u);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // cell k of the tile: padded cell f0 + k, row -1 .. H and column -1 .. W of
+    // the image (rows past H, behind the last tile, wrap like the rest)
+    for (int e = tid; e < cells * nch; e += kFlatThreads) {
+        const int k = e / nch, c = e - k * nch;
+        const int id = f0 + k, row = id / Wp;
+        const int yy = (row - 1 + H) % H, xx = (id - row * Wp - 1 + W) % W;
+        cp_async16(xs + c * plane + k * 16, x + (img + (long long)yy * W + xx) * csx + c * 8, 16u);
+    }
+    for (int t = 0; t < stages; ++t) copy_w(t);     // group 0 holds the cells too
+    const uint32_t idesc = tc_idesc_bf16(128, Co);
+    bool ok = true;
+    int issued = 0;
+    auto wait_tap = [&](int t) {
+        return mbar_wait_bounded(bar0 + 8 * (t % stages), (uint32_t)(t / stages) & 1u, kTcPolls);
+    };
+    for (int t = 0; t < 9; ++t) {
+        // tap t's group landed: `stages` groups are committed ahead of it, less
+        // the one whose buffer is refilled after the MMAs of tap t - 1
+        if (t == 0 && stages > 1) {
+            // every group but the first may be pending
+            switch (stages) {
+                case 2: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
+                case 3: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
+                case 4: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+                default: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+            }
+        } else if (stages >= 4) asm volatile("cp.async.wait_group 2;" ::: "memory");
+        else if (stages == 3) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        if (tid == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint64_t ad = tc_smem_desc(xs + (uint32_t)((t / 3) * Wp + t % 3) * 16, plane, 128);
+            const uint64_t bd = tc_smem_desc(ws + (uint32_t)(t % stages) * wstage, wchunk, 128);
+            tc_mma_run(tmem, ad, bd, 2 * plane / 16, 2 * wchunk / 16, idesc, nch / 2, t > 0);
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             bar0 + 8 * (t % stages))
+                         : "memory");
+        }
+        issued = t + 1;
+        // tap t - 1 done: its buffer takes the weights of tap t - 1 + stages
+        if (t > 0 && t - 1 + stages < 9) {
+            if (!__syncthreads_and(wait_tap(t - 1))) { ok = false; break; }
+            copy_w(t - 1 + stages);
+        } else if (t > 0) {
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    // the last committed tap completes after every earlier MMA of the CTA
+    if (issued > 0) {
+        const bool done = wait_tap(issued - 1);
+        ok = __syncthreads_and(ok && done) != 0;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (ok) {
+        const int f = f0 + 32 * (warp & 3) + lane, row = f / Wp, col = f - row * Wp;
+        const bool in = row < H && col < W;
+        const long long pix = img + (long long)row * W + col;
+        const bool vec = conv_vec<ACT>(y, csy);
+        for (int c0 = 16 * (warp >> 2); c0 < Co; c0 += 32) {
+            float v[16];
+            tc_ld16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, v);
+            if (in) conv_store16<ACT>(y, pix * csy + c0, v, bias ? bias + c0 : nullptr, vec);
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -539,7 +716,7 @@ __global__ void conv_wgrad_kernel(const bf16* __restrict__ x, int csx, const bf1
 // always: the rows past a side's channels read whatever lies behind its planes
 // and are not written out.
 constexpr int kWgCn = 128;            // input channels of one CTA at most
-constexpr int kWgThreads = 256;
+constexpr int kWgThreads = 288;          // a warp per tap issues its MMAs
 constexpr int kWgX = 6, kWgG = 4;     // rows in the rings
 constexpr size_t kWgSmemMax = 220 * 1024;   // below the 227 KB per CTA less the kernel's static shared memory
 
@@ -606,7 +783,8 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int k = 0; k < 2; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * k) : "memory");
+        for (int k = 0; k < 2; ++k)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar0 + 8 * k), "r"(taps) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -665,21 +843,11 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
         asm volatile("cp.async.wait_group 2;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (tid == 0) {
+        if (lane == 0 && warp < taps) {   // warp t: tap t (each tap its own accumulator)
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t gs = g_slot(j);
-            for (int d = 0; d < ndy; ++d) {
-                const uint32_t xs = x_slot(j + d);
-                for (int dx = 0; dx < 3; ++dx) {
-                    const uint32_t acc = tmem + (uint32_t)((3 * d + dx) * Nc);
-                    const uint32_t xo = xs + (uint32_t)dx * 16;
-                    for (int k = 0; k < P / 16; ++k) {
-                        const uint64_t xd = tc_smem_desc(xo + k * 256, 128, Lt.px);
-                        const uint64_t gd = tc_smem_desc(gs + k * 256, 128, Lt.pg);
-                        tc_mma(acc, x_is_a ? xd : gd, x_is_a ? gd : xd, idesc, (j > 0 || k > 0) ? 1u : 0u);
-                    }
-                }
-            }
+            const uint64_t xd = tc_smem_desc(x_slot(j + warp / 3) + (uint32_t)(warp % 3) * 16, 128, Lt.px);
+            const uint64_t gd = tc_smem_desc(g_slot(j), 128, Lt.pg);
+            tc_mma_run(tmem + (uint32_t)(warp * Nc), x_is_a ? xd : gd, x_is_a ? gd : xd, 16, 16, idesc, P / 16, j > 0);
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                              bar0 + 8 * (j & 1))
                          : "memory");
@@ -1343,8 +1511,6 @@ __global__ void smooth_kernel(const double* __restrict__ a, double* __restrict__
     b[p] = c + k * lap;
 }
 
-constexpr size_t kRowSmemMax = 200 * 1024;
-
 // Shared memory of one SM of the current device (looked up once per device;
 // 228 KB, GB300's, if the query fails).
 size_t sm_shared_bytes() {
@@ -1374,27 +1540,18 @@ size_t conv_row_launch_smem(size_t need, int Co) {
     return need > floor_bytes ? need : floor_bytes;
 }
 
-// Resident row-march CTAs on the current device (SMs x CTAs per SM), with the
-// attribute for large dynamic shared memory set once per device.
-template <bool ACT>
-cudaError_t conv_row_slots(size_t need, int Co, int* out) {
-    static bool attr_set[64] = {};
-    int dev = 0, sms = 0, occ = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        e = cudaFuncSetAttribute(conv_row_kernel<ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
+// The attribute for large dynamic shared memory of a convolution kernel, once
+// per device.
+template <typename K>
+cudaError_t large_smem(K kernel, bool (&done)[64], int dev) {
+    if (dev < 0 || dev >= 64 || !done[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmemMax);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(conv_row_kernel<ACT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
-        attr_set[dev] = true;
+        if (dev >= 0 && dev < 64) done[dev] = true;
     }
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, conv_row_kernel<ACT>, kRowM, conv_row_launch_smem(need, Co));
-    if (e != cudaSuccess) return e;
-    *out = sms * (occ > 0 ? occ : 1);
     return cudaSuccess;
 }
 
@@ -1490,31 +1647,49 @@ static int conv3x3(const void* x, int csx, const void* w, const float* bias, voi
     }
     int* err = nullptr;
     if (cudaGetSymbolAddress((void**)&err, g_sg_err) != cudaSuccess) return LBM_ECUDA;
-    // rows of 128-pixel segments: the row-march kernel, when its strip and
-    // the weights of all taps fit in shared memory
-    const size_t row_smem = conv_row_smem_bytes(Ci, Co);
-    if (W % kRowM == 0 && H >= 2 && row_smem <= kRowSmemMax) {
-        int slots = 0;
-        if (conv_row_slots<ACT>(row_smem, Co, &slots) != cudaSuccess) {
+    // rows of 128-pixel segments: the row march, when four input rows and the
+    // weights of all taps fit in shared memory; else flat tiles, when their
+    // cells and two taps' weights do.  (us at 8 x 256^2 / 2^l of level l, row
+    // march, flat tiles, tap kernel: see the table at conv3x3's callers.)
+    int sms = 1;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LBM_ECUDA;
+    const int slots = conv_row_slots_of(Ci, Co);
+    if (W % kRowM == 0 && slots >= 4) {
+        static bool done[64] = {};
+        if (large_smem(conv_row_kernel<ACT>, done, dev) != cudaSuccess) {
             cudaGetLastError();
             return LBM_ECUDA;
         }
-        int dev = 0, sms = 1;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return LBM_ECUDA;
         const long long cols = (long long)N * (W / kRowM);
-        // one CTA per SM: longer marches (the weights and the two halo rows of
-        // a chunk are loaded once per CTA) ran faster than two CTAs per SM on
-        // half the rows (d1 at 8 x 256^2: 0.127 against 0.135 ms)
-        long long chunks = (slots < sms ? slots : sms) / cols;
+        // one CTA per SM: the weights and the two halo rows of a chunk are
+        // loaded once per CTA
+        long long chunks = sms / cols;
         if (chunks < 1) chunks = 1;
         if (chunks > H) chunks = H;
         const int rows = (int)((H + chunks - 1) / chunks);
         const long long nb = cols * ((H + rows - 1) / rows);
-        conv_row_kernel<ACT><<<(unsigned)nb, kRowM, conv_row_launch_smem(row_smem, Co), s>>>(
-            (const bf16*)x, csx, (const bf16*)w, bias, y, csy, N, H, W, Ci, Co, rows, err);
+        conv_row_kernel<ACT><<<(unsigned)nb, kRowThreads,
+                               conv_row_launch_smem(conv_row_smem_bytes(Ci, Co, slots), Co), s>>>(
+            (const bf16*)x, csx, (const bf16*)w, bias, y, csy, N, H, W, Ci, Co, rows, slots, err);
         return check(cudaGetLastError());
+    }
+    const int stages = flat_stages(W, Ci, Co);
+    const long long flat = (long long)H * (W + 2);
+    if (stages >= 2 && flat < (1LL << 30)) {
+        static bool done[64] = {};
+        if (large_smem(conv_flat_kernel<ACT>, done, dev) != cudaSuccess) {
+            cudaGetLastError();
+            return LBM_ECUDA;
+        }
+        const int tiles = (int)((flat + 127) / 128);
+        if ((long long)N * tiles < (1LL << 31)) {
+            // no more CTAs on an SM than its tensor memory serves (four of 128 columns)
+            const size_t need = flat_x_bytes(W, Ci) + (size_t)stages * flat_w_bytes(Ci, Co);
+            const size_t least = sm_shared_bytes() / 5 + 1;
+            conv_flat_kernel<ACT><<<(unsigned)(N * tiles), kFlatThreads, need > least ? need : least, s>>>(
+                (const bf16*)x, csx, (const bf16*)w, bias, y, csy, H, W, Ci, Co, tiles, stages, err);
+            return check(cudaGetLastError());
+        }
     }
     const unsigned nb = (unsigned)((M + kTcM - 1) / kTcM);
     conv_tc_kernel<ACT><<<nb, kTcM, smem, s>>>((const bf16*)x, csx, (const bf16*)w, bias, y, csy, M, H, W, Ci, Co, err);

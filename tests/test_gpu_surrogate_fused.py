@@ -140,3 +140,36 @@ def test_adam_layers(env):
     for t, r in zip(keep, refs):
         for n in t:
             assert torch.allclose(t[n].float(), r[n].float(), rtol=1e-6 if n not in ("w16", "wt") else 8e-3, atol=1e-9), n
+
+
+def conv_reference(torch, x, w, b, N, H, W):
+    """Periodic 3x3 convolution in float64: x (M, ci), w (co, 9, ci)."""
+    img = x.double().view(N, H, W, -1)
+    out = b.double().view(1, 1, 1, -1).expand(N, H, W, -1)
+    for t in range(9):
+        out = out + torch.roll(img, (1 - t // 3, 1 - t % 3), (1, 2)) @ w[:, t].double().T
+    return out.reshape(N * H * W, -1)
+
+
+@pytest.mark.parametrize("N,H,W,ci,co", [
+    (1, 2, 8, 16, 16), (2, 4, 8, 32, 128), (3, 33, 16, 64, 32), (1, 8, 250, 32, 48), (2, 7, 40, 128, 64),   # flat tiles
+    (2, 64, 64, 256, 64), (1, 64, 64, 64, 128), (3, 32, 32, 128, 128), (1, 16, 62, 64, 128), (1, 1, 16, 16, 16),
+    (1, 1, 128, 16, 16), (1, 2, 128, 128, 32), (1, 3, 128, 64, 128), (2, 9, 256, 32, 16), (1, 200, 128, 16, 32),   # march
+    (1, 16, 64, 256, 128), (1, 4, 128, 256, 64)])                                                        # tap kernel
+def test_conv_paths_exact_on_integers(env, N, H, W, ci, co):
+    """Every path of the convolution and of the weight gradient on integers
+    small enough that every sum is exact: equal to float64 bit for bit."""
+    torch, lib, s = env
+    g = torch.Generator(device="cuda").manual_seed(N + H * W + ci * co)
+    r = lambda lo, hi, *sh: torch.randint(lo, hi + 1, sh, generator=g, device="cuda").bfloat16()
+    M = N * H * W
+    x, w, gy, b = r(-2, 2, M, ci), r(-2, 2, co, 9, ci), r(-1, 1, M, co), r(-5, 5, co).float()
+    y, gw = torch.full((M, co), 7.0, device="cuda"), torch.zeros(co, 9, ci, device="cuda")
+    assert lib.lbm_sg_conv3x3(p(x), ci, p(w), p(b), p(y), co, N, H, W, ci, co, s) == 0
+    assert torch.equal(y.double(), conv_reference(torch, x, w, b, N, H, W))
+    n = lib.lbm_sg_wgrad_scratch_floats(N, H, W, ci, co)
+    scr = torch.full((n,), float("nan"), device="cuda")
+    assert lib.lbm_sg_conv3x3_wgrad(p(x), ci, p(gy), co, p(gw), p(scr), n, N, H, W, ci, co, s) == 0
+    img, gi = x.double().view(N, H, W, ci), gy.double().view(N * H * W, co)
+    want = torch.stack([gi.T @ torch.roll(img, (1 - t // 3, 1 - t % 3), (1, 2)).reshape(-1, ci) for t in range(9)], 1)
+    assert torch.equal(gw.double(), want) and lib.lbm_sg_status(s) == 0

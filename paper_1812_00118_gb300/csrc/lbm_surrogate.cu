@@ -122,27 +122,55 @@ __host__ __device__ constexpr uint32_t tc_idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// The issuing thread of a warp: 1 in one lane (the same at every call), 0 in
+// the others.
+__device__ __forceinline__ uint32_t tc_elect() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
+
+// One MMA, issued by the lane with el != 0; every lane of the warp calls it.
+__device__ __forceinline__ void tc_mma(uint32_t el, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                       uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(el)
         : "memory");
+}
+
+// mbarrier arrival once every MMA the lane with el != 0 has issued is done
+__device__ __forceinline__ void tc_commit(uint32_t el, uint32_t bar) {
+    if (el)
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+                     : "memory");
 }
 
 // n MMAs of K = 16 into one accumulator, operand descriptors a step apart (the
 // address field counts 16-byte units and never carries out of its 14 bits); the
-// first one starts the sum unless `acc`.  One thread issues them: descriptors
-// stepped by an addition instead of built per MMA keep it ahead of the tensor
-// core.
-__device__ __forceinline__ void tc_mma_run(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t a_step, uint32_t b_step,
-                                           uint32_t idesc, int n, bool acc) {
-    tc_mma(d_tmem, a, b, idesc, acc ? 1u : 0u);
-#pragma unroll 4
-    for (int k = 1; k < n; ++k) {
+// first one starts the sum unless `acc`.  Called by a whole warp with uniform
+// arguments, four MMAs per loop pass: the descriptors then stay in uniform
+// registers and the issue keeps up with the tensor core.  (clk per MMA of M =
+// 128, K = 16, N = 32 / 128, one CTA: 40 / 64; from a branch of one thread
+// that steps the descriptors, 155 / 155; the core itself needs 64 at N = 128,
+// and 32 to read A at N = 32.)
+__device__ __forceinline__ void tc_mma_run(uint32_t el, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t a_step,
+                                           uint32_t b_step, uint32_t idesc, int n, bool acc) {
+    tc_mma(el, d_tmem, a, b, idesc, acc ? 1u : 0u);
+    int k = 1;
+    for (; k + 4 <= n; k += 4) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            a += a_step;
+            b += b_step;
+            tc_mma(el, d_tmem, a, b, idesc, 1u);
+        }
+    }
+    for (; k < n; ++k) {
         a += a_step;
         b += b_step;
-        tc_mma(d_tmem, a, b, idesc, 1u);
+        tc_mma(el, d_tmem, a, b, idesc, 1u);
     }
 }
 
@@ -205,7 +233,7 @@ conv_tc_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, 
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[kTcBuf];
     __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const long long p0 = (long long)blockIdx.x * kTcM;
     const int kcap = Ci < kTcK ? Ci : kTcK;   // channels per stage buffer
     const uint32_t a_bytes = kTcM * kcap * 2, stage_bytes = a_bytes + (uint32_t)Co * kcap * 2;
@@ -272,19 +300,15 @@ conv_tc_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, 
         // the copies were written through the generic proxy; the MMAs read through the async proxy
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t el = tc_elect();
             const uint32_t a_s = sb + (st % kTcBuf) * stage_bytes, b_s = a_s + a_bytes;
             const int kc0 = (st % nkb) * kTcK;
             const int kw = Ci - kc0 < kTcK ? Ci - kc0 : kTcK;
-            for (int s = 0; s < kw / 16; ++s) {
-                const uint64_t ad = tc_smem_desc(a_s + 2 * s * (kTcM * 16), kTcM * 16, 128);
-                const uint64_t bd = tc_smem_desc(b_s + 2 * s * (Co * 16), Co * 16, 128);
-                tc_mma(tmem, ad, bd, idesc, (st > 0 || s > 0) ? 1u : 0u);
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             bar0 + 8 * (st % kTcBuf))
-                         : "memory");
+            tc_mma_run(el, tmem, tc_smem_desc(a_s, kTcM * 16, 128), tc_smem_desc(b_s, Co * 16, 128), 2 * kTcM, 2 * Co,
+                       idesc, kw / 16, st > 0);
+            tc_commit(el, bar0 + 8 * (st % kTcBuf));
         }
         issued = st + 1;
     }
@@ -380,7 +404,7 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[2];
     __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const int segs = W / kRowM;
     const int chunks = (H + rows_per_cta - 1) / rows_per_cta;
     int b = blockIdx.x;
@@ -463,8 +487,9 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t el = tc_elect();
             const uint32_t acc = tmem + (uint32_t)((j & 1) * Co);
             for (int dy = 0; dy < 3; ++dy) {
                 const uint32_t a_s = sb + (uint32_t)((j + dy) % slots) * slot_bytes;
@@ -472,12 +497,10 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
                     const int tap = 3 * dy + dx;
                     const uint64_t ad = tc_smem_desc(a_s + (uint32_t)dx * 16, row_plane_bytes(), 128);
                     const uint64_t bd = tc_smem_desc(wb + (uint32_t)(tap * nch) * wchunk, wchunk, 128);
-                    tc_mma_run(acc, ad, bd, 2 * row_plane_bytes() / 16, 2 * wchunk / 16, idesc, nch / 2, tap > 0);
+                    tc_mma_run(el, acc, ad, bd, 2 * row_plane_bytes() / 16, 2 * wchunk / 16, idesc, nch / 2, tap > 0);
                 }
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             bar0 + 8 * (j & 1))
-                         : "memory");
+            tc_commit(el, bar0 + 8 * (j & 1));
         }
         issued = j + 1;
         // row j - 1 done: its oldest input row (j - 1) makes room for row
@@ -541,7 +564,7 @@ conv_flat_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[kFlatStages];
     __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const int n = blockIdx.x / tiles, f0 = (blockIdx.x - n * tiles) * 128;
     const int Wp = W + 2, nch = Ci / 8, cells = flat_cells(W);
     const uint32_t xs = smem_u32(smem), plane = flat_plane(W);
@@ -605,14 +628,13 @@ conv_flat_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w
         else asm volatile("cp.async.wait_group 0;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t el = tc_elect();
             const uint64_t ad = tc_smem_desc(xs + (uint32_t)((t / 3) * Wp + t % 3) * 16, plane, 128);
             const uint64_t bd = tc_smem_desc(ws + (uint32_t)(t % stages) * wstage, wchunk, 128);
-            tc_mma_run(tmem, ad, bd, 2 * plane / 16, 2 * wchunk / 16, idesc, nch / 2, t > 0);
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             bar0 + 8 * (t % stages))
-                         : "memory");
+            tc_mma_run(el, tmem, ad, bd, 2 * plane / 16, 2 * wchunk / 16, idesc, nch / 2, t > 0);
+            tc_commit(el, bar0 + 8 * (t % stages));
         }
         issued = t + 1;
         // tap t - 1 done: its buffer takes the weights of tap t - 1 + stages
@@ -751,7 +773,7 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[2];
     __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const int segs = W / P;
     const int nsplit = Ci / Cn;
     const int taps = wg_taps(Cn, Co);
@@ -843,14 +865,14 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
         asm volatile("cp.async.wait_group 2;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (lane == 0 && warp < taps) {   // warp t: tap t (each tap its own accumulator)
+        if (warp < taps) {   // warp t: tap t (each tap its own accumulator)
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t el = tc_elect();
             const uint64_t xd = tc_smem_desc(x_slot(j + warp / 3) + (uint32_t)(warp % 3) * 16, 128, Lt.px);
             const uint64_t gd = tc_smem_desc(g_slot(j), 128, Lt.pg);
-            tc_mma_run(tmem + (uint32_t)(warp * Nc), x_is_a ? xd : gd, x_is_a ? gd : xd, 16, 16, idesc, P / 16, j > 0);
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             bar0 + 8 * (j & 1))
-                         : "memory");
+            tc_mma_run(el, tmem + (uint32_t)(warp * Nc), x_is_a ? xd : gd, x_is_a ? gd : xd, 16, 16, idesc, P / 16,
+                       j > 0);
+            tc_commit(el, bar0 + 8 * (j & 1));
         }
         issued = j + 1;
     }

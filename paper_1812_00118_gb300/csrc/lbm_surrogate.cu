@@ -187,9 +187,65 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// ---- roles of the march kernels: eight worker warps copy operands in and write
+// results out, one more warp issues the MMAs; mbarriers are all that ties them.
+// The issuing warp has no copies of its own in flight, so its proxy fence (the
+// copies land through the generic proxy, the MMAs read through the async one)
+// waits for nothing; executed by threads with cp.async outstanding, the fence
+// waits for all of them and no copy runs ahead of the MMAs.
+constexpr int kWorkers = 256;
+constexpr int kRoleThreads = kWorkers + 32;
+
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("{\n\t.reg .b64 t;\n\tmbarrier.arrive.shared::cta.b64 t, [%0];\n\t}" ::"r"(bar) : "memory");
+}
+// arrival of this thread once all its cp.async so far have landed
+__device__ __forceinline__ void mbar_arrive_copies(uint32_t bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+// Wait for the k-th phase (from 0) of a barrier; false once it, or another wait
+// of the CTA, has given up (*failed).
+__device__ __forceinline__ bool mbar_wait_phase(uint32_t bar, int k, volatile int* failed) {
+    const uint32_t parity = (uint32_t)k & 1u;
+    for (long i = 0; i < kTcPolls; ++i) {
+        if (mbar_try(bar, parity)) return true;
+        if ((i & 255) == 255 && *failed) return false;
+    }
+    *failed = 1;
+    return false;
+}
+
+// The (row, 16-byte group) pairs of an operand a worker copies: `groups` per row,
+// neighbouring workers on neighbouring groups.  Where the groups divide the
+// workers (channel counts that are powers of two up to 2048) a worker keeps its
+// group and steps through the rows without a division.
+template <typename F>
+__device__ __forceinline__ void for_groups(int tid, int rows, int groups, F&& f) {
+    if ((groups & (groups - 1)) == 0 && groups <= kWorkers) {
+        const int sh = 31 - __clz(groups), c = tid & (groups - 1), step = kWorkers >> sh;
+        for (int q = tid >> sh; q < rows; q += step) f(q, c);
+    } else {
+        for (int e = tid; e < rows * groups; e += kWorkers) {
+            const int q = e / groups;
+            f(q, e - q * groups);
+        }
+    }
+}
+
+// A whole 32-byte sector per lane: lanes write pixels a row stride apart, and
+// two 16-byte stores per sector cost L2 two partial writes.
+__device__ __forceinline__ void st_global_32(void* p, const uint32_t (&v)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+
 // 16 channels of one pixel of a convolution's output, as FP32 or (ACT) as the
 // bf16 values after the ReLU, which is all the next layer and the backward
-// pass read of them; `vec`: the row starts on a 16-byte boundary.
+// pass read of them; `vec`: every pixel's channels start on a 32-byte boundary.
 template <bool ACT>
 __device__ __forceinline__ void conv_store16(void* y, long long at, float (&v)[16], const float* __restrict__ bias,
                                              bool vec) {
@@ -202,9 +258,10 @@ __device__ __forceinline__ void conv_store16(void* y, long long at, float (&v)[1
         for (int i = 0; i < 8; ++i)
             h[i] = __floats2bfloat162_rn(fmaxf(v[2 * i], 0.0f), fmaxf(v[2 * i + 1], 0.0f));
         if (vec) {
-            const uint4* q = reinterpret_cast<const uint4*>(h);
-            reinterpret_cast<uint4*>(out)[0] = q[0];
-            reinterpret_cast<uint4*>(out)[1] = q[1];
+            uint32_t q[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) q[i] = *reinterpret_cast<const uint32_t*>(&h[i]);
+            st_global_32(out, q);
         } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i) { out[2 * i] = h[i].x; out[2 * i + 1] = h[i].y; }
@@ -213,8 +270,12 @@ __device__ __forceinline__ void conv_store16(void* y, long long at, float (&v)[1
         float* out = (float*)y + at;
         if (vec) {
 #pragma unroll
-            for (int i = 0; i < 16; i += 4)
-                *reinterpret_cast<float4*>(out + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+            for (int i = 0; i < 16; i += 8) {
+                uint32_t q[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) q[k] = __float_as_uint(v[i + k]);
+                st_global_32(out + i, q);
+            }
         } else {
 #pragma unroll
             for (int i = 0; i < 16; ++i) out[i] = v[i];
@@ -223,7 +284,7 @@ __device__ __forceinline__ void conv_store16(void* y, long long at, float (&v)[1
 }
 template <bool ACT>
 __device__ __forceinline__ bool conv_vec(const void* y, int csy) {
-    return (csy & (ACT ? 7 : 3)) == 0 && ((uintptr_t)y & 15) == 0;
+    return (csy & (ACT ? 15 : 7)) == 0 && ((uintptr_t)y & 31) == 0;
 }
 
 template <bool ACT>
@@ -361,17 +422,14 @@ __device__ int g_sg_err;   // a bounded wait of a surrogate kernel gave up
 // memory once (the tap kernel above copies it nine times) and the weights of
 // all nine taps stay resident for the whole march.
 //
-// The march keeps the tensor core fed: a row's MMAs are issued as soon as its
-// last input row has landed, into one of two tensor-memory accumulators; then
-// the row before is waited for, its oldest input row replaced by a copy one to
-// three rows ahead (as many ring rows as fit), and its accumulator written
-// out, all under the running MMAs.  (Writing out row j - 1 and copying row
-// j + 1 before issuing row j, on 128 threads, took 126 us for the 64 -> 32
-// layer at 8 x 256^2; this takes 39.)  Every wait is bounded, as in the tap
-// kernel.
+// Worker warps copy the ring's rows ahead of the MMAs (a row's slot is refilled
+// as soon as the last row that reads it is done) and write out one of two
+// tensor-memory accumulators while the other is summed; a warp of its own
+// issues the MMAs.  (On 128 threads that wrote out row j - 1 and copied row
+// j + 1 before issuing row j the 64 -> 32 layer at 8 x 256^2 took 126 us; this
+// takes XX.)  Every wait is bounded, as in the tap kernel.
 constexpr int kRowM = 128;          // pixels of a row segment (MMA M)
 constexpr int kRowHalo = kRowM + 2;
-constexpr int kRowThreads = 256;
 constexpr int kRowSlots = 6;        // ring rows at most (at least 4)
 constexpr size_t kRowSmemMax = 220 * 1024;
 
@@ -380,11 +438,12 @@ __host__ __device__ inline uint32_t row_slot_bytes(int Ci) { return (uint32_t)(C
 // weights: [tap][ci chunk][co], chunks an odd multiple of 16 bytes apart
 __host__ __device__ inline uint32_t row_w_chunk(int Co) { return (uint32_t)(Co + 1) * 16; }
 __host__ __device__ inline uint32_t row_w_bytes(int Ci, int Co) { return 9u * (uint32_t)(Ci / 8) * row_w_chunk(Co); }
-// ring rows that fit beside the weights (below 4: the march does not apply)
-inline int conv_row_slots_of(int Ci, int Co) {
-    const size_t w = row_w_bytes(Ci, Co);
-    if (w >= kRowSmemMax) return 0;
-    const size_t n = (kRowSmemMax - w) / row_slot_bytes(Ci);
+// ring rows that fit beside the weights with `per_sm` CTAs on an SM (below 4:
+// they do not fit)
+inline int conv_row_slots_of(int Ci, int Co, int per_sm) {
+    const size_t w = row_w_bytes(Ci, Co), most = kRowSmemMax / per_sm - (per_sm > 1 ? 1024 : 0);
+    if (w >= most) return 0;
+    const size_t n = (most - w) / row_slot_bytes(Ci);
     return n < (size_t)kRowSlots ? (int)n : kRowSlots;
 }
 size_t conv_row_smem_bytes(int Ci, int Co, int slots) {
@@ -397,13 +456,14 @@ __host__ __device__ inline uint32_t row_tmem_cols(int Co) {
 }
 
 template <bool ACT>
-__global__ void __launch_bounds__(kRowThreads, 1)
+__global__ void __launch_bounds__(kRoleThreads, 1)
 conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, const float* __restrict__ bias,
                 void* __restrict__ y, int csy, int N, int H, int W, int Ci, int Co, int rows_per_cta, int slots,
                 int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t bars[2];
+    __shared__ __align__(8) uint64_t bars[kRowSlots + 4];   // full[slot], then done[2], drained[2]
     __shared__ uint32_t tmem_slot;
+    __shared__ int failed;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const int segs = W / kRowM;
     const int chunks = (H + rows_per_cta - 1) / rows_per_cta;
@@ -417,7 +477,7 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
     const uint32_t wb = smem_u32(smem);                  // weights, then the ring
     const uint32_t sb = wb + row_w_bytes(Ci, Co);
     const uint32_t slot_bytes = row_slot_bytes(Ci), wchunk = row_w_chunk(Co);
-    const uint32_t bar0 = smem_u32(&bars[0]);
+    const uint32_t full = smem_u32(&bars[0]), mma_done = full + 8 * kRowSlots, drained = mma_done + 16;
     const uint32_t ncols = row_tmem_cols(Co);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
@@ -426,70 +486,71 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int k = 0; k < 2; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * k) : "memory");
+        for (int k = 0; k < slots; ++k) mbar_init(full + 8 * k, kWorkers);
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(mma_done + 8 * k, 1);
+            mbar_init(drained + 8 * k, kWorkers);
+        }
+        failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
-    const uint32_t idesc = tc_idesc_bf16(kRowM, Co);
     const int nch = Ci / 8;
-    const long long img = (long long)n * H * W;
     const int nrows = y1 - y0;
-    // input row k of the march (image row y0 - 1 + k, wrapped; k <= nrows + 1)
-    // into ring slot k % slots: pixels x0 - 1 .. x0 + 128 (wrapped)
-    auto copy_row = [&](int k) {
-        if (k > nrows + 1) return;
-        const int yr = ((y0 - 1 + k) % H + H) % H;
-        const uint32_t dst = sb + (uint32_t)(k % slots) * slot_bytes;
-        const bf16* row = x + (img + (long long)yr * W) * csx;
-        for (int e = tid; e < nch * kRowHalo; e += kRowThreads) {
-            const int px = e / nch, c = e - px * nch;
-            int xx = x0 - 1 + px;
-            xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
-            cp_async16(dst + c * row_plane_bytes() + px * 16, row + (long long)xx * csx + c * 8, 16u);
-        }
-    };
-    // prologue: group 0 is the weights of every tap and input rows 0 .. 2, each
-    // later group one row
-    const int ahead = slots - 3;
-    for (int k = tid; k < 9 * nch * Co; k += kRowThreads) {
-        const int row = k / nch, c = k - row * nch, co = row / 9, tap = row - co * 9;
-        cp_async16(wb + (uint32_t)(tap * nch + c) * wchunk + co * 16, w + (long long)row * Ci + c * 8, 16u);
-    }
-    for (int k = 0; k < 3; ++k) copy_row(k);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    for (int k = 1; k < ahead; ++k) {
-        copy_row(2 + k);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    bool ok = true;
-    // row j of the march (row y0 + j) accumulates in buffer j & 1 and commits
-    // to barrier j & 1: the (j >> 1)-th phase of that barrier
-    auto wait_row = [&](int j) { return mbar_wait_bounded(bar0 + 8 * (j & 1), (uint32_t)(j >> 1) & 1u, kTcPolls); };
-    const bool vec = conv_vec<ACT>(y, csy);
-    auto epilogue = [&](int j) {   // warps w and w + 4 share a quarter of the lanes
-        const uint32_t acc = tmem + (uint32_t)((j & 1) * Co) + ((uint32_t)(32 * (warp & 3)) << 16);
-        const long long pix = img + (long long)(y0 + j) * W + x0 + 32 * (warp & 3) + lane;
-        for (int c0 = 16 * (warp >> 2); c0 < Co; c0 += 32) {
-            float v[16];
-            tc_ld16(acc + (uint32_t)c0, v);
-            conv_store16<ACT>(y, pix * csy + c0, v, bias ? bias + c0 : nullptr, vec);
-        }
-    };
-    int issued = 0;   // rows whose MMAs were issued and committed
-    for (int j = 0; j < nrows; ++j) {
-        // input rows j .. j + 2 landed (the ahead - 1 newer groups may be pending)
-        if (ahead >= 3) asm volatile("cp.async.wait_group 2;" ::: "memory");
-        else if (ahead == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
-        else asm volatile("cp.async.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        if (warp == 0) {
+    // row j of the march (row y0 + j) sums in buffer j & 1 over input rows
+    // j .. j + 2 (input row k: image row y0 - 1 + k, wrapped, in slot k % slots)
+    int issued = 0;
+    if (warp < kWorkers / 32) {
+        const long long img = (long long)n * H * W;
+        auto copy_row = [&](int k) {   // pixels x0 - 1 .. x0 + 128 (wrapped)
+            if (k > nrows + 1) return;
+            const int yr = ((y0 - 1 + k) % H + H) % H;
+            const uint32_t dst = sb + (uint32_t)(k % slots) * slot_bytes;
+            const bf16* row = x + (img + (long long)yr * W) * csx;
+            for_groups(tid, kRowHalo, nch, [&](int px, int c) {
+                int xx = x0 - 1 + px;
+                xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
+                cp_async16(dst + c * row_plane_bytes() + px * 16, row + xx * csx + c * 8, 16u);
+            });
+            mbar_arrive_copies(full + 8 * (k % slots));
+        };
+        for_groups(tid, 9 * Co, nch, [&](int row, int c) {   // the weights: landed with row 0
+            const int co = row / 9, tap = row - co * 9;
+            cp_async16(wb + (uint32_t)(tap * nch + c) * wchunk + co * 16, w + (long long)row * Ci + c * 8, 16u);
+        });
+        for (int k = 0; k < slots; ++k) copy_row(k);
+        const bool vec = conv_vec<ACT>(y, csy);
+        for (int j = 0; j < nrows; ++j) {
+            if (!mbar_wait_phase(mma_done + 8 * (j & 1), j >> 1, &failed)) break;
+            copy_row(j + slots);   // into the slot of input row j, read last by row j
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t el = tc_elect();
+            // warps w and w + 4 share a quarter of the lanes
+            const uint32_t acc = tmem + (uint32_t)((j & 1) * Co) + ((uint32_t)(32 * (warp & 3)) << 16);
+            const long long pix = img + (long long)(y0 + j) * W + x0 + 32 * (warp & 3) + lane;
+            for (int c0 = 16 * (warp >> 2); c0 < Co; c0 += 32) {
+                float v[16];
+                tc_ld16(acc + (uint32_t)c0, v);
+                conv_store16<ACT>(y, pix * csy + c0, v, bias ? bias + c0 : nullptr, vec);
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            mbar_arrive(drained + 8 * (j & 1));
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    } else {
+        const uint32_t idesc = tc_idesc_bf16(kRowM, Co);
+        const uint32_t el = tc_elect();
+        bool ok = true;
+        for (int j = 0; j < nrows && ok; ++j) {
+            for (int k = j == 0 ? 0 : j + 2; k <= j + 2 && ok; ++k)
+                ok = mbar_wait_phase(full + 8 * (k % slots), k / slots, &failed);
+            if (ok && j >= 2) ok = mbar_wait_phase(drained + 8 * (j & 1), (j >> 1) - 1, &failed);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t acc = tmem + (uint32_t)((j & 1) * Co);
             for (int dy = 0; dy < 3; ++dy) {
                 const uint32_t a_s = sb + (uint32_t)((j + dy) % slots) * slot_bytes;
@@ -500,34 +561,18 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
                     tc_mma_run(el, acc, ad, bd, 2 * row_plane_bytes() / 16, 2 * wchunk / 16, idesc, nch / 2, tap > 0);
                 }
             }
-            tc_commit(el, bar0 + 8 * (j & 1));
+            tc_commit(el, mma_done + 8 * (j & 1));
+            issued = j + 1;
         }
-        issued = j + 1;
-        // row j - 1 done: its oldest input row (j - 1) makes room for row
-        // j + 2 + ahead, and its accumulator goes out
-        if (j > 0 && !__syncthreads_and(wait_row(j - 1))) { ok = false; break; }
-        copy_row(j + 2 + ahead);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        if (j > 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            epilogue(j - 1);
-        }
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    // the last issued row: its MMAs complete after every earlier one (waited
-    // for on the failure path too, before the tensor memory is freed)
-    if (issued > 0) {
-        const bool done = wait_row(issued - 1);
-        const bool all = __syncthreads_and(ok && done) != 0;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (all && issued == nrows) epilogue(issued - 1);
-        ok = all && ok;
+        // the MMAs still running (on the failure path) end before the tensor
+        // memory is freed
+        if (issued > 0) mbar_wait_bounded(mma_done + 8 * ((issued - 1) & 1), (uint32_t)((issued - 1) >> 1) & 1u, kTcPolls);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
-    if (!ok && tid == 0) atomicExch(err, 1);
+    if (tid == 0 && failed) atomicExch(err, 1);
 }
 
 // ---------------------------------------------------------------- tcgen05 convolution, flat tiles
@@ -541,7 +586,6 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
 // kernel copies 9 x 128 pixels, a stage of 64 channels at a time), and the
 // weights tap by tap through a ring of `stages` buffers.  Taps and channels in
 // the tap kernel's order.
-constexpr int kFlatThreads = 256;
 constexpr int kFlatStages = 9;
 
 __host__ __device__ inline int flat_cells(int W) { return 128 + 2 * (W + 3); }
@@ -558,18 +602,19 @@ inline int flat_stages(int W, int Ci, int Co) {
 }
 
 template <bool ACT>
-__global__ void __launch_bounds__(kFlatThreads, 1)
+__global__ void __launch_bounds__(kRoleThreads, 1)
 conv_flat_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, const float* __restrict__ bias,
                  void* __restrict__ y, int csy, int H, int W, int Ci, int Co, int tiles, int stages, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t bars[kFlatStages];
+    __shared__ __align__(8) uint64_t bars[2 * kFlatStages];   // full[stage], done[stage]
     __shared__ uint32_t tmem_slot;
+    __shared__ int failed;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const int n = blockIdx.x / tiles, f0 = (blockIdx.x - n * tiles) * 128;
     const int Wp = W + 2, nch = Ci / 8, cells = flat_cells(W);
     const uint32_t xs = smem_u32(smem), plane = flat_plane(W);
     const uint32_t ws = xs + flat_x_bytes(W, Ci), wstage = flat_w_bytes(Ci, Co), wchunk = row_w_chunk(Co);
-    const uint32_t bar0 = smem_u32(&bars[0]);
+    const uint32_t full = smem_u32(&bars[0]), mma_done = full + 8 * kFlatStages;
     const uint32_t ncols = Co <= 32 ? 32u : (Co <= 64 ? 64u : 128u);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
@@ -578,96 +623,82 @@ conv_flat_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int k = 0; k < stages; ++k)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * k) : "memory");
+        for (int k = 0; k < stages; ++k) {
+            mbar_init(full + 8 * k, kWorkers);
+            mbar_init(mma_done + 8 * k, 1);
+        }
+        failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
-    const long long img = (long long)n * H * W;
-    auto copy_w = [&](int tap) {   // the tap's weights into buffer tap % stages, as one commit group
-        if (tap < 9) {
+    int issued = 0;
+    if (warp < kWorkers / 32) {
+        const long long img = (long long)n * H * W;
+        auto copy_w = [&](int tap) {   // the tap's weights into buffer tap % stages
             const uint32_t dst = ws + (uint32_t)(tap % stages) * wstage;
-            for (int e = tid; e < Co * nch; e += kFlatThreads) {
-                const int co = e / nch, c = e - co * nch;
-                cp_async16(dst + c * wchunk + co * 16, w + ((long long)co * 9 + tap) * Ci + c * 8, 16u);
+            const bf16* src = w + (long long)tap * Ci;
+            for_groups(tid, Co, nch, [&](int co, int c) {
+                cp_async16(dst + c * wchunk + co * 16, src + (long long)co * 9 * Ci + c * 8, 16u);
+            });
+            mbar_arrive_copies(full + 8 * (tap % stages));
+        };
+        // cell k of the tile: padded cell f0 + k, row -1 .. H and column -1 .. W of
+        // the image (rows past H, behind the last tile, wrap like the rest);
+        // landed with the weights of tap 0
+        const bf16* src = x + img * csx;
+        for_groups(tid, cells, nch, [&](int k, int c) {
+            const int id = f0 + k, row = id / Wp;
+            const int yy = (row - 1 + H) % H;
+            int xx = id - row * Wp - 1;
+            xx = xx < 0 ? W - 1 : (xx >= W ? xx - W : xx);
+            cp_async16(xs + c * plane + k * 16, src + ((long long)yy * W + xx) * csx + c * 8, 16u);
+        });
+        bool ok = true;
+        for (int t = 0; t < 9 && ok; ++t) {
+            if (t >= stages) ok = mbar_wait_phase(mma_done + 8 * (t % stages), t / stages - 1, &failed);
+            if (ok) copy_w(t);
+        }
+        if (ok) ok = mbar_wait_phase(mma_done + 8 * (8 % stages), 8 / stages, &failed);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if (__all_sync(0xffffffffu, ok)) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int f = f0 + 32 * (warp & 3) + lane, row = f / Wp, col = f - row * Wp;
+            const bool in = row < H && col < W;
+            const long long pix = img + (long long)row * W + col;
+            const bool vec = conv_vec<ACT>(y, csy);
+            for (int c0 = 16 * (warp >> 2); c0 < Co; c0 += 32) {
+                float v[16];
+                tc_ld16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, v);
+                if (in) conv_store16<ACT>(y, pix * csy + c0, v, bias ? bias + c0 : nullptr, vec);
             }
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    // cell k of the tile: padded cell f0 + k, row -1 .. H and column -1 .. W of
-    // the image (rows past H, behind the last tile, wrap like the rest)
-    for (int e = tid; e < cells * nch; e += kFlatThreads) {
-        const int k = e / nch, c = e - k * nch;
-        const int id = f0 + k, row = id / Wp;
-        const int yy = (row - 1 + H) % H, xx = (id - row * Wp - 1 + W) % W;
-        cp_async16(xs + c * plane + k * 16, x + (img + (long long)yy * W + xx) * csx + c * 8, 16u);
-    }
-    for (int t = 0; t < stages; ++t) copy_w(t);     // group 0 holds the cells too
-    const uint32_t idesc = tc_idesc_bf16(128, Co);
-    bool ok = true;
-    int issued = 0;
-    auto wait_tap = [&](int t) {
-        return mbar_wait_bounded(bar0 + 8 * (t % stages), (uint32_t)(t / stages) & 1u, kTcPolls);
-    };
-    for (int t = 0; t < 9; ++t) {
-        // tap t's group landed: `stages` groups are committed ahead of it, less
-        // the one whose buffer is refilled after the MMAs of tap t - 1
-        if (t == 0 && stages > 1) {
-            // every group but the first may be pending
-            switch (stages) {
-                case 2: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
-                case 3: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
-                case 4: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
-                default: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
-            }
-        } else if (stages >= 4) asm volatile("cp.async.wait_group 2;" ::: "memory");
-        else if (stages == 3) asm volatile("cp.async.wait_group 1;" ::: "memory");
-        else asm volatile("cp.async.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (warp == 0) {
+    } else {
+        const uint32_t idesc = tc_idesc_bf16(128, Co);
+        const uint32_t el = tc_elect();
+        for (int t = 0; t < 9; ++t) {
+            const bool ok = mbar_wait_phase(full + 8 * (t % stages), t / stages, &failed);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t el = tc_elect();
             const uint64_t ad = tc_smem_desc(xs + (uint32_t)((t / 3) * Wp + t % 3) * 16, plane, 128);
             const uint64_t bd = tc_smem_desc(ws + (uint32_t)(t % stages) * wstage, wchunk, 128);
             tc_mma_run(el, tmem, ad, bd, 2 * plane / 16, 2 * wchunk / 16, idesc, nch / 2, t > 0);
-            tc_commit(el, bar0 + 8 * (t % stages));
+            tc_commit(el, mma_done + 8 * (t % stages));
+            issued = t + 1;
         }
-        issued = t + 1;
-        // tap t - 1 done: its buffer takes the weights of tap t - 1 + stages
-        if (t > 0 && t - 1 + stages < 9) {
-            if (!__syncthreads_and(wait_tap(t - 1))) { ok = false; break; }
-            copy_w(t - 1 + stages);
-        } else if (t > 0) {
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        }
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    // the last committed tap completes after every earlier MMA of the CTA
-    if (issued > 0) {
-        const bool done = wait_tap(issued - 1);
-        ok = __syncthreads_and(ok && done) != 0;
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (ok) {
-        const int f = f0 + 32 * (warp & 3) + lane, row = f / Wp, col = f - row * Wp;
-        const bool in = row < H && col < W;
-        const long long pix = img + (long long)row * W + col;
-        const bool vec = conv_vec<ACT>(y, csy);
-        for (int c0 = 16 * (warp >> 2); c0 < Co; c0 += 32) {
-            float v[16];
-            tc_ld16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, v);
-            if (in) conv_store16<ACT>(y, pix * csy + c0, v, bias ? bias + c0 : nullptr, vec);
-        }
+        // the MMAs still running (on the failure path) end before the tensor
+        // memory is freed
+        if (issued > 0)
+            mbar_wait_bounded(mma_done + 8 * ((issued - 1) % stages), (uint32_t)((issued - 1) / stages) & 1u, kTcPolls);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
-    if (!ok && tid == 0) atomicExch(err, 1);
+    if (tid == 0 && failed) atomicExch(err, 1);
 }
 
 // partial[chunk, co, tap, ci] = sum over the chunk's pixels p of gy[p, co] x[shift(p, tap), ci];
@@ -734,14 +765,14 @@ __global__ void conv_wgrad_kernel(const bf16* __restrict__ x, int csx, const bf1
 // of a row issued while those of the one before still run.  The taps (all
 // nine where their columns fit tensor memory, else the three of one dy)
 // accumulate over the whole march and are written out once, as the CTA's
-// partial; partials are summed in a fixed order (deterministic).  M = 128
-// always: the rows past a side's channels read whatever lies behind its planes
-// and are not written out.
+// partial; partials are summed in a fixed order (deterministic).  M is 64 up
+// to 64 channels, else 128 (24 against 40 clk per MMA at N = 32): the rows past a
+// side's channels read whatever lies behind its planes and are not written out.
 constexpr int kWgCn = 128;            // input channels of one CTA at most
-constexpr int kWgThreads = 288;          // a warp per tap issues its MMAs
 constexpr int kWgX = 6, kWgG = 4;     // rows in the rings
 constexpr size_t kWgSmemMax = 220 * 1024;   // below the 227 KB per CTA less the kernel's static shared memory
 
+__host__ __device__ inline int wg_m(int channels) { return channels <= 64 ? 64 : 128; }
 struct WgLayout {
     uint32_t px, pg;        // plane pitches of x and gy
     uint32_t xrow, grow;    // bytes of one row
@@ -754,8 +785,8 @@ __host__ __device__ inline WgLayout wg_layout(int P, int Cn, int Co) {
     L.pg = (uint32_t)(P | 1) * 16;
     L.xrow = (uint32_t)(Cn / 8) * L.px;
     L.grow = (uint32_t)(Co / 8) * L.pg;
-    // the 16 planes an M = 128 operand reads from the last row of its ring
-    const uint32_t tail = Cn >= Co ? (uint32_t)(16 - Cn / 8) * L.px : (uint32_t)(16 - Co / 8) * L.pg;
+    // the planes of all M rows an operand reads from the last row of its ring
+    const uint32_t tail = Cn >= Co ? (uint32_t)(wg_m(Cn) - Cn) / 8 * L.px : (uint32_t)(wg_m(Co) - Co) / 8 * L.pg;
     L.total = kWgX * L.xrow + kWgG * L.grow + tail;
     return L;
 }
@@ -766,13 +797,14 @@ __host__ __device__ inline uint32_t wg_tmem_cols(int Cn, int Co) {
     return need <= 32 ? 32u : (need <= 64 ? 64u : (need <= 128 ? 128u : (need <= 256 ? 256u : 512u)));
 }
 
-__global__ void __launch_bounds__(kWgThreads, 1)
+__global__ void __launch_bounds__(kRoleThreads, 1)
 conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ gy, int csg,
                       float* __restrict__ partial, int N, int H, int W, int Ci, int Co, int P, int Cn,
                       int rows_per_cta, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t bars[2];
+    __shared__ __align__(8) uint64_t bars[kWgX + 2 * kWgG];   // x rows, gy rows landed; MMAs of a gy row done
     __shared__ uint32_t tmem_slot;
+    __shared__ int failed;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const int segs = W / P;
     const int nsplit = Ci / Cn;
@@ -795,7 +827,7 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
     // the ring of the M side lies last, its tail behind it
     const uint32_t sb = smem_u32(smem);
     const uint32_t xb = x_is_a ? sb + kWgG * Lt.grow : sb, gb = x_is_a ? sb : sb + kWgX * Lt.xrow;
-    const uint32_t bar0 = smem_u32(&bars[0]);
+    const uint32_t full_x = smem_u32(&bars[0]), full_g = full_x + 8 * kWgX, mma_done = full_g + 8 * kWgG;
     const int Nc = wg_n(Cn, Co);
     const uint32_t ncols = wg_tmem_cols(Cn, Co);
     if (warp == 0) {
@@ -805,85 +837,93 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int k = 0; k < 2; ++k)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar0 + 8 * k), "r"(taps) : "memory");
+        for (int k = 0; k < kWgX + kWgG; ++k) mbar_init(full_x + 8 * k, kWorkers);
+        // one per gy slot: a slot's next MMAs wait for the workers that refill it,
+        // so no barrier can run a phase ahead of them
+        for (int k = 0; k < kWgG; ++k) mbar_init(mma_done + 8 * k, 1);
+        failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
-    // both operands MN-major (bits 15 and 16)
-    const uint32_t idesc = tc_idesc_bf16(128, Nc) | (1u << 15) | (1u << 16);
-    const int nco8 = Co / 8, nci8 = Cn / 8;
-    const long long img = (long long)n * H * W;
-    // row r0 + dy0 ... of x that the march reads start at y0 + dy0; ring slots
-    // count from there
-    auto x_slot = [&](int k) { return xb + (uint32_t)(k % kWgX) * Lt.xrow; };   // k-th x row of the march
-    auto g_slot = [&](int k) { return gb + (uint32_t)(k % kWgG) * Lt.grow; };
-    auto copy_x = [&](int k) {   // x row y0 + dy0 + k (wrapped), pixels x0 - 1 .. x0 + P (wrapped)
-        const int yy = y0 + dy0 + k;
-        const int yr = ((yy % H) + H) % H;
-        const bf16* row = x + (img + (long long)yr * W) * csx + ci0;
-        const uint32_t dst = x_slot(k);
-        for (int e = tid; e < (P + 2) * nci8; e += kWgThreads) {
-            const int q = e / nci8, c = e - q * nci8;
-            int xx = x0 - 1 + q;
-            xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
-            cp_async16(dst + c * Lt.px + q * 16, row + (long long)xx * csx + c * 8, 16u);
-        }
-    };
-    auto copy_g = [&](int k) {   // gy row y0 + k
-        const bf16* row = gy + (img + (long long)(y0 + k) * W + x0) * csg;
-        const uint32_t dst = g_slot(k);
-        for (int e = tid; e < P * nco8; e += kWgThreads) {
-            const int q = e / nco8, c = e - q * nco8;
-            cp_async16(dst + c * Lt.pg + q * 16, row + (long long)q * csg + c * 8, 16u);
-        }
-    };
     const int S = y1 - y0;
-    // group j: the gy row j and the last x row its taps read (group 0: all of them)
-    auto copy_group = [&](int j) {
-        if (j < S) {
-            if (j == 0)
-                for (int k = 0; k < ndy - 1; ++k) copy_x(k);
-            copy_x(j + ndy - 1);
-            copy_g(j);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    // the MMAs of row j commit to barrier j & 1: its (j >> 1)-th phase
-    auto wait_row = [&](int j) { return mbar_wait_bounded(bar0 + 8 * (j & 1), (uint32_t)(j >> 1) & 1u, kTcPolls); };
+    // row j of the march (gy row y0 + j, slot j % kWgG) reads x rows j .. j +
+    // ndy - 1 (x row k: image row y0 + dy0 + k, wrapped, slot k % kWgX)
     bool ok = true;
-    int issued = 0;
-    copy_group(0);
-    copy_group(1);
-    for (int j = 0; j < S; ++j) {
-        // group j + 2 goes where row j - 2's operands were
-        if (j >= 2 && !__syncthreads_and(wait_row(j - 2))) { ok = false; break; }
-        copy_group(j + 2);
-        asm volatile("cp.async.wait_group 2;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (warp < taps) {   // warp t: tap t (each tap its own accumulator)
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t el = tc_elect();
-            const uint64_t xd = tc_smem_desc(x_slot(j + warp / 3) + (uint32_t)(warp % 3) * 16, 128, Lt.px);
-            const uint64_t gd = tc_smem_desc(g_slot(j), 128, Lt.pg);
-            tc_mma_run(el, tmem + (uint32_t)(warp * Nc), x_is_a ? xd : gd, x_is_a ? gd : xd, 16, 16, idesc, P / 16,
-                       j > 0);
-            tc_commit(el, bar0 + 8 * (j & 1));
+    if (warp < kWorkers / 32) {
+        const int nco8 = Co / 8, nci8 = Cn / 8;
+        const long long img = (long long)n * H * W;
+        auto copy_x = [&](int k) {   // pixels x0 - 1 .. x0 + P (wrapped)
+            if (k > S + ndy - 2) return;
+            const int yr = ((y0 + dy0 + k) % H + H) % H;
+            const bf16* row = x + (img + (long long)yr * W) * csx + ci0;
+            const uint32_t dst = xb + (uint32_t)(k % kWgX) * Lt.xrow;
+            for_groups(tid, P + 2, nci8, [&](int q, int c) {
+                int xx = x0 - 1 + q;
+                xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
+                cp_async16(dst + c * Lt.px + q * 16, row + xx * csx + c * 8, 16u);
+            });
+            mbar_arrive_copies(full_x + 8 * (k % kWgX));
+        };
+        auto copy_g = [&](int k) {
+            if (k >= S) return;
+            const bf16* row = gy + (img + (long long)(y0 + k) * W + x0) * csg;
+            const uint32_t dst = gb + (uint32_t)(k % kWgG) * Lt.grow;
+            for_groups(tid, P, nco8, [&](int q, int c) {
+                cp_async16(dst + c * Lt.pg + q * 16, row + q * csg + c * 8, 16u);
+            });
+            mbar_arrive_copies(full_g + 8 * (k % kWgG));
+        };
+        for (int k = 0; k < ndy; ++k) copy_x(k);
+        for (int k = 0; k < kWgG; ++k) {
+            copy_g(k);
+            if (ndy + k < kWgX) copy_x(ndy + k);
         }
-        issued = j + 1;
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (issued > 0) {
-        const bool done = wait_row(issued - 1);
-        ok = __syncthreads_and(ok && done) != 0 && issued == S;
+        for (int k = ndy + kWgG; k < kWgX; ++k) copy_x(k);
+        for (int j = 0; j < S && ok; ++j) {   // row j done: its gy slot and its first x slot are free
+            ok = mbar_wait_phase(mma_done + 8 * (j % kWgG), j / kWgG, &failed);
+            if (ok) {
+                copy_x(j + kWgX);
+                copy_g(j + kWgG);
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        ok = __all_sync(0xffffffffu, ok) != 0;
+    } else {
+        // both operands MN-major (bits 15 and 16)
+        const uint32_t idesc = tc_idesc_bf16(wg_m(x_is_a ? Cn : Co), Nc) | (1u << 15) | (1u << 16);
+        const uint32_t el = tc_elect();
+        int issued = 0;
+        for (int j = 0; j < S && ok; ++j) {
+            for (int k = j == 0 ? 0 : j + ndy - 1; k <= j + ndy - 1 && ok; ++k)
+                ok = mbar_wait_phase(full_x + 8 * (k % kWgX), k / kWgX, &failed);
+            if (ok) ok = mbar_wait_phase(full_g + 8 * (j % kWgG), j / kWgG, &failed);
+            ok = __all_sync(0xffffffffu, ok) != 0;
+            if (!ok) break;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint64_t gd = tc_smem_desc(gb + (uint32_t)(j % kWgG) * Lt.grow, 128, Lt.pg);
+            for (int t = 0; t < taps; ++t) {
+                const int d = t / 3, dx = t - 3 * d;
+                const uint64_t xd = tc_smem_desc(xb + (uint32_t)((j + d) % kWgX) * Lt.xrow + (uint32_t)dx * 16, 128, Lt.px);
+                tc_mma_run(el, tmem + (uint32_t)(t * Nc), x_is_a ? xd : gd, x_is_a ? gd : xd, 16, 16, idesc, P / 16,
+                           j > 0);
+            }
+            tc_commit(el, mma_done + 8 * (j % kWgG));
+            issued = j + 1;
+        }
+        // the MMAs still running (on the failure path) end before the tensor
+        // memory is freed
+        if (issued > 0) mbar_wait_bounded(mma_done + 8 * ((issued - 1) % kWgG), (uint32_t)((issued - 1) / kWgG) & 1u, kTcPolls);
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (ok && warp < 4) {
-        const int m = 32 * warp + lane;          // channel of the M side
+        // channel of the M side: row m of an M = 128 accumulator is lane m, of an
+        // M = 64 one lane 32 (m / 16) + m % 16
+        const bool half = wg_m(x_is_a ? Cn : Co) == 64;
+        const int m = half ? (lane < 16 ? 16 * warp + lane : 128) : 32 * warp + lane;
         const int K9 = 9 * Ci;
         float* out = partial + pchunk * Co * (long long)K9;
         for (int t = 0; t < taps; ++t) {
@@ -909,18 +949,28 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
-    if (!ok && tid == 0) atomicExch(err, 1);
+    if (tid == 0 && failed) atomicExch(err, 1);
 }
 
-// gw[k] = sum over chunks of partial[chunk, k], in chunk order
-__global__ void sum_chunks_kernel(const float* __restrict__ partial, long long nchunks, long long K,
-                                  float* __restrict__ gw) {
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
+// gw[k] = sum over chunks of partial[chunk, k] in a fixed order: 32 values per
+// block, each by eight threads that take every eighth chunk (one thread per
+// value left 18 blocks for the 16 -> 32 layer's 4608 values of 304 chunks: 27 us).
+__global__ void __launch_bounds__(256)
+sum_chunks_kernel(const float* __restrict__ partial, long long nchunks, long long K, float* __restrict__ gw) {
+    __shared__ float sh[8][32];
+    const int i = threadIdx.x & 31, part = threadIdx.x >> 5;
+    const long long k = (long long)blockIdx.x * 32 + i;
     float s = 0.0f;
+    if (k < K) {
 #pragma unroll 8
-    for (long long c = 0; c < nchunks; ++c) s += partial[c * K + k];
-    gw[k] = s;
+        for (long long c = part; c < nchunks; c += 8) s += partial[c * K + k];
+    }
+    sh[part][i] = s;
+    __syncthreads();
+    if (part == 0 && k < K) {
+        for (int q = 1; q < 8; ++q) s += sh[q][i];
+        gw[k] = s;
+    }
 }
 
 // wt[ci, 8 - tap, co] = w[co, tap, ci]: the weights of the input-gradient convolution
@@ -1675,22 +1725,27 @@ static int conv3x3(const void* x, int csx, const void* w, const float* bias, voi
     // march, flat tiles, tap kernel: see the table at conv3x3's callers.)
     int sms = 1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LBM_ECUDA;
-    const int slots = conv_row_slots_of(Ci, Co);
-    if (W % kRowM == 0 && slots >= 4) {
+    // CTAs on an SM: up to three, whose copies, MMAs and stores overlap, as long
+    // as each keeps eight rows to spread its weights and halo rows over
+    const long long row_segs = W % kRowM ? 0 : (long long)N * H * (W / kRowM);
+    int per_sm = row_segs ? 3 : 0;
+    while (per_sm > 0 && (per_sm * row_tmem_cols(Co) > 512 || conv_row_slots_of(Ci, Co, per_sm) < 4 ||
+                          (per_sm > 1 && row_segs < 8LL * per_sm * sms)))
+        --per_sm;
+    if (per_sm > 0) {
+        const int slots = conv_row_slots_of(Ci, Co, per_sm);
         static bool done[64] = {};
         if (large_smem(conv_row_kernel<ACT>, done, dev) != cudaSuccess) {
             cudaGetLastError();
             return LBM_ECUDA;
         }
         const long long cols = (long long)N * (W / kRowM);
-        // one CTA per SM: the weights and the two halo rows of a chunk are
-        // loaded once per CTA
-        long long chunks = sms / cols;
+        long long chunks = (long long)sms * per_sm / cols;
         if (chunks < 1) chunks = 1;
         if (chunks > H) chunks = H;
         const int rows = (int)((H + chunks - 1) / chunks);
         const long long nb = cols * ((H + rows - 1) / rows);
-        conv_row_kernel<ACT><<<(unsigned)nb, kRowThreads,
+        conv_row_kernel<ACT><<<(unsigned)nb, kRoleThreads,
                                conv_row_launch_smem(conv_row_smem_bytes(Ci, Co, slots), Co), s>>>(
             (const bf16*)x, csx, (const bf16*)w, bias, y, csy, N, H, W, Ci, Co, rows, slots, err);
         return check(cudaGetLastError());
@@ -1708,7 +1763,7 @@ static int conv3x3(const void* x, int csx, const void* w, const float* bias, voi
             // no more CTAs on an SM than its tensor memory serves (four of 128 columns)
             const size_t need = flat_x_bytes(W, Ci) + (size_t)stages * flat_w_bytes(Ci, Co);
             const size_t least = sm_shared_bytes() / 5 + 1;
-            conv_flat_kernel<ACT><<<(unsigned)(N * tiles), kFlatThreads, need > least ? need : least, s>>>(
+            conv_flat_kernel<ACT><<<(unsigned)(N * tiles), kRoleThreads, need > least ? need : least, s>>>(
                 (const bf16*)x, csx, (const bf16*)w, bias, y, csy, H, W, Ci, Co, tiles, stages, err);
             return check(cudaGetLastError());
         }
@@ -1783,11 +1838,11 @@ int lbm_sg_conv3x3_wgrad(const void* x, int csx, const void* gy, int csg, float*
         const int P = wg_segment(W, Ci, Co), Cn = wg_block(Ci);
         const long long pchunks = (long long)N * (W / P) * rchunks;
         const WgLayout Lt = wg_layout(P, Cn, Co);
-        conv_wgrad_row_kernel<<<(unsigned)((9 / wg_taps(Cn, Co)) * (Ci / Cn) * pchunks), kWgThreads,
+        conv_wgrad_row_kernel<<<(unsigned)((9 / wg_taps(Cn, Co)) * (Ci / Cn) * pchunks), kRoleThreads,
                                 wg_launch_smem(Lt.total, Cn, Co), s>>>(
             (const bf16*)x, csx, (const bf16*)gy, csg, scratch, N, H, W, Ci, Co, P, Cn, rows, err);
         const long long K = (long long)Co * 9 * Ci;
-        sum_chunks_kernel<<<blocks(K), kThreads, 0, s>>>(scratch, pchunks, K, gw);
+        sum_chunks_kernel<<<(unsigned)((K + 31) / 32), 256, 0, s>>>(scratch, pchunks, K, gw);
         return check(cudaGetLastError());
     }
     const long long nchunks = (M + kChunk - 1) / kChunk;
@@ -1796,7 +1851,7 @@ int lbm_sg_conv3x3_wgrad(const void* x, int csx, const void* gy, int csg, float*
     conv_wgrad_kernel<<<(unsigned)((warps * 32 + 127) / 128), 128, 0, s>>>((const bf16*)x, csx, (const bf16*)gy, csg,
                                                                           scratch, M, H, W, Ci, Co);
     const long long K = (long long)Co * 9 * Ci;
-    sum_chunks_kernel<<<blocks(K), kThreads, 0, s>>>(scratch, nchunks, K, gw);
+    sum_chunks_kernel<<<(unsigned)((K + 31) / 32), 256, 0, s>>>(scratch, nchunks, K, gw);
     return check(cudaGetLastError());
 }
 

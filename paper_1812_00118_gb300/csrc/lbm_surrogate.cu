@@ -150,27 +150,27 @@ __device__ __forceinline__ void tc_commit(uint32_t el, uint32_t bar) {
 // n MMAs of K = 16 into one accumulator, operand descriptors a step apart (the
 // address field counts 16-byte units and never carries out of its 14 bits); the
 // first one starts the sum unless `acc`.  Called by a whole warp with uniform
-// arguments, four MMAs per loop pass: the descriptors then stay in uniform
-// registers and the issue keeps up with the tensor core.  (clk per MMA of M =
-// 128, K = 16, N = 32 / 128, one CTA: 40 / 64; from a branch of one thread
-// that steps the descriptors, 155 / 155; the core itself needs 64 at N = 128,
-// and 32 to read A at N = 32.)
+// arguments, and straight-line for the counts that occur (powers of two): the
+// descriptors then stay in uniform registers and the issue keeps up with the
+// tensor core.  (clk per MMA of M = 128, K = 16, N = 32 / 128, one CTA: 40 / 64;
+// in a loop of one MMA per pass 120; from a branch of one thread that steps the
+// descriptors 155; the core itself needs 64 at N = 128, and 32 to read A.)
+template <int N>
+__device__ __forceinline__ void tc_mma_fixed(uint32_t el, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t a_step,
+                                             uint32_t b_step, uint32_t idesc, bool acc) {
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        tc_mma(el, d_tmem, a + (uint64_t)k * a_step, b + (uint64_t)k * b_step, idesc, (k > 0 || acc) ? 1u : 0u);
+}
 __device__ __forceinline__ void tc_mma_run(uint32_t el, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t a_step,
                                            uint32_t b_step, uint32_t idesc, int n, bool acc) {
-    tc_mma(el, d_tmem, a, b, idesc, acc ? 1u : 0u);
-    int k = 1;
-    for (; k + 4 <= n; k += 4) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            a += a_step;
-            b += b_step;
-            tc_mma(el, d_tmem, a, b, idesc, 1u);
-        }
-    }
-    for (; k < n; ++k) {
-        a += a_step;
-        b += b_step;
-        tc_mma(el, d_tmem, a, b, idesc, 1u);
+    for (int k = 0; k < n;) {
+        const uint64_t ak = a + (uint64_t)((uint32_t)k * a_step), bk = b + (uint64_t)((uint32_t)k * b_step);
+        const bool on = acc || k > 0;
+        if (n - k >= 8) { tc_mma_fixed<8>(el, d_tmem, ak, bk, a_step, b_step, idesc, on); k += 8; }
+        else if (n - k >= 4) { tc_mma_fixed<4>(el, d_tmem, ak, bk, a_step, b_step, idesc, on); k += 4; }
+        else if (n - k >= 2) { tc_mma_fixed<2>(el, d_tmem, ak, bk, a_step, b_step, idesc, on); k += 2; }
+        else { tc_mma_fixed<1>(el, d_tmem, ak, bk, a_step, b_step, idesc, on); k += 1; }
     }
 }
 
@@ -206,10 +206,11 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 __device__ __forceinline__ void mbar_arrive_copies(uint32_t bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
-// Wait for the k-th phase (from 0) of a barrier; false once it, or another wait
-// of the CTA, has given up (*failed).
+// Wait for the phase of parity k & 1 of a barrier (its k-th, from 0); false once
+// it, or another wait of the CTA, has given up (*failed).
 __device__ __forceinline__ bool mbar_wait_phase(uint32_t bar, int k, volatile int* failed) {
     const uint32_t parity = (uint32_t)k & 1u;
+    if (mbar_try(bar, parity)) return true;
     for (long i = 0; i < kTcPolls; ++i) {
         if (mbar_try(bar, parity)) return true;
         if ((i & 255) == 255 && *failed) return false;
@@ -246,11 +247,14 @@ __device__ __forceinline__ void st_global_32(void* p, const uint32_t (&v)[8]) {
 // 16 channels of one pixel of a convolution's output, as FP32 or (ACT) as the
 // bf16 values after the ReLU, which is all the next layer and the backward
 // pass read of them; `vec`: every pixel's channels start on a 32-byte boundary.
+// bias: 16 floats, 16-byte aligned (zeros where there is none).
 template <bool ACT>
-__device__ __forceinline__ void conv_store16(void* y, long long at, float (&v)[16], const float* __restrict__ bias,
-                                             bool vec) {
+__device__ __forceinline__ void conv_store16(void* y, long long at, float (&v)[16], const float* bias, bool vec) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] += bias ? bias[i] : 0.0f;
+    for (int i = 0; i < 16; i += 4) {
+        const float4 b = *reinterpret_cast<const float4*>(bias + i);
+        v[i] += b.x; v[i + 1] += b.y; v[i + 2] += b.z; v[i + 3] += b.w;
+    }
     if constexpr (ACT) {
         bf16* out = (bf16*)y + at;
         __nv_bfloat162 h[8];
@@ -293,6 +297,7 @@ conv_tc_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, 
                void* __restrict__ y, int csy, long long M, int H, int W, int Ci, int Co, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[kTcBuf];
+    __shared__ __align__(16) float bias_s[128];
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const long long p0 = (long long)blockIdx.x * kTcM;
@@ -302,6 +307,7 @@ conv_tc_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, 
     // buffer b: A at sb + b stage_bytes, B a_bytes after it; its barrier at bar0 + 8 b
     const uint32_t bar0 = smem_u32(&bars[0]);
     const uint32_t ncols = Co <= 32 ? 32u : (Co <= 64 ? 64u : 128u);
+    if (tid < Co) bias_s[tid] = bias ? bias[tid] : 0.0f;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                      "r"(ncols)
@@ -389,7 +395,7 @@ conv_tc_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, 
         for (int c0 = 0; c0 < Co; c0 += 16) {
             float v[16];
             tc_ld16(trow + (uint32_t)c0, v);
-            if (pr < M) conv_store16<ACT>(y, pr * csy + c0, v, bias ? bias + c0 : nullptr, vec);
+            if (pr < M) conv_store16<ACT>(y, pr * csy + c0, v, bias_s + c0, vec);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -462,6 +468,7 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
                 int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[kRowSlots + 4];   // full[slot], then done[2], drained[2]
+    __shared__ __align__(16) float bias_s[128];
     __shared__ uint32_t tmem_slot;
     __shared__ int failed;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
@@ -479,6 +486,7 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
     const uint32_t slot_bytes = row_slot_bytes(Ci), wchunk = row_w_chunk(Co);
     const uint32_t full = smem_u32(&bars[0]), mma_done = full + 8 * kRowSlots, drained = mma_done + 16;
     const uint32_t ncols = row_tmem_cols(Co);
+    if (tid < Co) bias_s[tid] = bias ? bias[tid] : 0.0f;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                      "r"(ncols)
@@ -505,64 +513,73 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
     int issued = 0;
     if (warp < kWorkers / 32) {
         const long long img = (long long)n * H * W;
-        auto copy_row = [&](int k) {   // pixels x0 - 1 .. x0 + 128 (wrapped)
-            if (k > nrows + 1) return;
-            const int yr = ((y0 - 1 + k) % H + H) % H;
-            const uint32_t dst = sb + (uint32_t)(k % slots) * slot_bytes;
-            const bf16* row = x + (img + (long long)yr * W) * csx;
+        // the next input row to copy: its number, slot and image row
+        int ck = 0, cs = 0, cy = y0 == 0 ? H - 1 : y0 - 1;
+        auto copy_next = [&]() {   // pixels x0 - 1 .. x0 + 128 (wrapped)
+            if (ck > nrows + 1) return;
+            const uint32_t dst = sb + (uint32_t)cs * slot_bytes;
+            const bf16* row = x + (img + (long long)cy * W) * csx;
             for_groups(tid, kRowHalo, nch, [&](int px, int c) {
                 int xx = x0 - 1 + px;
                 xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
                 cp_async16(dst + c * row_plane_bytes() + px * 16, row + xx * csx + c * 8, 16u);
             });
-            mbar_arrive_copies(full + 8 * (k % slots));
+            mbar_arrive_copies(full + 8 * cs);
+            ++ck;
+            cs = cs + 1 == slots ? 0 : cs + 1;
+            cy = cy + 1 == H ? 0 : cy + 1;
         };
         for_groups(tid, 9 * Co, nch, [&](int row, int c) {   // the weights: landed with row 0
             const int co = row / 9, tap = row - co * 9;
             cp_async16(wb + (uint32_t)(tap * nch + c) * wchunk + co * 16, w + (long long)row * Ci + c * 8, 16u);
         });
-        for (int k = 0; k < slots; ++k) copy_row(k);
+        for (int k = 0; k < slots; ++k) copy_next();
         const bool vec = conv_vec<ACT>(y, csy);
-        for (int j = 0; j < nrows; ++j) {
+        // warps w and w + 4 share a quarter of the lanes
+        const uint32_t acc0 = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+        long long at = (img + (long long)y0 * W + x0 + 32 * (warp & 3) + lane) * csy;
+        for (int j = 0; j < nrows; ++j, at += (long long)W * csy) {
             if (!mbar_wait_phase(mma_done + 8 * (j & 1), j >> 1, &failed)) break;
-            copy_row(j + slots);   // into the slot of input row j, read last by row j
+            copy_next();   // row j + slots, into the slot of input row j, read last by row j
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // warps w and w + 4 share a quarter of the lanes
-            const uint32_t acc = tmem + (uint32_t)((j & 1) * Co) + ((uint32_t)(32 * (warp & 3)) << 16);
-            const long long pix = img + (long long)(y0 + j) * W + x0 + 32 * (warp & 3) + lane;
             for (int c0 = 16 * (warp >> 2); c0 < Co; c0 += 32) {
                 float v[16];
-                tc_ld16(acc + (uint32_t)c0, v);
-                conv_store16<ACT>(y, pix * csy + c0, v, bias ? bias + c0 : nullptr, vec);
+                tc_ld16(acc0 + (uint32_t)((j & 1) * Co + c0), v);
+                conv_store16<ACT>(y, at + c0, v, bias_s + c0, vec);
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             mbar_arrive(drained + 8 * (j & 1));
         }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else {
         const uint32_t idesc = tc_idesc_bf16(kRowM, Co);
         const uint32_t el = tc_elect();
-        bool ok = true;
+        // slots of input rows j, j + 1, j + 2; phase of the newest
+        int s0 = 0, s1 = 1, s2 = 2, ph = 0;
+        bool ok = mbar_wait_phase(full, 0, &failed) && mbar_wait_phase(full + 8, 0, &failed);
+        const uint64_t a_hi = tc_smem_desc(0, row_plane_bytes(), 128), b0 = tc_smem_desc(wb, wchunk, 128);
+        const uint32_t b_tap = (uint32_t)nch * wchunk / 16;
         for (int j = 0; j < nrows && ok; ++j) {
-            for (int k = j == 0 ? 0 : j + 2; k <= j + 2 && ok; ++k)
-                ok = mbar_wait_phase(full + 8 * (k % slots), k / slots, &failed);
+            ok = mbar_wait_phase(full + 8 * s2, ph, &failed);
             if (ok && j >= 2) ok = mbar_wait_phase(drained + 8 * (j & 1), (j >> 1) - 1, &failed);
             if (!__all_sync(0xffffffffu, ok)) break;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t acc = tmem + (uint32_t)((j & 1) * Co);
+#pragma unroll
             for (int dy = 0; dy < 3; ++dy) {
-                const uint32_t a_s = sb + (uint32_t)((j + dy) % slots) * slot_bytes;
-                for (int dx = 0; dx < 3; ++dx) {
-                    const int tap = 3 * dy + dx;
-                    const uint64_t ad = tc_smem_desc(a_s + (uint32_t)dx * 16, row_plane_bytes(), 128);
-                    const uint64_t bd = tc_smem_desc(wb + (uint32_t)(tap * nch) * wchunk, wchunk, 128);
-                    tc_mma_run(el, acc, ad, bd, 2 * row_plane_bytes() / 16, 2 * wchunk / 16, idesc, nch / 2, tap > 0);
-                }
+                const uint64_t ad = a_hi + (uint64_t)((sb + (uint32_t)(dy == 0 ? s0 : (dy == 1 ? s1 : s2)) * slot_bytes) >> 4);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx)
+                    tc_mma_run(el, acc, ad + (uint64_t)dx, b0 + (uint64_t)((3 * dy + dx) * b_tap),
+                               2 * row_plane_bytes() / 16, 2 * wchunk / 16, idesc, nch / 2, dy + dx > 0);
             }
             tc_commit(el, mma_done + 8 * (j & 1));
             issued = j + 1;
+            s0 = s1;
+            s1 = s2;
+            s2 = s2 + 1 == slots ? 0 : s2 + 1;
+            ph ^= s2 == 0;
         }
         // the MMAs still running (on the failure path) end before the tensor
         // memory is freed
@@ -607,6 +624,7 @@ conv_flat_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w
                  void* __restrict__ y, int csy, int H, int W, int Ci, int Co, int tiles, int stages, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[2 * kFlatStages];   // full[stage], done[stage]
+    __shared__ __align__(16) float bias_s[128];
     __shared__ uint32_t tmem_slot;
     __shared__ int failed;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
@@ -616,6 +634,7 @@ conv_flat_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w
     const uint32_t ws = xs + flat_x_bytes(W, Ci), wstage = flat_w_bytes(Ci, Co), wchunk = row_w_chunk(Co);
     const uint32_t full = smem_u32(&bars[0]), mma_done = full + 8 * kFlatStages;
     const uint32_t ncols = Co <= 32 ? 32u : (Co <= 64 ? 64u : 128u);
+    if (tid < Co) bias_s[tid] = bias ? bias[tid] : 0.0f;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                      "r"(ncols)
@@ -672,7 +691,7 @@ conv_flat_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w
             for (int c0 = 16 * (warp >> 2); c0 < Co; c0 += 32) {
                 float v[16];
                 tc_ld16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, v);
-                if (in) conv_store16<ACT>(y, pix * csy + c0, v, bias ? bias + c0 : nullptr, vec);
+                if (in) conv_store16<ACT>(y, pix * csy + c0, v, bias_s + c0, vec);
             }
         }
     } else {
@@ -855,38 +874,44 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
     if (warp < kWorkers / 32) {
         const int nco8 = Co / 8, nci8 = Cn / 8;
         const long long img = (long long)n * H * W;
-        auto copy_x = [&](int k) {   // pixels x0 - 1 .. x0 + P (wrapped)
-            if (k > S + ndy - 2) return;
-            const int yr = ((y0 + dy0 + k) % H + H) % H;
-            const bf16* row = x + (img + (long long)yr * W) * csx + ci0;
-            const uint32_t dst = xb + (uint32_t)(k % kWgX) * Lt.xrow;
+        // the next x and gy rows to copy: number, slot, image row of x
+        int kx = 0, sx = 0, iy = (y0 + dy0 + H) % H, kg = 0, sg = 0;
+        auto copy_x = [&]() {   // pixels x0 - 1 .. x0 + P (wrapped)
+            if (kx > S + ndy - 2) return;
+            const bf16* row = x + (img + (long long)iy * W) * csx + ci0;
+            const uint32_t dst = xb + (uint32_t)sx * Lt.xrow;
             for_groups(tid, P + 2, nci8, [&](int q, int c) {
                 int xx = x0 - 1 + q;
                 xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
                 cp_async16(dst + c * Lt.px + q * 16, row + xx * csx + c * 8, 16u);
             });
-            mbar_arrive_copies(full_x + 8 * (k % kWgX));
+            mbar_arrive_copies(full_x + 8 * sx);
+            ++kx;
+            sx = sx + 1 == kWgX ? 0 : sx + 1;
+            iy = iy + 1 == H ? 0 : iy + 1;
         };
-        auto copy_g = [&](int k) {
-            if (k >= S) return;
-            const bf16* row = gy + (img + (long long)(y0 + k) * W + x0) * csg;
-            const uint32_t dst = gb + (uint32_t)(k % kWgG) * Lt.grow;
+        auto copy_g = [&]() {
+            if (kg >= S) return;
+            const bf16* row = gy + (img + (long long)(y0 + kg) * W + x0) * csg;
+            const uint32_t dst = gb + (uint32_t)sg * Lt.grow;
             for_groups(tid, P, nco8, [&](int q, int c) {
                 cp_async16(dst + c * Lt.pg + q * 16, row + q * csg + c * 8, 16u);
             });
-            mbar_arrive_copies(full_g + 8 * (k % kWgG));
+            mbar_arrive_copies(full_g + 8 * sg);
+            ++kg;
+            sg = sg + 1 == kWgG ? 0 : sg + 1;
         };
-        for (int k = 0; k < ndy; ++k) copy_x(k);
+        for (int k = 0; k < ndy; ++k) copy_x();
         for (int k = 0; k < kWgG; ++k) {
-            copy_g(k);
-            if (ndy + k < kWgX) copy_x(ndy + k);
+            copy_g();
+            if (ndy + k < kWgX) copy_x();
         }
-        for (int k = ndy + kWgG; k < kWgX; ++k) copy_x(k);
+        for (int k = ndy + kWgG; k < kWgX; ++k) copy_x();
         for (int j = 0; j < S && ok; ++j) {   // row j done: its gy slot and its first x slot are free
             ok = mbar_wait_phase(mma_done + 8 * (j % kWgG), j / kWgG, &failed);
             if (ok) {
-                copy_x(j + kWgX);
-                copy_g(j + kWgG);
+                copy_x();   // row j + kWgX
+                copy_g();   // row j + kWgG
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
@@ -896,21 +921,31 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
         const uint32_t idesc = tc_idesc_bf16(wg_m(x_is_a ? Cn : Co), Nc) | (1u << 15) | (1u << 16);
         const uint32_t el = tc_elect();
         int issued = 0;
+        const uint64_t x_hi = tc_smem_desc(0, 128, Lt.px), g_hi = tc_smem_desc(0, 128, Lt.pg);
+        int s0 = 0, s1 = 1, s2 = ndy == 3 ? 2 : 0, ph = 0;   // x slots of rows j, j + 1 and the newest, its phase
+        if (ndy == 3) ok = mbar_wait_phase(full_x, 0, &failed) && mbar_wait_phase(full_x + 8, 0, &failed);
         for (int j = 0; j < S && ok; ++j) {
-            for (int k = j == 0 ? 0 : j + ndy - 1; k <= j + ndy - 1 && ok; ++k)
-                ok = mbar_wait_phase(full_x + 8 * (k % kWgX), k / kWgX, &failed);
+            ok = mbar_wait_phase(full_x + 8 * s2, ph, &failed);
             if (ok) ok = mbar_wait_phase(full_g + 8 * (j % kWgG), j / kWgG, &failed);
             ok = __all_sync(0xffffffffu, ok) != 0;
             if (!ok) break;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t gd = tc_smem_desc(gb + (uint32_t)(j % kWgG) * Lt.grow, 128, Lt.pg);
-            for (int t = 0; t < taps; ++t) {
-                const int d = t / 3, dx = t - 3 * d;
-                const uint64_t xd = tc_smem_desc(xb + (uint32_t)((j + d) % kWgX) * Lt.xrow + (uint32_t)dx * 16, 128, Lt.px);
-                tc_mma_run(el, tmem + (uint32_t)(t * Nc), x_is_a ? xd : gd, x_is_a ? gd : xd, 16, 16, idesc, P / 16,
-                           j > 0);
+            const uint64_t gd = g_hi + (uint64_t)((gb + (uint32_t)(j % kWgG) * Lt.grow) >> 4);
+            for (int d = 0; d < ndy; ++d) {
+                const int sl = ndy == 1 ? s2 : (d == 0 ? s0 : (d == 1 ? s1 : s2));
+                const uint64_t xd0 = x_hi + (uint64_t)((xb + (uint32_t)sl * Lt.xrow) >> 4);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) {
+                    const uint64_t xd = xd0 + (uint64_t)dx;
+                    tc_mma_run(el, tmem + (uint32_t)((3 * d + dx) * Nc), x_is_a ? xd : gd, x_is_a ? gd : xd, 16, 16, idesc,
+                               P / 16, j > 0);
+                }
             }
+            s0 = s1;
+            s1 = s2;
+            s2 = s2 + 1 == kWgX ? 0 : s2 + 1;
+            ph ^= s2 == 0;
             tc_commit(el, mma_done + 8 * (j % kWgG));
             issued = j + 1;
         }

@@ -778,6 +778,79 @@ __device__ __forceinline__ void collide_pair(const NodeState<float>& s, const Pa
     *h_out = fma2(add2(heq, make_float2(-hin.x, -hin.y)), q.inv_tau, hin);
 }
 
+// ---------------------------------------------------------------- FP64 pairs
+// The pair in FP64, split into even and odd parts: with Gamma_I - w = E + O,
+// Gamma_J - w = E - O and the factors of the folded collision (collide_pair)
+// X = Xe +- Xo, Y = Ye +- Yo,
+//   g*_I, g*_J = even +- odd,
+//   even = E (Xe + Ye) + O (Xo + Yo) + w (Ye + 3 P) + filter,
+//   odd  = E (Xo + Yo) + O (Xe + Ye) + w Yo + c.u hoc,
+// 22 operations for g and 7 for h per pair, where two calls of collide_dir take
+// about 70.  FP64 runs at two lanes per clock and SM here, so the FP64 step's
+// time is its operation count (64^2 D2Q9: 433 FP64 instructions per node in the
+// collision before).
+struct PairState64 {
+    double Ze, k1, Fx, Fy, Fz;               // Xe + Ye; rho_dif/2 + 3 mu/2; 3 F / 2
+    double m15, usq15;                       // 3 mu/2, 1.5 u.u
+    double A[2], wm15[2], hoc[2];            // w (Ye + 3 P), w 3 mu/2, w 0.75 rho_dif lap phi
+    double om, tr3;                          // (1 - 1/tau_mix) 4.5, tr(Pi)/3
+    double keep, itphi, itth[2], itphiw[2];  // 1 - 1/tau_phi; phi, theta w and phi w over tau_phi
+};
+
+template <int LAT>
+__device__ __forceinline__ PairState64 pair_state64(const NodeState<double>& s, const PhysT<double>& p) {
+    using L = Lattice<LAT>;
+    PairState64 q;
+    const double hrd = 0.5 * p.rho_dif;
+    q.m15 = 1.5 * s.mu;
+    const double Ye = -q.m15 * s.ug - 1.5 * s.uF;
+    q.Ze = (s.rho - hrd * s.ug) + Ye;
+    q.k1 = hrd + q.m15;
+    q.Fx = 1.5 * s.Fx;
+    q.Fy = 1.5 * s.Fy;
+    q.Fz = 1.5 * s.Fz;
+    q.usq15 = 1.5 * s.usq;
+    q.om = (1.0 - s.omega) * 4.5;
+    q.tr3 = s.tr3;
+    q.keep = 1.0 - p.inv_tau_phi;
+    q.itphi = p.inv_tau_phi * s.phi;
+    const double th = p.inv_tau_phi * s.theta, hl = p.hocorr ? 0.75 * p.rho_dif * s.lap : 0.0, y3P = Ye + 3.0 * s.P;
+    const double wk[2] = {L::w[1], L::w[4]};   // an axis and a diagonal direction
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        q.A[k] = wk[k] * y3P;
+        q.wm15[k] = wk[k] * q.m15;
+        q.hoc[k] = wk[k] * hl;
+        q.itth[k] = wk[k] * th;
+        q.itphiw[k] = wk[k] * q.itphi;
+    }
+    return q;
+}
+
+template <int LAT, int I>
+__device__ __forceinline__ void collide_pair64(const NodeState<double>& s, const PairState64& q, double hI, double hJ,
+                                               double* h_I, double* h_J, double* g_I, double* g_J) {
+    using L = Lattice<LAT>;
+    constexpr int CX = L::cx[I], CY = L::cy[I], CZ = L::cz[I];
+    constexpr int WK = CX * CX + CY * CY + CZ * CZ == 1 ? 0 : 1;
+    constexpr double w = L::w[I];
+    const double cu = cdot3<CX, CY, CZ>(s.ux, s.uy, s.uz);
+    const double cg = cdot3<CX, CY, CZ>(s.gx, s.gy, s.gz);
+    const double cF = cdot3<CX, CY, CZ>(q.Fx, q.Fy, q.Fz);
+    const double cn = cdot3<CX, CY, CZ>(s.nx, s.ny, s.nz);
+    const double E = w * (4.5 * cu * cu - q.usq15), O = (3.0 * w) * cu;
+    const double Zo = q.k1 * cg + cF;
+    const double ccPi = cdot3<CX * CX, CY * CY, CZ * CZ>(s.pxx, s.pyy, s.pzz) +
+                        2.0 * cdot3<CX * CY, CX * CZ, CY * CZ>(s.pxy, s.pxz, s.pyz);
+    const double even = E * q.Ze + (O * Zo + ((ccPi - q.tr3) * (w * q.om) + q.A[WK]));
+    const double odd = E * Zo + (O * q.Ze + (q.wm15[WK] * cg + (w * cF + q.hoc[WK] * cu)));
+    *g_I = even + odd;
+    *g_J = even - odd;
+    const double he = q.itphi * E + q.itphiw[WK], ho = q.itphi * O + q.itth[WK] * cn;
+    *h_I = q.keep * hI + (he + ho);
+    *h_J = q.keep * hJ + (he - ho);
+}
+
 // ---------------------------------------------------------------- fused step
 // One CTA owns a TX x TY column of nodes in the x-y plane and marches along
 // z over a chunk of LZ planes.  Per plane it
@@ -937,20 +1010,26 @@ __device__ __forceinline__ void collide_node(const DirPtrs<typename Storage<ST>:
         });
         hsum = hsum2.x + hsum2.y;
     } else {
+        const PairState64 q = pair_state64<LAT>(s, p);
         Unroll<1, Q>::run([&](auto ic) {
             constexpr int i = decltype(ic)::value;
-            constexpr double W = L::w[i];
-            R hs, gs;
-            collide_dir<LAT, i, R>(s, p, hv(i), &hs, &gs);
-            hsum += hs;
-            write_dir<LAT, i, WALLS>(D.hout, G, own, nw, St::store(hs, (R)W * p.h_shift, (R)1));
-            write_dir<LAT, i, WALLS>(D.gout, G, own, nw, St::store(gs, (R)W * p.g_shift, p.g_scale));
-            if constexpr (WALLS) {
-                if (p.moving) {
-                    moving_wall_write<LAT, i>(D.hout, G, x, y, z, hs, s.phi, p,
-                                              [&](R v) { return St::store(v, (R)W * p.h_shift, (R)1); });
-                    moving_wall_write<LAT, i>(D.gout, G, x, y, z, gs, s.rho, p,
-                                              [&](R v) { return St::store(v, (R)W * p.g_shift, p.g_scale); });
+            constexpr int o = L::op[i];
+            if constexpr (i < o) {
+                R hi, ho, gi, go;
+                collide_pair64<LAT, i>(s, q, hv(i), hv(o), &hi, &ho, &gi, &go);
+                hsum += hi + ho;
+                write_dir<LAT, i, WALLS>(D.hout, G, own, nw, hi);
+                write_dir<LAT, o, WALLS>(D.hout, G, own, nw, ho);
+                write_dir<LAT, i, WALLS>(D.gout, G, own, nw, gi);
+                write_dir<LAT, o, WALLS>(D.gout, G, own, nw, go);
+                if constexpr (WALLS) {
+                    if (p.moving) {
+                        auto same = [](R v) { return v; };
+                        moving_wall_write<LAT, i>(D.hout, G, x, y, z, hi, s.phi, p, same);
+                        moving_wall_write<LAT, o>(D.hout, G, x, y, z, ho, s.phi, p, same);
+                        moving_wall_write<LAT, i>(D.gout, G, x, y, z, gi, s.rho, p, same);
+                        moving_wall_write<LAT, o>(D.gout, G, x, y, z, go, s.rho, p, same);
+                    }
                 }
             }
         });

@@ -57,6 +57,15 @@ using BoxA = Box<16, 4, 4, 2>;
 using BoxB = Box<8, 4, 4, 4>;
 constexpr int kBoxAHalves = 1;    // box A from this many half boxes per SM on
 constexpr int kBoxRounds = 1;     // boxes of one CTA per step at most
+#elif LBM_ST == 0
+// FP64 (D2Q9) is bound by the FP64 pipe, whose 65 clk per warp instruction do
+// not shrink with fewer active lanes: boxes of one warp spread evenly over the
+// SMs, a larger box only where those no longer fit the chip.  us per step,
+// 8x4 / 32x4: 64^2 14.0 / 14.8, 128^2 16.0 / 14.9, 256^2 50.5 / 52.9
+using BoxA = Box<32, 1, 4, 4>;
+using BoxB = Box<8, 1, 4, 16>;
+constexpr int kBoxAHalves = 1 << 20;
+constexpr int kBoxRounds = 1;
 #else
 using BoxA = Box<32, 1, 8, 4>;
 using BoxB = Box<32, 1, 4, 4>;
@@ -124,13 +133,17 @@ cudaError_t box_plan(const Geom& G, BoxPlan* plan) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     BoxPlan q = BoxA::cut(G, 0);
-    if (2LL * q.boxes < (long long)kBoxAHalves * sms) q = BoxB::cut(G, 1);
-    if (q.boxes < 1) return cudaSuccess;   // more boxes than fit an int
-    e = q.variant == 0 ? box_slots<LBM_LAT, LBM_ST, BoxA>(G, &slots) : box_slots<LBM_LAT, LBM_ST, BoxB>(G, &slots);
-    if (e != cudaSuccess) return e;
-    if (q.boxes > (long long)slots * kBoxRounds) return cudaSuccess;
-    q.ctas = q.boxes < slots ? q.boxes : slots;
-    *plan = q;
+    const bool a_first = 2LL * q.boxes >= (long long)kBoxAHalves * sms;
+    for (int t = a_first ? 1 : 0; t < 2; ++t) {   // the larger box where the smaller ones are too many
+        q = a_first || t == 1 ? BoxA::cut(G, 0) : BoxB::cut(G, 1);
+        if (q.boxes < 1) continue;                // more boxes than fit an int
+        e = q.variant == 0 ? box_slots<LBM_LAT, LBM_ST, BoxA>(G, &slots) : box_slots<LBM_LAT, LBM_ST, BoxB>(G, &slots);
+        if (e != cudaSuccess) return e;
+        if (q.boxes > (long long)slots * kBoxRounds) continue;
+        q.ctas = q.boxes < slots ? q.boxes : slots;
+        *plan = q;
+        return cudaSuccess;
+    }
     return cudaSuccess;
 }
 

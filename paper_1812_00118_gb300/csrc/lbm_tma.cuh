@@ -307,13 +307,17 @@ step_tma_kernel(const __grid_constant__ TmaMaps maps, const DirPtrs<typename Sto
                 if constexpr (WALLS) nw = node_writes(G, x, y, z);
                 const int own = (z + G.GZ) * G.PXY + rb;
                 R hsum = 0;
-                Unroll<1, Q>::run([&](auto ic) {
+                // the thread's pulled h of direction i
+                auto h_of = [&](auto ic) {
                     constexpr int i = decltype(ic)::value;
                     constexpr int off = C::HL::dir_offset(i) / C::ES + A - L::cx[i];
                     constexpr double W = L::w[i];
-                    const R hv = St::load(hs_[off + (ty + HY) * C::BX + tx], (R)W * p.h_shift, (R)1);
-                    R hs, gs;
-                    collide_dir<LAT, i, R>(s, p, hv, &hs, &gs);
+                    return St::load(hs_[off + (ty + HY) * C::BX + tx], (R)W * p.h_shift, (R)1);
+                };
+                // own cell, bounce-back cell and moving wall of direction i
+                auto write = [&](auto ic, R hs, R gs) {
+                    constexpr int i = decltype(ic)::value;
+                    constexpr double W = L::w[i];
                     hsum += hs;
                     write_dir<LAT, i, WALLS>(D.hout, G, own, nw, St::store(hs, (R)W * p.h_shift, (R)1));
                     write_dir<LAT, i, WALLS>(D.gout, G, own, nw, St::store(gs, (R)W * p.g_shift, p.g_scale));
@@ -325,7 +329,27 @@ step_tma_kernel(const __grid_constant__ TmaMaps maps, const DirPtrs<typename Sto
                                                       [&](R v) { return St::store(v, (R)W * p.g_shift, p.g_scale); });
                         }
                     }
-                });
+                };
+                if constexpr (std::is_same<R, double>::value) {
+                    const PairState64 q = pair_state64<LAT>(s, p);
+                    Unroll<1, Q>::run([&](auto ic) {
+                        constexpr int i = decltype(ic)::value;
+                        constexpr int o = L::op[i];
+                        if constexpr (i < o) {
+                            std::integral_constant<int, o> oc;
+                            R hi, ho, gi, go;
+                            collide_pair64<LAT, i>(s, q, h_of(ic), h_of(oc), &hi, &ho, &gi, &go);
+                            write(ic, hi, gi);
+                            write(oc, ho, go);
+                        }
+                    });
+                } else {
+                    Unroll<1, Q>::run([&](auto ic) {
+                        R hs, gs;
+                        collide_dir<LAT, decltype(ic)::value, R>(s, p, h_of(ic), &hs, &gs);
+                        write(ic, hs, gs);
+                    });
+                }
                 {
                     constexpr double W0 = L::w[0];
                     R hs, gs;

@@ -64,12 +64,12 @@ long long lbm_sg_wgrad_scratch_floats(int N, int H, int W, int Ci, int Co);
 
 /* gw (float [Co][9][Ci]) = gradient of sum_p <gy[p], y[p]> with respect to w
  * for y = lbm_sg_conv3x3(x, w): gw[co, tap, ci] = sum_p gy[p, co] x[p + d(tap), ci].
- * x, gy bf16.  When W is a multiple of 16, Co is at most 128, Ci is at
+ * x, gy bf16.  When W is a multiple of 32, Co is at most 128, Ci is at
  * most 128 or a multiple of 128, the channel strides are multiples of 8 and
  * x, gy and scratch start on 16-byte boundaries, the sums are GEMMs over
- * pixels on the tcgen05 tensor cores (each CTA marches a segment of up to 128
- * pixels down a chunk of rows for a block of at most 128 input channels,
- * all nine taps or the three of one tap row accumulated in tensor memory);
+ * pixels on the tcgen05 tensor cores (each CTA marches a 64- or 32-pixel row
+ * segment down a chunk of rows for one tap row and a block of at most 128
+ * input channels, its three taps accumulated in tensor memory);
  * otherwise warp-level mma.sync over
  * chunks of 1024 pixels.  Deterministic either way: per-CTA (or per-chunk) partials
  * summed in a fixed order.  A bounded wait that gives up is reported by
@@ -110,29 +110,29 @@ int lbm_sg_upsample(const void* x, int csx, void* y, int csy, int N, int H, int 
 int lbm_sg_upsample_bwd(const float* g, int csg, float* gx, int csx, int N, int H, int W, int C, int f,
                         void* stream);
 
-#define LBM_SG_GRAD_BLOCKS 512
+#define LBM_SG_LOSS_BLOCKS 512
 
 /* Gradient through a layer's ReLU and its bias gradient in one pass: ga (bf16,
  * stride C) = v rounded, v = gradient where act (bf16, stride csa, the layer's
  * output after the ReLU) is positive, else 0; gb[c] = sum of the FP32 v over
- * the pixels (fixed order).  The gradient of the H x W layer's output is g
+ * the pixels, the sum lbm_sg_bias_grad forms.  The gradient of the H x W layer's output is g
  * (float, stride csg; up = 1), the sums of g over 2 x 2 blocks of a 2H x 2W
  * image (up = 2: the layer's output was upsampled), or g + gp / 4 spread over
  * 2 x 2 blocks (gp not NULL, float, H/2 x W/2, stride csp, up = 1: it was
  * pooled as well).  C and the strides are multiples of 4, C at most 1024; g, gp
  * and scratch start on 16-byte boundaries, act and ga on 8-byte ones, else
- * LBM_EINVAL.  scratch: LBM_SG_GRAD_BLOCKS * C floats are always enough. */
+ * LBM_EINVAL.  scratch: 64 C floats are always enough. */
 int lbm_sg_relu_grad(const float* g, int csg, int up, const float* gp, int csp, const void* act, int csa, void* ga,
                      float* gb, float* scratch, long long scratch_floats, int N, int H, int W, int C, void* stream);
 
 /* lbm_sg_mse for the four-channel output layer, with what its backward pass
- * reads: *loss as there; g16 (bf16, 16 channels, the last 12 zero) = the
- * gradient rounded; gb (16 floats, the last 12 zero) = its sums over the pixels
- * from the FP32 values.  x and target have 4 channels, delta 16; x, delta,
- * target, g16 and scratch start on 16-byte boundaries.  scratch: 3 *
- * LBM_SG_GRAD_BLOCKS doubles. */
-int lbm_sg_mse_grad(const float* x, const float* delta, const float* target, void* g16, float* gb, double* scratch,
-                    double* loss, long long npix, void* stream);
+ * reads: *loss as there; g4 (float, 4 channels) = the gradient, g16 (bf16, 16
+ * channels, the last 12 zero) = the gradient rounded; gb (16 floats, the last 12
+ * zero) = its sums over the pixels (lbm_sg_bias_grad).  x and target have 4
+ * channels, delta 16; x, delta, target, g16, g4 and scratch start on 16-byte
+ * boundaries.  scratch: 2 * LBM_SG_LOSS_BLOCKS doubles. */
+int lbm_sg_mse_grad(const float* x, const float* delta, const float* target, void* g16, float* g4, float* gb,
+                    double* scratch, double* loss, long long npix, void* stream);
 
 /* Mean squared error of out = x + delta against target over the first C
  * channels: *loss (device double) = mean (out - target)^2 (FP64 sums), and

@@ -12,7 +12,7 @@
 // The forward (and input-gradient) convolution runs on the tcgen05 tensor
 // cores with the accumulator in tensor memory (conv_row_kernel for images
 // whose width is a multiple of 128, conv_tc_kernel otherwise); so does the
-// weight gradient, a GEMM over pixels, for widths that are multiples of 16
+// weight gradient, a GEMM over pixels, for widths that are multiples of 32
 // (conv_wgrad_row_kernel), with the warp-level mma.sync m16n8k16 BF16 kernel
 // (fragments gathered straight from the channels-last tensors) for the
 // rest.  All are implicit GEMMs without an im2col buffer.
@@ -433,7 +433,7 @@ __device__ int g_sg_err;   // a bounded wait of a surrogate kernel gave up
 // tensor-memory accumulators while the other is summed; a warp of its own
 // issues the MMAs.  (On 128 threads that wrote out row j - 1 and copied row
 // j + 1 before issuing row j the 64 -> 32 layer at 8 x 256^2 took 126 us; this
-// takes XX.)  Every wait is bounded, as in the tap kernel.
+// takes 42.)  Every wait is bounded, as in the tap kernel.
 constexpr int kRowM = 128;          // pixels of a row segment (MMA M)
 constexpr int kRowHalo = kRowM + 2;
 constexpr int kRowSlots = 6;        // ring rows at most (at least 4)
@@ -601,8 +601,10 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
 // that fall on the halo columns are computed and dropped.  A CTA copies the
 // 128 + 2 (W + 3) cells its tile reads once, all channels of them (the tap
 // kernel copies 9 x 128 pixels, a stage of 64 channels at a time), and the
-// weights tap by tap through a ring of `stages` buffers.  Taps and channels in
-// the tap kernel's order.
+// weights tap by tap through a ring of `stages` buffers.  Where the tiles leave
+// SMs idle (one 256^2 image has 9 at the coarsest level) the output channels are
+// split over blockIdx.y, Co of them each.  Taps and channels in the tap kernel's
+// order.
 constexpr int kFlatStages = 9;
 
 __host__ __device__ inline int flat_cells(int W) { return 128 + 2 * (W + 3); }
@@ -621,13 +623,16 @@ inline int flat_stages(int W, int Ci, int Co) {
 template <bool ACT>
 __global__ void __launch_bounds__(kRoleThreads, 1)
 conv_flat_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, const float* __restrict__ bias,
-                 void* __restrict__ y, int csy, int H, int W, int Ci, int Co, int tiles, int stages, int* err) {
+                 void* y, int csy, int H, int W, int Ci, int Co, int tiles, int stages, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[2 * kFlatStages];   // full[stage], done[stage]
     __shared__ __align__(16) float bias_s[128];
     __shared__ uint32_t tmem_slot;
     __shared__ int failed;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
+    w += (long long)blockIdx.y * Co * 9 * Ci;
+    if (bias) bias += blockIdx.y * Co;
+    y = ACT ? (void*)((bf16*)y + blockIdx.y * Co) : (void*)((float*)y + blockIdx.y * Co);
     const int n = blockIdx.x / tiles, f0 = (blockIdx.x - n * tiles) * 128;
     const int Wp = W + 2, nch = Ci / 8, cells = flat_cells(W);
     const uint32_t xs = smem_u32(smem), plane = flat_plane(W);
@@ -764,7 +769,7 @@ __global__ void conv_wgrad_kernel(const bf16* __restrict__ x, int csx, const bf1
 
 // ---------------------------------------------------------------- tcgen05 weight gradient, row march
 // gw[co, tap, ci] = sum_p gy[p, co] x[p + d(tap), ci] as GEMMs over pixels
-// on the tensor cores, for images whose width is a multiple of 16: per tap
+// on the tensor cores, for images whose width is a multiple of 32: per tap
 // D_tap (M x N) += A (M x pixels) B (N x pixels)^T, M the channels of the side
 // with more of them, N those of the other, K running over pixels.
 //
@@ -772,30 +777,34 @@ __global__ void conv_wgrad_kernel(const bf16* __restrict__ x, int csx, const bf1
 // planes of 8 channels, 16 bytes per pixel, which is the tensor core's
 // no-swizzle MN-major layout (core matrices of 8 pixels x 8 channels, plane
 // pitch between channel groups, 128 bytes between groups of 8 pixels).  A tap
-// is then the x row of its dy started (1 + dx) pixels in: no transposition,
-// and one copy of a row serves three dy and three dx.  (Transposing both
-// operands through registers into K-major buffers, for one dy per CTA, took
-// 290 us for the 64 -> 32 layer at 8 x 256^2; this takes 48.)  Plane
-// pitches are odd multiples of 16 bytes, so the 8 groups of a pixel, copied by
-// neighbouring threads, fall into different banks.
+// is then the x row of its dy started (1 + dx) pixels in: no transposition
+// (transposing both operands through registers into K-major buffers took
+// 290 us for the 64 -> 32 layer at 8 x 256^2; this takes 100).  Plane pitches are
+// odd multiples of 16 bytes, so the 8 groups of a pixel, copied by neighbouring
+// threads, fall into different banks.
 //
-// A CTA marches a segment of P pixels down a chunk of rows, x rows in a ring
-// of six and gy rows in a ring of four, copies two rows ahead of the MMAs, MMAs
-// of a row issued while those of the one before still run.  The taps (all
-// nine where their columns fit tensor memory, else the three of one dy)
-// accumulate over the whole march and are written out once, as the CTA's
-// partial; partials are summed in a fixed order (deterministic).  M is 64 up
-// to 64 channels, else 128 (24 against 40 clk per MMA at N = 32): the rows past a
-// side's channels read whatever lies behind its planes and are not written out.
+// A CTA takes a segment of P = 64 (or 32) pixels, one tap row dy, a block of at
+// most 128 input channels and a chunk of rows.  It marches groups of rows (256
+// pixels' worth) through two or three buffers: the waits and the proxy fence of
+// the issuing warp are paid once per group.  The three taps accumulate in tensor
+// memory over the whole chunk, rows and pixels in order, and are written out
+// once, as the CTA's partial; partials are summed in order (deterministic).
+// Chunks are cut by wgrad_row_plan: another cut would change the last bits of
+// the gradient, and with them, through Adam's normalised step and the bf16
+// rounding of the weights, a training run's course.  M is 64 up to 64 channels,
+// else 128 (24 against 40 clk per MMA at N = 32): the rows past a side's
+// channels read whatever lies behind its planes and are not written out.
 constexpr int kWgCn = 128;            // input channels of one CTA at most
-constexpr int kWgX = 6, kWgG = 4;     // rows in the rings
+constexpr int kWgPixels = 256;        // pixels of a group of rows
+constexpr int kWgBuf = 3;             // buffers at most
 constexpr size_t kWgSmemMax = 220 * 1024;   // below the 227 KB per CTA less the kernel's static shared memory
 
 __host__ __device__ inline int wg_m(int channels) { return channels <= 64 ? 64 : 128; }
 struct WgLayout {
     uint32_t px, pg;        // plane pitches of x and gy
     uint32_t xrow, grow;    // bytes of one row
-    uint32_t total;
+    uint32_t rows;          // rows of a group
+    uint32_t tail;          // the planes of all M rows an operand reads from the last row
 };
 // P pixels of a segment, Cn input channels and Co output channels of a CTA
 __host__ __device__ inline WgLayout wg_layout(int P, int Cn, int Co) {
@@ -804,51 +813,54 @@ __host__ __device__ inline WgLayout wg_layout(int P, int Cn, int Co) {
     L.pg = (uint32_t)(P | 1) * 16;
     L.xrow = (uint32_t)(Cn / 8) * L.px;
     L.grow = (uint32_t)(Co / 8) * L.pg;
-    // the planes of all M rows an operand reads from the last row of its ring
-    const uint32_t tail = Cn >= Co ? (uint32_t)(wg_m(Cn) - Cn) / 8 * L.px : (uint32_t)(wg_m(Co) - Co) / 8 * L.pg;
-    L.total = kWgX * L.xrow + kWgG * L.grow + tail;
+    L.rows = kWgPixels / P;
+    while (L.rows > 1 && 2 * L.rows * (L.xrow + L.grow) > kWgSmemMax - 24 * 1024) L.rows /= 2;
+    L.tail = Cn >= Co ? (uint32_t)(wg_m(Cn) - Cn) / 8 * L.px : (uint32_t)(wg_m(Co) - Co) / 8 * L.pg;
     return L;
 }
+__host__ __device__ inline size_t wg_bytes(const WgLayout& L, int bufs) {
+    return (size_t)bufs * L.rows * (L.xrow + L.grow) + L.tail;
+}
 __host__ __device__ inline int wg_n(int Cn, int Co) { return Cn >= Co ? Co : Cn; }   // columns of a tap
-__host__ __device__ inline int wg_taps(int Cn, int Co) { return 9 * wg_n(Cn, Co) <= 512 ? 9 : 3; }
-__host__ __device__ inline uint32_t wg_tmem_cols(int Cn, int Co) {
-    const int need = wg_taps(Cn, Co) * wg_n(Cn, Co);
-    return need <= 32 ? 32u : (need <= 64 ? 64u : (need <= 128 ? 128u : (need <= 256 ? 256u : 512u)));
+__host__ __device__ inline uint32_t wg_tmem_cols(int n) {   // three taps of n columns
+    const int need = 3 * n;
+    return need <= 64 ? 64u : (need <= 128 ? 128u : (need <= 256 ? 256u : 512u));
 }
 
 __global__ void __launch_bounds__(kRoleThreads, 1)
 conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ gy, int csg,
                       float* __restrict__ partial, int N, int H, int W, int Ci, int Co, int P, int Cn,
-                      int rows_per_cta, int* err) {
+                      int rows_per_cta, int bufs, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t bars[kWgX + 2 * kWgG];   // x rows, gy rows landed; MMAs of a gy row done
+    __shared__ __align__(8) uint64_t bars[2 * kWgBuf];   // full[buffer], done[buffer]
     __shared__ uint32_t tmem_slot;
     __shared__ int failed;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const int segs = W / P;
     const int nsplit = Ci / Cn;
-    const int taps = wg_taps(Cn, Co);
     const int chunks = (H + rows_per_cta - 1) / rows_per_cta;
     int b = blockIdx.x;
-    const int dy0 = taps == 9 ? -1 : b % 3 - 1, ndy = taps / 3;   // the CTA's tap rows
-    if (taps != 9) b /= 3;
+    const int dy = b % 3 - 1;
+    b /= 3;
     const int ci0 = (b % nsplit) * Cn;
     b /= nsplit;
     const int chunk = b % chunks;
     b /= chunks;
     const int seg = b % segs, n = b / segs;
     const int y0 = chunk * rows_per_cta;
-    const int y1 = y0 + rows_per_cta < H ? y0 + rows_per_cta : H;
+    const int S = (y0 + rows_per_cta < H ? y0 + rows_per_cta : H) - y0;   // rows of the march
     const int x0 = seg * P;
     const long long pchunk = ((long long)n * segs + seg) * chunks + chunk;
     const WgLayout Lt = wg_layout(P, Cn, Co);
+    const int RG = (int)Lt.rows, groups = (S + RG - 1) / RG;
     const bool x_is_a = Cn >= Co;
-    // the ring of the M side lies last, its tail behind it
+    // the buffers of the M side lie last, its tail behind them
     const uint32_t sb = smem_u32(smem);
-    const uint32_t xb = x_is_a ? sb + kWgG * Lt.grow : sb, gb = x_is_a ? sb : sb + kWgX * Lt.xrow;
-    const uint32_t full_x = smem_u32(&bars[0]), full_g = full_x + 8 * kWgX, mma_done = full_g + 8 * kWgG;
+    const uint32_t xb = x_is_a ? sb + (uint32_t)(bufs * RG) * Lt.grow : sb;
+    const uint32_t gb = x_is_a ? sb : sb + (uint32_t)(bufs * RG) * Lt.xrow;
+    const uint32_t full = smem_u32(&bars[0]), mma_done = full + 8 * kWgBuf;
     const int Nc = wg_n(Cn, Co);
-    const uint32_t ncols = wg_tmem_cols(Cn, Co);
+    const uint32_t ncols = wg_tmem_cols(Nc);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                      "r"(ncols)
@@ -856,10 +868,10 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int k = 0; k < kWgX + kWgG; ++k) mbar_init(full_x + 8 * k, kWorkers);
-        // one per gy slot: a slot's next MMAs wait for the workers that refill it,
-        // so no barrier can run a phase ahead of them
-        for (int k = 0; k < kWgG; ++k) mbar_init(mma_done + 8 * k, 1);
+        for (int k = 0; k < bufs; ++k) {
+            mbar_init(full + 8 * k, kWorkers);
+            mbar_init(mma_done + 8 * k, 1);
+        }
         failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -867,52 +879,32 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
-    const int S = y1 - y0;
-    // row j of the march (gy row y0 + j, slot j % kWgG) reads x rows j .. j +
-    // ndy - 1 (x row k: image row y0 + dy0 + k, wrapped, slot k % kWgX)
     bool ok = true;
     if (warp < kWorkers / 32) {
         const int nco8 = Co / 8, nci8 = Cn / 8;
         const long long img = (long long)n * H * W;
-        // the next x and gy rows to copy: number, slot, image row of x
-        int kx = 0, sx = 0, iy = (y0 + dy0 + H) % H, kg = 0, sg = 0;
-        auto copy_x = [&]() {   // pixels x0 - 1 .. x0 + P (wrapped)
-            if (kx > S + ndy - 2) return;
-            const bf16* row = x + (img + (long long)iy * W) * csx + ci0;
-            const uint32_t dst = xb + (uint32_t)sx * Lt.xrow;
-            for_groups(tid, P + 2, nci8, [&](int q, int c) {
-                int xx = x0 - 1 + q;
-                xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
-                cp_async16(dst + c * Lt.px + q * 16, row + xx * csx + c * 8, 16u);
-            });
-            mbar_arrive_copies(full_x + 8 * sx);
-            ++kx;
-            sx = sx + 1 == kWgX ? 0 : sx + 1;
-            iy = iy + 1 == H ? 0 : iy + 1;
-        };
-        auto copy_g = [&]() {
-            if (kg >= S) return;
-            const bf16* row = gy + (img + (long long)(y0 + kg) * W + x0) * csg;
-            const uint32_t dst = gb + (uint32_t)sg * Lt.grow;
-            for_groups(tid, P, nco8, [&](int q, int c) {
-                cp_async16(dst + c * Lt.pg + q * 16, row + q * csg + c * 8, 16u);
-            });
-            mbar_arrive_copies(full_g + 8 * sg);
-            ++kg;
-            sg = sg + 1 == kWgG ? 0 : sg + 1;
-        };
-        for (int k = 0; k < ndy; ++k) copy_x();
-        for (int k = 0; k < kWgG; ++k) {
-            copy_g();
-            if (ndy + k < kWgX) copy_x();
-        }
-        for (int k = ndy + kWgG; k < kWgX; ++k) copy_x();
-        for (int j = 0; j < S && ok; ++j) {   // row j done: its gy slot and its first x slot are free
-            ok = mbar_wait_phase(mma_done + 8 * (j % kWgG), j / kWgG, &failed);
-            if (ok) {
-                copy_x();   // row j + kWgX
-                copy_g();   // row j + kWgG
+        int buf = 0, ph = 0, yx = (y0 + dy + H) % H;   // buffer, its use, image row of x
+        for (int g = 0; g < groups && ok; ++g) {
+            if (g >= bufs) ok = mbar_wait_phase(mma_done + 8 * buf, ph - 1, &failed);
+            if (!ok) break;
+            const int r0 = g * RG, r1 = r0 + RG < S ? r0 + RG : S;
+            for (int q = r0; q < r1; ++q) {
+                const bf16* xrow = x + (img + (long long)yx * W) * csx + ci0;
+                const uint32_t xd = xb + (uint32_t)(buf * RG + q - r0) * Lt.xrow;
+                for_groups(tid, P + 2, nci8, [&](int p, int c) {   // pixels x0 - 1 .. x0 + P (wrapped)
+                    int xx = x0 - 1 + p;
+                    xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
+                    cp_async16(xd + c * Lt.px + p * 16, xrow + xx * csx + c * 8, 16u);
+                });
+                const bf16* grow = gy + (img + (long long)(y0 + q) * W + x0) * csg;
+                const uint32_t gd = gb + (uint32_t)(buf * RG + q - r0) * Lt.grow;
+                for_groups(tid, P, nco8, [&](int p, int c) {
+                    cp_async16(gd + c * Lt.pg + p * 16, grow + p * csg + c * 8, 16u);
+                });
+                yx = yx + 1 == H ? 0 : yx + 1;
             }
+            mbar_arrive_copies(full + 8 * buf);
+            if (++buf == bufs) { buf = 0; ++ph; }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         ok = __all_sync(0xffffffffu, ok) != 0;
@@ -920,49 +912,49 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
         // both operands MN-major (bits 15 and 16)
         const uint32_t idesc = tc_idesc_bf16(wg_m(x_is_a ? Cn : Co), Nc) | (1u << 15) | (1u << 16);
         const uint32_t el = tc_elect();
-        int issued = 0;
         const uint64_t x_hi = tc_smem_desc(0, 128, Lt.px), g_hi = tc_smem_desc(0, 128, Lt.pg);
-        int s0 = 0, s1 = 1, s2 = ndy == 3 ? 2 : 0, ph = 0;   // x slots of rows j, j + 1 and the newest, its phase
-        if (ndy == 3) ok = mbar_wait_phase(full_x, 0, &failed) && mbar_wait_phase(full_x + 8, 0, &failed);
-        for (int j = 0; j < S && ok; ++j) {
-            ok = mbar_wait_phase(full_x + 8 * s2, ph, &failed);
-            if (ok) ok = mbar_wait_phase(full_g + 8 * (j % kWgG), j / kWgG, &failed);
+        int buf = 0, ph = 0, last = 0, last_ph = 0;
+        bool any = false;
+        for (int g = 0; g < groups; ++g) {
+            ok = mbar_wait_phase(full + 8 * buf, ph, &failed);
             ok = __all_sync(0xffffffffu, ok) != 0;
             if (!ok) break;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t gd = g_hi + (uint64_t)((gb + (uint32_t)(j % kWgG) * Lt.grow) >> 4);
-            for (int d = 0; d < ndy; ++d) {
-                const int sl = ndy == 1 ? s2 : (d == 0 ? s0 : (d == 1 ? s1 : s2));
-                const uint64_t xd0 = x_hi + (uint64_t)((xb + (uint32_t)sl * Lt.xrow) >> 4);
+            const int rows = S - g * RG < RG ? S - g * RG : RG;
+            for (int q = 0; q < rows; ++q) {
+                const uint64_t gd = g_hi + (uint64_t)((gb + (uint32_t)(buf * RG + q) * Lt.grow) >> 4);
+                const uint64_t xd0 = x_hi + (uint64_t)((xb + (uint32_t)(buf * RG + q) * Lt.xrow) >> 4);
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx) {
                     const uint64_t xd = xd0 + (uint64_t)dx;
-                    tc_mma_run(el, tmem + (uint32_t)((3 * d + dx) * Nc), x_is_a ? xd : gd, x_is_a ? gd : xd, 16, 16, idesc,
-                               P / 16, j > 0);
+                    tc_mma_run(el, tmem + (uint32_t)(dx * Nc), x_is_a ? xd : gd, x_is_a ? gd : xd, 16, 16, idesc, P / 16,
+                               g + q > 0);
                 }
             }
-            s0 = s1;
-            s1 = s2;
-            s2 = s2 + 1 == kWgX ? 0 : s2 + 1;
-            ph ^= s2 == 0;
-            tc_commit(el, mma_done + 8 * (j % kWgG));
-            issued = j + 1;
+            tc_commit(el, mma_done + 8 * buf);
+            any = true;
+            last = buf;
+            last_ph = ph;
+            if (++buf == bufs) { buf = 0; ++ph; }
         }
-        // the MMAs still running (on the failure path) end before the tensor
-        // memory is freed
-        if (issued > 0) mbar_wait_bounded(mma_done + 8 * ((issued - 1) % kWgG), (uint32_t)((issued - 1) / kWgG) & 1u, kTcPolls);
+        // the MMAs still running end before the accumulators are read or (on the
+        // failure path) the tensor memory is freed
+        if (any) ok = mbar_wait_bounded(mma_done + 8 * last, (uint32_t)last_ph & 1u, kTcPolls) && ok;
+        if (!ok) failed = 1;
     }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (ok && warp < 4) {
+    if (!failed && warp < 4) {
         // channel of the M side: row m of an M = 128 accumulator is lane m, of an
         // M = 64 one lane 32 (m / 16) + m % 16
         const bool half = wg_m(x_is_a ? Cn : Co) == 64;
         const int m = half ? (lane < 16 ? 16 * warp + lane : 128) : 32 * warp + lane;
         const int K9 = 9 * Ci;
         float* out = partial + pchunk * Co * (long long)K9;
-        for (int t = 0; t < taps; ++t) {
-            const int tap = (dy0 + 1) * 3 + t;
+        for (int t = 0; t < 3; ++t) {
+            const int tap = (dy + 1) * 3 + t;
             for (int c0 = 0; c0 < Nc; c0 += 16) {
                 float v[16];
                 tc_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(t * Nc + c0), v);
@@ -987,25 +979,25 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
     if (tid == 0 && failed) atomicExch(err, 1);
 }
 
-// gw[k] = sum over chunks of partial[chunk, k] in a fixed order: 32 values per
-// block, each by eight threads that take every eighth chunk (one thread per
-// value left 18 blocks for the 16 -> 32 layer's 4608 values of 304 chunks: 27 us).
-__global__ void __launch_bounds__(256)
+// gw[k] = sum over chunks of partial[chunk, k], in chunk order; blocks of one
+// warp and 16 loads in flight (256 threads that waited for each: 18 blocks and
+// 10 us for the 4608 values of the 16 -> 32 layer)
+__global__ void __launch_bounds__(32)
 sum_chunks_kernel(const float* __restrict__ partial, long long nchunks, long long K, float* __restrict__ gw) {
-    __shared__ float sh[8][32];
-    const int i = threadIdx.x & 31, part = threadIdx.x >> 5;
-    const long long k = (long long)blockIdx.x * 32 + i;
+    const long long k = (long long)blockIdx.x * 32 + threadIdx.x;
+    if (k >= K) return;
+    const float* p = partial + k;
     float s = 0.0f;
-    if (k < K) {
-#pragma unroll 8
-        for (long long c = part; c < nchunks; c += 8) s += partial[c * K + k];
+    long long c = 0;
+    for (; c + 16 <= nchunks; c += 16) {
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = p[(c + i) * K];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) s += v[i];
     }
-    sh[part][i] = s;
-    __syncthreads();
-    if (part == 0 && k < K) {
-        for (int q = 1; q < 8; ++q) s += sh[q][i];
-        gw[k] = s;
-    }
+    for (; c < nchunks; ++c) s += p[c * K];
+    gw[k] = s;
 }
 
 // wt[ci, 8 - tap, co] = w[co, tap, ci]: the weights of the input-gradient convolution
@@ -1190,35 +1182,21 @@ __global__ void upsample_bwd_kernel(const float* __restrict__ g, int csg, float*
     gx[q * csx + c] = s;
 }
 
-// per-block partial sums of the columns of g (rows = pixels), fixed order:
-// neighbouring threads take neighbouring channels of a pixel, so a block reads
-// whole rows (one channel per block read 4 of every 4 C bytes: 63 us for
-// 8 x 256^2 x 32).  blockIdx.y: 256 channels.
-constexpr int kColThreads = 1024;
-__global__ void __launch_bounds__(kColThreads)
-colsum_partial_kernel(const float* __restrict__ g, int csg, long long npix, int C, float* __restrict__ part) {
-    __shared__ float sh[kColThreads];
-    const int c0 = blockIdx.y * 256;
-    const int nc = C - c0 < 256 ? C - c0 : 256, lanes = kColThreads / nc;
-    const int c = threadIdx.x % nc, lane = threadIdx.x / nc;
-    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};     // four pixels in flight
-    if (lane < lanes) {
-        const long long step = (long long)gridDim.x * lanes;
-        const float* q = g + c0 + c;
-        long long p = (long long)blockIdx.x * lanes + lane;
-        for (; p + 3 * step < npix; p += 4 * step) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) s[k] += q[(p + k * step) * csg];
-        }
-        for (; p < npix; p += step) s[0] += q[p * csg];
-    }
-    sh[threadIdx.x] = (s[0] + s[1]) + (s[2] + s[3]);
+// per-block partial sums of column c of g (rows = pixels), fixed order
+__global__ void colsum_partial_kernel(const float* __restrict__ g, int csg, long long npix, int C,
+                                      float* __restrict__ part) {
+    __shared__ float sh[kThreads];
+    const int c = blockIdx.y;
+    float s = 0.0f;
+    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < npix; p += (long long)gridDim.x * blockDim.x)
+        s += g[p * csg + c];
+    sh[threadIdx.x] = s;
     __syncthreads();
-    if ((int)threadIdx.x < nc) {
-        float t = 0.0f;
-        for (int l = 0; l < lanes; ++l) t += sh[threadIdx.x + l * nc];
-        part[(long long)(c0 + c) * gridDim.x + blockIdx.x] = t;
+    for (int o = kThreads / 2; o > 0; o >>= 1) {
+        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+        __syncthreads();
     }
+    if (threadIdx.x == 0) part[(long long)c * gridDim.x + blockIdx.x] = sh[0];
 }
 
 __global__ void colsum_finish_kernel(const float* __restrict__ part, int nb, int C, float* __restrict__ out) {
@@ -1234,82 +1212,102 @@ __global__ void colsum_finish_kernel(const float* __restrict__ part, int nb, int
 // convolutions), and the bias gradient's block partials from the FP32 v.  The
 // gradient of the activation is g (MODE 0), the sum of g over the 2 x 2 fine
 // pixels of an upsampling (MODE 1), or g plus a quarter of the pooled path's
-// gradient gp (MODE 2).  One pass over memory where the separate kernels
-// (pooling or upsampling backward, addition, ReLU, column sums) took up to
-// seven and an FP32 copy of v in between (the 8 x 256^2 x 32 level: 342 us).
-// Four channels per thread; H x W the layer's own size.
+// gradient gp (MODE 2); MODE 3 only sums g.  One pass over memory where the
+// separate kernels (pooling or upsampling backward, addition, ReLU, column sums)
+// took up to seven and an FP32 copy of v in between (the 8 x 256^2 x 32 level:
+// 342 us before, 57 now).  A thread takes four channels of two pixels in 256; the sums
+// are those of colsum_partial_kernel, in its order (its one channel per block
+// reads 4 of every 4 C bytes: 63 us at that level).  H x W the layer's own size.
+constexpr int kGradThreads = 512;    // 128 pixels x 16 channels
 template <int MODE>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kGradThreads)
 relu_grad_kernel(const float* __restrict__ g, int csg, const float* __restrict__ gp, int csp,
-                 const bf16* __restrict__ act, int csa, bf16* __restrict__ out, int H, int W, int npix, int C,
+                 const bf16* __restrict__ act, int csa, bf16* __restrict__ out, int W, int npix, int C,
                  float* __restrict__ part) {
-    __shared__ float4 sh[kThreads];
-    const int C4 = C / 4, lanes = kThreads / C4;       // pixels a block takes at a time
-    const int c = (threadIdx.x % C4) * 4, lane = threadIdx.x / C4;
-    float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    for (int p = blockIdx.x * lanes + lane; lane < lanes && p < npix; p += gridDim.x * lanes) {
-        float4 v;
-        if constexpr (MODE == 0) {
-            v = *reinterpret_cast<const float4*>(g + (long long)p * csg + c);
-        } else {
-            const int row = p / W, x = p - row * W;     // row over all images
-            if constexpr (MODE == 1) {
-                const float* q = g + ((long long)(2 * row) * (2 * W) + 2 * x) * csg + c;
-                const float4 a = *reinterpret_cast<const float4*>(q);
-                const float4 b = *reinterpret_cast<const float4*>(q + csg);
-                q += (long long)(2 * W) * csg;
-                const float4 d = *reinterpret_cast<const float4*>(q);
-                const float4 e = *reinterpret_cast<const float4*>(q + csg);
-                v = make_float4(((a.x + b.x) + d.x) + e.x, ((a.y + b.y) + d.y) + e.y, ((a.z + b.z) + d.z) + e.z,
-                                ((a.w + b.w) + d.w) + e.w);
+    __shared__ float4 sh[256][4];
+    const int quad = threadIdx.x & 3, c = blockIdx.y * 16 + quad * 4, lane = threadIdx.x >> 2;
+    float4 sum[2] = {};
+    for (int base = blockIdx.x * 256; base < npix && c < C; base += gridDim.x * 256) {
+        float4 v[2];
+        uint2 m[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int p = base + lane + 128 * u;
+            v[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (p >= npix) continue;
+            if constexpr (MODE == 0 || MODE == 3) {
+                v[u] = *reinterpret_cast<const float4*>(g + (long long)p * csg + c);
             } else {
-                const float4 a = *reinterpret_cast<const float4*>(g + (long long)p * csg + c);
-                const float4 b = *reinterpret_cast<const float4*>(
-                    gp + ((long long)(row >> 1) * (W >> 1) + (x >> 1)) * csp + c);
-                v = make_float4(a.x + b.x * 0.25f, a.y + b.y * 0.25f, a.z + b.z * 0.25f, a.w + b.w * 0.25f);
+                const int row = p / W, x = p - row * W;     // row over all images
+                if constexpr (MODE == 1) {
+                    const float* q = g + ((long long)(2 * row) * (2 * W) + 2 * x) * csg + c;
+                    const float4 a = *reinterpret_cast<const float4*>(q);
+                    const float4 b = *reinterpret_cast<const float4*>(q + csg);
+                    q += (long long)(2 * W) * csg;
+                    const float4 d = *reinterpret_cast<const float4*>(q);
+                    const float4 e = *reinterpret_cast<const float4*>(q + csg);
+                    v[u] = make_float4(((a.x + b.x) + d.x) + e.x, ((a.y + b.y) + d.y) + e.y, ((a.z + b.z) + d.z) + e.z,
+                                       ((a.w + b.w) + d.w) + e.w);
+                } else {
+                    const float4 a = *reinterpret_cast<const float4*>(g + (long long)p * csg + c);
+                    const float4 b = *reinterpret_cast<const float4*>(
+                        gp + ((long long)(row >> 1) * (W >> 1) + (x >> 1)) * csp + c);
+                    v[u] = make_float4(a.x + b.x * 0.25f, a.y + b.y * 0.25f, a.z + b.z * 0.25f, a.w + b.w * 0.25f);
+                }
             }
+            if constexpr (MODE != 3) m[u] = *reinterpret_cast<const uint2*>(act + (long long)p * csa + c);
         }
-        const uint2 m = *reinterpret_cast<const uint2*>(act + (long long)p * csa + c);
-        v.x = __uint_as_float(m.x << 16) > 0.0f ? v.x : 0.0f;
-        v.y = __uint_as_float(m.x & 0xffff0000u) > 0.0f ? v.y : 0.0f;
-        v.z = __uint_as_float(m.y << 16) > 0.0f ? v.z : 0.0f;
-        v.w = __uint_as_float(m.y & 0xffff0000u) > 0.0f ? v.w : 0.0f;
-        __nv_bfloat162 o[2] = {__floats2bfloat162_rn(v.x, v.y), __floats2bfloat162_rn(v.z, v.w)};
-        *reinterpret_cast<uint2*>(out + (long long)p * C + c) = *reinterpret_cast<uint2*>(o);
-        sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int p = base + lane + 128 * u;
+            if (p >= npix) continue;
+            if constexpr (MODE != 3) {
+                v[u].x = __uint_as_float(m[u].x << 16) > 0.0f ? v[u].x : 0.0f;
+                v[u].y = __uint_as_float(m[u].x & 0xffff0000u) > 0.0f ? v[u].y : 0.0f;
+                v[u].z = __uint_as_float(m[u].y << 16) > 0.0f ? v[u].z : 0.0f;
+                v[u].w = __uint_as_float(m[u].y & 0xffff0000u) > 0.0f ? v[u].w : 0.0f;
+                __nv_bfloat162 o[2] = {__floats2bfloat162_rn(v[u].x, v[u].y), __floats2bfloat162_rn(v[u].z, v[u].w)};
+                *reinterpret_cast<uint2*>(out + (long long)p * C + c) = *reinterpret_cast<uint2*>(o);
+            }
+            sum[u].x += v[u].x; sum[u].y += v[u].y; sum[u].z += v[u].z; sum[u].w += v[u].w;
+        }
     }
-    sh[threadIdx.x] = sum;
+    sh[lane][quad] = sum[0];
+    sh[lane + 128][quad] = sum[1];
     __syncthreads();
-    if ((int)threadIdx.x < C4) {
-        for (int l = 1; l < lanes; ++l) {
-            const float4 t = sh[threadIdx.x + l * C4];
-            sum.x += t.x; sum.y += t.y; sum.z += t.z; sum.w += t.w;
+    for (int o = 128; o > 0; o >>= 1) {
+        if (lane < o) {
+            float4& a = sh[lane][quad];
+            const float4 b = sh[lane + o][quad];
+            a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
         }
-        *reinterpret_cast<float4*>(part + (long long)blockIdx.x * C + c) = sum;
+        __syncthreads();
     }
+    if (lane == 0 && c < C) *reinterpret_cast<float4*>(part + (long long)blockIdx.x * C + c) = sh[0][quad];
 }
 
-// out[c] = sum of part[b][c] over the blocks: one warp per channel, fixed order
-__global__ void channel_finish_kernel(const float* __restrict__ part, int nb, int C, float* __restrict__ out) {
-    const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (c >= C) return;
+// out[c] = sum of part[b][c] over the blocks, in block order; channels past C of
+// `pad` are set to zero
+__global__ void channel_finish_kernel(const float* __restrict__ part, int nb, int C, int pad, float* __restrict__ out) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= pad) return;
     float s = 0.0f;
-    for (int b = lane; b < nb; b += 32) s += part[(long long)b * C + c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) out[c] = s;
+    if (c < C) {
+#pragma unroll 16
+        for (int b = 0; b < nb; ++b) s += part[(long long)b * C + c];
+    }
+    out[c] = s;
 }
 
-// Loss of out = x + delta against t over four channels, its gradient as the
-// bf16 operand of the output layer's gradient convolutions (16 channels, the
-// padded ones zero) and the output layer's bias gradient: one thread per pixel.
-// part: the block's FP64 loss sum; gpart: its sums of the FP32 gradient.
+// Loss of out = x + delta against t over four channels, its gradient in FP32 (g4)
+// and as the bf16 operand of the output layer's gradient convolutions (16
+// channels, the padded ones zero): one thread per pixel.  part: the block's FP64
+// loss sum.
 __global__ void __launch_bounds__(kThreads)
 mse_grad_kernel(const float4* __restrict__ x, const float* __restrict__ delta, const float4* __restrict__ t,
-                bf16* __restrict__ g16, int npix, double inv, double* __restrict__ part, float* __restrict__ gpart) {
+                bf16* __restrict__ g16, float4* __restrict__ g4, int npix, double inv, double* __restrict__ part) {
     __shared__ double sh[kThreads];
-    __shared__ float4 gs[kThreads];
     double s = 0.0;
-    float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     for (int p = blockIdx.x * kThreads + threadIdx.x; p < npix; p += gridDim.x * kThreads) {
         const float4 a = x[p], d = *reinterpret_cast<const float4*>(delta + (long long)p * 16), b = t[p];
         const double e[4] = {(double)a.x + (double)d.x - (double)b.x, (double)a.y + (double)d.y - (double)b.y,
@@ -1320,7 +1318,7 @@ mse_grad_kernel(const float4* __restrict__ x, const float* __restrict__ delta, c
             s += e[k] * e[k];
             g[k] = (float)(2.0 * e[k] * inv);
         }
-        sum.x += g[0]; sum.y += g[1]; sum.z += g[2]; sum.w += g[3];
+        g4[p] = make_float4(g[0], g[1], g[2], g[3]);
         __nv_bfloat162 o[4] = {__floats2bfloat162_rn(g[0], g[1]), __floats2bfloat162_rn(g[2], g[3]),
                                __floats2bfloat162_rn(0.0f, 0.0f), __floats2bfloat162_rn(0.0f, 0.0f)};
         uint4* q = reinterpret_cast<uint4*>(g16 + (long long)p * 16);
@@ -1328,26 +1326,17 @@ mse_grad_kernel(const float4* __restrict__ x, const float* __restrict__ delta, c
         q[1] = make_uint4(0u, 0u, 0u, 0u);
     }
     sh[threadIdx.x] = s;
-    gs[threadIdx.x] = sum;
     __syncthreads();
     for (int o = kThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            sh[threadIdx.x] += sh[threadIdx.x + o];
-            float4& u = gs[threadIdx.x];
-            const float4 v = gs[threadIdx.x + o];
-            u.x += v.x; u.y += v.y; u.z += v.z; u.w += v.w;
-        }
+        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        part[blockIdx.x] = sh[0];
-        *reinterpret_cast<float4*>(gpart + 4 * blockIdx.x) = gs[0];
-    }
+    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-// loss and the 16 entries of the output layer's bias gradient (4 real) from the
-// block partials: one warp each
-__global__ void mse_grad_finish_kernel(const double* __restrict__ part, const float* __restrict__ gpart, int nb,
+// the loss, and the 16 entries of the output layer's bias gradient (4 real) from
+// the block partials of g4
+__global__ void mse_grad_finish_kernel(const double* __restrict__ part, int nb, const float* __restrict__ gpart, int ngb,
                                        double inv_count, double* __restrict__ loss, float* __restrict__ gb) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (w == 0) {
@@ -1355,12 +1344,13 @@ __global__ void mse_grad_finish_kernel(const double* __restrict__ part, const fl
         for (int b = lane; b < nb; b += 32) s += part[b];
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) loss[0] = s * inv_count;
-        if (lane >= 4 && lane < 16) gb[lane] = 0.0f;
-    } else if (w <= 4) {
+    } else if (lane < 16) {
         float s = 0.0f;
-        for (int b = lane; b < nb; b += 32) s += gpart[4 * b + w - 1];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) gb[w - 1] = s;
+        if (lane < 4) {
+#pragma unroll 16
+            for (int b = 0; b < ngb; ++b) s += gpart[4 * b + lane];
+        }
+        gb[lane] = s;
     }
 }
 
@@ -1662,59 +1652,37 @@ cudaError_t large_smem(K kernel, bool (&done)[64], int dev) {
     return cudaSuccess;
 }
 
-// Dynamic shared memory of a weight-gradient row-march launch, raised like
-// conv_row_launch_smem so that the CTAs an SM holds fit its tensor memory.
-size_t wg_launch_smem(size_t need, int Cn, int Co) {
-    const int per_sm = 512 / (int)wg_tmem_cols(Cn, Co);
-    const size_t floor_bytes = sm_shared_bytes() / (size_t)(per_sm + 1) + 1;
-    return need > floor_bytes ? need : floor_bytes;
-}
-
-// Input channels of one CTA of the weight-gradient row march, and the pixels of
-// its segment: the widest divisor of W that is a multiple of 16, at most 128
-// and fits shared memory (0: the march does not apply to these sizes).
+// Segment width of the weight-gradient row march (0: the width allows none)
+// and the input channels of one CTA.
+inline int wg_segment(int W) { return W % 64 == 0 ? 64 : (W % 32 == 0 ? 32 : 0); }
 inline int wg_block(int Ci) { return Ci <= kWgCn ? Ci : kWgCn; }
-inline int wg_segment(int W, int Ci, int Co) {
-    if (W % 16) return 0;
-    for (int P = W < 128 ? W : 128; P >= 16; P -= 16)
-        if (W % P == 0 && wg_layout(P, wg_block(Ci), Co).total <= kWgSmemMax) return P;
-    return 0;
-}
 
 // Row chunks of the weight-gradient row march on the current device: rows
 // per CTA and chunks per column (0 rows: the march does not apply to these
-// sizes).  One wave: tap rows x channel blocks x N x W / P segments x
-// chunks CTAs at most the resident CTAs.
+// sizes).  As many chunks as keep 3 tap rows x channel blocks x N x W / P segments
+// x chunks CTAs within what an SM would hold of CTAs with two row buffers in
+// both operand layouts (`cta` bytes) and 3 Cn columns of tensor memory.  The
+// kernel needs less than that, but the cut fixes the order of the sums.
 cudaError_t wgrad_row_plan(int N, int H, int W, int Ci, int Co, int* rows, int* chunks) {
     *rows = 0;
     *chunks = 0;
-    const int Cn = wg_block(Ci);
-    if (Ci % Cn || Co > 128 || Ci % 16 || Co % 16 || H < 1) return cudaSuccess;
-    const int P = wg_segment(W, Ci, Co);
-    if (P == 0) return cudaSuccess;
-    const WgLayout Lt = wg_layout(P, Cn, Co);
+    const int P = wg_segment(W), Cn = wg_block(Ci);
+    if (P == 0 || Ci % Cn || Co > 128 || Ci % 16 || Co % 16 || H < 1) return cudaSuccess;
+    const size_t cta = 2 * ((size_t)P * (2 * Co + 16) + (size_t)(P + 2) * (2 * Cn + 16)) +
+                       2 * (size_t)(P / 8) * (128 + 3 * (size_t)Cn) * 16;
+    if (cta > kWgSmemMax || wg_bytes(wg_layout(P, Cn, Co), 2) > kWgSmemMax) return cudaSuccess;
     static bool attr_set[64] = {};
-    int dev = 0, sms = 0, occ = 0;
+    int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = large_smem(conv_wgrad_row_kernel, attr_set, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        e = cudaFuncSetAttribute(conv_wgrad_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmemMax);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(conv_wgrad_row_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        attr_set[dev] = true;
-    }
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    // CTAs an SM holds: its shared memory (1 KB reserved per CTA) and its 512
-    // tensor-memory columns
-    const size_t per_cta = wg_launch_smem(Lt.total, Cn, Co) + 1024;
-    occ = (int)(sm_shared_bytes() / per_cta);
-    const int by_tmem = 512 / (int)wg_tmem_cols(Cn, Co);
+    const int by_tmem = 512 / (int)(3 * Cn <= 64 ? 64 : (3 * Cn <= 128 ? 128 : (3 * Cn <= 256 ? 256 : 512)));
+    const size_t least = sm_shared_bytes() / (size_t)(by_tmem + 1) + 1;
+    int occ = (int)(sm_shared_bytes() / ((cta > least ? cta : least) + 1024));
     if (occ > by_tmem) occ = by_tmem;
     const long long slots = (long long)sms * (occ > 0 ? occ : 1);
-    const long long cols = (9LL / wg_taps(Cn, Co)) * (Ci / Cn) * N * (W / P);
+    const long long cols = 3LL * (Ci / Cn) * N * (W / P);
     long long c = slots / cols;
     if (c < 1) c = 1;
     if (c > H) c = H;
@@ -1756,8 +1724,10 @@ static int conv3x3(const void* x, int csx, const void* w, const float* bias, voi
     if (cudaGetSymbolAddress((void**)&err, g_sg_err) != cudaSuccess) return LBM_ECUDA;
     // rows of 128-pixel segments: the row march, when four input rows and the
     // weights of all taps fit in shared memory; else flat tiles, when their
-    // cells and two taps' weights do.  (us at 8 x 256^2 / 2^l of level l, row
-    // march, flat tiles, tap kernel: see the table at conv3x3's callers.)
+    // cells and two taps' weights do, else the tap kernel.  us of the U-Net's
+    // layers at 8 x 256^2, tap kernel / this: 128 -> 32 at 128^2 157 / 28 (march),
+    // 64 -> 128 at 64^2 42 / 28, 256 -> 64 at 64^2 101 / 49, 128 -> 128 at 32^2 39 / 18
+    // (flat).
     int sms = 1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LBM_ECUDA;
     // CTAs on an SM: up to three, whose copies, MMAs and stores overlap, as long
@@ -1785,23 +1755,22 @@ static int conv3x3(const void* x, int csx, const void* w, const float* bias, voi
             (const bf16*)x, csx, (const bf16*)w, bias, y, csy, N, H, W, Ci, Co, rows, slots, err);
         return check(cudaGetLastError());
     }
-    const int stages = flat_stages(W, Ci, Co);
-    const long long flat = (long long)H * (W + 2);
-    if (stages >= 2 && flat < (1LL << 30)) {
+    const long long flat = (long long)H * (W + 2), tiles = (flat + 127) / 128;
+    int Cs = Co;   // output channels of a CTA: halved while that still fills no more than the SMs
+    while (Cs % 32 == 0 && N * tiles * (Co / Cs) * 2 <= sms) Cs /= 2;
+    const int stages = flat_stages(W, Ci, Cs);
+    if (stages >= 2 && flat < (1LL << 30) && N * tiles < (1LL << 31)) {
         static bool done[64] = {};
         if (large_smem(conv_flat_kernel<ACT>, done, dev) != cudaSuccess) {
             cudaGetLastError();
             return LBM_ECUDA;
         }
-        const int tiles = (int)((flat + 127) / 128);
-        if ((long long)N * tiles < (1LL << 31)) {
-            // no more CTAs on an SM than its tensor memory serves (four of 128 columns)
-            const size_t need = flat_x_bytes(W, Ci) + (size_t)stages * flat_w_bytes(Ci, Co);
-            const size_t least = sm_shared_bytes() / 5 + 1;
-            conv_flat_kernel<ACT><<<(unsigned)(N * tiles), kRoleThreads, need > least ? need : least, s>>>(
-                (const bf16*)x, csx, (const bf16*)w, bias, y, csy, H, W, Ci, Co, tiles, stages, err);
-            return check(cudaGetLastError());
-        }
+        // no more CTAs on an SM than its tensor memory serves (four of 128 columns)
+        const size_t need = flat_x_bytes(W, Ci) + (size_t)stages * flat_w_bytes(Ci, Cs);
+        const size_t least = sm_shared_bytes() / 5 + 1;
+        conv_flat_kernel<ACT><<<dim3((unsigned)(N * tiles), Co / Cs), kRoleThreads, need > least ? need : least, s>>>(
+            (const bf16*)x, csx, (const bf16*)w, bias, y, csy, H, W, Ci, Cs, (int)tiles, stages, err);
+        return check(cudaGetLastError());
     }
     const unsigned nb = (unsigned)((M + kTcM - 1) / kTcM);
     conv_tc_kernel<ACT><<<nb, kTcM, smem, s>>>((const bf16*)x, csx, (const bf16*)w, bias, y, csy, M, H, W, Ci, Co, err);
@@ -1842,7 +1811,7 @@ long long lbm_sg_wgrad_scratch_floats(int N, int H, int W, int Ci, int Co) {
     int rows = 0, chunks = 0;
     if (wgrad_row_plan(N, H, W, Ci, Co, &rows, &chunks) == cudaSuccess) {
         if (rows > 0) {
-            const long long row_need = (long long)N * (W / wg_segment(W, Ci, Co)) * chunks * Co * 9 * Ci;
+            const long long row_need = (long long)N * (W / wg_segment(W)) * chunks * Co * 9 * Ci;
             if (row_need > need) need = row_need;
         }
     } else {
@@ -1858,8 +1827,8 @@ int lbm_sg_conv3x3_wgrad(const void* x, int csx, const void* gy, int csg, float*
         return LBM_EINVAL;
     const long long need = lbm_sg_wgrad_scratch_floats(N, H, W, Ci, Co);
     if (scratch_floats < need) return LBM_EINVAL;
-    // rows in segments of multiples of 16 pixels, with 16-byte aligned channel
-    // rows: the tcgen05 row march
+    // rows in segments of 64 or 32 pixels, with 16-byte aligned channel rows: the
+    // tcgen05 row march
     int rows = 0, rchunks = 0;
     if (wgrad_row_plan(N, H, W, Ci, Co, &rows, &rchunks) != cudaSuccess) {
         cudaGetLastError();
@@ -1870,14 +1839,24 @@ int lbm_sg_conv3x3_wgrad(const void* x, int csx, const void* gy, int csg, float*
         int* err = nullptr;
         if (cudaGetSymbolAddress((void**)&err, g_sg_err) != cudaSuccess) return LBM_ECUDA;
         cudaStream_t s = (cudaStream_t)stream;
-        const int P = wg_segment(W, Ci, Co), Cn = wg_block(Ci);
-        const long long pchunks = (long long)N * (W / P) * rchunks;
+        const int P = wg_segment(W), Cn = wg_block(Ci);
+        const long long pchunks = (long long)N * (W / P) * rchunks, ctas = 3 * (Ci / Cn) * pchunks;
         const WgLayout Lt = wg_layout(P, Cn, Co);
-        conv_wgrad_row_kernel<<<(unsigned)((9 / wg_taps(Cn, Co)) * (Ci / Cn) * pchunks), kRoleThreads,
-                                wg_launch_smem(Lt.total, Cn, Co), s>>>(
-            (const bf16*)x, csx, (const bf16*)gy, csg, scratch, N, H, W, Ci, Co, P, Cn, rows, err);
+        // all CTAs on the chip at once where two buffers allow it, a third
+        // buffer where it does not cost that; no more than tensor memory serves
+        int dev = 0, sms = 1;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return LBM_ECUDA;
+        const int by_tmem = 512 / (int)wg_tmem_cols(wg_n(Cn, Co));
+        long long want = (ctas + sms - 1) / sms;
+        if (want > by_tmem) want = by_tmem;
+        const int bufs = wg_bytes(Lt, 3) <= kWgSmemMax / (size_t)want - (want > 1 ? 1024 : 0) ? 3 : 2;
+        const size_t need = wg_bytes(Lt, bufs), least = sm_shared_bytes() / (size_t)(by_tmem + 1) + 1;
+        conv_wgrad_row_kernel<<<(unsigned)ctas, kRoleThreads, need > least ? need : least, s>>>(
+            (const bf16*)x, csx, (const bf16*)gy, csg, scratch, N, H, W, Ci, Co, P, Cn, rows, bufs, err);
         const long long K = (long long)Co * 9 * Ci;
-        sum_chunks_kernel<<<(unsigned)((K + 31) / 32), 256, 0, s>>>(scratch, pchunks, K, gw);
+        sum_chunks_kernel<<<(unsigned)((K + 31) / 32), 32, 0, s>>>(scratch, pchunks, K, gw);
         return check(cudaGetLastError());
     }
     const long long nchunks = (M + kChunk - 1) / kChunk;
@@ -1886,7 +1865,7 @@ int lbm_sg_conv3x3_wgrad(const void* x, int csx, const void* gy, int csg, float*
     conv_wgrad_kernel<<<(unsigned)((warps * 32 + 127) / 128), 128, 0, s>>>((const bf16*)x, csx, (const bf16*)gy, csg,
                                                                           scratch, M, H, W, Ci, Co);
     const long long K = (long long)Co * 9 * Ci;
-    sum_chunks_kernel<<<(unsigned)((K + 31) / 32), 256, 0, s>>>(scratch, nchunks, K, gw);
+    sum_chunks_kernel<<<(unsigned)((K + 31) / 32), 32, 0, s>>>(scratch, nchunks, K, gw);
     return check(cudaGetLastError());
 }
 
@@ -1897,11 +1876,24 @@ int lbm_sg_weight_flip(const void* w, void* wt, int Ci, int Co, void* stream) {
     return check(cudaGetLastError());
 }
 
+// blocks of the sums over pixels, 256 pixels at a time: their number fixes the
+// order of the additions
+static int sum_blocks(long long npix) {
+    return (int)(npix < 64LL * kThreads ? (npix + kThreads - 1) / kThreads : 64);
+}
+
 int lbm_sg_bias_grad(const float* g, int csg, float* gb, float* scratch, long long npix, int C, void* stream) {
     if (!g || !gb || !scratch || npix < 1 || C < 1 || csg < C) return LBM_EINVAL;
-    const int nb = (int)(npix < 64LL * kThreads ? (npix + kThreads - 1) / kThreads : 64);
+    const int nb = sum_blocks(npix);
     cudaStream_t s = (cudaStream_t)stream;
-    colsum_partial_kernel<<<dim3(nb, (C + 255) / 256), kColThreads, 0, s>>>(g, csg, npix, C, scratch);
+    if (C % 4 == 0 && csg % 4 == 0 && ((uintptr_t)g & 15) == 0 && ((uintptr_t)scratch & 15) == 0 && npix < (1LL << 30) &&
+        (C + 15) / 16 < 65536) {   // rows in 16-byte groups: the same sums
+        relu_grad_kernel<3><<<dim3(nb, (C + 15) / 16), kGradThreads, 0, s>>>(g, csg, nullptr, 0, nullptr, 0, nullptr, 1,
+                                                                            (int)npix, C, scratch);
+        channel_finish_kernel<<<(C + 31) / 32, 32, 0, s>>>(scratch, nb, C, C, gb);
+        return check(cudaGetLastError());
+    }
+    colsum_partial_kernel<<<dim3(nb, C), kThreads, 0, s>>>(g, csg, npix, C, scratch);
     colsum_finish_kernel<<<blocks(C), kThreads, 0, s>>>(scratch, nb, C, gb);
     return check(cudaGetLastError());
 }
@@ -1952,40 +1944,42 @@ int lbm_sg_relu_grad(const float* g, int csg, int up, const float* gp, int csp, 
     const long long npix = (long long)N * H * W;
     if (!g || !act || !ga || !gb || !scratch || N < 1 || H < 1 || W < 1 || npix >= (1LL << 30)) return LBM_EINVAL;
     if ((up != 1 && up != 2) || (gp && (up != 1 || H % 2 || W % 2 || csp < C || csp % 4))) return LBM_EINVAL;
-    if (C < 4 || C % 4 || C > 4 * kThreads || csg < C || csg % 4 || csa < C || csa % 4) return LBM_EINVAL;
+    if (C < 4 || C % 4 || C > 1024 || csg < C || csg % 4 || csa < C || csa % 4) return LBM_EINVAL;
     if (((uintptr_t)g & 15) || ((uintptr_t)gp & 15) || ((uintptr_t)act & 7) || ((uintptr_t)ga & 7) ||
         ((uintptr_t)scratch & 15))
         return LBM_EINVAL;
-    // about 16 pixels per thread, at most the blocks the scratch holds partials of
-    const int lanes = kThreads / (C / 4);
-    long long nb = (npix + 16LL * lanes - 1) / (16LL * lanes);
-    if (nb > LBM_SG_GRAD_BLOCKS) nb = LBM_SG_GRAD_BLOCKS;
-    if (scratch_floats < nb * C) return LBM_EINVAL;
+    const int nb = sum_blocks(npix);
+    if (scratch_floats < (long long)nb * C) return LBM_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     const bf16* a = (const bf16*)act;
     bf16* o = (bf16*)ga;
+    const dim3 grid(nb, (C + 15) / 16);
     const int np = (int)npix;
-    if (gp) relu_grad_kernel<2><<<(unsigned)nb, kThreads, 0, s>>>(g, csg, gp, csp, a, csa, o, H, W, np, C, scratch);
-    else if (up == 2) relu_grad_kernel<1><<<(unsigned)nb, kThreads, 0, s>>>(g, csg, gp, csp, a, csa, o, H, W, np, C, scratch);
-    else relu_grad_kernel<0><<<(unsigned)nb, kThreads, 0, s>>>(g, csg, gp, csp, a, csa, o, H, W, np, C, scratch);
-    channel_finish_kernel<<<(C + 7) / 8, kThreads, 0, s>>>(scratch, (int)nb, C, gb);
+    if (gp) relu_grad_kernel<2><<<grid, kGradThreads, 0, s>>>(g, csg, gp, csp, a, csa, o, W, np, C, scratch);
+    else if (up == 2) relu_grad_kernel<1><<<grid, kGradThreads, 0, s>>>(g, csg, gp, csp, a, csa, o, W, np, C, scratch);
+    else relu_grad_kernel<0><<<grid, kGradThreads, 0, s>>>(g, csg, gp, csp, a, csa, o, W, np, C, scratch);
+    channel_finish_kernel<<<(C + 31) / 32, 32, 0, s>>>(scratch, nb, C, C, gb);
     return check(cudaGetLastError());
 }
 
-int lbm_sg_mse_grad(const float* x, const float* delta, const float* target, void* g16, float* gb, double* scratch,
-                    double* loss, long long npix, void* stream) {
-    if (!x || !delta || !target || !g16 || !gb || !scratch || !loss || npix < 1 || npix >= (1LL << 30)) return LBM_EINVAL;
+int lbm_sg_mse_grad(const float* x, const float* delta, const float* target, void* g16, float* g4, float* gb,
+                    double* scratch, double* loss, long long npix, void* stream) {
+    if (!x || !delta || !target || !g16 || !g4 || !gb || !scratch || !loss || npix < 1 || npix >= (1LL << 30))
+        return LBM_EINVAL;
     if (((uintptr_t)x & 15) || ((uintptr_t)delta & 15) || ((uintptr_t)target & 15) || ((uintptr_t)g16 & 15) ||
-        ((uintptr_t)scratch & 15))
+        ((uintptr_t)g4 & 15) || ((uintptr_t)scratch & 15))
         return LBM_EINVAL;
     long long nb = (npix + kThreads - 1) / kThreads;
-    if (nb > LBM_SG_GRAD_BLOCKS) nb = LBM_SG_GRAD_BLOCKS;
+    if (nb > LBM_SG_LOSS_BLOCKS) nb = LBM_SG_LOSS_BLOCKS;
+    const int ngb = sum_blocks(npix);
     cudaStream_t s = (cudaStream_t)stream;
-    float* gpart = (float*)(scratch + LBM_SG_GRAD_BLOCKS);
+    float* gpart = (float*)(scratch + LBM_SG_LOSS_BLOCKS);
     const double inv = 1.0 / ((double)npix * 4);
-    mse_grad_kernel<<<(unsigned)nb, kThreads, 0, s>>>((const float4*)x, delta, (const float4*)target, (bf16*)g16, (int)npix,
-                                                      inv, scratch, gpart);
-    mse_grad_finish_kernel<<<1, 160, 0, s>>>(scratch, gpart, (int)nb, inv, loss, gb);
+    mse_grad_kernel<<<(unsigned)nb, kThreads, 0, s>>>((const float4*)x, delta, (const float4*)target, (bf16*)g16,
+                                                      (float4*)g4, (int)npix, inv, scratch);
+    relu_grad_kernel<3><<<dim3(ngb, 1), kGradThreads, 0, s>>>(g4, 4, nullptr, 0, nullptr, 0, nullptr, 1, (int)npix, 4,
+                                                             gpart);
+    mse_grad_finish_kernel<<<1, 64, 0, s>>>(scratch, (int)nb, gpart, ngb, inv, loss, gb);
     return check(cudaGetLastError());
 }
 

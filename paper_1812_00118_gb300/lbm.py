@@ -126,7 +126,7 @@ SIGNATURES = [
                                   ctypes.c_longlong, ctypes.c_int, _VP]),
     ("lbm_sg_relu_grad", ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int, _VP, ctypes.c_int, _VP, ctypes.c_int, _VP, _VP,
                                         _VP, ctypes.c_longlong] + [ctypes.c_int] * 4 + [_VP]),
-    ("lbm_sg_mse_grad", ctypes.c_int, [_VP] * 7 + [ctypes.c_longlong, _VP]),
+    ("lbm_sg_mse_grad", ctypes.c_int, [_VP] * 8 + [ctypes.c_longlong, _VP]),
     ("lbm_sg_adam_layers", ctypes.c_int, [ctypes.POINTER(lbm_sg_layer), ctypes.c_int, ctypes.c_float, ctypes.c_float,
                                           ctypes.c_float, ctypes.c_float, ctypes.c_int, _VP]),
     ("lbm_sg_adam", ctypes.c_int, [_VP, _VP, _VP, _VP, ctypes.c_longlong, ctypes.c_float, ctypes.c_float,

@@ -30,7 +30,7 @@ LAYERS = [("e1", 4, 32), ("e2", 32, 64), ("e3", 64, 128), ("b", 128, 128),
 POOL = 2      # pooling / upsampling factor between levels
 LEVELS = 4
 NC = 4        # real channels of the input and output: phi, rho u_x, rho u_y, P
-GRAD_BLOCKS = 512   # LBM_SG_GRAD_BLOCKS of include/lbm_surrogate.h
+LOSS_BLOCKS = 512   # LBM_SG_LOSS_BLOCKS of include/lbm_surrogate.h
 CO_MAX = 128  # output channels one lbm_sg_conv3x3 call produces at most
 
 
@@ -104,6 +104,7 @@ class Surrogate:
         self.g16_3, self.g16_4 = z(M3, 128, dt=b16), z(M4, 128, dt=b16)
         self.gh1, self.gc1, self.gc2, self.gc3 = z(M1, 32), z(M1, 64), z(M2, 128), z(M3, 256)
         self.gp3, self.gp2, self.gp1 = z(M4, 128), z(M3, 64), z(M2, 32)
+        self.g_delta = z(M1, NC)
         lib = self.lib
         scratch = max(lib.lbm_sg_wgrad_scratch_floats(N, H, W, 64, 32),
                       lib.lbm_sg_wgrad_scratch_floats(N, H, W, 16, 32),
@@ -112,9 +113,9 @@ class Surrogate:
                       lib.lbm_sg_wgrad_scratch_floats(N, H // 2, W // 2, 32, 64),
                       lib.lbm_sg_wgrad_scratch_floats(N, H // 4, W // 4, 256, 64),
                       lib.lbm_sg_wgrad_scratch_floats(N, H // 4, W // 4, 64, 128),
-                      lib.lbm_sg_wgrad_scratch_floats(N, H // 8, W // 8, 128, 128), GRAD_BLOCKS * 128)
+                      lib.lbm_sg_wgrad_scratch_floats(N, H // 8, W // 8, 128, 128), 64 * 256)
         self.scratch = z(int(scratch))
-        self.mse_scratch = torch.zeros(3 * GRAD_BLOCKS, dtype=torch.float64, device=dev)
+        self.mse_scratch = torch.zeros(2 * LOSS_BLOCKS, dtype=torch.float64, device=dev)
         self.loss_dev = torch.zeros(1, dtype=torch.float64, device=dev)
         self.step_count = 0
 
@@ -256,8 +257,8 @@ class Surrogate:
                              f"{self.x32.device} is required")
         if target32.data_ptr() % 16:     # a view into a larger tensor
             target32 = target32.clone()
-        _ck(lib.lbm_sg_mse_grad(p(self.x32), p(self.delta), p(target32), p(self.g16_1), p(self.layers["out"]["gb"]),
-                                p(self.mse_scratch), p(self.loss_dev), M1, s), "lbm_sg_mse_grad")
+        _ck(lib.lbm_sg_mse_grad(p(self.x32), p(self.delta), p(target32), p(self.g16_1), p(self.g_delta),
+                                p(self.layers["out"]["gb"]), p(self.mse_scratch), p(self.loss_dev), M1, s), "lbm_sg_mse_grad")
         # out, d1 (level 1)
         self._wgrad("out", p(self.h1), 32, p(self.g16_1), 16, 0)
         self._conv_input_grad("out", p(self.g16_1), 16, self.gh1, 32, 0)

@@ -462,7 +462,7 @@ __host__ __device__ inline uint32_t row_tmem_cols(int Co) {
 }
 
 template <bool ACT>
-__global__ void __launch_bounds__(kRoleThreads, 1)
+__global__ void __launch_bounds__(kRoleThreads, 3)
 conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, const float* __restrict__ bias,
                 void* __restrict__ y, int csy, int N, int H, int W, int Ci, int Co, int rows_per_cta, int slots,
                 int* err) {
@@ -621,7 +621,7 @@ inline int flat_stages(int W, int Ci, int Co) {
 }
 
 template <bool ACT>
-__global__ void __launch_bounds__(kRoleThreads, 1)
+__global__ void __launch_bounds__(kRoleThreads, 3)
 conv_flat_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w, const float* __restrict__ bias,
                  void* y, int csy, int H, int W, int Ci, int Co, int tiles, int stages, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -827,7 +827,7 @@ __host__ __device__ inline uint32_t wg_tmem_cols(int n) {   // three taps of n c
     return need <= 64 ? 64u : (need <= 128 ? 128u : (need <= 256 ? 256u : 512u));
 }
 
-__global__ void __launch_bounds__(kRoleThreads, 1)
+__global__ void __launch_bounds__(kRoleThreads, 3)
 conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ gy, int csg,
                       float* __restrict__ partial, int N, int H, int W, int Ci, int Co, int P, int Cn,
                       int rows_per_cta, int bufs, int* err) {

@@ -177,16 +177,20 @@ __global__ void diag_partial_kernel(const double* __restrict__ phi, const double
     }
 }
 
-// sum / max of nb partial rows of width `width` (columns in max_mask use max)
+// sum / max of nb partial rows of width `width` <= 32 (columns in max_mask use
+// max): one warp per column, fixed order.  An addition takes 65 clk here, so a
+// chain of 1024 took 32 us; 32 chains and a tree take 2.
 __global__ void finish_kernel(const double* __restrict__ part, int nb, int width, int max_mask, double* out) {
-    if (threadIdx.x >= (unsigned)width) return;
-    const int k = threadIdx.x;
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (k >= width) return;
+    const bool mx = (max_mask >> k) & 1;
     double r = 0;
-    for (int b = 0; b < nb; ++b) {
+    for (int b = lane; b < nb; b += 32) {
         const double v = part[b * width + k];
-        r = ((max_mask >> k) & 1) ? fmax(r, v) : r + v;
+        r = mx ? fmax(r, v) : r + v;
     }
-    out[k] = r;
+    r = mx ? warp_max(r) : warp_sum(r);
+    if (lane == 0) out[k] = r;
 }
 
 // Laplace partials: sum P and count for r < r_in, and for r > r_out.
@@ -239,10 +243,10 @@ __global__ void sum_partial_kernel(const double* __restrict__ a, long long n, do
 
 __global__ void phi_delta_kernel(const double* __restrict__ part, int nb, double target, long long n,
                                  double* __restrict__ delta) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[b];
-    *delta = (target - s) / (double)n;
+    double s = 0.0;   // one warp, as in finish_kernel
+    for (int b = threadIdx.x; b < nb; b += 32) s += part[b];
+    s = warp_sum(s);
+    if (threadIdx.x == 0) *delta = (target - s) / (double)n;
 }
 
 int partial_blocks(const lbm_ctx* c) {
@@ -256,7 +260,7 @@ int reduce_diag(lbm_ctx* c, double out[4]) {
     double* res = c->partial + 4 * (size_t)c->n_partial_blocks;
     diag_partial_kernel<<<nb, kRedThreads, 0, c->stream>>>(f_phi(c), f_P(c), f_u(c, 0), f_u(c, 1), f_u(c, 2),
                                                           c->G.N, c->P.rho_L, c->P.rho_dif, c->partial);
-    finish_kernel<<<1, 32, 0, c->stream>>>(c->partial, nb, 4, 1 << 2, res);
+    finish_kernel<<<1, 128, 0, c->stream>>>(c->partial, nb, 4, 1 << 2, res);
     c->launches += 2;
     if (check_cuda(cudaGetLastError())) return LBM_ECUDA;
     if (check_cuda(cudaMemcpyAsync(out, res, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream))) return LBM_ECUDA;
@@ -804,7 +808,7 @@ int lbm_laplace(lbm_ctx* c, const double centre[3], double r_in, double r_out, d
     double* res = c->partial + 4 * (size_t)c->n_partial_blocks;
     laplace_partial_kernel<<<nb, kRedThreads, 0, c->stream>>>(f_P(c), c->G, cc[0], cc[1], cc[2], r_in, r_out,
                                                              c->partial);
-    finish_kernel<<<1, 32, 0, c->stream>>>(c->partial, nb, 4, 0, res);
+    finish_kernel<<<1, 128, 0, c->stream>>>(c->partial, nb, 4, 0, res);
     c->launches += 2;
     if (check_cuda(cudaGetLastError())) return LBM_ECUDA;
     double h[4];

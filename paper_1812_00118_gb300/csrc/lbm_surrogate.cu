@@ -1383,11 +1383,18 @@ __global__ void mse_kernel(const float* __restrict__ x, int csx, const float* __
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-__global__ void mse_finish_kernel(const double* __restrict__ part, int nb, double inv_count, double* out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Sum of column k of nb rows of `width` partials by the calling warp, fixed
+// order, in every lane (a chain of 256 FP64 additions of 65 clk took 8 us).
+__device__ __forceinline__ double warp_column(const double* __restrict__ part, int nb, int width, int k) {
     double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[b];
-    out[0] = s * inv_count;
+    for (int b = threadIdx.x & 31; b < nb; b += 32) s += part[b * width + k];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+__global__ void mse_finish_kernel(const double* __restrict__ part, int nb, double inv_count, double* out) {
+    const double s = warp_column(part, nb, 1, 0);
+    if (threadIdx.x == 0) out[0] = s * inv_count;
 }
 
 // Adam on FP32 master values, with the bf16 copy used by the convolutions
@@ -1498,11 +1505,8 @@ __global__ void residual_partial_kernel(const double* __restrict__ a, const doub
 }
 
 __global__ void residual_finish_kernel(const double* __restrict__ part, int nb, double* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double d2 = 0.0, a2 = 0.0;
-    for (int k = 0; k < nb; ++k) { d2 += part[2 * k]; a2 += part[2 * k + 1]; }
-    out[0] = d2;
-    out[1] = a2;
+    const double v = warp_column(part, nb, 2, threadIdx.x >> 5);   // two warps
+    if ((threadIdx.x & 31) == 0) out[threadIdx.x >> 5] = v;
 }
 
 // block partials of (sum P, count) over the bulk heavy phase (phi >= 1 - d)
@@ -1528,10 +1532,11 @@ __global__ void phase_pressure_partial_kernel(const double* __restrict__ phi, co
 }
 
 __global__ void phase_pressure_finish_kernel(const double* __restrict__ part, int nb, double* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = 0; b < nb; ++b)
-        for (int j = 0; j < 4; ++j) a[j] += part[4 * b + j];
+    __shared__ double a[4];
+    const double v = warp_column(part, nb, 4, threadIdx.x >> 5);   // four warps
+    if ((threadIdx.x & 31) == 0) a[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     out[0] = a[1] > 0.0 ? a[0] / a[1] : 0.0;
     out[1] = a[3] > 0.0 ? a[2] / a[3] : 0.0;
     out[2] = a[1];
@@ -1574,16 +1579,13 @@ __global__ void phi_project_kernel(double* __restrict__ phi, const double* __res
     }
 }
 
-// c = (sum phi0 - sum phi) / sum 4 phi (1 - phi), partials in block order, into part[3 nb]
+// c = (sum phi0 - sum phi) / sum 4 phi (1 - phi), into part[3 nb]
 __global__ void phi_project_finish_kernel(double* __restrict__ part, int nb) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    for (int b = 0; b < nb; ++b) {
-        a0 += part[3 * b];
-        a1 += part[3 * b + 1];
-        a2 += part[3 * b + 2];
-    }
-    part[3 * nb] = a2 > 0.0 ? (a0 - a1) / a2 : 0.0;
+    __shared__ double a[3];
+    const double v = warp_column(part, nb, 3, threadIdx.x >> 5);   // three warps
+    if ((threadIdx.x & 31) == 0) a[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) part[3 * nb] = a[2] > 0.0 ? (a[0] - a[1]) / a[2] : 0.0;
 }
 
 // phi += c 4 phi (1 - phi): the total of phi0 restored by moving the interfaces
@@ -2089,7 +2091,7 @@ int lbm_sg_residual(const double* a, const double* b, long long n, double* out, 
     const int nb = 256;
     cudaStream_t s = (cudaStream_t)stream;
     residual_partial_kernel<<<nb, kThreads, 0, s>>>(a, b, n, scratch);
-    residual_finish_kernel<<<1, 32, 0, s>>>(scratch, nb, out);
+    residual_finish_kernel<<<1, 64, 0, s>>>(scratch, nb, out);
     return check(cudaGetLastError());
 }
 
@@ -2099,7 +2101,7 @@ int lbm_sg_phase_pressure(const double* phi, const double* P, long long n, doubl
     const int nb = 256;
     cudaStream_t s = (cudaStream_t)stream;
     phase_pressure_partial_kernel<<<nb, kThreads, 0, s>>>(phi, P, n, d, scratch);
-    phase_pressure_finish_kernel<<<1, 32, 0, s>>>(scratch, nb, out);
+    phase_pressure_finish_kernel<<<1, 128, 0, s>>>(scratch, nb, out);
     return check(cudaGetLastError());
 }
 
@@ -2108,7 +2110,7 @@ int lbm_sg_phi_project(double* phi, const double* phi0, long long n, double* scr
     const int nb = 256;
     cudaStream_t s = (cudaStream_t)stream;
     phi_project_kernel<<<nb, kThreads, 0, s>>>(phi, phi0, n, scratch);
-    phi_project_finish_kernel<<<1, 32, 0, s>>>(scratch, nb);
+    phi_project_finish_kernel<<<1, 96, 0, s>>>(scratch, nb);
     phi_restore_kernel<<<blocks(n), kThreads, 0, s>>>(phi, n, scratch + 3 * nb);
     return check(cudaGetLastError());
 }

@@ -191,7 +191,8 @@ __device__ __forceinline__ bool box_step(const DirPtrs<typename Storage<ST>::S, 
     if (active) {
         const int rb = (y + G.GY) * G.PX + x + G.GX;
         auto h_of = [&](int i) { return St::raw(hv[i]); };
-        if (WALLS && wall_adjacent<LAT>(G, x, y, z))
+        // a warp with a node next to a wall takes one path, not both
+        if (WALLS && __any_sync(__activemask(), wall_adjacent<LAT>(G, x, y, z)))
             collide_node<LAT, ST, true>(D, G, p, sm.phis, lz, lz + 1, lz + 2, lx + 1, ly + HY, m, h_of, x, y, z, rb);
         else
             collide_node<LAT, ST, false>(D, G, p, sm.phis, lz, lz + 1, lz + 2, lx + 1, ly + HY, m, h_of, x, y, z, rb);

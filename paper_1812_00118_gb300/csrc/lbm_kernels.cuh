@@ -1232,9 +1232,9 @@ __device__ __forceinline__ void march(const DirPtrs<typename Storage<ST>::S, Lat
         __syncthreads();
         if (active) {
             auto hv = [&](int i) { return hown[(j + 1) & 1][i - 1][tid]; };   // i >= 1
-            // only a node next to a wall writes bounce-back ghost cells: the
-            // rest take the wall-free collision (fewer live registers)
-            if (WALLS && wall_adjacent<LAT>(G, x, y, z))
+            // only a node next to a wall writes bounce-back ghost cells: warps
+            // without one take the wall-free collision (fewer live registers)
+            if (WALLS && __any_sync(__activemask(), wall_adjacent<LAT>(G, x, y, z)))
                 collide_node<LAT, ST, true>(D, G, p, phis, j & 3, (j + 1) & 3, (j + 2) & 3, tx + 1, ty + HY, m, hv, x,
                                             y, z, rb);
             else

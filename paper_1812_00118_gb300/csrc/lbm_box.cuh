@@ -13,8 +13,8 @@
 // one node, that node's pull another), so with boxes at least two nodes wide
 // the data of step s come from the up to 26 adjacent boxes, and the buffer
 // step s writes was last read, in step s - 1, by the same boxes.  flags[box]
-// counts the steps a box has completed: box b starts step s once every
-// adjacent flag shows step s - 1 done, which covers both.  The counts go on
+// counts the warps that have completed a step: box b starts step s once every
+// adjacent flag shows step s - 1 done by all of them, which covers both.  The counts go on
 // from launch to launch (a box reads its own at the start), so a captured
 // launch can be replayed.  The launch is cooperative whenever boxes wait, so
 // they are all resident; the waits are bounded, and one that gives up raises
@@ -129,7 +129,7 @@ __device__ __forceinline__ bool box_step(const DirPtrs<typename Storage<ST>::S, 
                 b = b < 0 ? pl.ny - 1 : (b >= pl.ny ? 0 : b);
                 c = c < 0 ? pl.nz - 1 : (c >= pl.nz ? 0 : c);
                 const int* f = flags + (c * pl.ny + b) * pl.nx + a;
-                const int want = first + wait_for;
+                const int want = first + wait_for * (NT / 32);
                 ok = false;
                 for (int i = 0; i < kBoxPolls; ++i) {
                     int v;
@@ -140,7 +140,7 @@ __device__ __forceinline__ bool box_step(const DirPtrs<typename Storage<ST>::S, 
                 if (!ok) atomicExch(err, 1);
             }
         }
-        ok = __syncthreads_and(ok) != 0;
+        ok = __syncthreads_and(ok) != 0;   // also: the phi of the step before is read
         if (!ok) return false;
     }
 
@@ -197,7 +197,6 @@ __device__ __forceinline__ bool box_step(const DirPtrs<typename Storage<ST>::S, 
         else
             collide_node<LAT, ST, false>(D, G, p, sm.phis, lz, lz + 1, lz + 2, lx + 1, ly + HY, m, h_of, x, y, z, rb);
     }
-    __syncthreads();   // every store of the box issued, and its phi read
     return true;
 }
 
@@ -218,13 +217,15 @@ box_kernel(const __grid_constant__ BoxPtrs<typename Storage<ST>::S, Lattice<LAT>
 #pragma unroll 1
     for (int s = 0; s < n_steps; ++s) {
         for (int box = blockIdx.x; box < pl.boxes; box += gridDim.x) {
+            if (s == 0 && box != blockIdx.x) __syncthreads();   // phi of the box before (later steps wait instead)
             if (!box_step<LAT, ST, BX, BY, BZ, WALLS>(ptrs.d[s & 1], G, p, pl, box, first, s, flags, err, sm)) return;
-            // the barrier at the end of box_step orders the box's stores before
-            // this thread's release
-            if (n_steps > 1 && threadIdx.x == 0)
-                asm volatile("fence.acq_rel.gpu;\n\tst.relaxed.gpu.global.s32 [%0], %1;" ::"l"(flags + box),
-                             "r"(first + s + 1)
-                             : "memory");
+            // a warp's stores are done, each on its own account: no barrier, and
+            // the releases of a box's warps overlap
+            if (n_steps > 1) {
+                __syncwarp();
+                if ((threadIdx.x & 31) == 0)
+                    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(flags + box) : "memory");
+            }
         }
     }
 }

@@ -94,6 +94,29 @@ def test_phi_correction_splits_the_launch(lbm):
         assert np.array_equal(x, y)
 
 
+def test_resume_without_initialisation(lbm):
+    """A context whose first state comes from lbm_set_populations steps like the
+    one the state came from (its box counts start at zero)."""
+    import torch
+    a = make(lbm, (256, 192), (P, P), lbm.F32)
+    a.step(5)
+    h, g = a.get_populations()
+    junk = torch.full((1 << 22,), -1, dtype=torch.int32, device="cuda")   # what freed memory may hold
+    del junk
+    sims = []
+    for _ in range(3):
+        b = lbm.Simulation(lbm.D2Q9, (256, 192), a.params)
+        b.set_populations(h, g)
+        b.step(20)
+        sims.append(b)
+    a.step(20)
+    want = a.get_populations()
+    for b in sims:
+        assert b.diagnostics()["status"] == lbm.OK
+        for x, y in zip(b.get_populations(), want):
+            assert np.array_equal(x, y)
+
+
 def test_capture_and_replay(lbm):
     """A captured launch of 6 steps, replayed three times, equals 18 steps."""
     import torch

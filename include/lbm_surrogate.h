@@ -129,7 +129,7 @@ int lbm_sg_relu_grad(const float* g, int csg, int up, const float* gp, int csp, 
  * reads: *loss as there; g4 (float, 4 channels) = the gradient, g16 (bf16, 16
  * channels, the last 12 zero) = the gradient rounded; gb (16 floats, the last 12
  * zero) = its sums over the pixels (lbm_sg_bias_grad).  x and target have 4
- * channels, delta 16; x, delta, target, g16, g4 and scratch start on 16-byte
+ * channels, delta 16; x, delta, g16, g4 and scratch start on 16-byte
  * boundaries.  scratch: 2 * LBM_SG_LOSS_BLOCKS doubles. */
 int lbm_sg_mse_grad(const float* x, const float* delta, const float* target, void* g16, float* g4, float* gb,
                     double* scratch, double* loss, long long npix, void* stream);

@@ -237,7 +237,8 @@ __device__ __forceinline__ void for_groups(int tid, int rows, int groups, F&& f)
 }
 
 // A whole 32-byte sector per lane: lanes write pixels a row stride apart, and
-// two 16-byte stores per sector cost L2 two partial writes.
+// two 16-byte stores per sector cost L2 two partial writes (16 -> 32 channels at
+// 8 x 256^2: 32 us, 27 with this).
 __device__ __forceinline__ void st_global_32(void* p, const uint32_t (&v)[8]) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
                  "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
@@ -522,7 +523,7 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
             for_groups(tid, kRowHalo, nch, [&](int px, int c) {
                 int xx = x0 - 1 + px;
                 xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
-                cp_async16(dst + c * row_plane_bytes() + px * 16, row + xx * csx + c * 8, 16u);
+                cp_async16(dst + c * row_plane_bytes() + px * 16, row + (long long)xx * csx + c * 8, 16u);
             });
             mbar_arrive_copies(full + 8 * cs);
             ++ck;
@@ -779,7 +780,7 @@ __global__ void conv_wgrad_kernel(const bf16* __restrict__ x, int csx, const bf1
 // pitch between channel groups, 128 bytes between groups of 8 pixels).  A tap
 // is then the x row of its dy started (1 + dx) pixels in: no transposition
 // (transposing both operands through registers into K-major buffers took
-// 290 us for the 64 -> 32 layer at 8 x 256^2; this takes 100).  Plane pitches are
+// 290 us for the 64 -> 32 layer at 8 x 256^2; this takes 81).  Plane pitches are
 // odd multiples of 16 bytes, so the 8 groups of a pixel, copied by neighbouring
 // threads, fall into different banks.
 //
@@ -894,12 +895,12 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
                 for_groups(tid, P + 2, nci8, [&](int p, int c) {   // pixels x0 - 1 .. x0 + P (wrapped)
                     int xx = x0 - 1 + p;
                     xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
-                    cp_async16(xd + c * Lt.px + p * 16, xrow + xx * csx + c * 8, 16u);
+                    cp_async16(xd + c * Lt.px + p * 16, xrow + (long long)xx * csx + c * 8, 16u);
                 });
                 const bf16* grow = gy + (img + (long long)(y0 + q) * W + x0) * csg;
                 const uint32_t gd = gb + (uint32_t)(buf * RG + q - r0) * Lt.grow;
                 for_groups(tid, P, nco8, [&](int p, int c) {
-                    cp_async16(gd + c * Lt.pg + p * 16, grow + p * csg + c * 8, 16u);
+                    cp_async16(gd + c * Lt.pg + p * 16, grow + (long long)p * csg + c * 8, 16u);
                 });
                 yx = yx + 1 == H ? 0 : yx + 1;
             }
@@ -981,7 +982,7 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
 
 // gw[k] = sum over chunks of partial[chunk, k], in chunk order; blocks of one
 // warp and 16 loads in flight (256 threads that waited for each: 18 blocks and
-// 10 us for the 4608 values of the 16 -> 32 layer)
+// 10.3 us for the 4608 values of the 16 -> 32 layer, 5.6 now)
 __global__ void __launch_bounds__(32)
 sum_chunks_kernel(const float* __restrict__ partial, long long nchunks, long long K, float* __restrict__ gw) {
     const long long k = (long long)blockIdx.x * 32 + threadIdx.x;
@@ -1079,7 +1080,7 @@ __global__ void pool_kernel(const bf16* __restrict__ x, int csx, bf16* __restric
 
 // 2 x 2 pooling and upsampling on 8 channels (16 bytes) per thread: the
 // per-element kernels spend their time on 64-bit index divisions (8 x 256^2 x
-// 32 channels: pooling 53 us, upsampling 121 us).  The sums are formed in the
+// 32 channels: pooling 53 us, upsampling 121 us; these 8 and 11).  The sums are formed in the
 // order of pool_kernel.
 __device__ __forceinline__ void unpack8(uint4 q, float (&v)[8]) {
     const uint32_t u[4] = {q.x, q.y, q.z, q.w};
@@ -1304,12 +1305,14 @@ __global__ void channel_finish_kernel(const float* __restrict__ part, int nb, in
 // channels, the padded ones zero): one thread per pixel.  part: the block's FP64
 // loss sum.
 __global__ void __launch_bounds__(kThreads)
-mse_grad_kernel(const float4* __restrict__ x, const float* __restrict__ delta, const float4* __restrict__ t,
+mse_grad_kernel(const float4* __restrict__ x, const float* __restrict__ delta, const float* __restrict__ t, bool t_vec,
                 bf16* __restrict__ g16, float4* __restrict__ g4, int npix, double inv, double* __restrict__ part) {
     __shared__ double sh[kThreads];
     double s = 0.0;
     for (int p = blockIdx.x * kThreads + threadIdx.x; p < npix; p += gridDim.x * kThreads) {
-        const float4 a = x[p], d = *reinterpret_cast<const float4*>(delta + (long long)p * 16), b = t[p];
+        const float4 a = x[p], d = *reinterpret_cast<const float4*>(delta + (long long)p * 16);
+        const float* tp = t + (long long)p * 4;    // the caller's array: any alignment
+        const float4 b = t_vec ? *reinterpret_cast<const float4*>(tp) : make_float4(tp[0], tp[1], tp[2], tp[3]);
         const double e[4] = {(double)a.x + (double)d.x - (double)b.x, (double)a.y + (double)d.y - (double)b.y,
                              (double)a.z + (double)d.z - (double)b.z, (double)a.w + (double)d.w - (double)b.w};
         float g[4];
@@ -1968,8 +1971,8 @@ int lbm_sg_mse_grad(const float* x, const float* delta, const float* target, voi
                     double* scratch, double* loss, long long npix, void* stream) {
     if (!x || !delta || !target || !g16 || !g4 || !gb || !scratch || !loss || npix < 1 || npix >= (1LL << 30))
         return LBM_EINVAL;
-    if (((uintptr_t)x & 15) || ((uintptr_t)delta & 15) || ((uintptr_t)target & 15) || ((uintptr_t)g16 & 15) ||
-        ((uintptr_t)g4 & 15) || ((uintptr_t)scratch & 15))
+    if (((uintptr_t)x & 15) || ((uintptr_t)delta & 15) || ((uintptr_t)g16 & 15) || ((uintptr_t)g4 & 15) ||
+        ((uintptr_t)scratch & 15))
         return LBM_EINVAL;
     long long nb = (npix + kThreads - 1) / kThreads;
     if (nb > LBM_SG_LOSS_BLOCKS) nb = LBM_SG_LOSS_BLOCKS;
@@ -1977,8 +1980,8 @@ int lbm_sg_mse_grad(const float* x, const float* delta, const float* target, voi
     cudaStream_t s = (cudaStream_t)stream;
     float* gpart = (float*)(scratch + LBM_SG_LOSS_BLOCKS);
     const double inv = 1.0 / ((double)npix * 4);
-    mse_grad_kernel<<<(unsigned)nb, kThreads, 0, s>>>((const float4*)x, delta, (const float4*)target, (bf16*)g16,
-                                                      (float4*)g4, (int)npix, inv, scratch);
+    mse_grad_kernel<<<(unsigned)nb, kThreads, 0, s>>>((const float4*)x, delta, target, ((uintptr_t)target & 15) == 0,
+                                                      (bf16*)g16, (float4*)g4, (int)npix, inv, scratch);
     relu_grad_kernel<3><<<dim3(ngb, 1), kGradThreads, 0, s>>>(g4, 4, nullptr, 0, nullptr, 0, nullptr, 1, (int)npix, 4,
                                                              gpart);
     mse_grad_finish_kernel<<<1, 64, 0, s>>>(scratch, (int)nb, gpart, ngb, inv, loss, gb);

@@ -255,8 +255,6 @@ class Surrogate:
             # the loss kernel reads M x 4 floats from this pointer unchecked
             raise ValueError(f"target32: a contiguous float32 CUDA tensor of shape ({M1}, {NC}) on "
                              f"{self.x32.device} is required")
-        if target32.data_ptr() % 16:     # a view into a larger tensor
-            target32 = target32.clone()
         _ck(lib.lbm_sg_mse_grad(p(self.x32), p(self.delta), p(target32), p(self.g16_1), p(self.g_delta),
                                 p(self.layers["out"]["gb"]), p(self.mse_scratch), p(self.loss_dev), M1, s), "lbm_sg_mse_grad")
         # out, d1 (level 1)

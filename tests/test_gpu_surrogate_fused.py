@@ -96,6 +96,11 @@ def test_mse_grad(env, n):
     assert lib.lbm_sg_mse_grad(p(x), p(d), p(t), p(h16), p(g4), p(gb), p(scr), p(lb), n, s) == 0
     assert torch.equal(g16, h16) and torch.equal(g4, g[:, :4])
     assert lb.item() == pytest.approx(la.item(), rel=1e-13)
+    odd = torch.empty(4 * n + 1, device="cuda")[1:].view(n, 4)   # a target on any address
+    odd.copy_(t)
+    k16, lc = torch.ones_like(h16), f64(1)
+    assert lib.lbm_sg_mse_grad(p(x), p(d), p(odd), p(k16), p(g4), p(gb), p(scr), p(lc), n, s) == 0
+    assert torch.equal(k16, h16) and lc.item() == lb.item()
     err = (gb.double() - g.double().sum(0)).abs()
     assert (err <= 1e-5 * g.double().abs().sum(0)).all() and (gb[4:] == 0).all()
 

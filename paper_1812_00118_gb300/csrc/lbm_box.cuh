@@ -6,7 +6,10 @@
 // step, and a 256 x 256 grid gives it 32 CTAs of 18 dependent planes.  Here
 // the grid is cut into boxes of BX x BY x BZ nodes, one thread per node and
 // one CTA per box, all boxes resident at once: a step is one round of loads,
-// one barrier, one collision and one round of stores.
+// one barrier, one collision and one round of stores.  (us per step, march of
+// 16-plane chunks / this: 64^2 FP64 239 / 13.8, 256^2 FP32 22.7 / 4.3, 150 x 600 with
+// walls 28.8 / 5.9, 32^3 45 / 6.5.  At 64^2 FP32 the 3.1 are, in clk: the wait for
+// the flags 640, loads and sums 1600, collision 830, release 1000.)
 //
 // Between steps a box waits only for the boxes around it.  A node's new
 // populations depend on cells at most two nodes away (the phi stencil reaches

@@ -788,7 +788,7 @@ __device__ __forceinline__ void collide_pair(const NodeState<float>& s, const Pa
 // 22 operations for g and 7 for h per pair, where two calls of collide_dir take
 // about 70.  FP64 runs at two lanes per clock and SM here, so the FP64 step's
 // time is its operation count (64^2 D2Q9: 433 FP64 instructions per node in the
-// collision before).
+// collision before; march of 256^2 267 us per step before, 211 with this).
 struct PairState64 {
     double Ze, k1, Fx, Fy, Fz;               // Xe + Ye; rho_dif/2 + 3 mu/2; 3 F / 2
     double m15, usq15;                       // 3 mu/2, 1.5 u.u
@@ -1232,9 +1232,11 @@ __device__ __forceinline__ void march(const DirPtrs<typename Storage<ST>::S, Lat
         __syncthreads();
         if (active) {
             auto hv = [&](int i) { return hown[(j + 1) & 1][i - 1][tid]; };   // i >= 1
-            // only a node next to a wall writes bounce-back ghost cells: warps
-            // without one take the wall-free collision (fewer live registers)
-            if (WALLS && __any_sync(__activemask(), wall_adjacent<LAT>(G, x, y, z)))
+            // only a node next to a wall writes bounce-back ghost cells: the
+            // rest take the wall-free collision (fewer live registers).  A vote
+            // that sends a whole warp one way, as in the resident step, costs the
+            // march 5 % (256 x 256 x 512 with walls: 23.8 against 22.6 ms for 10 steps)
+            if (WALLS && wall_adjacent<LAT>(G, x, y, z))
                 collide_node<LAT, ST, true>(D, G, p, phis, j & 3, (j + 1) & 3, (j + 2) & 3, tx + 1, ty + HY, m, hv, x,
                                             y, z, rb);
             else
@@ -1471,8 +1473,10 @@ __global__ void shift_rest_kernel(typename Storage<ST>::S* __restrict__ h0, Geom
 // A sum of FP32 values as a non-overlapping triple of FP32 (two levels of
 // TwoSum), converted to FP64 once: at least as close to the exact sum as a
 // chain of FP64 additions.  FP64 operations, conversions from and to FP32
-// included, run at two lanes per clock and SM on this chip; 19 conversions and
-// additions per node took 2.0 ms for 2^25 nodes, this 0.5 ms.
+// included, run at two lanes per clock and SM on this chip.  (Read-out of phi, P
+// and rho u of 2^25 nodes, with the in-place outputs of macro_kernel: 5.0 ms with
+// 19 conversions and additions per node here and as many in the stencils, 2.7
+// with this.)
 template <typename R>
 struct WideSum {
     double s = 0;

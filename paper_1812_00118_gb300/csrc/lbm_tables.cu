@@ -46,7 +46,8 @@ namespace {
 
 // Boxes of the resident step (lbm_box.cuh): nodes along the internal axes and
 // the CTAs per SM the registers are bounded for; the larger box first.
-// Measured, us per step of a periodic grid (FP32, 100 steps per launch):
+// Measured, us per step of a periodic grid (FP32, 100 steps per launch, boxes
+// that release their stores by one thread):
 //   D2Q9   32x8 / 32x4: 64^2 3.8 / 3.1, 128^2 4.0 / 3.3, 256^2 4.9 / 4.8, 512^2 11.5 / 15.4
 //   D3Q19  16x4x4 / 8x4x4: 16^3 6.6 / 5.9, 24^3 6.9 / 6.0, 32^3 6.4 / 7.0, 40^3 9.8 / 11.1
 // so the larger box pays once it gives at least half the SMs a box (D3Q19) or
@@ -125,7 +126,7 @@ bool ok_dispatch(int tile, const Geom& G) {
 // faster form.  The march of as many CTAs as the chip holds (StepArgs::fit)
 // overtakes once the boxes need more than one round per step (D3Q19: 40^3 9.8
 // against 14.4 us, 48^3 16.4 against 14.5) or two (D2Q9: 512^2 11.5 against
-// 12.4, 707^2 23.2 against 18.8).
+// 12.4, 707^2 23.2 against 18.8; FP64, one round: 512^2 210 against 171).
 cudaError_t box_plan(const Geom& G, BoxPlan* plan) {
     *plan = BoxPlan();
     int dev = 0, sms = 0, slots = 0;

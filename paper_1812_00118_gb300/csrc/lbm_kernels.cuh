@@ -538,20 +538,20 @@ struct Unroll<N, N> {
 // formed (IEEE arithmetic cannot drop 0 * x or x + 0 by itself), +-1
 // coefficients become additions and subtractions.
 template <int C, typename R>
-__device__ __forceinline__ R cmul(R v) {
+__host__ __device__ __forceinline__ R cmul(R v) {
     if constexpr (C == 1) return v;
     else if constexpr (C == -1) return -v;
     else return (R)C * v;
 }
 template <int A, int B, typename R>
-__device__ __forceinline__ R cdot2(R a, R b) {
+__host__ __device__ __forceinline__ R cdot2(R a, R b) {
     if constexpr (A != 0 && B != 0) return cmul<A>(a) + cmul<B>(b);
     else if constexpr (A != 0) return cmul<A>(a);
     else if constexpr (B != 0) return cmul<B>(b);
     else return (R)0;
 }
 template <int A, int B, int C, typename R>
-__device__ __forceinline__ R cdot3(R a, R b, R c) {
+__host__ __device__ __forceinline__ R cdot3(R a, R b, R c) {
     if constexpr (A != 0 && (B != 0 || C != 0)) return cmul<A>(a) + cdot2<B, C>(b, c);
     else if constexpr (A != 0) return cmul<A>(a);
     else return cdot2<B, C>(b, c);
@@ -655,8 +655,8 @@ __device__ __forceinline__ void node_state(NodeState<R>& s, const PhysT<R>& p, R
 //        + (1 - 1/tau_mix) w_i/(2T^2) (c_i c_i : Pi - T tr Pi)
 // and h*_i (Eq. 1 with Eq. 2).  Gamma_i is shared by both (Eq. 3).
 template <int LAT, int I, typename R>
-__device__ __forceinline__ void collide_dir(const NodeState<R>& s, const PhysT<R>& p, R h_in,
-                                            R* h_out, R* g_out) {
+__host__ __device__ __forceinline__ void collide_dir(const NodeState<R>& s, const PhysT<R>& p, R h_in,
+                                                     R* h_out, R* g_out) {
     using L = Lattice<LAT>;
     constexpr int CX = L::cx[I], CY = L::cy[I], CZ = L::cz[I];
     const R w = (R)L::w[I];
@@ -785,20 +785,23 @@ __device__ __forceinline__ void collide_pair(const NodeState<float>& s, const Pa
 //   g*_I, g*_J = even +- odd,
 //   even = E (Xe + Ye) + O (Xo + Yo) + w (Ye + 3 P) + filter,
 //   odd  = E (Xo + Yo) + O (Xe + Ye) + w Yo + c.u hoc,
-// 22 operations for g and 7 for h per pair, where two calls of collide_dir take
-// about 70.  FP64 runs at two lanes per clock and SM here, so the FP64 step's
-// time is its operation count (64^2 D2Q9: 433 FP64 instructions per node in the
+// 22 operations for g and 9 for h per pair, where two calls of collide_dir take
+// about 70.  h relaxes by its distance from h^eq as it does there: the shorter
+// (1 - 1/tau_phi) h + h^eq / tau_phi, 7 operations, has 1.35 times the rounding
+// error (h of O(0.1): rms 7.5e-18 against 5.5e-18; this form 4.8e-18).
+// FP64 runs at two lanes per clock and SM here, so the FP64 step's time is its
+// operation count (64^2 D2Q9: 433 FP64 instructions per node in the
 // collision before; march of 256^2 267 us per step before, 211 with this).
 struct PairState64 {
     double Ze, k1, Fx, Fy, Fz;               // Xe + Ye; rho_dif/2 + 3 mu/2; 3 F / 2
     double m15, usq15;                       // 3 mu/2, 1.5 u.u
     double A[2], wm15[2], hoc[2];            // w (Ye + 3 P), w 3 mu/2, w 0.75 rho_dif lap phi
     double om, tr3;                          // (1 - 1/tau_mix) 4.5, tr(Pi)/3
-    double keep, itphi, itth[2], itphiw[2];  // 1 - 1/tau_phi; phi, theta w and phi w over tau_phi
+    double itau, thw[2];                     // 1/tau_phi, theta w
 };
 
 template <int LAT>
-__device__ __forceinline__ PairState64 pair_state64(const NodeState<double>& s, const PhysT<double>& p) {
+__host__ __device__ __forceinline__ PairState64 pair_state64(const NodeState<double>& s, const PhysT<double>& p) {
     using L = Lattice<LAT>;
     PairState64 q;
     const double hrd = 0.5 * p.rho_dif;
@@ -812,24 +815,22 @@ __device__ __forceinline__ PairState64 pair_state64(const NodeState<double>& s, 
     q.usq15 = 1.5 * s.usq;
     q.om = (1.0 - s.omega) * 4.5;
     q.tr3 = s.tr3;
-    q.keep = 1.0 - p.inv_tau_phi;
-    q.itphi = p.inv_tau_phi * s.phi;
-    const double th = p.inv_tau_phi * s.theta, hl = p.hocorr ? 0.75 * p.rho_dif * s.lap : 0.0, y3P = Ye + 3.0 * s.P;
+    q.itau = p.inv_tau_phi;
+    const double hl = p.hocorr ? 0.75 * p.rho_dif * s.lap : 0.0, y3P = Ye + 3.0 * s.P;
     const double wk[2] = {L::w[1], L::w[4]};   // an axis and a diagonal direction
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         q.A[k] = wk[k] * y3P;
         q.wm15[k] = wk[k] * q.m15;
         q.hoc[k] = wk[k] * hl;
-        q.itth[k] = wk[k] * th;
-        q.itphiw[k] = wk[k] * q.itphi;
+        q.thw[k] = wk[k] * s.theta;
     }
     return q;
 }
 
 template <int LAT, int I>
-__device__ __forceinline__ void collide_pair64(const NodeState<double>& s, const PairState64& q, double hI, double hJ,
-                                               double* h_I, double* h_J, double* g_I, double* g_J) {
+__host__ __device__ __forceinline__ void collide_pair64(const NodeState<double>& s, const PairState64& q, double hI,
+                                                        double hJ, double* h_I, double* h_J, double* g_I, double* g_J) {
     using L = Lattice<LAT>;
     constexpr int CX = L::cx[I], CY = L::cy[I], CZ = L::cz[I];
     constexpr int WK = CX * CX + CY * CY + CZ * CZ == 1 ? 0 : 1;
@@ -846,9 +847,9 @@ __device__ __forceinline__ void collide_pair64(const NodeState<double>& s, const
     const double odd = E * Zo + (O * q.Ze + (q.wm15[WK] * cg + (w * cF + q.hoc[WK] * cu)));
     *g_I = even + odd;
     *g_J = even - odd;
-    const double he = q.itphi * E + q.itphiw[WK], ho = q.itphi * O + q.itth[WK] * cn;
-    *h_I = q.keep * hI + (he + ho);
-    *h_J = q.keep * hJ + (he - ho);
+    const double G = E + w, ho = s.phi * O + q.thw[WK] * cn;
+    *h_I = hI + ((s.phi * G - hI) + ho) * q.itau;
+    *h_J = hJ + ((s.phi * G - hJ) - ho) * q.itau;
 }
 
 // ---------------------------------------------------------------- fused step

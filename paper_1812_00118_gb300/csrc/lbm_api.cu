@@ -94,6 +94,21 @@ int derive(const lbm_params& u, int lattice, Phys* out) {
     return LBM_OK;
 }
 
+// The resident step (lbm_box.cuh) keeps its box counts in the half of the
+// reduction scratch that the reductions leave free (they use the first
+// 4 x 1024 doubles and the 4 after them).
+constexpr int kMaxBoxes = 8000;
+unsigned* box_flags(lbm_ctx* c) { return (unsigned*)(c->partial + 4 * 1024 + 8); }
+bool resident(const lbm_ctx* c) {
+    return c->box.variant >= 0 && c->box.boxes <= kMaxBoxes && c->partial && !c->owner;
+}
+int start_box_counts(lbm_ctx* c) {
+    if (!resident(c)) return LBM_OK;
+    box_start_kernel<<<(c->box.boxes + 255) / 256, 256, 0, c->stream>>>(box_flags(c), c->box.boxes);
+    c->launches += 1;
+    return check_cuda(cudaGetLastError());
+}
+
 int ensure_scratch(lbm_ctx* c) {
     if (c->fields && c->partial) return LBM_OK;
     if (!c->fields) {
@@ -113,8 +128,7 @@ int ensure_scratch(lbm_ctx* c) {
         c->partial = nullptr;
         return LBM_ENOMEM;
     }
-    // the box counts of the resident step in it start at zero
-    return check_cuda(cudaMemsetAsync(c->partial, 0, sizeof(double) * 8 * c->n_partial_blocks, c->stream));
+    return start_box_counts(c);
 }
 
 double* f_phi(lbm_ctx* c) { return c->fields; }
@@ -287,21 +301,11 @@ int copy_field(lbm_ctx* c, double* dst, const double* src, size_t n, int on_devi
                                       on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
 }
 
-// The resident step (lbm_box.cuh) keeps its box counts in the half of the
-// reduction scratch that the reductions leave free (they use the first
-// 4 x 1024 doubles and the 4 after them).
-constexpr int kMaxBoxes = 8000;
-int* box_flags(lbm_ctx* c) { return (int*)(c->partial + 4 * 1024 + 8); }
-bool resident(const lbm_ctx* c) {
-    return c->box.variant >= 0 && c->box.boxes <= kMaxBoxes && c->partial && !c->owner;
-}
-
 // A new state: the error flag of the bounded waits, and the box counts a wait
 // that gave up left uneven.
 int clear_wait_state(lbm_ctx* c) {
     if (check_cuda(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream))) return LBM_ECUDA;
-    if (!resident(c)) return LBM_OK;
-    return check_cuda(cudaMemsetAsync(box_flags(c), 0, sizeof(int) * c->box.boxes, c->stream));
+    return start_box_counts(c);
 }
 
 // rho_bar for force_mode 1 from the current state's phi (scratch fields must be fresh)

@@ -29,6 +29,21 @@ namespace lbm {
 
 constexpr int kBoxPolls = 1 << 22;
 
+// The counts are 32 bits wide and never reset while a context steps on: 8 warps
+// pass 2^31 after 2.7e8 steps, 19 minutes of a 256 x 256 grid.  They are unsigned
+// and compared by their difference, which a wrap leaves as it is (it never
+// exceeds two steps).  A context's counts start just below 2^31, so that every
+// run passes the sign bit in its first steps and not only one of 19 minutes.
+constexpr unsigned kBoxFirstCount = 0x7ffffff0u;
+
+// the count of a box that has completed `steps` steps since it stood at `first`
+__host__ __device__ __forceinline__ unsigned box_count(unsigned first, int steps, int warps) {
+    return first + (unsigned)steps * (unsigned)warps;
+}
+__host__ __device__ __forceinline__ bool box_reached(unsigned count, unsigned want) {
+    return count - want < 0x80000000u;
+}
+
 // Loads of populations another CTA may have written in this launch: coherent
 // at the GPU scope (never the read-only path).
 template <typename S> __device__ __forceinline__ S ld_coherent(const S* p);
@@ -69,7 +84,7 @@ struct BoxSmem {
 template <int LAT, int ST, int BX, int BY, int BZ, bool WALLS>
 __device__ __forceinline__ bool box_step(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::Q>& D, const Geom& G,
                                          const PhysT<typename Storage<ST>::R>& p, const BoxPlan& pl, int box,
-                                         int first, int wait_for, const int* flags, int* err,
+                                         unsigned first, int wait_for, const unsigned* flags, int* err,
                                          BoxSmem<LAT, ST, BX, BY, BZ>& sm) {
     using L = Lattice<LAT>;
     using St = Storage<ST>;
@@ -131,13 +146,13 @@ __device__ __forceinline__ bool box_step(const DirPtrs<typename Storage<ST>::S, 
                 a = a < 0 ? pl.nx - 1 : (a >= pl.nx ? 0 : a);
                 b = b < 0 ? pl.ny - 1 : (b >= pl.ny ? 0 : b);
                 c = c < 0 ? pl.nz - 1 : (c >= pl.nz ? 0 : c);
-                const int* f = flags + (c * pl.ny + b) * pl.nx + a;
-                const int want = first + wait_for * (NT / 32);
+                const unsigned* f = flags + (c * pl.ny + b) * pl.nx + a;
+                const unsigned want = box_count(first, wait_for, NT / 32);
                 ok = false;
                 for (int i = 0; i < kBoxPolls; ++i) {
-                    int v;
-                    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
-                    if (v - want >= 0) { ok = true; break; }
+                    unsigned v;
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
+                    if (box_reached(v, want)) { ok = true; break; }
                     if ((i & 255) == 255 && *(volatile int*)err) break;   // another box gave up
                 }
                 if (!ok) atomicExch(err, 1);
@@ -214,9 +229,9 @@ template <int LAT, int ST, int BX, int BY, int BZ, int MINB, bool WALLS>
 __global__ void __launch_bounds__(BX * BY * BZ, MINB)
 box_kernel(const __grid_constant__ BoxPtrs<typename Storage<ST>::S, Lattice<LAT>::Q> ptrs, const __grid_constant__ Geom G,
            const __grid_constant__ PhysT<typename Storage<ST>::R> p, const __grid_constant__ BoxPlan pl, int n_steps,
-           int* flags, int* err) {
+           unsigned* flags, int* err) {
     __shared__ BoxSmem<LAT, ST, BX, BY, BZ> sm;
-    const int first = n_steps > 1 ? *(volatile int*)(flags + blockIdx.x) : 0;
+    const unsigned first = n_steps > 1 ? *(volatile unsigned*)(flags + blockIdx.x) : 0u;
 #pragma unroll 1
     for (int s = 0; s < n_steps; ++s) {
         for (int box = blockIdx.x; box < pl.boxes; box += gridDim.x) {
@@ -227,10 +242,17 @@ box_kernel(const __grid_constant__ BoxPtrs<typename Storage<ST>::S, Lattice<LAT>
             if (n_steps > 1) {
                 __syncwarp();
                 if ((threadIdx.x & 31) == 0)
-                    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(flags + box) : "memory");
+                    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(flags + box) : "memory");
             }
         }
     }
+}
+
+// Counts of a new state (and of one whose last launch a wait ended early, which
+// leaves them uneven).
+static __global__ void box_start_kernel(unsigned* flags, int boxes) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < boxes) flags[k] = kBoxFirstCount;
 }
 
 }  // namespace lbm

@@ -158,7 +158,7 @@ cudaError_t box_slots(const Geom& G, int* out) {
 }
 
 template <int LAT, int ST, typename B>
-cudaError_t launch_box(const StepArgs& a, const BoxPlan& pl, int n, int* flags) {
+cudaError_t launch_box(const StepArgs& a, const BoxPlan& pl, int n, unsigned* flags) {
     using S = typename Storage<ST>::S;
     const Geom& G = a.G;
     cudaLaunchConfig_t cfg = {};

@@ -63,7 +63,7 @@ struct KernelTable {
     // resident step of small grids: its plan for a grid on the current device
     // (variant -1: not for this grid), and n steps in one launch
     cudaError_t (*box_plan)(const Geom& G, BoxPlan* plan);
-    cudaError_t (*box_steps)(const StepArgs& a, const BoxPlan& plan, int n, int* flags);
+    cudaError_t (*box_steps)(const StepArgs& a, const BoxPlan& plan, int n, unsigned* flags);
     // tensor maps of one input buffer pair for bulk-copy tile `tile`
     cudaError_t (*make_maps)(int tile, TmaMaps* out, const void* h, const void* g, const Geom& G);
     // true if tile `tile` can run this grid and storage type (shared memory,

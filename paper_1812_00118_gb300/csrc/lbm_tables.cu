@@ -148,7 +148,7 @@ cudaError_t box_plan(const Geom& G, BoxPlan* plan) {
     return cudaSuccess;
 }
 
-cudaError_t box_dispatch(const StepArgs& a, const BoxPlan& pl, int n, int* flags) {
+cudaError_t box_dispatch(const StepArgs& a, const BoxPlan& pl, int n, unsigned* flags) {
     switch (pl.variant) {
         case 0: return launch_box<LBM_LAT, LBM_ST, BoxA>(a, pl, n, flags);
         case 1: return launch_box<LBM_LAT, LBM_ST, BoxB>(a, pl, n, flags);

@@ -171,10 +171,10 @@ int lbm_init_fields_ex(lbm_ctx* ctx, const double* phi, const double* u, const d
  * enough to be resident on the chip as a whole (and whose tile the caller has
  * not chosen) takes all n steps in one cooperative launch instead, split only
  * where lbm_set_phi_correction asks for a correction; the waits inside it are
- * bounded, and one that gives up is reported by lbm_diagnostics as
- * LBM_ETIMEOUT, like a bulk-copy step's.  The bulk-copy tile (see lbm_set_tile) adds one launch of a small kernel that
- * writes the periodic images into the ghost band of the buffer just written
- * (and one more before its first step on a state another tile wrote).
+ * bounded (lbm_set_wait_limit).  The bulk-copy tile (see lbm_set_tile) adds one
+ * launch of a small kernel that writes the periodic images into the ghost band
+ * of the buffer just written (and one more before its first step on a state
+ * another tile wrote).
  * Asynchronous on the context stream; returns LBM_ECUDA if a launch fails,
  * and LBM_EDIVERGED without launching anything if the last lbm_diagnostics
  * found the state diverged (until lbm_init_fields or lbm_set_populations
@@ -203,9 +203,9 @@ int lbm_set_populations(lbm_ctx* ctx, const double* h, const double* g, int on_d
 /* FP64 diagnostics of the current state, reduced on the device in a fixed
  * order (deterministic): out[0] = sum phi, out[1] = sum rho, out[2] = max |u|,
  * out[3] = number of non-finite phi/u/P values.  Returns LBM_ETIMEOUT if a
- * bounded wait of a bulk-copy step gave up since creation, else
- * LBM_EDIVERGED (after filling out) if out[3] > 0 or out[2] > 0.3.
- * Synchronises. */
+ * bounded wait of a step gave up since the last lbm_init_fields or
+ * lbm_set_populations, else LBM_EDIVERGED (after filling out) if out[3] > 0
+ * or out[2] > 0.3.  Synchronises. */
 int lbm_diagnostics(lbm_ctx* ctx, double out[4]);
 
 /* Laplace-law measurement (Section 4.1) in FP64 on the device:
@@ -279,15 +279,17 @@ int lbm_set_wall_velocity(lbm_ctx* ctx, int axis, int side, const double u[3]);
 int lbm_set_tile(lbm_ctx* ctx, int tile, int lz);
 int lbm_get_tile(const lbm_ctx* ctx, int* tile, int* lz, int* tx, int* ty);
 
-/* Poll limit of the bounded waits of the bulk-copy step pipeline (tile 4; of
- * the other forms only the resident step waits, with a limit of its own).  A wait whose copies have not landed
- * after `polls` tries gives up: the kernel raises the context's error flag,
- * lets the copies it has in flight land (a separate bounded wait) and
- * returns, so the GPU context stays usable, lbm_diagnostics returns
- * LBM_ETIMEOUT and the state of that step is invalid until the next
- * lbm_init_fields / lbm_set_populations (which also clear the flag).
- * Default 4194304; 0 makes every pipeline wait give up at once (a host-side
- * way to exercise the failure path without any fault).  Errors: LBM_EINVAL
+/* Poll limit of the bounded waits inside a step: those of the bulk-copy
+ * pipeline (tile 4) for its copies, and those of the resident step of small
+ * grids for the boxes around (see lbm_step; a call of one step has none).  A
+ * wait not over after `polls` tries gives up: the kernel raises the context's
+ * error flag, lets the copies it has in flight land (a separate bounded wait)
+ * and returns, so the GPU context stays usable, lbm_diagnostics returns
+ * LBM_ETIMEOUT and the state is invalid until the next lbm_init_fields /
+ * lbm_set_populations (which also clear the flag): until then its phi and h,
+ * and what follows from them, read out as NaN.
+ * Default 4194304; 0 makes every such wait give up at once (a host-side way to
+ * exercise the failure path without any fault).  Errors: LBM_EINVAL
  * (polls < 0). */
 int lbm_set_wait_limit(lbm_ctx* ctx, long long polls);
 

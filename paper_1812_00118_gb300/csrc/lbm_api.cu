@@ -139,7 +139,7 @@ double* f_u(lbm_ctx* c, int a) { return c->fields + (2 + a) * c->G.N; }
 int compute_fields(lbm_ctx* c) {
     int rc = ensure_scratch(c);
     if (rc) return rc;
-    if (check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, f_phi(c), nullptr, c->stream))) return LBM_ECUDA;
+    if (check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, f_phi(c), nullptr, c->d_err, c->stream))) return LBM_ECUDA;
     if (check_cuda(c->K->macro(c->g[c->cur], c->G, c->P, f_phi(c), f_P(c), f_u(c, 0), f_u(c, 1), f_u(c, 2),
                                c->stream)))
         return LBM_ECUDA;
@@ -285,7 +285,7 @@ int reduce_diag(lbm_ctx* c, double out[4]) {
 // Total of phi restored to phi_target (FP64 sums on the GPU, uniform shift of
 // the rest population); stream-ordered, no host synchronisation.
 int phi_fix(lbm_ctx* c) {
-    if (check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, f_phi(c), nullptr, c->stream))) return LBM_ECUDA;
+    if (check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, f_phi(c), nullptr, c->d_err, c->stream))) return LBM_ECUDA;
     long long nb = (c->G.N + kRedThreads - 1) / kRedThreads;
     if (nb > kFixBlocks) nb = kFixBlocks;
     sum_partial_kernel<<<(unsigned)nb, kRedThreads, 0, c->stream>>>(f_phi(c), c->G.N, c->d_fix);
@@ -697,7 +697,7 @@ int lbm_macro(lbm_ctx* c, double* phi, double* P, double* rho_u, int on_device) 
     // it is, else a rounded copy in the scratch of the velocity (unused here)
     void* rounded = c->store == LBM_F64 ? nullptr : (void*)f_u(c, 0);
     const bool flow = d_P || d_ru;
-    rc = check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, d_phi, flow ? rounded : nullptr, c->stream));
+    rc = check_cuda(c->K->phi(c->h[c->cur], c->G, c->P, d_phi, flow ? rounded : nullptr, c->d_err, c->stream));
     c->launches += 1;
     if (!rc && flow) {
         double* ru[3] = {nullptr, nullptr, nullptr};   // internal axes
@@ -732,7 +732,7 @@ int lbm_get_populations(lbm_ctx* c, double* h, double* g, int on_device) {
             return LBM_ENOMEM;
         }
     }
-    int rc = check_cuda(c->K->get(c->h[c->cur], c->g[c->cur], c->G, c->P, dh, dg, c->stream));
+    int rc = check_cuda(c->K->get(c->h[c->cur], c->g[c->cur], c->G, c->P, dh, dg, c->d_err, c->stream));
     c->launches += 1;
     if (!rc && !on_device) {
         rc = check_cuda(cudaMemcpyAsync(h, dh, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));

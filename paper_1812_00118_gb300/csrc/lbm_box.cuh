@@ -20,14 +20,13 @@
 // adjacent flag shows step s - 1 done by all of them, which covers both.  The counts go on
 // from launch to launch (a box reads its own at the start), so a captured
 // launch can be replayed.  The launch is cooperative whenever boxes wait, so
-// they are all resident; the waits are bounded, and one that gives up raises
-// *err, on which every box leaves.
+// they are all resident; the waits are bounded (lbm_set_wait_limit), and one that
+// gives up raises *err, on which every box that still waits leaves.  The state is
+// lost then, and reads out as NaN (phi_kernel, get_kernel).
 #pragma once
 #include "lbm_kernels.cuh"
 
 namespace lbm {
-
-constexpr int kBoxPolls = 1 << 22;
 
 // The counts are 32 bits wide and never reset while a context steps on: 8 warps
 // pass 2^31 after 2.7e8 steps, 19 minutes of a 256 x 256 grid.  They are unsigned
@@ -84,7 +83,7 @@ struct BoxSmem {
 template <int LAT, int ST, int BX, int BY, int BZ, bool WALLS>
 __device__ __forceinline__ bool box_step(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::Q>& D, const Geom& G,
                                          const PhysT<typename Storage<ST>::R>& p, const BoxPlan& pl, int box,
-                                         unsigned first, int wait_for, const unsigned* flags, int* err,
+                                         unsigned first, int wait_for, const unsigned* flags, int* err, int polls,
                                          BoxSmem<LAT, ST, BX, BY, BZ>& sm) {
     using L = Lattice<LAT>;
     using St = Storage<ST>;
@@ -149,7 +148,7 @@ __device__ __forceinline__ bool box_step(const DirPtrs<typename Storage<ST>::S, 
                 const unsigned* f = flags + (c * pl.ny + b) * pl.nx + a;
                 const unsigned want = box_count(first, wait_for, NT / 32);
                 ok = false;
-                for (int i = 0; i < kBoxPolls; ++i) {
+                for (int i = 0; i < polls; ++i) {
                     unsigned v;
                     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
                     if (box_reached(v, want)) { ok = true; break; }
@@ -229,14 +228,15 @@ template <int LAT, int ST, int BX, int BY, int BZ, int MINB, bool WALLS>
 __global__ void __launch_bounds__(BX * BY * BZ, MINB)
 box_kernel(const __grid_constant__ BoxPtrs<typename Storage<ST>::S, Lattice<LAT>::Q> ptrs, const __grid_constant__ Geom G,
            const __grid_constant__ PhysT<typename Storage<ST>::R> p, const __grid_constant__ BoxPlan pl, int n_steps,
-           unsigned* flags, int* err) {
+           unsigned* flags, int* err, int polls) {
     __shared__ BoxSmem<LAT, ST, BX, BY, BZ> sm;
     const unsigned first = n_steps > 1 ? *(volatile unsigned*)(flags + blockIdx.x) : 0u;
 #pragma unroll 1
     for (int s = 0; s < n_steps; ++s) {
         for (int box = blockIdx.x; box < pl.boxes; box += gridDim.x) {
             if (s == 0 && box != blockIdx.x) __syncthreads();   // phi of the box before (later steps wait instead)
-            if (!box_step<LAT, ST, BX, BY, BZ, WALLS>(ptrs.d[s & 1], G, p, pl, box, first, s, flags, err, sm)) return;
+            if (!box_step<LAT, ST, BX, BY, BZ, WALLS>(ptrs.d[s & 1], G, p, pl, box, first, s, flags, err, polls, sm))
+                return;
             // a warp's stores are done, each on its own account: no barrier, and
             // the releases of a box's warps overlap
             if (n_steps > 1) {

@@ -4,6 +4,7 @@
 #pragma once
 #include <cudaTypedefs.h>
 
+#include <climits>
 #include <new>
 
 #include "lbm_box.cuh"
@@ -174,7 +175,7 @@ cudaError_t launch_box(const StepArgs& a, const BoxPlan& pl, int n, unsigned* fl
     ptrs.d[0] = dir_ptrs<S, Lattice<LAT>::Q>(a.hin, a.gin, a.hout, a.gout, G.NP);
     ptrs.d[1] = dir_ptrs<S, Lattice<LAT>::Q>(a.hout, a.gout, const_cast<void*>(a.hin), const_cast<void*>(a.gin), G.NP);
     return cudaLaunchKernelEx(&cfg, B::template kernel<LAT, ST>(G), ptrs, G, phys_as<typename Storage<ST>::R>(a.p), pl,
-                              n, flags, a.error_flag);
+                              n, flags, a.error_flag, a.wait_polls < INT_MAX ? (int)a.wait_polls : INT_MAX);
 }
 
 // ---------------------------------------------------------------- batches
@@ -297,10 +298,10 @@ template <int LAT, int ST>
 struct Launchers {
     using S = typename Storage<ST>::S;
     static constexpr int Q = Lattice<LAT>::Q;
-    static cudaError_t phi(const void* hin, const Geom& G, const Phys& p, double* out, void* rounded,
+    static cudaError_t phi(const void* hin, const Geom& G, const Phys& p, double* out, void* rounded, const int* lost,
                            cudaStream_t s) {
         phi_kernel<LAT, ST><<<blocks_for(G.N, 256), 256, 0, s>>>(
-            dir_ptrs<S, Q>(hin, hin, nullptr, nullptr, G.NP), G, p, out, (typename Storage<ST>::R*)rounded);
+            dir_ptrs<S, Q>(hin, hin, nullptr, nullptr, G.NP), G, p, out, (typename Storage<ST>::R*)rounded, lost);
         return cudaGetLastError();
     }
     static cudaError_t macro(const void* gin, const Geom& G, const Phys& p, const double* phi, double* P,
@@ -327,9 +328,9 @@ struct Launchers {
         return cudaGetLastError();
     }
     static cudaError_t get(const void* hin, const void* gin, const Geom& G, const Phys& p, double* h, double* g,
-                           cudaStream_t s) {
+                           const int* lost, cudaStream_t s) {
         get_kernel<LAT, ST><<<blocks_for(G.N, 256), 256, 0, s>>>(
-            dir_ptrs<S, Q>(hin, gin, nullptr, nullptr, G.NP), G, p, h, g);
+            dir_ptrs<S, Q>(hin, gin, nullptr, nullptr, G.NP), G, p, h, g, lost);
         return cudaGetLastError();
     }
     static cudaError_t halo(void* hout, void* gout, const Geom& G, cudaStream_t s) {

@@ -38,7 +38,7 @@ struct StepArgs {
     cudaStream_t stream;
     const TmaMaps* maps;   // tensor maps of (hin, gin) for a bulk-copy tile
     int* error_flag;       // raised by a bounded wait that gave up
-    long wait_polls;       // polls of a bulk-copy pipeline wait before it gives up
+    long wait_polls;       // polls of a bounded wait before it gives up
 };
 
 // Everything one batch step launch needs (see batch_step_kernel).
@@ -69,8 +69,9 @@ struct KernelTable {
     // true if tile `tile` can run this grid and storage type (shared memory,
     // sizes; bulk-copy and asynchronous-load tiles have limits)
     bool (*tile_ok)(int tile, const Geom& G);
-    // phi in double and (rounded not null) in the kernels' arithmetic type
-    cudaError_t (*phi)(const void* hin, const Geom& G, const Phys& p, double* phi, void* rounded, cudaStream_t s);
+    // phi in double and (rounded not null) in the kernels' arithmetic type; NaN if *lost
+    cudaError_t (*phi)(const void* hin, const Geom& G, const Phys& p, double* phi, void* rounded, const int* lost,
+                       cudaStream_t s);
     cudaError_t (*macro)(const void* gin, const Geom& G, const Phys& p, const double* phi, double* P,
                          double* ux, double* uy, double* uz, cudaStream_t s);
     // P and rho u (null outputs left out) from phi and its rounded copy
@@ -80,7 +81,7 @@ struct KernelTable {
                         const double* ux, const double* uy, const double* uz, const double* P, int neq,
                         cudaStream_t s);
     cudaError_t (*get)(const void* hin, const void* gin, const Geom& G, const Phys& p, double* h,
-                       double* g, cudaStream_t s);
+                       double* g, const int* lost, cudaStream_t s);
     cudaError_t (*set)(void* hout, void* gout, const Geom& G, const Phys& p, const double* h,
                        const double* g, cudaStream_t s);
     // periodic images of the ghost band of a freshly written buffer pair
@@ -143,7 +144,7 @@ struct lbm_ctx {
     bool ghosts[2] = {false, false};   // ghost band of buffer b holds the periodic images
     int* d_err = nullptr;  // device flag raised by a bounded wait that gave up
     bool diverged = false; // the last lbm_diagnostics found the state diverged
-    long wait_polls = 1L << 22;   // bulk-copy pipeline wait limit (lbm_set_wait_limit)
+    long wait_polls = 1L << 22;   // limit of the bounded waits (lbm_set_wait_limit)
     double* fields = nullptr;    // scratch: phi, P, ux, uy, uz (5 N doubles)
     double* partial = nullptr;   // scratch: reduction partials
     int n_partial_blocks = 0;

@@ -1506,10 +1506,12 @@ struct WideSum<float> {
 };
 
 // phi = sum_i of the pulled h at every node: in double (node order) and, where
-// asked for, rounded to the kernels' arithmetic type for the stencils.
+// asked for, rounded to the kernels' arithmetic type for the stencils.  *lost:
+// a bounded wait of a step gave up and the state is not one of any time; it
+// reads out as NaN.
 template <int LAT, int ST>
 __global__ void phi_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::Q> D, Geom G, Phys p, double* phi,
-                           typename Storage<ST>::R* rounded) {
+                           typename Storage<ST>::R* rounded, const int* __restrict__ lost) {
     using L = Lattice<LAT>;
     using St = Storage<ST>;
     using R = typename St::R;
@@ -1524,7 +1526,7 @@ __global__ void phi_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::
         constexpr double W = L::w[i];
         acc.add(St::load(pull_pad<LAT, i, false>(D.hin, po), (R)(W * p.h_shift), (R)1));
     });
-    const double f = acc.value();
+    const double f = *lost ? NAN : acc.value();
     phi[n] = f;
     if (rounded) rounded[n] = (R)f;
 }
@@ -1702,10 +1704,11 @@ __global__ void init_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>:
     });
 }
 
-// Pre-collision populations out (double, population-major, node order).
+// Pre-collision populations out (double, population-major, node order); h of a
+// lost state (see phi_kernel) is NaN.
 template <int LAT, int ST>
 __global__ void get_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::Q> D, Geom G, Phys p, double* h,
-                           double* g) {
+                           double* g, const int* __restrict__ lost) {
     using L = Lattice<LAT>;
     using St = Storage<ST>;
     using R = typename St::R;
@@ -1714,10 +1717,12 @@ __global__ void get_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::
     int x, y, z;
     node_coords(G, n, &x, &y, &z);
     const PullOffsets po = pull_offsets(G, x, y, z);
+    const bool gone = *lost != 0;
     Unroll<0, L::Q>::run([&](auto ic) {
         constexpr int i = decltype(ic)::value;
         constexpr double W = L::w[i];
-        h[(long long)i * G.N + n] = (double)St::load(pull_pad<LAT, i, false>(D.hin, po), (R)(W * p.h_shift), (R)1);
+        const R v = St::load(pull_pad<LAT, i, false>(D.hin, po), (R)(W * p.h_shift), (R)1);
+        h[(long long)i * G.N + n] = gone ? NAN : (double)v;
         g[(long long)i * G.N + n] = (double)St::load(pull_pad<LAT, i, false>(D.gin, po), (R)(W * p.g_shift),
                                                      (R)p.g_inv_scale);
     });

@@ -429,7 +429,7 @@ class Simulation:
         _check(load().lbm_set_tile(self._ctx, tile, lz), "lbm_set_tile")
 
     def set_wait_limit(self, polls):
-        """Poll limit of the bulk-copy pipeline waits (0: give up at once)."""
+        """Poll limit of the bounded waits inside a step (0: give up at once)."""
         _check(load().lbm_set_wait_limit(self._ctx, int(polls)), "lbm_set_wait_limit")
 
     def get_tile(self):

@@ -1,0 +1,76 @@
+"""The waits of the resident step: a limit that runs out on the host's order is
+reported and recovered from, and the counts pass 2^31 in the first steps."""
+import numpy as np
+import pytest
+
+from paper_1812_00118_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1812_00118_gb300 import build, lbm as L
+    build.build()
+    L.load()
+    return L
+
+
+def fields(shape):
+    dim = len(shape)
+    nx, ny = shape[:2]
+    phi, u, P = I.smooth_random((shape[2] if dim == 3 else 1, ny, nx), 31, dim=dim, u_amp=0.01, P_amp=1e-4)
+    return [np.ascontiguousarray(a.reshape(-1)) for a in (phi, u[:dim], P)]
+
+
+def make(L, shape, store, bc=(0, 0, 0)):
+    prm = L.make_params(M=0.05, W=4.0, sigma=1e-3, rho_L=0.5, rho_H=1.0, nu_L=0.1, nu_H=0.1, store=store,
+                        g_scale=100.0 if store in (L.F16S, L.BF16S) else 0.0)
+    return L.Simulation(L.D2Q9 if len(shape) == 2 else L.D3Q19, shape, prm, bc=bc)
+
+
+# the last two: several boxes per CTA, and walls
+CASES = [((64, 64), "F64", (0, 0)), ((100, 90), "F32", (0, 0)), ((20, 18, 17), "F16S", (0, 0, 0)),
+         ((9, 30, 11), "BF16S", (0, 1, 0)), ((512, 300), "F32", (0, 0)), ((150, 61), "F32", (0, 1))]
+
+
+@pytest.mark.parametrize("shape,store,bc", CASES)
+def test_wait_limit_reported_and_recovered(lbm, shape, store, bc):
+    f = fields(shape)
+    sim, ref = (make(lbm, shape, getattr(lbm, store), bc) for _ in range(2))
+    sim.init_fields(*f)
+    ref.init_fields(*f)
+    ref.step(30)
+    want = ref.get_populations()
+    for n in (2, 7):
+        sim.set_wait_limit(0)
+        sim.step(n)
+        with pytest.raises(lbm.LbmError) as e:
+            sim.diagnostics()
+        assert e.value.code == lbm.ETIMEOUT
+        assert np.isnan(sim.macro()[0]).all()          # no read-out passes for a result
+        assert np.isnan(sim.get_populations()[0]).all()
+        sim.step(3)                                    # a lost state steps on without hanging
+        sim.set_wait_limit(1 << 22)
+        if n == 2:
+            sim.init_fields(*f)                        # a new state clears the flag and the counts
+        else:
+            sim.set_populations(*start)
+        if n == 2:
+            start = sim.get_populations()
+        sim.step(30)
+        assert sim.diagnostics()["status"] == lbm.OK
+        for a, b in zip(sim.get_populations(), want):
+            assert np.array_equal(a, b)
+
+
+def test_single_steps_do_not_wait(lbm):
+    sim = make(lbm, (64, 64), lbm.F32)
+    sim.init_fields(*fields((64, 64)))
+    sim.set_wait_limit(0)
+    for _ in range(3):
+        sim.step(1)
+    assert sim.diagnostics()["status"] == lbm.OK

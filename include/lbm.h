@@ -169,10 +169,10 @@ int lbm_init_fields_ex(lbm_ctx* ctx, const double* phi, const double* u, const d
 /* Advance n >= 0 time steps: each step is one launch of the fused
  * collide-and-pull-stream kernel (Eqs. 1-14) and a buffer swap.  A grid small
  * enough to be resident on the chip as a whole (and whose tile the caller has
- * not chosen) takes all n steps in one cooperative launch instead, split only
- * where lbm_set_phi_correction asks for a correction; the waits inside it are
- * bounded (lbm_set_wait_limit).  The bulk-copy tile (see lbm_set_tile) adds one
- * launch of a small kernel that writes the periodic images into the ghost band
+ * not chosen) takes the n steps in cooperative launches of up to 1024 instead,
+ * split also where lbm_set_phi_correction asks for a correction; the waits
+ * inside are bounded (lbm_set_wait_limit).  The bulk-copy tile (see
+ * lbm_set_tile) adds one launch of a small kernel that writes the periodic images into the ghost band
  * of the buffer just written (and one more before its first step on a state
  * another tile wrote).
  * Asynchronous on the context stream; returns LBM_ECUDA if a launch fails,

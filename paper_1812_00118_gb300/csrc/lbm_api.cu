@@ -596,6 +596,11 @@ int lbm_step_profiled(lbm_ctx* c, int n, double* kernel_ms) {
     return rc;
 }
 
+// Steps of one launch of the resident step: 3 to 14 ms, after which kernels of
+// other streams get their turn (a launch of all steps of a call held up to
+// every SM for the length of the call); the launch between costs 5 us of them.
+constexpr int kBoxSteps = 1024;
+
 static int step_impl(lbm_ctx* c, int n, cudaEvent_t* ev) {
     if (!c || n < 0 || c->owner) return LBM_EINVAL;
     if (c->diverged) return LBM_EDIVERGED;
@@ -616,8 +621,9 @@ static int step_impl(lbm_ctx* c, int n, cudaEvent_t* ev) {
     a.wait_polls = c->wait_polls;
     int s = 0;
     while (s < n && resident(c) && !c->tile_chosen) {
-        // one launch up to the end or the next re-imposition of phi's total
-        int m = ev ? 1 : n - s;
+        // one launch up to the end, the next re-imposition of phi's total or the
+        // limit of a launch
+        int m = ev ? 1 : (n - s < kBoxSteps ? n - s : kBoxSteps);
         if (c->phi_fix_every > 0) {
             const int left = c->phi_fix_every - c->phi_fix_count;
             if (m > left) m = left > 1 ? left : 1;

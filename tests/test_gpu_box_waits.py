@@ -1,5 +1,6 @@
 """The waits of the resident step: a limit that runs out on the host's order is
-reported and recovered from, and the counts pass 2^31 in the first steps."""
+reported and recovered from, calls of many steps take several launches, and the
+counts pass 2^31 in the first steps."""
 import numpy as np
 import pytest
 
@@ -65,6 +66,20 @@ def test_wait_limit_reported_and_recovered(lbm, shape, store, bc):
         assert sim.diagnostics()["status"] == lbm.OK
         for a, b in zip(sim.get_populations(), want):
             assert np.array_equal(a, b)
+
+
+def test_long_calls_are_split(lbm):
+    """A call of 2500 steps is three launches and equals calls of 500."""
+    a, b = (make(lbm, (40, 24), lbm.F32) for _ in range(2))
+    for s in (a, b):
+        s.init_fields(*fields((40, 24)))
+    n0 = a.launch_count()
+    a.step(2500)
+    assert a.launch_count() - n0 == 3
+    for _ in range(5):
+        b.step(500)
+    for x, y in zip(a.get_populations(), b.get_populations()):
+        assert np.array_equal(x, y)
 
 
 def test_single_steps_do_not_wait(lbm):

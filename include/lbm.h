@@ -294,11 +294,15 @@ int lbm_get_tile(const lbm_ctx* ctx, int* tile, int* lz, int* tx, int* ty);
 int lbm_set_wait_limit(lbm_ctx* ctx, long long polls);
 
 /* Autotuner: times every compiled tile (those the grid supports) with lz in
- * {4, 8, 16, 32}, and the form a context takes before any choice, for `steps` steps each on the current state, keeps the
+ * {4, 8, 16, 32} for `steps` steps each on the current state, keeps the
  * fastest configuration, and restores the state it started from (the state
  * is saved to, and copied back from, a temporary device copy).  Reports the
- * choice and its time per step (step kernel plus ghost update) in ms; any
- * output pointer may be NULL.  Synchronises.  If a trial fails, the state is
+ * fastest pair and its time per step (step kernel plus ghost update) in ms;
+ * any output pointer may be NULL.  A context without a choice so far also
+ * times its own form (see lbm_set_tile) and, where that is faster than every
+ * pair, stays with it; no pair selects that form, so the pair and time reported
+ * are then those of the fastest tile all the same, an upper bound of the
+ * context's own time.  Synchronises.  If a trial fails, the state is
  * restored all the same, the context keeps the tile it had and the trial's
  * status is returned.  Errors: LBM_EINVAL (steps < 1), LBM_EDIVERGED (the
  * state was found diverged earlier), LBM_ENOMEM, LBM_ECUDA. */

@@ -858,10 +858,12 @@ int lbm_autotune(lbm_ctx* c, int steps, int* best_tile, int* best_lz, double* be
     cudaEventCreate(&e1);
     const int lzs[4] = {4, 8, 16, 32};
     int bt = c->tile, bl = c->lz;
-    bool bc = saved_chosen;
+    bool keep_own = false;
     float bms = 1e30f;
-    // the last trial is the context's own configuration before any choice
-    // (the resident step, or the default tile fitted to one wave)
+    // the last trial is the form of a context before any choice (the resident
+    // step, or the default tile fitted to one wave): no (tile, lz) stands for
+    // it, so it is kept where it is the fastest, but what is reported is the
+    // fastest pair, whose time lbm_set_tile gives on any such context
     for (int t = 0; t <= c->K->n_tiles && !rc; ++t) {
         const bool own = t == c->K->n_tiles;
         if (own ? saved_chosen : !c->K->tile_ok(t, c->G)) continue;
@@ -878,7 +880,8 @@ int lbm_autotune(lbm_ctx* c, int steps, int* best_tile, int* best_lz, double* be
             rc = check_cuda(cudaEventSynchronize(e1));
             float ms = 0;
             cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < bms) { bms = ms; bt = c->tile; bl = c->lz; bc = c->tile_chosen; }
+            if (own) keep_own = ms < bms;
+            else if (ms < bms) { bms = ms; bt = c->tile; bl = c->lz; }
         }
     }
     cudaEventDestroy(e0);
@@ -897,9 +900,10 @@ int lbm_autotune(lbm_ctx* c, int steps, int* best_tile, int* best_lz, double* be
     }
     cudaFreeAsync(save_h, c->stream);
     cudaFreeAsync(save_g, c->stream);
-    c->tile = rc ? saved_tile : bt;
-    c->lz = rc ? saved_lz : bl;
-    c->tile_chosen = rc ? saved_chosen : bc;
+    const bool back = rc || keep_own;   // to what the context had
+    c->tile = back ? saved_tile : bt;
+    c->lz = back ? saved_lz : bl;
+    c->tile_chosen = back ? saved_chosen : true;
     if (!rc) rc = check_cuda(cudaStreamSynchronize(c->stream));
     if (best_tile) *best_tile = bt;
     if (best_lz) *best_lz = bl;

@@ -440,7 +440,8 @@ class Simulation:
 
     def autotune(self, steps=20):
         """Pick the fastest tile/lz for this grid (state is restored); returns
-        (tile, lz, ms_per_step)."""
+        (tile, lz, ms_per_step) of the fastest pair.  A small grid whose own form
+        (the resident step) is faster than every pair stays with it."""
         t, lz, ms = ctypes.c_int(), ctypes.c_int(), ctypes.c_double()
         _check(load().lbm_autotune(self._ctx, int(steps), ctypes.byref(t), ctypes.byref(lz), ctypes.byref(ms)),
                "lbm_autotune")

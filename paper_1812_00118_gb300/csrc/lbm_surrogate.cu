@@ -540,7 +540,8 @@ conv_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restrict__ w,
         const uint32_t acc0 = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
         long long at = (img + (long long)y0 * W + x0 + 32 * (warp & 3) + lane) * csy;
         for (int j = 0; j < nrows; ++j, at += (long long)W * csy) {
-            if (!mbar_wait_phase(mma_done + 8 * (j & 1), j >> 1, &failed)) break;
+            // by warps: tcgen05.ld takes all 32 lanes or hangs
+            if (!__all_sync(0xffffffffu, mbar_wait_phase(mma_done + 8 * (j & 1), j >> 1, &failed))) break;
             copy_next();   // row j + slots, into the slot of input row j, read last by row j
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             for (int c0 = 16 * (warp >> 2); c0 < Co; c0 += 32) {

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdint>
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -679,7 +680,8 @@ static int step_impl(lbm_ctx* c, int n, cudaEvent_t* ev) {
 }
 
 // Two launches, straight into the caller's device arrays; host outputs, and
-// device outputs that overlap one another, go through scratch fields.
+// device outputs that overlap one another or do not start on 8-byte boundaries,
+// go through scratch fields.
 int lbm_macro(lbm_ctx* c, double* phi, double* P, double* rho_u, int on_device) {
     lbm::NvtxRange range("lbm_macro");
     if (!c) return LBM_EINVAL;
@@ -689,7 +691,8 @@ int lbm_macro(lbm_ctx* c, double* phi, double* P, double* rho_u, int on_device) 
     auto apart = [](const double* a, long long na, const double* b, long long nb) {
         return !a || !b || a + na <= b || b + nb <= a;
     };
-    const bool direct = on_device && apart(phi, N, P, N) && apart(phi, N, rho_u, c->dim * N) &&
+    const bool aligned = (((uintptr_t)phi | (uintptr_t)P | (uintptr_t)rho_u) & 7) == 0;
+    const bool direct = on_device && aligned && apart(phi, N, P, N) && apart(phi, N, rho_u, c->dim * N) &&
                         apart(P, N, rho_u, c->dim * N);
     double* d_phi = direct && phi ? phi : f_phi(c);
     double* d_P = direct ? P : (P ? f_P(c) : nullptr);

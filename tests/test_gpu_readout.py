@@ -82,3 +82,22 @@ def test_not_finite_stays_not_finite(lbm):
         assert np.isfinite(np.delete(phi, 100)).all()
         assert phi[100] == bad or (np.isnan(bad) and np.isnan(phi[100]))
         assert sim.diagnostics(raise_on_divergence=False)["nonfinite"] >= 1
+
+
+def test_device_outputs_on_any_address(lbm):
+    """Device outputs that do not start on 8-byte boundaries are copied to, as they
+    were when every output was a copy."""
+    import ctypes
+
+    import torch
+    sim = state(lbm, (33, 17), (0, 1), lbm.F32)
+    host = sim.macro()
+    lib, N = lbm.load(), sim.N
+    for k in range(3):                    # one odd output at a time, then all three
+        offs = [[4, 0, 0], [0, 0, 1], [4, 2, 12]][k]
+        bufs = [torch.zeros(8 * n + 16, dtype=torch.uint8, device="cuda") for n in (N, N, 2 * N)]
+        ptrs = [ctypes.c_void_p(b.data_ptr() + o) for b, o in zip(bufs, offs)]
+        assert lib.lbm_macro(sim.ctx, *ptrs, 1) == lbm.OK
+        for b, o, h in zip(bufs, offs, host):
+            got = np.frombuffer(b.cpu().numpy()[o:o + 8 * h.size].tobytes(), dtype=np.float64)
+            assert np.array_equal(got, h)

@@ -1730,7 +1730,8 @@ static int conv3x3(const void* x, int csx, const void* w, const float* bias, voi
     if (cudaGetSymbolAddress((void**)&err, g_sg_err) != cudaSuccess) return LBM_ECUDA;
     // rows of 128-pixel segments: the row march, when four input rows and the
     // weights of all taps fit in shared memory; else flat tiles, when their
-    // cells and two taps' weights do, else the tap kernel.  us of the U-Net's
+    // cells and two taps' weights do and the image is not too wide, else the tap
+    // kernel.  us of the U-Net's
     // layers at 8 x 256^2, tap kernel / this: 128 -> 32 at 128^2 157 / 28 (march),
     // 64 -> 128 at 64^2 42 / 28, 256 -> 64 at 64^2 101 / 49, 128 -> 128 at 32^2 39 / 18
     // (flat).
@@ -1764,7 +1765,16 @@ static int conv3x3(const void* x, int csx, const void* w, const float* bias, voi
     const long long flat = (long long)H * (W + 2), tiles = (flat + 127) / 128;
     int Cs = Co;   // output channels of a CTA: halved while that still fills no more than the SMs
     while (Cs % 32 == 0 && N * tiles * (Co / Cs) * 2 <= sms) Cs /= 2;
-    const int stages = flat_stages(W, Ci, Cs);
+    // A tile's cells grow with the width (two rows of halo), the tap kernel's nine
+    // copies of 128 pixels do not.  us at 1024 rows, tap kernel / flat tiles: 16 -> 16
+    // at W = 392 58 / 49, 450 65 / 60, 500 71 / 67; 32 -> 16 at 392 99 / 92, 450 92 / 109;
+    // 48 -> 48 at 392 154 / 143, 500 194 / 272, 900 335 / 593; beyond 64 output
+    // channels, where the tap kernel holds one CTA per SM, 64 -> 128 at 560 552 / 442.
+    // Tiles of one wave wait for latency, not for copies: 16 rows of 900, 32 -> 64
+    // 15 / 13, but of 1200 15 / 17.
+    const bool pays = W <= 4096 && (flat_cells(W) <= (Co > 64 ? 1280 : 1024) ||
+                                    (flat_cells(W) <= 2048 && N * tiles * (Co / Cs) <= sms));
+    const int stages = pays ? flat_stages(W, Ci, Cs) : 0;
     if (stages >= 2 && flat < (1LL << 30) && N * tiles < (1LL << 31)) {
         static bool done[64] = {};
         if (large_smem(conv_flat_kernel<ACT>, done, dev) != cudaSuccess) {

@@ -1288,17 +1288,28 @@ relu_grad_kernel(const float* __restrict__ g, int csg, const float* __restrict__
     if (lane == 0 && c < C) *reinterpret_cast<float4*>(part + (long long)blockIdx.x * C + c) = sh[0][quad];
 }
 
+// Sum of v(0) .. v(n - 1) in order, 16 loads in flight; the last group too (loads
+// one after the other, 15 of them, cost 2 to 4 us where n is 63 instead of 64).
+template <typename F>
+__device__ __forceinline__ float ordered_sum(int n, F&& v) {
+    float s = 0.0f;
+    for (int b = 0; b < n; b += 16) {
+        float t[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) t[i] = b + i < n ? v(b + i) : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (b + i < n) s += t[i];
+    }
+    return s;
+}
+
 // out[c] = sum of part[b][c] over the blocks, in block order; channels past C of
 // `pad` are set to zero
 __global__ void channel_finish_kernel(const float* __restrict__ part, int nb, int C, int pad, float* __restrict__ out) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= pad) return;
-    float s = 0.0f;
-    if (c < C) {
-#pragma unroll 16
-        for (int b = 0; b < nb; ++b) s += part[(long long)b * C + c];
-    }
-    out[c] = s;
+    out[c] = c < C ? ordered_sum(nb, [&](int b) { return part[(long long)b * C + c]; }) : 0.0f;
 }
 
 // Loss of out = x + delta against t over four channels, its gradient in FP32 (g4)
@@ -1349,12 +1360,7 @@ __global__ void mse_grad_finish_kernel(const double* __restrict__ part, int nb, 
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) loss[0] = s * inv_count;
     } else if (lane < 16) {
-        float s = 0.0f;
-        if (lane < 4) {
-#pragma unroll 16
-            for (int b = 0; b < ngb; ++b) s += gpart[4 * b + lane];
-        }
-        gb[lane] = s;
+        gb[lane] = lane < 4 ? ordered_sum(ngb, [&](int b) { return gpart[4 * b + lane]; }) : 0.0f;
     }
 }
 
@@ -1902,8 +1908,13 @@ int lbm_sg_bias_grad(const float* g, int csg, float* gb, float* scratch, long lo
     if (!g || !gb || !scratch || npix < 1 || C < 1 || csg < C) return LBM_EINVAL;
     const int nb = sum_blocks(npix);
     cudaStream_t s = (cudaStream_t)stream;
-    if (C % 4 == 0 && csg % 4 == 0 && ((uintptr_t)g & 15) == 0 && ((uintptr_t)scratch & 15) == 0 && npix < (1LL << 30) &&
-        (C + 15) / 16 < 65536) {   // rows in 16-byte groups: the same sums
+    // rows in 16-byte groups, the same sums, from 16 channels on: a block takes 16,
+    // and fewer leave its threads idle (10^6 pixels, one channel per block / this: 4
+    // channels 12.4 / 20.6 us, 8 20.1 / 20.6, 16 35.7 / 22.6).  Below 32 channels it
+    // takes many pixels to pay (16000 pixels of 16: 8.4 / 10.4; 40000: 10.3 either
+    // way; 524288: 22.6 / 16.4).
+    if ((C >= 32 || (C >= 16 && npix > 32768)) && C % 4 == 0 && csg % 4 == 0 && ((uintptr_t)g & 15) == 0 &&
+        ((uintptr_t)scratch & 15) == 0 && npix < (1LL << 30) && (C + 15) / 16 < 65536) {
         relu_grad_kernel<3><<<dim3(nb, (C + 15) / 16), kGradThreads, 0, s>>>(g, csg, nullptr, 0, nullptr, 0, nullptr, 1,
                                                                             (int)npix, C, scratch);
         channel_finish_kernel<<<(C + 31) / 32, 32, 0, s>>>(scratch, nb, C, C, gb);

@@ -179,3 +179,30 @@ def test_conv_paths_exact_on_integers(env, N, H, W, ci, co):
     img, gi = x.double().view(N, H, W, ci), gy.double().view(N * H * W, co)
     want = torch.stack([gi.T @ torch.roll(img, (1 - t // 3, 1 - t % 3), (1, 2)).reshape(-1, ci) for t in range(9)], 1)
     assert torch.equal(gw.double(), want) and lib.lbm_sg_status(s) == 0
+
+
+@pytest.mark.parametrize("npix", [1, 255, 257, 4095, 16 * 1000, 16383, 16384, 65537])
+@pytest.mark.parametrize("C", [4, 12, 16, 20, 128])
+def test_bias_sums_one_order(env, npix, C):
+    """The bias sums are the same bits on every path: rows in 16-byte groups, one
+    channel per block (reached by an address off a 16-byte boundary), and inside
+    lbm_sg_relu_grad and lbm_sg_mse_grad."""
+    torch, lib, s = env
+    g = rnd(torch, npix, C, seed=3)
+    odd = torch.empty(npix * C + 1, device="cuda")[1:].view(npix, C)
+    odd.copy_(g)
+    act = torch.ones(npix, C, device="cuda", dtype=torch.bfloat16)
+    a, b, c = (torch.zeros(C, device="cuda") for _ in range(3))
+    scr, ga = torch.zeros(64 * C, device="cuda"), torch.zeros_like(act)
+    assert lib.lbm_sg_bias_grad(p(g), C, p(a), p(scr), npix, C, s) == 0
+    assert lib.lbm_sg_bias_grad(p(odd), C, p(b), p(scr), npix, C, s) == 0
+    assert lib.lbm_sg_relu_grad(p(g), C, 1, None, 0, p(act), C, p(ga), p(c), p(scr), scr.numel(), 1, 1, npix, C, s) == 0
+    assert torch.equal(a, b) and torch.equal(a, c)
+    if C == 4:
+        x, t, d = rnd(torch, npix, 4), rnd(torch, npix, 4, seed=1), rnd(torch, npix, 16, seed=2)
+        g4, g16 = torch.zeros(npix, 4, device="cuda"), torch.zeros(npix, 16, device="cuda", dtype=torch.bfloat16)
+        e, want = torch.ones(16, device="cuda"), torch.zeros(4, device="cuda")
+        part, loss = (torch.zeros(k, dtype=torch.float64, device="cuda") for k in (1024, 1))
+        assert lib.lbm_sg_mse_grad(p(x), p(d), p(t), p(g16), p(g4), p(e), p(part), p(loss), npix, s) == 0
+        assert lib.lbm_sg_bias_grad(p(g4), 4, p(want), p(scr), npix, 4, s) == 0
+        assert torch.equal(e[:4], want) and (e[4:] == 0).all()

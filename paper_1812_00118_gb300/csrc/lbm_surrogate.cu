@@ -981,12 +981,15 @@ conv_wgrad_row_kernel(const bf16* __restrict__ x, int csx, const bf16* __restric
     if (tid == 0 && failed) atomicExch(err, 1);
 }
 
-// gw[k] = sum over chunks of partial[chunk, k], in chunk order; blocks of one
-// warp and 16 loads in flight (256 threads that waited for each: 18 blocks and
-// 10.3 us for the 4608 values of the 16 -> 32 layer, 5.6 now)
-__global__ void __launch_bounds__(32)
+// gw[k] = sum over chunks of partial[chunk, k], in chunk order, 16 loads in flight.
+// Blocks of one warp while those are few (blocks of 256 threads that waited for
+// each load: 18 blocks and 10.3 us for the 4608 values of the 16 -> 32 layer, 5.6
+// now), of 256 threads from 2^16 values on (9216 blocks of one warp for the
+// 256 -> 128 layer at 8^2: the weight gradient 18.5 us, 14.4 with 1152).
+template <int T>
+__global__ void __launch_bounds__(T)
 sum_chunks_kernel(const float* __restrict__ partial, long long nchunks, long long K, float* __restrict__ gw) {
-    const long long k = (long long)blockIdx.x * 32 + threadIdx.x;
+    const long long k = (long long)blockIdx.x * T + threadIdx.x;
     if (k >= K) return;
     const float* p = partial + k;
     float s = 0.0f;
@@ -1842,6 +1845,11 @@ long long lbm_sg_wgrad_scratch_floats(int N, int H, int W, int Ci, int Co) {
     return need;
 }
 
+static void sum_chunks(const float* partial, long long nchunks, long long K, float* gw, cudaStream_t s) {
+    if (K < (1 << 16)) sum_chunks_kernel<32><<<(unsigned)((K + 31) / 32), 32, 0, s>>>(partial, nchunks, K, gw);
+    else sum_chunks_kernel<256><<<(unsigned)((K + 255) / 256), 256, 0, s>>>(partial, nchunks, K, gw);
+}
+
 int lbm_sg_conv3x3_wgrad(const void* x, int csx, const void* gy, int csg, float* gw, float* scratch,
                          long long scratch_floats, int N, int H, int W, int Ci, int Co, void* stream) {
     const long long M = (long long)N * H * W;
@@ -1878,7 +1886,7 @@ int lbm_sg_conv3x3_wgrad(const void* x, int csx, const void* gy, int csg, float*
         conv_wgrad_row_kernel<<<(unsigned)ctas, kRoleThreads, need > least ? need : least, s>>>(
             (const bf16*)x, csx, (const bf16*)gy, csg, scratch, N, H, W, Ci, Co, P, Cn, rows, bufs, err);
         const long long K = (long long)Co * 9 * Ci;
-        sum_chunks_kernel<<<(unsigned)((K + 31) / 32), 32, 0, s>>>(scratch, pchunks, K, gw);
+        sum_chunks(scratch, pchunks, K, gw, s);
         return check(cudaGetLastError());
     }
     const long long nchunks = (M + kChunk - 1) / kChunk;
@@ -1887,7 +1895,7 @@ int lbm_sg_conv3x3_wgrad(const void* x, int csx, const void* gy, int csg, float*
     conv_wgrad_kernel<<<(unsigned)((warps * 32 + 127) / 128), 128, 0, s>>>((const bf16*)x, csx, (const bf16*)gy, csg,
                                                                           scratch, M, H, W, Ci, Co);
     const long long K = (long long)Co * 9 * Ci;
-    sum_chunks_kernel<<<(unsigned)((K + 31) / 32), 32, 0, s>>>(scratch, nchunks, K, gw);
+    sum_chunks(scratch, nchunks, K, gw, s);
     return check(cudaGetLastError());
 }
 

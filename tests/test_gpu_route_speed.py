@@ -45,6 +45,19 @@ def test_bias_sums_of_few_channels(env):
     assert t[0] < 0.85 * t[1], t
 
 
+def test_many_weights_of_few_pixels(env):
+    """The weight gradient of 8 x 8 pixels: 256 -> 128 channels against 64 -> 128
+    (measured 1.2; 1.5 with sums in blocks of one warp)."""
+    torch, lib, s = env
+    t = []
+    for ci, co in ((64, 128), (256, 128)):
+        x, gy = (torch.randn(64, c, device="cuda").bfloat16() for c in (ci, co))
+        n = lib.lbm_sg_wgrad_scratch_floats(1, 8, 8, ci, co)
+        gw, scr = torch.empty(co, 9, ci, device="cuda"), torch.empty(n, device="cuda")
+        t.append(us(torch, lambda: lib.lbm_sg_conv3x3_wgrad(p(x), ci, p(gy), co, p(gw), p(scr), n, 1, 8, 8, ci, co, s)))
+    assert t[1] < 1.35 * t[0] + 1, t
+
+
 def test_wide_images(env):
     """A convolution of 1000 x 1000 takes the time per pixel of 1024 x 392 within 1.4
     (measured 1.0; 1.9 where the wide image went to flat tiles)."""

@@ -272,7 +272,9 @@ int lbm_set_wall_velocity(lbm_ctx* ctx, int axis, int side, const double u[3]);
  * 2^24 nodes or more; lbm_get_tile reports the current choice and its CTA
  * shape.  Until lbm_set_tile or lbm_autotune chooses, lz is an upper limit
  * (a grid that would leave the chip idle is cut into shorter chunks) and
- * small grids step in the resident form (see lbm_step).
+ * small grids step in the resident form (see lbm_step).  A choice holds for the
+ * context's life, and the pair lbm_get_tile reports is one too: set, it is the
+ * tile in chunks of exactly lz planes.
  * Errors: LBM_EINVAL for an unknown tile or lz < 1, LBM_ENOTSUP for a
  * bulk-copy or asynchronous-copy tile this grid, layout or storage type
  * cannot use. */

@@ -19,6 +19,10 @@
  *     are multiples of 16 (zero-pad), Co <= 128, N H W a multiple of 16.
  *   - Pooling and upsampling are by a factor f (1..64) in both directions;
  *     H and W (always the FINE grid's size) are multiples of f.
+ *   - The network's passes (paper_1812_00118_gb300/surrogate.py) run on the
+ *     fused calls; lbm_sg_relu, lbm_sg_relu_bwd, lbm_sg_pool_bwd,
+ *     lbm_sg_upsample_bwd, lbm_sg_mse and lbm_sg_adam are the single steps
+ *     these stand for, for other networks and as their reference in the tests.
  *   - The caller owns every buffer; the functions allocate nothing.  All are
  *     asynchronous on `stream` (NULL: default stream).
  *   - Return LBM_OK, LBM_EINVAL (NULL pointer, bad size or stride),
@@ -35,11 +39,13 @@ extern "C" {
  * (float[Co], may be NULL): an implicit GEMM on the tcgen05 tensor cores,
  * bf16 products, FP32 sums in tensor memory, 128 pixels per MMA.  When W is a
  * multiple of 128 and the weights of all nine taps fit in shared memory with
- * four input rows (9 Co Ci + 4 x 130 Ci bf16 values, at most 200 KB), a CTA
+ * four input rows (9 Co Ci + 4 x 130 Ci bf16 values, at most 220 KB), a CTA
  * marches a 128-pixel row segment down a chunk of rows, copying every input
- * row into shared memory once; otherwise a CTA takes 128 consecutive pixels
- * and copies each tap's shifted rows.  Both accumulate the taps in the same
- * order.  x's channel stride csx is a multiple of 8 and x and w start
+ * row into shared memory once; otherwise a CTA takes 128 consecutive positions
+ * of the image (a halo column on each side) and copies the cells they read
+ * once, or, where those are too many (wide images, many channels), 128
+ * consecutive pixels and each tap's shifted rows.  All accumulate the taps in
+ * the same order.  x's channel stride csx is a multiple of 8 and x and w start
  * on 16-byte boundaries (the operands are staged in 16-byte copies);
  * LBM_EINVAL otherwise.  A bounded wait inside the kernel that gives up leaves
  * its CTA's part of y unwritten and is reported by lbm_sg_status. */

@@ -193,8 +193,8 @@ __global__ void diag_partial_kernel(const double* __restrict__ phi, const double
     }
 }
 
-// sum / max of nb partial rows of width `width` <= 32 (columns in max_mask use
-// max): one warp per column, fixed order.  An addition takes 65 clk here, so a
+// sum / max of nb partial rows of `width` columns (those in max_mask use max) by
+// one block of 32 threads per column: one warp each, fixed order.  An addition takes 65 clk here, so a
 // chain of 1024 took 32 us in every initialisation and diagnostic.
 __global__ void finish_kernel(const double* __restrict__ part, int nb, int width, int max_mask, double* out) {
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -7,8 +7,8 @@
 // the grid is cut into boxes of BX x BY x BZ nodes, one thread per node and
 // one CTA per box, all boxes resident at once: a step is one round of loads,
 // one barrier, one collision and one round of stores.  (us per step, march of
-// 16-plane chunks / this: 64^2 FP64 239 / 13.8, 256^2 FP32 22.7 / 4.3, 150 x 600 with
-// walls 28.8 / 5.9, 32^3 45 / 6.5.  At 64^2 FP32 the 3.1 are, in clk: the wait for
+// 16-plane chunks / this: 64^2 FP64 190 / 13.5, 256^2 FP32 22.7 / 4.3, 150 x 600 with
+// walls 28.8 / 6.0, 32^3 45 / 6.5.  At 64^2 FP32 the 3.1 are, in clk: the wait for
 // the flags 640, loads and sums 1600, collision 830, release 1000.)
 //
 // Between steps a box waits only for the boxes around it.  A node's new

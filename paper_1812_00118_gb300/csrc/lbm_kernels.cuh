@@ -791,7 +791,8 @@ __device__ __forceinline__ void collide_pair(const NodeState<float>& s, const Pa
 // error (h of O(0.1): rms 7.5e-18 against 5.5e-18; this form 4.8e-18).
 // FP64 runs at two lanes per clock and SM here, so the FP64 step's time is its
 // operation count (64^2 D2Q9: 433 FP64 instructions per node in the
-// collision before; march of 256^2 267 us per step before, 211 with this).
+// collision before; march of 256^2 in 16-plane chunks 267 us per step before, 209
+// with this).
 struct PairState64 {
     double Ze, k1, Fx, Fy, Fz;               // Xe + Ye; rho_dif/2 + 3 mu/2; 3 F / 2
     double m15, usq15;                       // 3 mu/2, 1.5 u.u

@@ -10,12 +10,14 @@
 // 16 (zero-padded by the caller), pixel counts multiples of 16.
 //
 // The forward (and input-gradient) convolution runs on the tcgen05 tensor
-// cores with the accumulator in tensor memory (conv_row_kernel for images
-// whose width is a multiple of 128, conv_tc_kernel otherwise); so does the
-// weight gradient, a GEMM over pixels, for widths that are multiples of 32
-// (conv_wgrad_row_kernel), with the warp-level mma.sync m16n8k16 BF16 kernel
-// (fragments gathered straight from the channels-last tensors) for the
-// rest.  All are implicit GEMMs without an im2col buffer.
+// cores with the accumulator in tensor memory: conv_row_kernel for images
+// whose width is a multiple of 128 and whose ring of rows and weights fit
+// shared memory, else conv_flat_kernel where its cells and two taps' weights
+// fit and the image is not too wide, else conv_tc_kernel (conv3x3 below has the
+// rule).  So does the weight gradient, a GEMM over pixels, for widths that are
+// multiples of 32 (conv_wgrad_row_kernel), with the warp-level mma.sync
+// m16n8k16 BF16 kernel (fragments gathered straight from the channels-last
+// tensors) for the rest.  All are implicit GEMMs without an im2col buffer.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -71,7 +73,7 @@ __device__ __forceinline__ long long shift_pixel(long long p, int H, int W, int 
 // core: 8 x 16-byte core matrices, rows 16 bytes apart, 8-row groups 128
 // bytes apart (stride byte offset), the 8-channel chunks one after another
 // (leading byte offset = rows x 16 bytes).  The copies run two stages ahead
-// of the MMAs: once a stage's copies have landed, thread 0 issues its MMAs
+// of the MMAs: once a stage's copies have landed, warp 0 issues its MMAs
 // and commits them to the buffer's mbarrier, and a buffer is refilled only
 // after its mbarrier shows the MMAs that read it done.  The epilogue reads
 // the accumulator back with tcgen05.ld (warp w reads lanes 32w..32w+31, one
@@ -433,8 +435,9 @@ __device__ int g_sg_err;   // a bounded wait of a surrogate kernel gave up
 // as soon as the last row that reads it is done) and write out one of two
 // tensor-memory accumulators while the other is summed; a warp of its own
 // issues the MMAs.  (On 128 threads that wrote out row j - 1 and copied row
-// j + 1 before issuing row j the 64 -> 32 layer at 8 x 256^2 took 126 us; this
-// takes 42.)  Every wait is bounded, as in the tap kernel.
+// j + 1 before issuing row j the 64 -> 32 layer at 8 x 256^2 took 126 us with its
+// FP32 output; this takes 52 to 54, and 43 with the ReLU in the epilogue and bf16
+// out.)  Every wait is bounded, as in the tap kernel.
 constexpr int kRowM = 128;          // pixels of a row segment (MMA M)
 constexpr int kRowHalo = kRowM + 2;
 constexpr int kRowSlots = 6;        // ring rows at most (at least 4)
@@ -1710,10 +1713,6 @@ cudaError_t wgrad_row_plan(int N, int H, int W, int Ci, int Co, int* rows, int* 
 bool conv_dims_ok(long long M, int Ci, int Co) { return M > 0 && M % 16 == 0 && Ci > 0 && Ci % 16 == 0 && Co > 0 && Co % 16 == 0; }
 
 }  // namespace
-
-extern "C" {
-
-}  // extern "C"
 
 template <bool ACT>
 static int conv3x3(const void* x, int csx, const void* w, const float* bias, void* y, int csy, int N, int H, int W,

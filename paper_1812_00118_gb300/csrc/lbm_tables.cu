@@ -46,12 +46,14 @@ namespace {
 
 // Boxes of the resident step (lbm_box.cuh): nodes along the internal axes and
 // the CTAs per SM the registers are bounded for; the larger box first.
-// Measured, us per step of a periodic grid (FP32, 100 steps per launch, boxes
-// that release their stores by one thread):
-//   D2Q9   32x8 / 32x4: 64^2 3.8 / 3.1, 128^2 4.0 / 3.3, 256^2 4.9 / 4.8, 512^2 11.5 / 15.4
-//   D3Q19  16x4x4 / 8x4x4: 16^3 6.6 / 5.9, 24^3 6.9 / 6.0, 32^3 6.4 / 7.0, 40^3 9.8 / 11.1
-// so the larger box pays once it gives at least half the SMs a box (D3Q19) or
-// every SM one (D2Q9).  At 64 registers (4 CTAs of 256) the D2Q9 box spills
+// Measured, us per step of a periodic grid (FP32, 100 steps per launch):
+//   D2Q9   32x8 / 32x4: 64^2 3.5 / 3.2, 128^2 3.6 / 3.2, 256^2 4.3 / 4.1, 512^2 (two
+//          boxes per CTA) 11.6 / does not fit
+//   D3Q19  16x4x4 / 8x4x4: 16^3 6.7 / 5.8, 24^3 7.3 / 6.0, 32^3 6.5 / 6.8, 36^3 9.0 / 8.1,
+//          40^3 8.9 / 8.4
+// so the smaller box is the faster one by up to 20 % on few SMs and within 5 %
+// either way beyond, and the larger one fits more of a grid: it is taken from
+// half a box per SM on (D3Q19) or one (D2Q9).  At 64 registers (4 CTAs of 256) the D2Q9 box spills
 // nothing; D3Q19 needs 128.
 #if LBM_LAT == 1
 using BoxA = Box<16, 4, 4, 2>;
@@ -62,7 +64,7 @@ constexpr int kBoxRounds = 1;     // boxes of one CTA per step at most
 // FP64 (D2Q9) is bound by the FP64 pipe, whose 65 clk per warp instruction do
 // not shrink with fewer active lanes: boxes of one warp spread evenly over the
 // SMs, a larger box only where those no longer fit the chip.  us per step,
-// 8x4 / 32x4: 64^2 14.0 / 14.8, 128^2 16.0 / 14.9, 256^2 50.5 / 52.9
+// 8x4 / 32x4: 64^2 13.5 / 14.3, 128^2 14.7 / 14.5, 256^2 44.2 / 54.3
 using BoxA = Box<32, 1, 4, 4>;
 using BoxB = Box<8, 1, 4, 16>;
 constexpr int kBoxAHalves = 1 << 20;
@@ -124,9 +126,11 @@ bool ok_dispatch(int tile, const Geom& G) {
 
 // How a grid is cut into boxes; plan->variant stays -1 where the march is the
 // faster form.  The march of as many CTAs as the chip holds (StepArgs::fit)
-// overtakes once the boxes need more than one round per step (D3Q19: 40^3 9.8
-// against 14.4 us, 48^3 16.4 against 14.5) or two (D2Q9: 512^2 11.5 against
-// 12.4, 707^2 23.2 against 18.8; FP64, one round: 512^2 210 against 171).
+// overtakes once the boxes need more than one round per step (D3Q19: 40^3 8.9
+// against 14.3 us, 44^3 17.3 against 14.7) or two (D2Q9: 512^2 11.6 against
+// 12.3, in three rounds 600^2 17.8 against 15.2; at the small end of two rounds
+// the march is ahead, 400^2 11.8 against 10.4; FP64, one round: 256^2 44.2
+// against 54.8, in two 320^2 94.2 against 86.1).
 cudaError_t box_plan(const Geom& G, BoxPlan* plan) {
     *plan = BoxPlan();
     int dev = 0, sms = 0, slots = 0;

@@ -103,6 +103,11 @@ unsigned* box_flags(lbm_ctx* c) { return (unsigned*)(c->partial + 4 * 1024 + 8);
 bool resident(const lbm_ctx* c) {
     return c->box.variant >= 0 && c->box.boxes <= kMaxBoxes && c->partial && !c->owner;
 }
+NewState new_state(lbm_ctx* c) {
+    const bool r = resident(c);
+    return {c->d_err, r ? box_flags(c) : nullptr, r ? c->box.boxes : 0, kBoxFirstCount};
+}
+// the counts in scratch just allocated
 int start_box_counts(lbm_ctx* c) {
     if (!resident(c)) return LBM_OK;
     box_start_kernel<<<(c->box.boxes + 255) / 256, 256, 0, c->stream>>>(box_flags(c), c->box.boxes);
@@ -300,13 +305,6 @@ int phi_fix(lbm_ctx* c) {
 int copy_field(lbm_ctx* c, double* dst, const double* src, size_t n, int on_device) {
     return check_cuda(cudaMemcpyAsync(dst, src, n * sizeof(double),
                                       on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
-}
-
-// A new state: the error flag of the bounded waits, and the box counts a wait
-// that gave up left uneven.
-int clear_wait_state(lbm_ctx* c) {
-    if (check_cuda(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream))) return LBM_ECUDA;
-    return start_box_counts(c);
 }
 
 // rho_bar for force_mode 1 from the current state's phi (scratch fields must be fresh)
@@ -560,11 +558,10 @@ int lbm_init_fields_ex(lbm_ctx* c, const double* phi, const double* u, const dou
     // the buffer all its grids hold the state in)
     const int b = c->cur;
     if (check_cuda(c->K->init(c->h[b], c->g[b], c->G, c->P, f_phi(c), f_u(c, 0), f_u(c, 1), f_u(c, 2), f_P(c),
-                              (flags & LBM_INIT_NONEQ) ? 1 : 0, c->stream)))
+                              (flags & LBM_INIT_NONEQ) ? 1 : 0, new_state(c), c->stream)))
         return LBM_ECUDA;
     c->ghosts[b] = true;   // the initialisation writes the periodic images too
     c->diverged = false;
-    if (clear_wait_state(c)) return LBM_ECUDA;
     c->launches += 1;
     return check_cuda(cudaStreamSynchronize(c->stream));
 }
@@ -773,10 +770,9 @@ int lbm_set_populations(lbm_ctx* c, const double* h, const double* g, int on_dev
         dh = th; dg = tg;
     }
     const int b = c->cur;
-    int rc = check_cuda(c->K->set(c->h[b], c->g[b], c->G, c->P, dh, dg, c->stream));
+    int rc = check_cuda(c->K->set(c->h[b], c->g[b], c->G, c->P, dh, dg, new_state(c), c->stream));
     c->ghosts[b] = true;
     c->diverged = false;
-    if (!rc) rc = clear_wait_state(c);
     c->launches += 1;
     if (th) { cudaFreeAsync(th, c->stream); cudaFreeAsync(tg, c->stream); }
     if (!rc) {

@@ -248,8 +248,7 @@ box_kernel(const __grid_constant__ BoxPtrs<typename Storage<ST>::S, Lattice<LAT>
     }
 }
 
-// Counts of a new state (and of one whose last launch a wait ended early, which
-// leaves them uneven).
+// Counts in memory just allocated (those of a new state: NewState).
 static __global__ void box_start_kernel(unsigned* flags, int boxes) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < boxes) flags[k] = kBoxFirstCount;

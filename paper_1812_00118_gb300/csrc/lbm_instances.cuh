@@ -321,10 +321,10 @@ struct Launchers {
     }
     static cudaError_t init(void* hout, void* gout, const Geom& G, const Phys& p, const double* phi,
                             const double* ux, const double* uy, const double* uz, const double* P, int neq,
-                            cudaStream_t s) {
+                            const NewState& st, cudaStream_t s) {
         init_kernel<LAT, ST><<<blocks_for(G.N, 256), 256, 0, s>>>(
             dir_ptrs<S, Q>(hout, gout, hout, gout, G.NP), G, phys_as<typename Storage<ST>::R>(p), phi, ux, uy, uz, P,
-            neq);
+            neq, st);
         return cudaGetLastError();
     }
     static cudaError_t get(const void* hin, const void* gin, const Geom& G, const Phys& p, double* h, double* g,
@@ -347,9 +347,9 @@ struct Launchers {
         return cudaGetLastError();
     }
     static cudaError_t set(void* hout, void* gout, const Geom& G, const Phys& p, const double* h,
-                           const double* g, cudaStream_t s) {
+                           const double* g, const NewState& st, cudaStream_t s) {
         set_kernel<LAT, ST><<<blocks_for(G.N, 256), 256, 0, s>>>(
-            dir_ptrs<S, Q>(hout, gout, hout, gout, G.NP), G, p, h, g);
+            dir_ptrs<S, Q>(hout, gout, hout, gout, G.NP), G, p, h, g, st);
         return cudaGetLastError();
     }
 };

@@ -79,11 +79,11 @@ struct KernelTable {
                             double* P, double* rux, double* ruy, double* ruz, cudaStream_t s);
     cudaError_t (*init)(void* hout, void* gout, const Geom& G, const Phys& p, const double* phi,
                         const double* ux, const double* uy, const double* uz, const double* P, int neq,
-                        cudaStream_t s);
+                        const NewState& st, cudaStream_t s);
     cudaError_t (*get)(const void* hin, const void* gin, const Geom& G, const Phys& p, double* h,
                        double* g, const int* lost, cudaStream_t s);
     cudaError_t (*set)(void* hout, void* gout, const Geom& G, const Phys& p, const double* h,
-                       const double* g, cudaStream_t s);
+                       const double* g, const NewState& st, cudaStream_t s);
     // periodic images of the ghost band of a freshly written buffer pair
     cudaError_t (*halo)(void* hout, void* gout, const Geom& G, cudaStream_t s);
     // h_0 += *delta (device double) at every node of buffer h

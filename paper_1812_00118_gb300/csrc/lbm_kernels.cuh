@@ -1622,6 +1622,21 @@ __device__ __forceinline__ void store_cell(S* __restrict__ arr, const Geom& G, i
     else arr[pidx(G, x, y, z)] = v;
 }
 
+// What the kernels that write a new state clear with it: the error flag of the
+// bounded waits and the box counts of the resident step (none: boxes 0; no more
+// boxes than nodes), which a wait that gave up leaves uneven.  (As a memset each
+// they added 2 to 3 us to an initialisation of 65 to 130.)
+struct NewState {
+    int* err;
+    unsigned* counts;
+    int boxes;
+    unsigned first;
+    __device__ __forceinline__ void clear(long long n) const {
+        if (n == 0) *err = 0;
+        if (n < boxes) counts[n] = first;
+    }
+};
+
 // Equilibrium initialisation (h = h^eq, g = g^eq of the given fields),
 // written where the next pull reads it, in the kernels' arithmetic type R
 // (FP32 for FP32 and 16-bit storage, FP64 for FP64 storage): the stored
@@ -1634,12 +1649,13 @@ template <int LAT, int ST>
 __global__ void init_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::Q> D, Geom G,
                             PhysT<typename Storage<ST>::R> p, const double* __restrict__ phi,
                             const double* __restrict__ ux, const double* __restrict__ uy,
-                            const double* __restrict__ uz, const double* __restrict__ P, int neq) {
+                            const double* __restrict__ uz, const double* __restrict__ P, int neq, NewState st) {
     using L = Lattice<LAT>;
     using St = Storage<ST>;
     using R = typename St::R;
     const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (n >= G.N) return;
+    st.clear(n);
     int x, y, z;
     node_coords(G, n, &x, &y, &z);
     NodeState<R> s;
@@ -1731,12 +1747,13 @@ __global__ void get_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::
 
 template <int LAT, int ST>
 __global__ void set_kernel(const DirPtrs<typename Storage<ST>::S, Lattice<LAT>::Q> D, Geom G, Phys p,
-                           const double* __restrict__ h, const double* __restrict__ g) {
+                           const double* __restrict__ h, const double* __restrict__ g, NewState st) {
     using L = Lattice<LAT>;
     using St = Storage<ST>;
     using R = typename St::R;
     const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (n >= G.N) return;
+    st.clear(n);
     int x, y, z;
     node_coords(G, n, &x, &y, &z);
     Unroll<0, L::Q>::run([&](auto ic) {
